@@ -142,17 +142,24 @@ def lib() -> ctypes.CDLL:
 
 
 def _ptr(t) -> Optional[int]:
-    if t is None:
-        return None
-    if isinstance(t, int):
+    if t is None or isinstance(t, int):
         return t
     return t.data_ptr()
 
 
+_raw_stream = _device_index = None
+
+
 def _stream(stream) -> Optional[int]:
+    """The stream's handle; None is the current stream of the current device. The two raw getters take 0.1 us where building a
+    torch.cuda.Stream object takes 3 us, a third of what a whole call of this binding used to cost the host."""
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        global _raw_stream, _device_index
+        if _raw_stream is None:
+            import torch
+            torch.cuda.init()
+            _raw_stream, _device_index = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+        return _raw_stream(_device_index())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
@@ -214,7 +221,7 @@ def pt_conv_workspace_bytes(ctx: Context, d: pt_conv_desc, which: int) -> int:
 
 
 def _ws(ws):
-    return (None, 0) if ws is None else (ws.data_ptr(), ws.numel() * ws.element_size())
+    return (None, 0) if ws is None else (ws.data_ptr(), ws.nbytes)
 
 
 def pt_conv_fwd(ctx, d, x, w, y, ws=None, stream=None):
