@@ -122,3 +122,28 @@ def test_bad_arguments_and_indices():
     with pytest.raises(B.PtError):
         c.poll()
     c.poll()                                                          # the status word was cleared
+
+
+# (npix, source channels, selected): one and several column blocks of the staged form (pitch 768 is one block of 384 pairs), a partial
+# last chunk, fewer pixels than SMs, and a source row too long for shared memory, which takes the direct form
+@pytest.mark.parametrize("npix,c_src,n_sel", [(5, 768, 768), (301, 776, 769), (149, 4096, 4096), (2000, 9, 8), (7, 12296, 300)])
+def test_gather_and_scatter_add_at_the_edges_of_the_staged_form(npix, c_src, n_sel):
+    g = np.random.default_rng(npix)
+    idx = g.permutation(c_src)[:n_sel].astype(np.int32)
+    d_idx = torch.from_numpy(idx).cuda()
+    ld, ld_s = W.pad8(c_src), W.pad8(n_sel)
+    gen = torch.Generator().manual_seed(npix)
+    node, branch = (W.bf16_round(torch.randn((npix, k), generator=gen)).numpy() for k in (c_src, n_sel))
+    c = Hh.ctx()
+    out = torch.full((npix, ld_s), float("nan"), dtype=torch.bfloat16, device="cuda")
+    B.pt_channel_gather(c, _dev_act(node, ld), ld, c_src, d_idx, n_sel, out, ld_s, npix)
+    torch.cuda.synchronize()
+    got = out.float().cpu().numpy()
+    assert np.array_equal(got[:, :n_sel], oracle.channel_gather(node, idx)) and np.all(got[:, n_sel:] == 0)
+    if ld <= 4096:
+        res = torch.full((npix, ld), float("nan"), dtype=torch.bfloat16, device="cuda")
+        B.pt_channel_scatter_add(c, _dev_act(branch, ld_s), ld_s, d_idx, n_sel, _dev_act(node, ld), res, ld, c_src, npix, True)
+        torch.cuda.synchronize()
+        got = res.float().cpu().numpy()
+        assert np.array_equal(got[:, :c_src], oracle.channel_scatter_add(branch, idx, node, relu=True)) and np.all(got[:, c_src:] == 0)
+    c.poll()
