@@ -84,8 +84,8 @@ struct GemmP {
     int test_skip;      // test hook (pt_test_skip_next_arrive): the A producer leaves out the first stage of its first tile
     int stats_off;      // byte offset in shared memory of the epilogue warps' statistics accumulators (stats != nullptr)
     int stats_warp;     // bytes of one warp's accumulators: 512 per 64-channel chunk of the tile
-    float *stats;       // optional: per (pixel tile, warp quarter) and output channel, sum and sum of squares of the bf16 values
-                        // stored, as [part][2][ld_out] floats (the batch-normalisation statistics of the layer that follows)
+    float *stats;       // optional: rows [2][ld_out] of floats, one per n_tiles CTAs: per output channel, sum and sum of squares of
+                        // the bf16 values they stored (the batch-normalisation statistics of the layer that follows)
     void *out;
     unsigned int *status;
     unsigned char tap_oh[kMaxTaps], tap_ow[kMaxTaps];   // im2col offsets of each visited tap
@@ -119,8 +119,8 @@ constexpr uint32_t kSlabs = 2;                          // staging slabs per epi
 // Batch-normalisation statistics of a staged output chunk: `rows` is a bit mask of the warp's 32 staged rows (128 bytes each,
 // 128-byte swizzle, first row `row0` of the slab) that are real output pixels. Lane l owns channels 2l and 2l + 1 of the
 // 64-channel chunk and adds the bf16 values exactly as they were stored, rows in ascending order: sum and sum of squares,
-// accumulated in the warp's own shared-memory slots (acc: 128 floats per chunk of the tile, four per lane) and written to the
-// warp's row of partial sums by stats_flush. Feature normalisation (Sec. 2.1) reads its input twice; taking the sums here,
+// accumulated in the warp's own shared-memory slots (acc: 128 floats per chunk of the tile, four per lane); stats_store_cta
+// combines the warps of a CTA at the end. Feature normalisation (Sec. 2.1) reads its input twice; taking the sums here,
 // from the tile that is still in shared memory, removes the first of the two passes.
 constexpr uint32_t kStatsChunkBytes = 128u * 4u;              // per 64-channel chunk: 32 lanes x (sum, sum of squares) x two channels
 
@@ -162,32 +162,29 @@ __device__ __forceinline__ void stats_clear(uint32_t acc0, int lane, int n_chunk
             asm volatile("st.shared.v4.f32 [%0], {%1, %1, %1, %1};" ::"r"(acc0 + (uint32_t)ch * 512u + (uint32_t)lane * 16u), "f"(0.f) : "memory");
 }
 
-// Adds the warp's shared-memory sums of the channels n0 .. n0 + 64 * n_chunks into its row of partial sums (zeroed by the warp
-// at kernel start; a column is always this lane's: read, add, write) and clears them.
-__device__ __forceinline__ void stats_flush(uint32_t acc0, int lane, float *dst, int ld, int n0, int n_chunks, int n_cols, bool add)
+// The sums of a CTA's epilogue warps (accumulators of `stride` bytes each, from `acc0` on) are added in the order of the warps and
+// leave for a row of partial sums, [2][ld] floats. A CTA's tiles all have the same output channels n0 .. (its grid is a multiple of
+// the number of channel tiles), so that it writes once, and the CTAs of a row, one per channel tile, write disjoint columns; the
+// last one also writes the zeros up to ld. `tid` of `nthr` epilogue threads; a barrier of theirs comes before the call. (One row
+// per epilogue warp made up to 1776 rows, a few megabytes, for the normalisation to add up.)
+__device__ __forceinline__ void stats_store_cta(uint32_t acc0, uint32_t stride, int n_warps, int tid, int nthr, float *dst, int ld, int n_cols,
+                                                int n0, int n_end)
 {
-    float4 t[4];
-    float o[4][4];
-#pragma unroll
-    for (int ch = 0; ch < 4; ++ch) {
-        if (ch >= n_chunks) break;
-        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(t[ch].x), "=f"(t[ch].y), "=f"(t[ch].z), "=f"(t[ch].w)
-                     : "r"(acc0 + (uint32_t)ch * 512u + (uint32_t)lane * 16u) : "memory");
-        const int c = n0 + ch * 64 + 2 * lane;
-        // (a warp that visits its columns once, at the very end, has nothing to add to: the row still holds its zeros)
-        o[ch][0] = (add && c < n_cols) ? dst[c] : 0.f;
-        o[ch][1] = (add && c < n_cols) ? dst[ld + c] : 0.f;
-        o[ch][2] = (add && c + 1 < n_cols) ? dst[c + 1] : 0.f;
-        o[ch][3] = (add && c + 1 < n_cols) ? dst[ld + c + 1] : 0.f;
+    for (int c = n0 + tid; c < n_end; c += nthr) {
+        float s0 = 0.f, s1 = 0.f;
+        if (c < n_cols) {
+            // a chunk is 64 channels: lane (c % 64) / 2 keeps (sum, sum of squares) of its two channels
+            const int e = c - n0;
+            const uint32_t a = acc0 + (uint32_t)(e >> 6) * 512u + (uint32_t)((e & 63) >> 1) * 16u + (uint32_t)(e & 1) * 8u;
+            for (int w = 0; w < n_warps; ++w) {
+                float u0, u1;
+                asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(u0), "=f"(u1) : "r"(a + (uint32_t)w * stride) : "memory");
+                s0 += u0; s1 += u1;
+            }
+        }
+        dst[c] = s0;
+        dst[ld + c] = s1;
     }
-#pragma unroll
-    for (int ch = 0; ch < 4; ++ch) {
-        if (ch >= n_chunks) break;
-        const int c = n0 + ch * 64 + 2 * lane;
-        if (c < n_cols) { dst[c] = o[ch][0] + t[ch].x; dst[ld + c] = o[ch][1] + t[ch].y; }
-        if (c + 1 < n_cols) { dst[c + 1] = o[ch][2] + t[ch].z; dst[ld + c + 1] = o[ch][3] + t[ch].w; }
-    }
-    stats_clear(acc0, lane, n_chunks);
 }
 
 // Device-side timeline of CTA 0 (a build with -DPT_DEVICE_TRACE; read back with pt_debug_gemm_trace): per pipeline stage in
@@ -416,11 +413,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) conv_gemm_kernel(const __grid
         // i.e. the tiles tc = g, g + G, g + 2G, ... of this CTA
         const int quarter = warp & 3, group = (warp - 2) >> 2, G = p.epi_groups;
         const uint32_t slab0 = (p.alias_staging ? data_base : staging_base) + (uint32_t)(warp - 2) * (kSlabs * 4096u);
-        // statistics: one row of partial sums per epilogue warp of the grid, [2][ld_out] floats, accumulated over the warp's tiles
-        float *my_stats = (STATS && p.stats) ? p.stats + ((size_t)blockIdx.x * (4 * G) + (warp - 2)) * 2 * p.ld_out : nullptr;
+        // statistics: accumulated over the warp's tiles in shared memory, combined at the end
         const uint32_t st_acc = smem_base + (uint32_t)p.stats_off + (uint32_t)(warp - 2) * (uint32_t)p.stats_warp;
-        if (my_stats) {
-            for (int e = lane; e < 2 * p.ld_out; e += 32) my_stats[e] = 0.f;
+        if (STATS && p.stats) {
             stats_clear(st_acc, lane, (p.BN + 63) / 64);
             __syncwarp();
         }
@@ -527,8 +522,6 @@ __global__ void __launch_bounds__(kGemmThreads, 1) conv_gemm_kernel(const __grid
                         chunk_stats(slab, 0, rows, lane, st_acc + (uint32_t)ch * 512u);
                     }
                 }
-                // several channel tiles: the sums of this tile's columns leave shared memory now; one tile: after the last tile
-                if (my_stats && p.n_tiles > 1) stats_flush(st_acc, lane, my_stats, p.ld_out, n0, n_chunks, p.n_cols, true);
                 if (quarter == 0) GTRACE(7, tc);
                 continue;
             }
@@ -577,7 +570,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1) conv_gemm_kernel(const __grid
                 }
             }
         }
-        if (my_stats && p.n_tiles == 1) stats_flush(st_acc, lane, my_stats, p.ld_out, 0, (p.BN + 63) / 64, p.n_cols, false);
+        if (STATS && p.stats) {
+            named_barrier(1, 128 * G);
+            const int nt = (int)blockIdx.x % p.n_tiles;
+            stats_store_cta(smem_base + (uint32_t)p.stats_off, (uint32_t)p.stats_warp, 4 * G, (int)threadIdx.x - 64, 128 * G,
+                            p.stats + (size_t)(blockIdx.x / p.n_tiles) * 2 * p.ld_out, p.ld_out, p.n_cols, nt * p.BN,
+                            nt + 1 < p.n_tiles ? (nt + 1) * p.BN : p.ld_out);
+        }
         if (p.tma_store && lane == 0) tma_store_wait_read();     // the staging slabs must outlive the stores' reads
         if (warp == 2) CTRACE(6);
         tc_fence_before();
@@ -614,7 +613,7 @@ struct HaloP {
     int oH, oW, o_step, o_h0, o_w0;      // direct stores: raster (n, i, j) -> out[((n*oH + i*o_step + o_h0)*oW + j*o_step + o_w0)*ld_out]
     int stats_off;                       // byte offset in shared memory of the epilogue warps' statistics accumulators
     int stats_warp;                      // bytes of one warp's accumulators: 512 per 64-channel chunk of the tile
-    float *stats;                        // optional: per epilogue warp and channel, sum and sum of squares of the stored bf16
+    float *stats;                        // optional: rows [2][ld_out], one per n_tiles CTAs: sums and sums of squares of the stored bf16
     void *out;
     unsigned int *status;
     unsigned char tap_oh[kMaxTaps], tap_ow[kMaxTaps];
@@ -903,11 +902,9 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
         const int quarter = warp & 3, group = (warp - 2) >> 2;
         const int gtid = (warp - 2 - group * 4) * 32 + lane;         // 0..127 within the group
         const uint32_t slab = staging_base + (uint32_t)group * (uint32_t)p.staging;
-        // statistics: one row of partial sums per epilogue warp of the grid, [2][ld_out] floats, accumulated over the warp's tiles
-        float *my_stats = (STATS && p.stats) ? p.stats + ((size_t)blockIdx.x * 8 + (warp - 2)) * 2 * p.ld_out : nullptr;
+        // statistics: accumulated over the warp's tiles in shared memory, combined at the end
         const uint32_t st_acc = smem_base + (uint32_t)p.stats_off + (uint32_t)(warp - 2) * (uint32_t)p.stats_warp;
-        if (my_stats) {
-            for (int e = lane; e < 2 * p.ld_out; e += 32) my_stats[e] = 0.f;
+        if (STATS && p.stats) {
             stats_clear(st_acc, lane, (p.BN + 63) / 64);
             __syncwarp();
         }
@@ -980,7 +977,6 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
                         chunk_stats(slab, quarter * 32, rows, lane, st_acc + (uint32_t)ch * 512u);
                     }
                 }
-                if (my_stats && p.n_tiles > 1) stats_flush(st_acc, lane, my_stats, p.ld_out, n0, n_chunks, p.n_cols, true);
                 continue;
             }
             // ---- direct stores (fp32 outputs)
@@ -1008,7 +1004,13 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
                 }
             }
         }
-        if (my_stats && p.n_tiles == 1) stats_flush(st_acc, lane, my_stats, p.ld_out, 0, (p.BN + 63) / 64, p.n_cols, false);
+        if (STATS && p.stats) {
+            named_barrier(3, 256);
+            const int nt = (int)blockIdx.x % p.n_tiles;
+            stats_store_cta(smem_base + (uint32_t)p.stats_off, (uint32_t)p.stats_warp, 8, (int)threadIdx.x - 64, 256,
+                            p.stats + (size_t)(blockIdx.x / p.n_tiles) * 2 * p.ld_out, p.ld_out, p.n_cols, nt * p.BN,
+                            nt + 1 < p.n_tiles ? (nt + 1) * p.BN : p.ld_out);
+        }
         if (p.tma_store && gtid == 0) tma_store_wait_read();
         tc_fence_before();
     }
@@ -1905,10 +1907,11 @@ pt_status launch_gemm(pt_ctx *c, const CUtensorMap &tmA, const CUtensorMap &tmB,
         PT_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
         attr_set[kid] = true;
     }
-    const int grid = total_tiles < c->sm_count ? total_tiles : c->sm_count;
+    int grid = total_tiles < c->sm_count ? total_tiles : c->sm_count;
     if (c->stats_mode) {
         if (!p.tma_store) return PT_ERR_UNSUPPORTED;
-        c->stats_parts = grid * 4 * p.epi_groups;
+        if (grid > p.n_tiles) grid = grid / p.n_tiles * p.n_tiles;     // every CTA keeps one channel tile
+        c->stats_parts = grid / p.n_tiles;
         if ((size_t)c->stats_parts * 2 * p.ld_out * sizeof(float) > c->stats_cap) return PT_ERR_WORKSPACE;
         p.stats = c->stats_out;
     }
@@ -2087,7 +2090,8 @@ pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const
     if (h.max_ctas > 0 && grid > h.max_ctas) grid = h.max_ctas;
     if (c->stats_mode) {
         if (!p.tma_store || B_MN) return PT_ERR_UNSUPPORTED;
-        c->stats_parts = grid * 8;
+        if (grid > p.n_tiles) grid = grid / p.n_tiles * p.n_tiles;     // every CTA keeps one channel tile
+        c->stats_parts = grid / p.n_tiles;
         if ((size_t)c->stats_parts * 2 * p.ld_out * sizeof(float) > c->stats_cap) return PT_ERR_WORKSPACE;
         p.stats = c->stats_out;
     }

@@ -85,6 +85,22 @@ static inline int pt_out_dim(int H, int R, int stride, int pad) {
     return t < 0 ? 0 : t / stride + 1;
 }
 
+// Launch with programmatic stream serialization: the kernel may be scheduled while the previous kernel of the stream is still
+// draining, so that its launch latency and prologue overlap that kernel's tail. Every kernel launched this way executes
+// griddepcontrol.wait before it touches anything a predecessor wrote, and before it releases its own dependents.
+template <typename... KArgs, typename... Args>
+cudaError_t pt_launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args)
+{
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // Copies `bytes` of host data into the region's slot of the arena if it differs from what is there.
 // Returns the device address of the slot.
 pt_status pt_upload_table(pt_ctx *ctx, pt_region *reg, const void *host, size_t bytes, cudaStream_t st, char **dev);

@@ -102,3 +102,11 @@ def test_bn_is_run_to_run_identical_and_validates():
     if B.pt_bn_workspace_bytes(c, d) > 16:
         with pytest.raises(B.PtError):
             B.pt_bn_relu_fwd(c, d, xd, None, g, b, None, None, sm, si, y, small)
+
+
+# channel slabs of unequal width (9, 17 and 18 vectors of 8 channels), the widest pitch, fewer pixels than a block's rows, a ragged
+# last chunk, and one slab that is the whole row with a chunk per block and several chunks per block
+@pytest.mark.parametrize("shape", [(1, 3, 3, 65), (2, 9, 7, 133), (3, 37, 41, 141), (3, 5, 5, 2041), (2, 33, 65, 5), (16, 97, 61, 19)])
+def test_bn_relu_at_the_edges_of_the_channel_slabs(shape):
+    test_bn_relu_forward_and_backward(shape, True, True)
+    test_bn_relu_forward_and_backward(shape, False, True)
