@@ -55,6 +55,8 @@ extern "C" pt_status pt_create(pt_ctx **out, int device)
               cudaMemset(c->d_sync, 0, kSyncWords * sizeof(unsigned int)) == cudaSuccess &&
               cudaEventCreateWithFlags(&c->upload_done, cudaEventDisableTiming) == cudaSuccess;
     if (!ok) { (void)cudaGetLastError(); pt_destroy(c); return PT_ERR_CUDA; }
+    // pinned memory comes back from an earlier context with what it held: a flag left there must not look like this context's first plan
+    memset(c->h_counts, 0, (65536 + 16) * sizeof(int32_t));
     size_t off = 0;
     for (int i = 0; i < 3; ++i) { c->lasso_tab[i].off = off; c->lasso_tab[i].cap = kSlotBytes; off += kSlotBytes; }
     for (int i = 0; i < 2; ++i) { c->detect_tab[i].off = off; c->detect_tab[i].cap = kSlotBytes; off += kSlotBytes; }

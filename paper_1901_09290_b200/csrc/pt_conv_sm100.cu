@@ -1051,9 +1051,11 @@ struct WgradP {
     int pair;               // row-block form, C <= 64: the M side of an MMA is TWO taps x 64 input channels of the x tile
                             // (the second tap is the first one shifted: the operand's 64-element block stride is that shift)
                             // and the N side is the output channels; accumulator lanes = (tap, c), columns = k
+    int cluster;            // 1: the splits of a tile are one thread-block cluster and meet in shared memory (no workspace)
     int apc;                // accumulators per CTA (= tpc, or tpc / 2 in the paired form)
     int acc_cols;           // columns of one accumulator (= BN, or the padded K in the paired form)
     unsigned a_box, b_box;  // bytes reserved per dy box and per x box (multiples of 1024)
+    unsigned data_bytes;    // shared memory behind the control block: the stages, and what the exchange of the splits may use
     float *out;             // dw
     int test_skip;          // test hook (pt_test_skip_next_arrive): split 0 does not announce its partial tile
     float *partial;         // splits > 1: workspace [blockIdx.x][tap in group][split][128][BN] fp32
@@ -1077,6 +1079,106 @@ __device__ __forceinline__ int fast_div(int n, int d, float inv_d)
     return q;
 }
 
+__device__ __forceinline__ int pt_ceil_div_dev(int a, int b) { return (a + b - 1) / b; }
+
+// 32 columns (16 where the accumulator ends) of a warp's 32 TMEM lanes; zeros for a CTA that had no work.
+__device__ __forceinline__ void wgrad_load32(uint32_t taddr, bool second, bool any, uint32_t (&v)[32])
+{
+    uint32_t lo[16], hi[16];
+    if (any) {
+        tmem_ld16(taddr, lo);
+        if (second) tmem_ld16(taddr + 16u, hi);
+        tmem_ld_wait();
+    }
+#pragma unroll
+    for (int e = 0; e < 16; ++e) { v[e] = any ? lo[e] : 0u; v[16 + e] = any && second ? hi[e] : 0u; }
+}
+
+// Four consecutive floats of dw, nv of which exist (a dw row starts on a 16-byte boundary only if C allows it).
+__device__ __forceinline__ void wgrad_store4(float *dst, const float4 &v, int nv)
+{
+    if (nv == 4 && ((uintptr_t)dst & 15) == 0) { *reinterpret_cast<float4 *>(dst) = v; return; }
+    if (nv == 4 && ((uintptr_t)dst & 7) == 0) {
+        reinterpret_cast<float2 *>(dst)[0] = make_float2(v.x, v.y);
+        reinterpret_cast<float2 *>(dst)[1] = make_float2(v.z, v.w);
+        return;
+    }
+    dst[0] = v.x;
+    if (nv > 1) dst[1] = v.y;
+    if (nv > 2) dst[2] = v.z;
+    if (nv > 3) dst[3] = v.w;
+}
+
+// The splits of a tile as one cluster: the accumulators, cut into slots of 32 lanes x 32 columns, are dealt out to the CTAs; every
+// CTA writes each of its slots straight from its registers into the shared memory of the slot's owner (in that CTA's then idle
+// stage memory, the sources side by side), and the owner adds the sources in ascending order and stores dw. Through the workspace the
+// same exchange costs three round trips to L2 (store the partial tile, wait for its arrival counter, load: 7 us whatever the size);
+// here it is two cluster barriers and the bytes (about 2.5 us). At most eight splits: what a portable cluster can be.
+// Every thread of every CTA of the cluster calls this, with the same trip counts, and aborting CTAs too (they hand on zeros; dw is
+// then undefined and the time-out already recorded): the barriers always complete.
+__device__ __forceinline__ void wgrad_cluster_sum(const WgradP &p, Ctl *ctl, uint32_t data_base, uint32_t tmem_base, int ntap, int tap0, int k0,
+                                                  int c0, int split, int iters, uint32_t ring_bytes, int n_acc, int acc_cols)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int S = p.splits, nch = pt_ceil_div_dev(acc_cols, 32);
+    // quarters of the 128 lanes that hold something: output channels below K; in the paired form channel lanes below C of both taps
+    const int nq = p.pair ? (p.C > 32 ? 4 : 2) : min(4, pt_ceil_div_dev(p.K - k0, 32));
+    const int qstep = p.pair && p.C <= 32 ? 2 : 1;
+    const int slots = n_acc * nch * nq, mine = pt_ceil_div_dev(slots, S);              // slot u: owner u % S, its (u / S)-th
+    const int cap = (int)(ring_bytes / ((uint32_t)S * 4096u));                         // slots an owner can receive at a time
+    const bool any = iters > 0 && !*(volatile int *)&ctl->abort_flag;
+    for (int base = 0; base < mine; base += cap) {
+        cluster_barrier();                     // every ring is idle (first round), every sum has been read (later rounds)
+        const int n = min(cap, mine - base);
+        if (warp >= 1) {
+            const int quarter = warp & 3, wset = (warp >= 2 && warp < 6) ? 0 : 1;
+            if (quarter % qstep == 0 && quarter / qstep < nq) {
+                const uint32_t lane_addr = tmem_base + ((uint32_t)(quarter * 32) << 16);
+                for (int ci = wset; ci < n_acc * nch; ci += 2) {
+                    const int u = ci * nq + quarter / qstep, pos = u / S - base;
+                    if (pos < 0 || pos >= n) continue;
+                    const int tt = ci / nch, cc = (ci - tt * nch) * 32;
+                    uint32_t v[32];
+                    wgrad_load32(lane_addr + (uint32_t)(tt * acc_cols + cc), cc + 16 < acc_cols, any, v);
+                    const uint32_t slab = map_to_rank(data_base + ((uint32_t)pos * (uint32_t)S + (uint32_t)split) * 4096u, (uint32_t)(u % S));
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        st_cluster_v4(slab + (uint32_t)lane * 128u + (((uint32_t)j ^ ((uint32_t)lane & 7u)) << 4), v[4 * j], v[4 * j + 1],
+                                      v[4 * j + 2], v[4 * j + 3]);
+                }
+            }
+        }
+        cluster_barrier();                     // everything this CTA owns has arrived
+        // a slot has 32 rows x 8 float4: in the paired form the row (input channel) varies fastest, so that lanes write consecutive
+        // floats of dw; else the column
+        for (int i = threadIdx.x; i < n * 256; i += kThreads) {
+            const int pos = i >> 8, u = (base + pos) * S + split;
+            if (u >= slots) break;
+            const int ci = u / nq, quarter = (u - ci * nq) * qstep, tt = ci / nch, cc = (ci - tt * nch) * 32;
+            const int r = p.pair ? i & 31 : (i >> 3) & 31, j = p.pair ? (i >> 5) & 7 : i & 7;
+            const int row = quarter * 32 + r, col = cc + j * 4;
+            const uint32_t a = data_base + (uint32_t)pos * (uint32_t)S * 4096u + (uint32_t)r * 128u + ((uint32_t)(j ^ (r & 7)) << 4);
+            float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int z = 0; z < S; ++z) {
+                float4 t;
+                asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(t.x), "=f"(t.y), "=f"(t.z), "=f"(t.w) : "r"(a + (uint32_t)z * 4096u) : "memory");
+                sum.x += t.x; sum.y += t.y; sum.z += t.z; sum.w += t.w;
+            }
+            if (p.pair) {
+                const int tap = tap0 + 2 * tt + (row >> 6), c = row & 63;
+                if (c < p.C && tap < tap0 + ntap) {
+                    const float v4[4] = {sum.x, sum.y, sum.z, sum.w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        if (col + e < p.K) p.out[((size_t)(col + e) * p.taps + tap) * p.C + c] = v4[e];
+                }
+            } else if (k0 + row < p.K && col < acc_cols && c0 + col < p.C) {
+                wgrad_store4(p.out + ((size_t)(k0 + row) * p.taps + tap0 + tt) * p.C + c0 + col, sum, min(4, p.C - (c0 + col)));
+            }
+        }
+    }
+}
+
 // Everything after the main loop of a weight-gradient kernel: the accumulators leave TMEM (directly to dw, or as this
 // split's partial tile), the splits of a tile meet, and every CTA sums its share of the tile over the splits.
 // `ring_bytes` of shared memory at `data_base` are free by then and serve as staging.
@@ -1098,33 +1200,28 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, const CUtensorMap 
             const bool row_ok = k < p.K;
             (void)row_ok;
             const uint32_t lane_addr = tmem_base + ((uint32_t)(quarter * 32) << 16);
-            if (p.splits > 1) {
-                // ---- (1) this CTA's fp32 partial tile goes to the workspace through swizzled staging + TMA stores
+            if (p.cluster) {
+                // the exchange is below: every thread of the cluster takes part in its barriers
+            } else if (p.splits > 1) {
+                // ---- (1) this CTA's fp32 partial tile goes to the workspace through swizzled staging + TMA stores (the rows that
+                // hold something: not the output channels past K, in the paired form not the channel lanes past C)
                 const int gtid = (warp - 1) * 32 + lane;
+                const bool rows_used = p.pair ? (quarter & 1) * 32 < p.C : k0 + quarter * 32 < p.K;
                 int sl = 0, ci = 0;
-                for (int tt = 0; tt < n_acc; ++tt)
+                for (int tt = 0; tt < n_acc && rows_used; ++tt)
                 for (int cc = 0; cc < acc_cols; cc += 32, ++ci) {
                     if ((ci & 1) != wset) continue;
                     sl ^= 1;
                     const uint32_t slab = data_base + (uint32_t)((wset * 4 + quarter) * 2 + sl) * 4096u;
                     if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
                     __syncwarp();
-                    uint32_t lo[16], hi[16];
-                    if (iters > 0) {
-                        tmem_ld16(lane_addr + (uint32_t)(tt * acc_cols + cc), lo);
-                        if (cc + 16 < acc_cols) tmem_ld16(lane_addr + (uint32_t)(tt * acc_cols + cc) + 16u, hi);
-                        tmem_ld_wait();
-                    }
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) {
-                        if (iters <= 0) lo[e] = 0u;
-                        if (iters <= 0 || cc + 16 >= acc_cols) hi[e] = 0u;
-                    }
+                    uint32_t v[32];
+                    wgrad_load32(lane_addr + (uint32_t)(tt * acc_cols + cc), cc + 16 < acc_cols, iters > 0, v);
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
-                        const uint32_t *src = j < 4 ? &lo[4 * j] : &hi[4 * (j - 4)];
                         const uint32_t addr = slab + (uint32_t)lane * 128u + (((uint32_t)j ^ ((uint32_t)lane & 7u)) << 4);
-                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(src[0]), "r"(src[1]), "r"(src[2]), "r"(src[3])
+                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v[4 * j]), "r"(v[4 * j + 1]), "r"(v[4 * j + 2]),
+                                     "r"(v[4 * j + 3])
                                      : "memory");
                     }
                     fence_proxy_async();
@@ -1144,10 +1241,15 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, const CUtensorMap 
                     // (test hook: split 0 stays silent, so that every split of the tile runs into the bounded wait below)
                     if (!(p.test_skip && split == 0)) atomicAdd(arrived, 1u);
                     const uint64_t t0 = globaltimer_ns();
-                    while (atomicAdd(arrived, 0u) < (unsigned)p.splits) {
-                        if (*abort_flag) break;
-                        if (globaltimer_ns() - t0 > *(volatile unsigned long long *)&g_wait_limit_ns) { record_timeout(p.status, 8); *abort_flag = 1; break; }
-                        __nanosleep(64);
+                    unsigned int seen, polls = 0;
+                    for (;;) {
+                        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(arrived) : "memory");
+                        if (seen >= (unsigned)p.splits || *abort_flag) break;
+                        if ((++polls & 63u) == 0u && globaltimer_ns() - t0 > *(volatile unsigned long long *)&g_wait_limit_ns) {
+                            record_timeout(p.status, 8);
+                            *abort_flag = 1;
+                            break;
+                        }
                     }
                 }
                 named_barrier(1, 256);
@@ -1214,6 +1316,10 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, const CUtensorMap 
         }
         tc_fence_before();
     }
+    if (p.cluster) {
+        wgrad_cluster_sum(p, ctl, data_base, tmem_base, ntap, tap0, k0, c0, split, iters, ring_bytes, n_acc, acc_cols);
+        return;
+    }
     __syncthreads();
     if (p.splits > 1 && !*abort_flag) {
         // ---- (3) all threads: this CTA sums its share of the tile's elements over the splits
@@ -1222,8 +1328,9 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, const CUtensorMap 
         // The partial tiles sit in L2; what costs time is a chain of dependent loads, so every thread first issues the
         // asynchronous 16-byte copies of its items for ALL splits into the (now idle) stage memory, and only then are the
         // copies summed from shared memory in ascending split order: deterministic, whichever CTA does the work.
-        const int rows_real = p.pair ? 128 : min(128, p.K - k0);
-        const int ngrp = acc_cols / 4;                               // float4 groups per row (a multiple of 16 columns)
+        // In the paired form an item's row varies fastest: its lanes then write consecutive floats of dw (rows are input channels).
+        const int rows_real = p.pair ? 2 * p.C : min(128, p.K - k0);
+        const int ngrp = pt_ceil_div_dev(p.pair ? p.K : min(acc_cols, p.C - c0), 4);     // float4 groups per row
         const int items = rows_real * ngrp;
         const int total = n_acc * items;
         const int per_cta = (total + p.splits - 1) / p.splits;
@@ -1231,12 +1338,25 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, const CUtensorMap 
         const size_t zstride = (size_t)128 * acc_cols;
         const float *pbase = p.partial + (size_t)blockIdx.x * p.apc * p.splits * zstride;
         const int cap = (int)(((size_t)ring_bytes) / ((size_t)p.splits * 16));   // items the stage memory holds
-        const float inv_items = 1.0f / (float)items, inv_ngrp = 1.0f / (float)ngrp;
+        const float inv_items = 1.0f / (float)items, inv_ngrp = 1.0f / (float)ngrp, inv_rows = 1.0f / (float)rows_real;
+        // row of the partial tile and first column of an item
+        auto place = [&](int item, int &r, int &col) {
+            if (p.pair) {
+                const int gq = fast_div(item, rows_real, inv_rows), rr = item - gq * rows_real;
+                r = rr >= p.C ? 64 + rr - p.C : rr;
+                col = gq * 4;
+            } else {
+                r = fast_div(item, ngrp, inv_ngrp);
+                col = (item - r * ngrp) * 4;
+            }
+        };
         for (int c_beg = it_beg; c_beg < it_end; c_beg += cap) {
             const int n_chunk = min(cap, it_end - c_beg);
             for (int i = threadIdx.x; i < n_chunk; i += kThreads) {
                 const int idx = c_beg + i, tt = fast_div(idx, items, inv_items), item = idx - tt * items;
-                const float *src = pbase + (size_t)tt * p.splits * zstride + (size_t)item * 4;
+                int r, col;
+                place(item, r, col);
+                const float *src = pbase + (size_t)tt * p.splits * zstride + (size_t)r * acc_cols + col;
                 uint32_t dst = data_base + (uint32_t)i * 16u;
                 for (int z = 0; z < p.splits; ++z, src += zstride, dst += (uint32_t)n_chunk * 16u)
                     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
@@ -1245,8 +1365,8 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, const CUtensorMap 
             __syncthreads();
             for (int i = threadIdx.x; i < n_chunk; i += kThreads) {
                 const int idx = c_beg + i, tt = fast_div(idx, items, inv_items), item = idx - tt * items;
-                const int r = fast_div(item, ngrp, inv_ngrp), col = (item - r * ngrp) * 4;
-                if (!p.pair && c0 + col >= p.C) continue;
+                int r, col;
+                place(item, r, col);
                 float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
                 uint32_t a = data_base + (uint32_t)i * 16u;
                 for (int z = 0; z < p.splits; ++z, a += (uint32_t)n_chunk * 16u) {
@@ -1265,21 +1385,7 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, const CUtensorMap 
                     }
                     continue;
                 }
-                float *dst = p.out + ((size_t)(k0 + r) * p.taps + tap0 + tt) * p.C + c0 + col;
-                const int nv = min(4, p.C - (c0 + col));
-                if (nv == 4 && ((uintptr_t)dst & 15) == 0) {
-                    *reinterpret_cast<float4 *>(dst) = sum;           // a dw row starts on a 16-byte boundary only if C allows it
-                    continue;
-                }
-                if (nv == 4 && ((uintptr_t)dst & 7) == 0) {
-                    reinterpret_cast<float2 *>(dst)[0] = make_float2(sum.x, sum.y);
-                    reinterpret_cast<float2 *>(dst)[1] = make_float2(sum.z, sum.w);
-                    continue;
-                }
-                dst[0] = sum.x;
-                if (nv > 1) dst[1] = sum.y;
-                if (nv > 2) dst[2] = sum.z;
-                if (nv > 3) dst[3] = sum.w;
+                wgrad_store4(p.out + ((size_t)(k0 + r) * p.taps + tap0 + tt) * p.C + c0 + col, sum, min(4, p.C - (c0 + col)));
             }
             __syncthreads();
         }
@@ -1451,7 +1557,7 @@ __global__ void __launch_bounds__(kThreads) conv_wgrad_kernel(const __grid_const
         if (ok) umma_commit_lead(smem_u32(&ctl->accum), leader);
         if (warp == 1) WTRACE(2);
     }
-    wgrad_finish(p, tmP, ctl, data_base, tmem_base, ntap, tap0, k0, c0, split, iters, (uint32_t)p.stages * stage_bytes, ntap, p.BN);
+    wgrad_finish(p, tmP, ctl, data_base, tmem_base, ntap, tap0, k0, c0, split, iters, p.data_bytes, ntap, p.BN);
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem_base, (uint32_t)p.tmem_cols);
@@ -1509,10 +1615,19 @@ __global__ void __launch_bounds__(kThreads) conv_wgrad_rows_kernel(const __grid_
         prefetch_tmap(&tmDy);
         prefetch_tmap(&tmX);
     }
-    // the ring starts as zeros: the rows between the end of a box and the end of the last 16-pixel step are read by the
-    // MMAs (times zero) and must be finite
-    for (uint32_t off = threadIdx.x * 16u; off < (uint32_t)p.stages * stage_bytes; off += kThreads * 16u)
-        asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(data_base + off), "r"(0u) : "memory");
+    // the rows between the end of a box and the end of the last 16-pixel step are read by the MMAs (times zero) and must be finite
+    {
+        const uint32_t a_used = (uint32_t)(p.nr * p.Wp) * 128u, b_used = (uint32_t)((p.nr + p.lo_span) * p.Wp) * 128u;
+        const uint32_t a_rest = (p.a_box - a_used) / 16u, b_rest = (p.b_box - b_used) / 16u;
+        const uint32_t per_stage = (uint32_t)p.nb_a * a_rest + nb_b * b_rest;
+        for (uint32_t i = threadIdx.x; i < (uint32_t)p.stages * per_stage; i += kThreads) {
+            const uint32_t st = i / per_stage, o = i - st * per_stage;
+            const uint32_t at = o < (uint32_t)p.nb_a * a_rest ? (o / a_rest) * p.a_box + a_used + (o % a_rest) * 16u
+                                                              : a_bytes + ((o - (uint32_t)p.nb_a * a_rest) / b_rest) * p.b_box + b_used +
+                                                                    ((o - (uint32_t)p.nb_a * a_rest) % b_rest) * 16u;
+            asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(data_base + st * stage_bytes + at), "r"(0u) : "memory");
+        }
+    }
     fence_proxy_async();
     if (warp == 1) {
         tmem_alloc(smem_u32(&ctl->tmem_base), (uint32_t)p.tmem_cols);
@@ -1606,7 +1721,7 @@ __global__ void __launch_bounds__(kThreads) conv_wgrad_rows_kernel(const __grid_
         if (ok) umma_commit_lead(smem_u32(&ctl->accum), leader);
         if (warp == 1) WTRACE(2);
     }
-    wgrad_finish(p, tmP, ctl, data_base, tmem_base, ntap, tap0, k0, c0, split, iters, (uint32_t)p.stages * stage_bytes, n_acc, p.acc_cols);
+    wgrad_finish(p, tmP, ctl, data_base, tmem_base, ntap, tap0, k0, c0, split, iters, p.data_bytes, n_acc, p.acc_cols);
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem_base, (uint32_t)p.tmem_cols);
@@ -2123,6 +2238,25 @@ void halo_spec_stride1(const pt_conv_desc *d, HaloSpec *h, const void *src, int 
 // memory: at most one of them per SM, whatever else runs beside it (kernels that wait for nobody always finish).
 constexpr size_t kSplitSmemFloor = 116 * 1024;
 
+// ---- launch shape of a weight gradient
+// Both kernels cut the work three ways: tiles of dw (channels), groups of taps, and the pixels of the reduction over `splits` CTAs
+// that exchange partial sums at the end. The shape is chosen by a rough time of one CTA (microseconds; the constants are measured):
+//   first load 1.4, then per stage the larger of its MMAs (55 cycles each at N <= 64, N/2 + 8 above) and its bytes at 100 KB/us,
+//   plus 0.12 of waiting and issuing; then the exchange:
+//   none (one split): 1; in a cluster (2..8 splits): 1.8 + bytes of the accumulators at 120 KB/us;
+//   through the workspace: 6 + bytes at 60 KB/us (partial tile to L2, arrival counter, sum: three round trips).
+// A cluster needs its CTAs free at the same time in one GPC: used while the device can hold all of the launch's clusters at once.
+constexpr double kWgSearch = 400.0;      // layers whose tile takes one CTA less than this (us) also choose tap groups and unit size
+
+double wg_mma_us(int n) { return (n <= 64 ? 55.0 : n * 0.5 + 8.0) / 1900.0; }
+double wg_exchange_us(int splits, bool cluster, double acc_bytes)
+{
+    if (splits <= 1) return 1.0 + acc_bytes / 200e3;
+    return cluster ? 1.8 + acc_bytes / 120e3 : 6.0 + acc_bytes / 60e3;
+}
+
+int wg_max_clusters(const pt_ctx *c, int size);
+
 // Taps handled by one weight-gradient CTA: they share the dy tile and get one TMEM accumulator of BN columns each.
 // Bounded by the 512 TMEM columns and by a stage of 16 KB (dy) + taps x BN/64 x 8 KB (x) staying at or below 48 KB, so
 // that at least four pipeline stages fit (measured: with two stages the kernel is slower than with one tap per CTA);
@@ -2138,109 +2272,169 @@ int wgrad_taps_per_cta(int taps, int bn)
     return pt_ceil_div(taps, groups);
 }
 
-int wgrad_splits(const pt_ctx *c, const pt_conv_desc *d, int P, int Q)
+int wgrad_budget(const pt_ctx *c) { return (c->wgrad_ctas > 0 && c->wgrad_ctas < c->sm_count) ? c->wgrad_ctas : c->sm_count; }
+
+// Splits of a launch with `tiles` CTAs per split, at most `max_s`: all the budget holds through the workspace, or up to eight as
+// clusters, whichever is estimated faster; `main_us(s)` is the main loop with s splits.
+template <typename F>
+double wg_pick_splits(const pt_ctx *c, int tiles, int max_s, double acc_bytes, F main_us, int *splits, int *cluster)
 {
-    int n_tiles;
-    const int bn = tile_n(d->C, &n_tiles);
-    const int tpc = wgrad_taps_per_cta(d->R * d->S, bn);
-    const int tiles = pt_ceil_div(d->K, 128) * n_tiles * pt_ceil_div(d->R * d->S, tpc);
-    const long long npix = (long long)d->N * P * Q;
-    const int budget = (c->wgrad_ctas > 0 && c->wgrad_ctas < c->sm_count) ? c->wgrad_ctas : c->sm_count;
-    long long s = budget / tiles;                          // at most one CTA per SM, one wave
-    const long long max_s = (npix + 255) / 256;          // at least four 64-pixel stages per split
+    int s = wgrad_budget(c) / tiles;                       // at most one CTA per SM, one wave
     if (s > max_s) s = max_s;
-    if (s < 1) s = 1;
     if (s > 512) s = 512;
-    return (int)s;
+    if (s < 1) s = 1;
+    double best = main_us(s) + wg_exchange_us(s, false, acc_bytes);
+    *splits = s; *cluster = 0;
+    for (int k = s < 8 ? s : 8; k >= 2; --k) {
+        if (tiles > wg_max_clusters(c, k)) continue;
+        const double t = main_us(k) + wg_exchange_us(k, true, acc_bytes);
+        if (t < best) { best = t; *splits = k; *cluster = 1; }
+        break;                                             // the largest cluster that fits
+    }
+    return best;
 }
 
-// Plan of the row-block weight gradient (stride-1 filters with at most 64 input channels); ok = 0 where the generic kernel is used.
-struct WgRows {
-    int ok;
-    int bn, n_tiles, m_tiles, tpc, tap_groups, apc, acc_cols;
-    int nr, Wp, RB, units, units_per_split, splits, ksteps, nb_a, stages;
-    unsigned a_box, b_box;
-    size_t stage_bytes, smem;
-};
-
-WgRows wgrad_rows_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q)
+// The generic kernel: 64 pixels per stage.
+void wgrad_gen_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, pt_wgrad_plan *w)
 {
-    WgRows w;
-    memset(&w, 0, sizeof(w));
+    memset(w, 0, sizeof(*w));
     const int taps = d->R * d->S;
-    if (d->stride != 1 || taps > kMaxTaps) return w;
+    w->bn = tile_n(d->C, &w->n_tiles);
+    w->m_tiles = pt_ceil_div(d->K, 128);
+    w->acc_cols = w->bn;
+    const long long npix = (long long)d->N * P * Q;
+    long long max_s = (npix + 255) / 256;                  // at least four 64-pixel stages per split
+    if (max_s > 512) max_s = 512;
+    const int nb = pt_ceil_div(w->bn, 64), base = wgrad_taps_per_cta(taps, w->bn), groups0 = pt_ceil_div(taps, base);
+    double best = 1e30;
+    for (int g = groups0; g <= taps; g += groups0) {
+        const int tpc = pt_ceil_div(taps, g), tiles = w->m_tiles * w->n_tiles * pt_ceil_div(taps, tpc);
+        if (g > groups0 && (tiles > wgrad_budget(c) || pt_ceil_div(taps, tpc) != g)) continue;
+        const double load = ((d->K > 64 ? 16384.0 : 8192.0) + tpc * nb * 8192.0) / 100e3, mma = tpc * 4 * wg_mma_us(w->bn);
+        const double stage = (load > mma ? load : mma) + 0.12;
+        int s, cl;
+        const double t = wg_pick_splits(c, tiles, (int)max_s, (double)tpc * w->bn * 512.0,
+                                        [&](int k) { return 1.4 + (double)((npix + 63) / 64 + k - 1) / k * stage; }, &s, &cl);
+        if (t < best) {
+            best = t;
+            w->tpc = w->apc = tpc; w->tap_groups = pt_ceil_div(taps, tpc);
+            w->splits = s; w->cluster = cl;
+        }
+        if ((double)((npix + 63) / 64) * stage > kWgSearch) break;      // large: the fewest groups read the least
+    }
+}
+
+// The row-block kernel (stride-1 filters with at most 64 input channels); false where the generic kernel is used.
+bool wgrad_rows_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, pt_wgrad_plan *w)
+{
+    memset(w, 0, sizeof(*w));
+    const int taps = d->R * d->S;
+    if (d->stride != 1 || taps > kMaxTaps) return false;
     // a 1x1 filter has no halo to save, but the orientation (x on the M side, all of dy's channels on the N side: one tile
     // where the generic kernel needs two for K > 128) and the plain tiled loads (no im2col boxes on 96-byte pixel pitches)
     // still pay on large maps (56x56, 59 -> 143: 53 -> 31 us at 49 CTAs); small maps have too few units to split
-    if (taps < 2 && P * Q < 784) return w;
-    w.Wp = Q + d->S - 1;
-    if (w.Wp > 256 || P < 1 || Q < 1) return w;
+    if (taps < 2 && P * Q < 784) return false;
+    w->Wp = Q + d->S - 1;
+    if (w->Wp > 256 || P < 1 || Q < 1) return false;
     // paired form only: the x tile is the M side (two taps x 64 channel lanes), dy's output channels the N side
-    w.acc_cols = pt_ceil_div(d->K, 16) * 16;
-    if (d->C > 64 || w.acc_cols > 256) return w;
-    w.bn = tile_n(d->C, &w.n_tiles);
-    w.m_tiles = 1;
+    w->acc_cols = pt_ceil_div(d->K, 16) * 16;
+    if (d->C > 64 || w->acc_cols > 256) return false;
+    w->bn = tile_n(d->C, &w->n_tiles);
+    w->m_tiles = 1;
     const int pairs = pt_ceil_div(taps, 2);
-    int t = 512 / w.acc_cols;
+    int t = 512 / w->acc_cols;
     if (t > 16) t = 16;                                   // four issuer warps x four accumulators
     if (t > pairs) t = pairs;
-    w.tap_groups = pt_ceil_div(pairs, t);
-    w.apc = pt_ceil_div(pairs, w.tap_groups);
-    w.tpc = 2 * w.apc;
-    w.tap_groups = pt_ceil_div(taps, w.tpc);
-    w.nb_a = pt_ceil_div(w.acc_cols, 64);
-    const int nb_b = 1;
-    // rows per unit: the least traffic per useful row (dy rows + x halo rows, the last unit of an image padded) times
-    // the MMA steps spent per useful pixel, among the sizes that leave at least two stages
-    double best = 1e30;
-    for (int nr = 1; nr <= P && nr + d->R - 1 <= 256; ++nr) {
-        const int ks = pt_ceil_div(nr * w.Wp, 16);
-        const size_t a_box = (size_t)ks * 2048;
-        const size_t b_box = pt_align_up(((size_t)(d->R - 1) * w.Wp + d->S + (size_t)ks * 16) * 128, 1024);
-        const size_t stage = w.nb_a * a_box + nb_b * b_box;
-        const int st = (int)((220 * 1024 - 2048) / stage);
-        if (st < 2) break;
-        const int rb = pt_ceil_div(P, nr);
-        const double traffic = (double)(w.nb_a * nr + nb_b * (nr + d->R - 1)) * rb / P;
-        const double steps = (double)ks * 16 * rb / ((double)P * w.Wp);
-        const double cost = traffic * steps;
-        if (cost < best) {
-            best = cost;
-            w.nr = nr; w.ksteps = ks; w.a_box = (unsigned)a_box; w.b_box = (unsigned)b_box;
-            w.stages = st > kMaxStages ? kMaxStages : st;
-            w.stage_bytes = stage;
+    const int groups0 = pt_ceil_div(pairs, t);
+    w->nb_a = pt_ceil_div(w->acc_cols, 64);
+    const double cyc = wg_mma_us(w->acc_cols);
+    // Rows per unit. Large layers: the least traffic per useful row (dy rows + x halo rows, the last unit of an image padded) times
+    // the MMA steps spent per useful pixel. Small ones: with the tap groups and the splits, by the estimated time.
+    double best_cost = 1e30, best_us = 1e30;
+    bool large = false;
+    for (int pass = 0; pass < 2 && !large; ++pass) {
+        for (int nr = 1; nr <= P && nr + d->R - 1 <= 256; ++nr) {
+            const int ks = pt_ceil_div(nr * w->Wp, 16);
+            const size_t a_box = (size_t)ks * 2048;
+            const size_t b_box = pt_align_up(((size_t)(d->R - 1) * w->Wp + d->S + (size_t)ks * 16) * 128, 1024);
+            const size_t stage = w->nb_a * a_box + b_box;
+            const int st = (int)((220 * 1024 - 2048) / stage);
+            if (st < 2) break;
+            const int rb = pt_ceil_div(P, nr), units = d->N * rb;
+            auto take = [&](int apc, int s, int cl) {
+                w->nr = nr; w->ksteps = ks; w->a_box = (unsigned)a_box; w->b_box = (unsigned)b_box;
+                w->stages = st > kMaxStages ? kMaxStages : st;
+                w->stage_bytes = stage; w->RB = rb; w->units = units;
+                w->apc = apc; w->tpc = 2 * apc; w->tap_groups = pt_ceil_div(taps, w->tpc);
+                w->splits = s; w->cluster = cl;
+            };
+            const double load = (double)(w->nb_a * nr + nr + d->R - 1) * w->Wp * 128.0 / 100e3;
+            if (pass == 0) {
+                const double traffic = (double)(w->nb_a * nr + nr + d->R - 1) * rb / P, steps = (double)ks * 16 * rb / ((double)P * w->Wp);
+                if (traffic * steps >= best_cost) continue;
+                best_cost = traffic * steps;
+                take(pt_ceil_div(pairs, groups0), 1, 0);
+                continue;
+            }
+            for (int g = groups0; g <= pairs; g += groups0) {
+                const int apc = pt_ceil_div(pairs, g), tiles = pt_ceil_div(pairs, apc);
+                if (g > groups0 && (tiles > wgrad_budget(c) || tiles != g)) continue;
+                const double mma = ks * apc * cyc, unit = (load > mma ? load : mma) + 0.12;
+                int s, cl;
+                const double us = wg_pick_splits(c, tiles, units > 3 ? units / 2 : 1, (double)apc * w->acc_cols * 512.0,
+                                                 [&](int k) { return 1.4 + pt_ceil_div(units, k) * unit; }, &s, &cl);
+                if (us < best_us) { best_us = us; take(apc, s, cl); }
+            }
+        }
+        if (w->nr == 0) return false;
+        if (pass == 0) {
+            const double unit = w->ksteps * w->apc * cyc;
+            large = unit * w->units > kWgSearch;
+            if (large) {
+                int s, cl;
+                wg_pick_splits(c, w->tap_groups, w->units > 3 ? w->units / 2 : 1, (double)w->apc * w->acc_cols * 512.0,
+                               [&](int k) { return 1.4 + pt_ceil_div(w->units, k) * (unit + 0.12); }, &s, &cl);
+                w->splits = s; w->cluster = cl;
+            }
         }
     }
-    if (w.nr == 0) return w;
-    w.RB = pt_ceil_div(P, w.nr);
-    w.units = d->N * w.RB;
-    const int tiles = w.m_tiles * w.n_tiles * w.tap_groups;
-    const int budget = (c->wgrad_ctas > 0 && c->wgrad_ctas < c->sm_count) ? c->wgrad_ctas : c->sm_count;
-    int s = budget / tiles;                                // at most one CTA per SM, one wave
-    if (s > w.units / 2) s = w.units / 2;                  // at least two units per split
-    if (s < 1) s = 1;
-    if (s > 512) s = 512;
-    w.units_per_split = pt_ceil_div(w.units, s);
-    w.splits = pt_ceil_div(w.units, w.units_per_split);
-    if (w.stages > w.units_per_split && w.units_per_split >= 2) w.stages = w.units_per_split;
-    w.smem = 2048 + (size_t)w.stages * w.stage_bytes;
-    if (w.smem < 2048 + 8 * 2 * 4096) w.smem = 2048 + 8 * 2 * 4096;    // the epilogue's staging slabs reuse the ring
-    w.ok = 1;
+    w->units_per_split = pt_ceil_div(w->units, w->splits);
+    w->splits = pt_ceil_div(w->units, w->units_per_split);
+    if (w->splits < 2) w->cluster = 0;
+    if (w->stages > w->units_per_split && w->units_per_split >= 2) w->stages = w->units_per_split;
+    w->smem = 2048 + (size_t)w->stages * w->stage_bytes;
+    if (w->smem < 2048 + 8 * 2 * 4096) w->smem = 2048 + 8 * 2 * 4096;    // the epilogue's staging slabs reuse the ring
+    w->rows = 1;
+    return true;
+}
+
+// The plan of a descriptor at the context's CTA limit. rows_only: only a row-block plan is asked for (its `rows` is 0 if there is none).
+pt_wgrad_plan wgrad_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, bool rows_only = false)
+{
+    pt_conv_desc key = *d;
+    key.ldw = key.out_f32 = 0; key.algo = rows_only ? 1 : 0;
+    const int limit = wgrad_budget(c);
+    unsigned h = 2166136261u;
+    for (size_t i = 0; i < sizeof(key) / 4; ++i) h = (h ^ (unsigned)reinterpret_cast<const int32_t *>(&key)[i]) * 16777619u;
+    h = (h ^ (unsigned)limit) * 16777619u;
+    std::lock_guard<std::mutex> lock(c->wgrad_mutex);
+    pt_ctx::WgradSlot &slot = c->wgrad_slot[(h >> 8) & 127];
+    if (slot.valid && slot.limit == limit && slot.P == P && slot.Q == Q && memcmp(&slot.d, &key, sizeof(key)) == 0) return slot.plan;
+    pt_wgrad_plan w;
+    if (!wgrad_rows_plan(c, d, P, Q, &w)) {
+        w.rows = 0;
+        if (!rows_only) wgrad_gen_plan(c, d, P, Q, &w);
+    }
+    slot.d = key; slot.limit = limit; slot.P = P; slot.Q = Q; slot.plan = w; slot.valid = true;
     return w;
 }
 
-// Workspace of the split weight gradient: one padded 128 x BN fp32 tile per (tile, split).
-size_t wgrad_partial_bytes(const pt_ctx *c, const pt_conv_desc *d, int P, int Q)
+// Workspace of the split weight gradient: one padded 128 x columns fp32 tile per (tile, split). (A cluster needs none, but the test
+// hook of the arrival wait turns one into an exchange through the workspace.)
+size_t wgrad_partial_bytes(const pt_wgrad_plan &w)
 {
-    const WgRows wr = wgrad_rows_plan(c, d, P, Q);
-    if (wr.ok)
-        return wr.splits <= 1 ? 0 : (size_t)wr.tap_groups * wr.apc * wr.splits * 128 * wr.acc_cols * sizeof(float);
-    const int s = wgrad_splits(c, d, P, Q);
-    if (s <= 1) return 0;
-    int n_tiles;
-    const int bn = tile_n(d->C, &n_tiles);
-    const int tpc = wgrad_taps_per_cta(d->R * d->S, bn);
-    return (size_t)n_tiles * pt_ceil_div(d->K, 128) * pt_ceil_div(d->R * d->S, tpc) * tpc * s * 128 * bn * sizeof(float);
+    if (w.splits <= 1) return 0;
+    return (size_t)w.n_tiles * w.m_tiles * w.tap_groups * w.apc * w.splits * 128 * w.acc_cols * sizeof(float);
 }
 
 // The splits' fp32 partial tiles as a 2-D tensor (BN columns, rows): box 32 x 32, 128-byte swizzle.
@@ -2256,41 +2450,99 @@ bool make_partial_map(const pt_ctx *c, CUtensorMap *tm, void *ws, int bn, size_t
     return map_ok(r, __LINE__);
 }
 
-// Launches the weight-gradient kernel for a problem whose x operand is described by `tmX` (64 pixels x 64 channels boxes).
-pt_status run_wgrad(pt_ctx *c, const pt_conv_desc *d, int P, int Q, int stride, int lo_h, int lo_w, const CUtensorMap &tmX,
-                    const void *dy, float *out, void *ws, size_t ws_bytes, cudaStream_t st, bool x_tiled = false)
+// Launch of a weight-gradient kernel: with programmatic stream serialization and, where the splits of a tile meet in shared memory,
+// as clusters of `cluster` CTAs along y.
+cudaError_t launch_wgrad(void (*kernel)(CUtensorMap, CUtensorMap, CUtensorMap, WgradP), dim3 grid, int cluster, size_t smem, cudaStream_t st,
+                         const CUtensorMap &a, const CUtensorMap &b, const CUtensorMap &q, const WgradP &p)
 {
-    WgradP p;
-    memset(&p, 0, sizeof(p));
-    p.x_tiled = x_tiled ? 1 : 0;
-    p.K = d->K; p.C = d->C; p.taps = d->R * d->S; p.S = d->S;
-    p.BN = tile_n(d->C, &p.n_tiles);
-    p.m_tiles = pt_ceil_div(d->K, 128);
-    p.tpc = wgrad_taps_per_cta(p.taps, p.BN);
-    p.tap_groups = pt_ceil_div(p.taps, p.tpc);
-    p.apc = p.tpc; p.acc_cols = p.BN;
-    p.npix = d->N * P * Q;
-    p.splits = wgrad_splits(c, d, P, Q);
-    p.pix_per_split = pt_ceil_div(pt_ceil_div(p.npix, p.splits), 64) * 64;
-    p.Pd = P; p.Qd = Q; p.stride = stride; p.lo_h = lo_h; p.lo_w = lo_w;
-    p.tmem_cols = pow2_cols(p.tpc * p.BN);
-    p.status = c->d_status;
-    const int gx = p.n_tiles * p.m_tiles * p.tap_groups;
-    p.out = out;
-    CUtensorMap tmP;
-    memset(&tmP, 0, sizeof(tmP));
-    if (p.splits > 1) {
-        const size_t need = (size_t)gx * p.tpc * p.splits * 128 * p.BN * sizeof(float);
-        if (!ws || ws_bytes < need) return PT_ERR_WORKSPACE;
-        p.partial = (float *)ws;
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = grid; cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 1; attr[1].val.clusterDim.y = (unsigned)cluster; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = cluster > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kernel, a, b, q, p);
+}
+
+pt_status wgrad_attr()
+{
+    static bool attr_set = false;
+    if (!attr_set) {
+        PT_CUDA_OK(cudaFuncSetAttribute(conv_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
+        PT_CUDA_OK(cudaFuncSetAttribute(conv_wgrad_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
+        attr_set = true;
+    }
+    return PT_OK;
+}
+
+// Clusters of `size` weight-gradient CTAs the device holds at once (one CTA per SM; a GPC whose SM count is no multiple leaves some over).
+int wg_max_clusters(const pt_ctx *c, int size)
+{
+    if (size < 2 || size > 8) return 0;
+    if (c->max_clusters[size] == 0) {
+        int n = 0;
+        cudaLaunchConfig_t cfg;
+        memset(&cfg, 0, sizeof(cfg));
+        cfg.gridDim = dim3(1, (unsigned)size); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = 220 * 1024;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = (unsigned)size; attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr; cfg.numAttrs = 1;
+        if (wgrad_attr() != PT_OK || cudaOccupancyMaxActiveClusters(&n, conv_wgrad_kernel, &cfg) != cudaSuccess || n < 1) {
+            (void)cudaGetLastError();
+            n = -1;
+        }
+        c->max_clusters[size] = n;
+    }
+    return c->max_clusters[size] < 0 ? 0 : c->max_clusters[size];
+}
+
+// What both forms have in common: tiles, splits and where the partial tiles go.
+pt_status wgrad_common(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const pt_wgrad_plan &w, float *out, void *ws, size_t ws_bytes, WgradP *p,
+                       CUtensorMap *tmP)
+{
+    memset(p, 0, sizeof(*p));
+    p->K = d->K; p->C = d->C; p->taps = d->R * d->S; p->S = d->S;
+    p->BN = w.bn; p->n_tiles = w.n_tiles; p->m_tiles = w.m_tiles;
+    p->tpc = w.tpc; p->tap_groups = w.tap_groups; p->apc = w.apc; p->acc_cols = w.acc_cols;
+    p->npix = d->N * P * Q;
+    p->splits = w.splits; p->cluster = w.cluster;
+    p->Pd = P; p->Qd = Q;
+    p->tmem_cols = pow2_cols(w.apc * w.acc_cols);
+    p->status = c->d_status;
+    p->out = out;
+    memset(tmP, 0, sizeof(*tmP));
+    if (c->test_skip == 1 && p->splits > 1) { p->test_skip = 1; p->cluster = 0; c->test_skip = 0; }
+    if (p->splits > 1 && !p->cluster) {
+        const int gx = p->n_tiles * p->m_tiles * p->tap_groups;
+        if (!ws || ws_bytes < wgrad_partial_bytes(w)) return PT_ERR_WORKSPACE;
+        p->partial = (float *)ws;
         // two self-resetting counters per tile from the context's ring (kernels of one stream run in order, and the ring
         // is far larger than the tiles of the few launches that can be in flight)
         if (2 * gx > 8192) return PT_ERR_UNSUPPORTED;
         if (c->sync_next + 2 * gx > 16384) c->sync_next = 0;
-        p.sync = c->d_sync + c->sync_next;
+        p->sync = c->d_sync + c->sync_next;
         c->sync_next += 2 * gx;
-        if (!make_partial_map(c, &tmP, ws, p.BN, (size_t)gx * p.tpc * p.splits * 128)) return PT_ERR_CUDA;
+        if (!make_partial_map(c, tmP, ws, w.acc_cols, (size_t)gx * w.apc * w.splits * 128)) return PT_ERR_CUDA;
     }
+    return wgrad_attr();
+}
+
+// Launches the weight-gradient kernel for a problem whose x operand is described by `tmX` (64 pixels x 64 channels boxes).
+pt_status run_wgrad(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const pt_wgrad_plan &w, int stride, int lo_h, int lo_w, const CUtensorMap &tmX,
+                    const void *dy, float *out, void *ws, size_t ws_bytes, cudaStream_t st, bool x_tiled = false)
+{
+    WgradP p;
+    CUtensorMap tmP;
+    const pt_status r0 = wgrad_common(c, d, P, Q, w, out, ws, ws_bytes, &p, &tmP);
+    if (r0 != PT_OK) return r0;
+    p.x_tiled = x_tiled ? 1 : 0;
+    p.pix_per_split = pt_ceil_div(pt_ceil_div(p.npix, p.splits), 64) * 64;
+    p.stride = stride; p.lo_h = lo_h; p.lo_w = lo_w;
+    const int gx = p.n_tiles * p.m_tiles * p.tap_groups;
     // A: dy as a 2-D tensor (K channels, N*P*Q pixels), box 64 channels x 64 pixels
     if (!c->encode_tiled) return PT_ERR_CUDA;
     CUtensorMap tmA;
@@ -2308,68 +2560,39 @@ pt_status run_wgrad(pt_ctx *c, const pt_conv_desc *d, int P, int Q, int stride, 
     p.stages = pick_stages(stage, pt_ceil_div(p.pix_per_split, 64), 0, &smem);
     if (smem < 2048 + 8 * 2 * 4096) smem = 2048 + 8 * 2 * 4096;        // the epilogue's staging slabs reuse the stage memory
     if (p.splits > 1 && smem < kSplitSmemFloor) smem = kSplitSmemFloor;
-    static bool attr_set = false;
-    if (!attr_set) {
-        PT_CUDA_OK(cudaFuncSetAttribute(conv_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
-        attr_set = true;
-    }
     dim3 grid((unsigned)gx, (unsigned)p.splits);
-    if (c->test_skip == 1 && p.splits > 1) { p.test_skip = 1; c->test_skip = 0; }
-    PT_CUDA_OK(launch_pdl(conv_wgrad_kernel, grid, dim3(kThreads), smem, st, tmA, tmX, tmP, p));
+    p.data_bytes = (unsigned)(smem - 2048);
+    PT_CUDA_OK(launch_wgrad(conv_wgrad_kernel, grid, p.cluster ? p.splits : 1, smem, st, tmA, tmX, tmP, p));
     c->launches += 1;
     PT_CUDA_OK(cudaGetLastError());
     return PT_OK;
 }
 
-// Launches the row-block weight-gradient kernel; PT_ERR_UNSUPPORTED (nothing launched) where the plan declines the shape.
+// Launches the row-block weight-gradient kernel.
 // `x_row_pixels` > 0 and (lo_h, lo_w): x is a view whose rows are x_row_pixels apart and whose raster origin for tap (0, 0)
 // is at (lo_h, lo_w) instead of (-pad, -pad) -- the space-to-depth stem, whose "pixels" are overlapping 4-pixel windows.
-pt_status run_wgrad_rows(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const void *x, const void *dy, float *out, void *ws,
+pt_status run_wgrad_rows(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const pt_wgrad_plan &wr, const void *x, const void *dy, float *out, void *ws,
                          size_t ws_bytes, cudaStream_t st, int x_row_pixels = 0, int lo_h = 0, int lo_w = 0)
 {
-    const WgRows wr = wgrad_rows_plan(c, d, P, Q);
-    if (!wr.ok || !c->encode_tiled) return PT_ERR_UNSUPPORTED;
+    if (!c->encode_tiled) return PT_ERR_CUDA;
     WgradP p;
-    memset(&p, 0, sizeof(p));
-    p.K = d->K; p.C = d->C; p.taps = d->R * d->S; p.S = d->S;
-    p.BN = wr.bn; p.n_tiles = wr.n_tiles; p.m_tiles = wr.m_tiles;
-    p.tpc = wr.tpc; p.tap_groups = wr.tap_groups;
-    p.pair = 1; p.apc = wr.apc; p.acc_cols = wr.acc_cols;
-    p.npix = d->N * P * Q;
-    p.splits = wr.splits;
-    p.Pd = P; p.Qd = Q; p.stride = 1; p.lo_h = -d->pad; p.lo_w = -d->pad;
+    CUtensorMap tmP, tmA, tmX;
+    const pt_status r0 = wgrad_common(c, d, P, Q, wr, out, ws, ws_bytes, &p, &tmP);
+    if (r0 != PT_OK) return r0;
+    p.pair = 1;
+    p.stride = 1; p.lo_h = -d->pad; p.lo_w = -d->pad;
     if (x_row_pixels > 0) { p.lo_h = lo_h; p.lo_w = lo_w; }
     p.nr = wr.nr; p.Wp = wr.Wp; p.RB = wr.RB; p.units = wr.units; p.units_per_split = wr.units_per_split;
     p.ksteps = wr.ksteps; p.nb_a = wr.nb_a; p.lo_span = d->R - 1; p.a_box = wr.a_box; p.b_box = wr.b_box;
     p.stages = wr.stages;
-    p.tmem_cols = pow2_cols(p.apc * p.acc_cols);
-    p.status = c->d_status;
-    p.out = out;
     const int gx = p.n_tiles * p.m_tiles * p.tap_groups;
-    CUtensorMap tmP, tmA, tmX;
-    memset(&tmP, 0, sizeof(tmP));
-    if (p.splits > 1) {
-        const size_t need = (size_t)gx * p.apc * p.splits * 128 * p.acc_cols * sizeof(float);
-        if (!ws || ws_bytes < need) return PT_ERR_WORKSPACE;
-        p.partial = (float *)ws;
-        if (2 * gx > 8192) return PT_ERR_UNSUPPORTED;
-        if (c->sync_next + 2 * gx > 16384) c->sync_next = 0;
-        p.sync = c->d_sync + c->sync_next;
-        c->sync_next += 2 * gx;
-        if (!make_partial_map(c, &tmP, ws, p.acc_cols, (size_t)gx * p.apc * p.splits * 128)) return PT_ERR_CUDA;
-    }
     // dy: box of nr rows x Wp columns (Wp > Q: the extra columns are out of bounds and read as zeros); x: the halo box
     if (!make_halo_in_map(c, &tmA, dy, d->K, Q, P, d->N, d->ldy, wr.Wp, wr.nr)) return PT_ERR_UNSUPPORTED;
     if (!make_halo_in_map(c, &tmX, x, d->C, d->W, d->H, d->N, d->ldx, wr.Wp, wr.nr + d->R - 1, kKC, x_row_pixels)) return PT_ERR_UNSUPPORTED;
-    static bool attr_set = false;
-    if (!attr_set) {
-        PT_CUDA_OK(cudaFuncSetAttribute(conv_wgrad_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
-        attr_set = true;
-    }
     dim3 grid((unsigned)gx, (unsigned)p.splits);
     const size_t smem = (p.splits > 1 && wr.smem < kSplitSmemFloor) ? kSplitSmemFloor : wr.smem;
-    if (c->test_skip == 1 && p.splits > 1) { p.test_skip = 1; c->test_skip = 0; }
-    PT_CUDA_OK(launch_pdl(conv_wgrad_rows_kernel, grid, dim3(kThreads), smem, st, tmA, tmX, tmP, p));
+    p.data_bytes = (unsigned)(smem - 2048);
+    PT_CUDA_OK(launch_wgrad(conv_wgrad_rows_kernel, grid, p.cluster ? p.splits : 1, smem, st, tmA, tmX, tmP, p));
     c->launches += 1;
     PT_CUDA_OK(cudaGetLastError());
     return PT_OK;
@@ -2497,21 +2720,11 @@ int pt_sm100_wgrad_ctas(const pt_ctx *c, const pt_conv_desc *d, int *waits)
     const StemPlan sp = stem_plan(d);
     pt_conv_desc v = sp.ok ? stem_virtual_desc(d, sp) : *d;
     const int P = sp.ok ? sp.P : pt_out_dim(d->H, d->R, d->stride, d->pad), Q = sp.ok ? sp.Q : pt_out_dim(d->W, d->S, d->stride, d->pad);
-    int tiles, splits;
     const pt_conv_desc vr = sp.ok ? stem_rows_desc(d, sp) : v;
-    const WgRows wr = wgrad_rows_plan(c, &vr, P, Q);
-    if (wr.ok) {
-        tiles = wr.n_tiles * wr.m_tiles * wr.tap_groups;
-        splits = wr.splits;
-    } else {
-        int n_tiles;
-        const int bn = tile_n(v.C, &n_tiles);
-        const int tpc = wgrad_taps_per_cta(v.R * v.S, bn);
-        tiles = pt_ceil_div(v.K, 128) * n_tiles * pt_ceil_div(v.R * v.S, tpc);
-        splits = wgrad_splits(c, &v, P, Q);
-    }
-    if (waits) *waits = splits > 1 ? 1 : 0;
-    return tiles * splits;
+    pt_wgrad_plan w = wgrad_plan(c, &vr, P, Q, sp.ok);
+    if (sp.ok && !w.rows) w = wgrad_plan(c, &v, P, Q);
+    if (waits) *waits = w.splits > 1 ? 1 : 0;
+    return w.n_tiles * w.m_tiles * w.tap_groups * w.splits;
 }
 
 size_t pt_sm100_conv_workspace(const pt_ctx *c, const pt_conv_desc *d, int which)
@@ -2520,12 +2733,12 @@ size_t pt_sm100_conv_workspace(const pt_ctx *c, const pt_conv_desc *d, int which
     if (sp.ok && which == PT_CONV_FWD) return sp.xs_bytes + pt_align_up(sp.w2_elems * 2, 1024);
     if (sp.ok && which == PT_CONV_WGRAD) {
         const pt_conv_desc v = stem_virtual_desc(d, sp), vr = stem_rows_desc(d, sp);
-        const size_t pa = wgrad_partial_bytes(c, &v, sp.P, sp.Q), pb = wgrad_partial_bytes(c, &vr, sp.P, sp.Q);
+        const size_t pa = wgrad_partial_bytes(wgrad_plan(c, &v, sp.P, sp.Q)), pb = wgrad_partial_bytes(wgrad_plan(c, &vr, sp.P, sp.Q, true));
         return sp.xs_bytes + pt_align_up(sp.w2_elems * 4, 1024) + (pa > pb ? pa : pb);
     }
     if (which != PT_CONV_WGRAD) return 0;
     const int P = pt_out_dim(d->H, d->R, d->stride, d->pad), Q = pt_out_dim(d->W, d->S, d->stride, d->pad);
-    return wgrad_partial_bytes(c, d, P, Q);
+    return wgrad_partial_bytes(wgrad_plan(c, d, P, Q));
 }
 
 pt_status pt_sm100_conv(pt_ctx *c, const pt_conv_desc *d, int which, const void *a, const void *b, void *out, void *ws,
@@ -2549,12 +2762,14 @@ pt_status pt_sm100_conv(pt_ctx *c, const pt_conv_desc *d, int which, const void 
             // the row-block kernel first: the windows of a unit of rows are staged once for all U vertical taps and two taps share
             // an MMA (M = 128 lanes where the generic kernel has 55 output channels on its M side)
             const pt_conv_desc vr = stem_rows_desc(d, sp);
-            pt_status r = run_wgrad_rows(c, &vr, sp.P, sp.Q, xs, b, dw2, part, ws_bytes - (size_t)(part - wsb), st, sp.Wp, -sp.pl, 0);
+            const pt_wgrad_plan wr = wgrad_plan(c, &vr, sp.P, sp.Q, true);
+            pt_status r = PT_ERR_UNSUPPORTED;
+            if (wr.rows) r = run_wgrad_rows(c, &vr, sp.P, sp.Q, wr, xs, b, dw2, part, ws_bytes - (size_t)(part - wsb), st, sp.Wp, -sp.pl, 0);
             if (r == PT_ERR_UNSUPPORTED) {
                 CUtensorMap tmX;
                 const int up_h = (sp.P - 1) - sp.pl - (sp.Hs - 1);
                 if (!make_im2col_map(c, &tmX, xs, 64, sp.Q, sp.Hs, d->N, 16, 0, -sp.pl, 0, up_h, 1, 64, sp.Wp)) return PT_ERR_CUDA;
-                r = run_wgrad(c, &v, sp.P, sp.Q, 1, -sp.pl, 0, tmX, b, dw2, part, ws_bytes - (size_t)(part - wsb), st);
+                r = run_wgrad(c, &v, sp.P, sp.Q, wgrad_plan(c, &v, sp.P, sp.Q), 1, -sp.pl, 0, tmX, b, dw2, part, ws_bytes - (size_t)(part - wsb), st);
             }
             if (r != PT_OK) return r;
             const int n = d->K * d->R * d->S * d->C;
@@ -2563,9 +2778,11 @@ pt_status pt_sm100_conv(pt_ctx *c, const pt_conv_desc *d, int which, const void 
             PT_CUDA_OK(cudaGetLastError());
             return PT_OK;
         }
-        {
-            const pt_status r = run_wgrad_rows(c, d, P, Q, a, b, (float *)out, ws, ws_bytes, st);
+        pt_wgrad_plan w = wgrad_plan(c, d, P, Q);
+        if (w.rows) {
+            const pt_status r = run_wgrad_rows(c, d, P, Q, w, a, b, (float *)out, ws, ws_bytes, st);
             if (r != PT_ERR_UNSUPPORTED) return r;
+            wgrad_gen_plan(c, d, P, Q, &w);
         }
         CUtensorMap tmX;
         const int up_w = (Q - 1) * d->stride - d->pad - (d->W - 1), up_h = (P - 1) * d->stride - d->pad - (d->H - 1);
@@ -2573,7 +2790,7 @@ pt_status pt_sm100_conv(pt_ctx *c, const pt_conv_desc *d, int which, const void 
         if (plain) {
             if (!make_act2d_map(c, &tmX, a, d->C, (long long)d->N * d->H * d->W, d->ldx, 64)) return PT_ERR_CUDA;
         } else if (!make_im2col_map(c, &tmX, a, d->C, d->W, d->H, d->N, d->ldx, -d->pad, -d->pad, up_w, up_h, d->stride, 64)) return PT_ERR_CUDA;
-        return run_wgrad(c, d, P, Q, d->stride, -d->pad, -d->pad, tmX, b, (float *)out, ws, ws_bytes, st, plain);
+        return run_wgrad(c, d, P, Q, w, d->stride, -d->pad, -d->pad, tmX, b, (float *)out, ws, ws_bytes, st, plain);
     }
 
     GemmP p;

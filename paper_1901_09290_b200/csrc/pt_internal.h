@@ -4,6 +4,7 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 #include <string.h>
+#include <mutex>
 #include <vector>
 
 #include "../../include/pt.h"
@@ -29,6 +30,17 @@ struct pt_region {              // one cached table in the arena
     size_t off = 0, cap = 0;    // byte range inside the arena
     std::vector<char> key;      // host bytes the current device copy was built from
     bool valid = false;
+};
+
+// Launch shape of a weight gradient. rows = 1: the row-block kernel (stride-1 filters with at most 64 input channels).
+struct pt_wgrad_plan {
+    int rows;
+    int bn, n_tiles, m_tiles, tpc, tap_groups, apc, acc_cols;
+    int splits, cluster;            // CTAs that share a tile's pixels; 1: they are one thread-block cluster
+    // row-block form
+    int nr, Wp, RB, units, units_per_split, ksteps, nb_a, stages;
+    unsigned a_box, b_box;
+    size_t stage_bytes, smem;
 };
 
 struct pt_ctx {
@@ -69,6 +81,16 @@ struct pt_ctx {
     float *stats_out = nullptr;
     size_t stats_cap = 0;
     int test_skip = 0;                  // pt_test_skip_next_arrive: 1 = next split weight gradient, 2 = next fwd/dgrad GEMM-form launch
+    // Plans of recent weight-gradient descriptors: choosing one walks a few hundred candidates (about 10 us), a call must not.
+    struct WgradSlot {
+        pt_conv_desc d;
+        int limit, P, Q;
+        bool valid = false;
+        pt_wgrad_plan plan;
+    };
+    mutable WgradSlot wgrad_slot[128];
+    mutable std::mutex wgrad_mutex;
+    mutable int max_clusters[9] = {0};  // co-resident weight-gradient clusters of 2..8 CTAs (0: not asked yet)
     // Helper streams for independent launches inside one call (the parity classes of a stride-2 data gradient): the caller's
     // stream forks to them and joins them back through events, which a stream capture records as graph edges.
     cudaStream_t fork_stream[3] = {nullptr, nullptr, nullptr};

@@ -150,6 +150,25 @@ __device__ __forceinline__ void prefetch_tmap(const CUtensorMap *tm)
     asm volatile("prefetch.tensormap [%0];" ::"l"(tm) : "memory");
 }
 
+// ---------------------------------------------------------------- thread-block clusters
+// Barrier of every thread of the cluster (a CTA that has left counts as arrived); what was written before it, to a peer's shared
+// memory too, is visible behind it.
+__device__ __forceinline__ void cluster_barrier()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// The shared-memory address `addr` of this CTA in the CTA of the given rank of the cluster.
+__device__ __forceinline__ uint32_t map_to_rank(uint32_t addr, uint32_t rank)
+{
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void st_cluster_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
+{
+    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+
 // ---------------------------------------------------------------- programmatic dependent launch
 // Blocks until every kernel this one depends on has completed and its memory operations are visible.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

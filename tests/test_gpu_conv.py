@@ -235,3 +235,30 @@ def test_tcgen05_path_takes_all_three_passes_when_forced(stride):
     with pytest.raises(B.PtError) as e:
         B.pt_conv_fwd(Hh.ctx(), d9, buf, buf, buf)
     assert e.value.status == 2
+
+
+# Weight gradients whose splits meet as a thread-block cluster: lane quarters that are partly or wholly empty (C or K just above and
+# below 32, 64 and 128), an odd last tap, one and several channel tiles, two to eight splits (the CTA limit), and accumulators larger
+# than the shared memory of the owners (several rounds: 8 x 512 columns)
+@pytest.mark.parametrize("N,H,C,K,R,stride", [(4, 12, 31, 33, 3, 1), (4, 12, 33, 129, 3, 1), (8, 9, 64, 256, 3, 1), (5, 10, 65, 127, 3, 1),
+                                              (6, 14, 300, 260, 1, 1), (8, 15, 128, 96, 3, 2), (16, 8, 256, 128, 1, 1), (3, 28, 40, 20, 1, 1)])
+def test_weight_gradient_splits_as_a_cluster(N, H, C, K, R, stride):
+    c = Hh.ctx()
+    x, w, dy, pad = _case(N, H, H, C, K, R, stride, W.BASE_SEED + C)
+    ref = oracle.conv_wgrad(x.numpy(), dy.numpy(), R, R, stride, pad)
+    d = B.make_conv_desc(N, H, H, C, K, R, R, stride, pad, algo=2)
+    xd, dyd = Hh.to_dev_padded(x, d.ldx), Hh.to_dev_padded(dy, d.ldy)
+    try:
+        for lim in (0, 2, 7, 40):
+            B.pt_set_wgrad_cta_limit(c, lim)
+            dw = torch.full((K, R, R, C), 7680.0, device="cuda")
+            B.pt_conv_wgrad(c, d, xd, dyd, dw, Hh.conv_ws(d, B.PT_CONV_WGRAD))
+            torch.cuda.synchronize()
+            c.poll()
+            Hh.check_conv(dw, C, ref, what=f"wgrad at limit {lim}")
+            again = torch.full_like(dw, 7680.0)
+            B.pt_conv_wgrad(c, d, xd, dyd, again, Hh.conv_ws(d, B.PT_CONV_WGRAD))
+            torch.cuda.synchronize()
+            assert torch.equal(dw, again)                        # fixed order of the sums
+    finally:
+        B.pt_set_wgrad_cta_limit(c, 0)
