@@ -372,6 +372,12 @@ typedef struct {
  * the kept indices in ascending order (entries past the count are -1); new_sizes (HOST, n_spaces) receives the
  * counts. This call synchronises `stream` once to return the counts. A count of 0 is reported, not clamped. */
 pt_status pt_reconfigure_plan(pt_ctx *ctx, const pt_graph *g, int32_t *new2old, int32_t *new_sizes /*host*/, void *stream);
+/* The same in two calls, for a caller that has more work to enqueue behind the plan: the first enqueues it and returns, the second
+ * waits for the counts of the context's last plan (n_spaces as in its graph; stream: the one it was enqueued on). A training loop that
+ * expects the sizes it allocated for can enqueue the gather and the whole step between the two and check the counts afterwards: the
+ * GPU does not idle while the host wakes up. PT_ERR_INVALID_ARG if no plan was enqueued or n_spaces differs. */
+pt_status pt_reconfigure_plan_enqueue(pt_ctx *ctx, const pt_graph *g, int32_t *new2old, void *stream);
+pt_status pt_reconfigure_plan_wait(pt_ctx *ctx, int32_t n_spaces, int32_t *new_sizes /*host*/, void *stream);
 
 /* Phase 1. Gather every layer of old_g into the caller-allocated tensors of new_g:
  *   new.w[k',rs,c'] = old.w[new2old_out[k'], rs, new2old_in[c']]   (same for v and the bf16 shadow, bit for bit)

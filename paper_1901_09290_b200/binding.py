@@ -120,6 +120,8 @@ EXPORTS = {
     "pt_channel_scatter_add": (c_int32, [c_void_p, c_void_p, c_int32, c_void_p, c_int32, c_void_p, c_void_p, c_int32, c_int32, c_int64,
                                          c_int32, c_void_p]),
     "pt_reconfigure_plan": (c_int32, [c_void_p, POINTER(pt_graph), c_void_p, POINTER(c_int32), c_void_p]),
+    "pt_reconfigure_plan_enqueue": (c_int32, [c_void_p, POINTER(pt_graph), c_void_p, c_void_p]),
+    "pt_reconfigure_plan_wait": (c_int32, [c_void_p, c_int32, POINTER(c_int32), c_void_p]),
     "pt_reconfigure": (c_int32, [c_void_p, POINTER(pt_graph), c_void_p, POINTER(pt_graph), c_void_p]),
 }
 
@@ -442,6 +444,17 @@ def pt_reconfigure_plan(ctx, graph: GraphHandle, new2old, stream=None) -> List[i
     sizes = (c_int32 * n)()
     _check(lib().pt_reconfigure_plan(ctx.handle, byref(graph.graph), _ptr(new2old), sizes, _stream(stream)),
            "pt_reconfigure_plan")
+    return list(sizes)
+
+
+def pt_reconfigure_plan_enqueue(ctx, graph: GraphHandle, new2old, stream=None):
+    _check(lib().pt_reconfigure_plan_enqueue(ctx.handle, byref(graph.graph), _ptr(new2old), _stream(stream)), "pt_reconfigure_plan_enqueue")
+
+
+def pt_reconfigure_plan_wait(ctx, graph: GraphHandle, stream=None) -> List[int]:
+    n = graph.graph.n_spaces
+    sizes = (c_int32 * n)()
+    _check(lib().pt_reconfigure_plan_wait(ctx.handle, n, sizes, _stream(stream)), "pt_reconfigure_plan_wait")
     return list(sizes)
 
 

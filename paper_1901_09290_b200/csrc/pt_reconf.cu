@@ -204,9 +204,9 @@ pt_status check_graph(const pt_graph *g)
 
 }  // namespace
 
-extern "C" pt_status pt_reconfigure_plan(pt_ctx *c, const pt_graph *g, int32_t *new2old, int32_t *new_sizes, void *stream)
+extern "C" pt_status pt_reconfigure_plan_enqueue(pt_ctx *c, const pt_graph *g, int32_t *new2old, void *stream)
 {
-    if (!c || !new2old || !new_sizes) return PT_ERR_INVALID_ARG;
+    if (!c || !new2old) return PT_ERR_INVALID_ARG;
     pt_status s = check_graph(g);
     if (s != PT_OK) return s;
     if (g->n_spaces > 65536) return PT_ERR_UNSUPPORTED;
@@ -257,28 +257,44 @@ extern "C" pt_status pt_reconfigure_plan(pt_ctx *c, const pt_graph *g, int32_t *
                                   (volatile int32_t *)counts, (volatile unsigned int *)flag, seq, c->d_status + 2));
     c->launches += 1;
     PT_CUDA_OK(cudaGetLastError());
-    // The documented synchronisation: the host needs the new sizes. It waits for the kernel's flag (bounded), looking at the
-    // stream now and then so that an error upstream ends the wait.
-    {
-        const auto t0 = std::chrono::steady_clock::now();
-        unsigned spins = 0;
-        bool seen = false;
-        while (!(seen = (*flag == seq))) {
-            if ((++spins & 0x3fffu) == 0u) {
-                const cudaError_t q = cudaStreamQuery(st);
-                if (q == cudaSuccess) { seen = (*flag == seq); break; }
-                if (q != cudaErrorNotReady) { (void)cudaGetLastError(); return PT_ERR_CUDA; }
-                if (std::chrono::steady_clock::now() - t0 > std::chrono::seconds(30)) break;
-            }
-        }
-        if (!seen) {
-            PT_CUDA_OK(cudaStreamSynchronize(st));
-            if (*flag != seq) return PT_ERR_CUDA;
+    c->plan_spaces = g->n_spaces;
+    return PT_OK;
+}
+
+// The documented synchronisation: the host needs the new sizes. It waits for the kernel's flag (bounded), looking at the
+// stream now and then so that an error upstream ends the wait.
+extern "C" pt_status pt_reconfigure_plan_wait(pt_ctx *c, int32_t n_spaces, int32_t *new_sizes, void *stream)
+{
+    if (!c || !new_sizes || n_spaces < 1 || c->plan_spaces != n_spaces) return PT_ERR_INVALID_ARG;
+    cudaStream_t st = (cudaStream_t)stream;
+    const volatile unsigned int *flag = (const volatile unsigned int *)c->h_counts;
+    const volatile int32_t *counts = (const volatile int32_t *)c->h_counts + 16;
+    const unsigned int seq = c->plan_seq;
+    const auto t0 = std::chrono::steady_clock::now();
+    unsigned spins = 0;
+    bool seen = false;
+    while (!(seen = (*flag == seq))) {
+        if ((++spins & 0x3fffu) == 0u) {
+            const cudaError_t q = cudaStreamQuery(st);
+            if (q == cudaSuccess) { seen = (*flag == seq); break; }
+            if (q != cudaErrorNotReady) { (void)cudaGetLastError(); return PT_ERR_CUDA; }
+            if (std::chrono::steady_clock::now() - t0 > std::chrono::seconds(30)) break;
         }
     }
+    if (!seen) {
+        PT_CUDA_OK(cudaStreamSynchronize(st));
+        if (*flag != seq) return PT_ERR_CUDA;
+    }
     std::atomic_thread_fence(std::memory_order_acquire);
-    for (int i = 0; i < g->n_spaces; ++i) new_sizes[i] = counts[i];
+    for (int i = 0; i < n_spaces; ++i) new_sizes[i] = counts[i];
     return PT_OK;
+}
+
+extern "C" pt_status pt_reconfigure_plan(pt_ctx *c, const pt_graph *g, int32_t *new2old, int32_t *new_sizes, void *stream)
+{
+    if (!new_sizes) return PT_ERR_INVALID_ARG;
+    const pt_status s = pt_reconfigure_plan_enqueue(c, g, new2old, stream);
+    return s != PT_OK ? s : pt_reconfigure_plan_wait(c, g->n_spaces, new_sizes, stream);
 }
 
 extern "C" pt_status pt_reconfigure(pt_ctx *c, const pt_graph *og, const int32_t *new2old, const pt_graph *ng, void *stream)

@@ -284,7 +284,9 @@ class TrainStep:
         """Detection and keep-set scan: everything up to (and including) the host synchronisation that returns the new sizes."""
         c = self.ctx
         B.pt_find_zero_groups(c, self.md.arr, 1e-4, False, self.md.ws, stream)
-        sizes = B.pt_reconfigure_plan(c, self.md.graph(), self.new2old, stream)
+        self._check_sizes(B.pt_reconfigure_plan(c, self.md.graph(), self.new2old, stream))
+
+    def _check_sizes(self, sizes):
         if sizes != self.counts:
             raise RuntimeError(f"reconfiguration plan returned {sizes}, expected {self.counts}")
 
@@ -473,8 +475,13 @@ class TrainStep:
         return self.graph
 
     def step(self, stream=None, before_train=None):
-        if getattr(self, "graph", None) is not None and getattr(self, "_graph_has_gather", False):
-            self.reconfigure_plan(stream)                 # the gather is part of the graph (in two parts, beside the first layers)
+        # With the gather inside the graph (in two parts, beside the first layers) nothing of the step needs the host before the sizes are
+        # checked: the whole step is enqueued first, so that the GPU goes from the plan to the gather without waiting for the host to
+        # wake up and launch a graph of ~180 nodes (60 to 90 us of the step). A plan that disagrees raises as before.
+        ahead = getattr(self, "graph", None) is not None and getattr(self, "_graph_has_gather", False)
+        if ahead:
+            B.pt_find_zero_groups(self.ctx, self.md.arr, 1e-4, False, self.md.ws, stream)
+            B.pt_reconfigure_plan_enqueue(self.ctx, self.md.graph(), self.new2old, stream)
         else:
             self.reconfigure(stream)
         if before_train is not None:
@@ -484,6 +491,8 @@ class TrainStep:
             if not self._graph_has_update:
                 allreduce_mean(self.mp.g_flat, self.world)       # the one exchange of a data-parallel step
                 self.lasso(stream)
+            if ahead:
+                self._check_sizes(B.pt_reconfigure_plan_wait(self.ctx, self.md.graph(), stream))
         else:
             self.train(stream)
 
