@@ -58,8 +58,8 @@ extern "C" pt_status pt_create(pt_ctx **out, int device)
     // pinned memory comes back from an earlier context with what it held: a flag left there must not look like this context's first plan
     memset(c->h_counts, 0, (65536 + 16) * sizeof(int32_t));
     size_t off = 0;
-    for (int i = 0; i < 3; ++i) { c->lasso_tab[i].off = off; c->lasso_tab[i].cap = kSlotBytes; off += kSlotBytes; }
-    for (int i = 0; i < 2; ++i) { c->detect_tab[i].off = off; c->detect_tab[i].cap = kSlotBytes; off += kSlotBytes; }
+    for (int i = 0; i < 3; ++i) { c->lasso_tab[i].reg.off = off; c->lasso_tab[i].reg.cap = kSlotBytes; off += kSlotBytes; }
+    for (int i = 0; i < 2; ++i) { c->detect_tab[i].reg.off = off; c->detect_tab[i].reg.cap = kSlotBytes; off += kSlotBytes; }
     c->graph_tab.off = off;  c->graph_tab.cap = kSlotBytes; off += kSlotBytes;
     for (int i = 0; i < 4; ++i) { c->gather_slot[i].reg.off = off; c->gather_slot[i].reg.cap = kSlotBytes; off += kSlotBytes; }
     // Driver entry points for tensor-map encoding, looked up at run time so the library loads without libcuda.
@@ -156,17 +156,6 @@ pt_status pt_upload_table(pt_ctx *c, pt_region *reg, const void *host, size_t by
     reg->key.assign((const char *)host, (const char *)host + bytes);
     reg->valid = true;
     return PT_OK;
-}
-
-pt_status pt_upload_table_slots(pt_ctx *c, pt_region *slots, int n_slots, int *next, const void *host, size_t bytes,
-                                cudaStream_t st, char **dev)
-{
-    for (int i = 0; i < n_slots; ++i)
-        if (slots[i].valid && slots[i].key.size() == bytes && memcmp(slots[i].key.data(), host, bytes) == 0)
-            return pt_upload_table(c, &slots[i], host, bytes, st, dev);
-    pt_region *victim = &slots[*next % n_slots];
-    *next = (*next + 1) % n_slots;
-    return pt_upload_table(c, victim, host, bytes, st, dev);
 }
 
 // ------------------------------------------------------------------------------------------ conv dispatch

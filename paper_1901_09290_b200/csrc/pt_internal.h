@@ -32,6 +32,17 @@ struct pt_region {              // one cached table in the arena
     bool valid = false;
 };
 
+// One cached table of the lasso step or the detection: the layers array it was built from, and what the launches need to know of it.
+struct pt_group_slot {
+    pt_region reg;
+    std::vector<char> args;
+    size_t chunks_off = 0, jobs_off = 0;
+    unsigned n_chunks = 0, n_jobs = 0;
+    bool small = false;
+    std::vector<int> first_chunk;
+    size_t ws[10];                  // offsets of the workspace's parts
+};
+
 // Launch shape of a weight gradient. rows = 1: the row-block kernel (stride-1 filters with at most 64 input channels).
 struct pt_wgrad_plan {
     int rows;
@@ -56,7 +67,8 @@ struct pt_ctx {
     bool upload_pending = false;
     // Cached device tables. A captured CUDA graph embeds the device address of the table its kernels read, so tables of
     // different callers must not evict each other: the lasso step and the detection have their own slot sets.
-    pt_region lasso_tab[3], detect_tab[2], graph_tab;
+    pt_group_slot lasso_tab[3], detect_tab[2];
+    pt_region graph_tab;
     int lasso_next = 0, detect_next = 0;
     // pt_reconfigure: four cached gather tables, each with the argument bytes it was built from and its launch shape. A call
     // with the same arguments (every reconfiguration of a fixed pair of models, or of a fixed part of them) launches straight
@@ -64,8 +76,8 @@ struct pt_ctx {
     struct GatherSlot {
         pt_region reg;
         std::vector<char> args;
-        unsigned chunks = 0, grid = 0;
-        size_t jobs_bytes = 0, first_off = 0;
+        unsigned chunks = 0;
+        size_t jobs_bytes = 0;
     } gather_slot[4];
     int gather_next = 0;
     int32_t *h_counts = nullptr;        // pinned, for pt_reconfigure_plan: [0] = flag the kernel raises, [16..] = counts
@@ -127,10 +139,6 @@ cudaError_t pt_launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_
 // Copies `bytes` of host data into the region's slot of the arena if it differs from what is there.
 // Returns the device address of the slot.
 pt_status pt_upload_table(pt_ctx *ctx, pt_region *reg, const void *host, size_t bytes, cudaStream_t st, char **dev);
-// Same over a set of slots: a slot already holding these bytes is reused, otherwise the oldest one is overwritten.
-pt_status pt_upload_table_slots(pt_ctx *ctx, pt_region *slots, int n_slots, int *next, const void *host, size_t bytes,
-                                cudaStream_t st, char **dev);
-
 // Validation shared by the conv entry points. Fills P, Q.
 pt_status pt_conv_validate(const pt_ctx *ctx, const pt_conv_desc *d, int *P, int *Q);
 
