@@ -607,8 +607,10 @@ struct HaloP {
     int stages_a, stages_b, resident;    // ring depths; resident: weights loaded once
     int n_issuers, acc_per;              // MMA issuer warps (each with its own A ring of stages_a / n_issuers stages); accumulators per issuer (1 or 2)
     int shared_b;                        // two pipelines fed by ONE weight stream: a stage is read by both issuers (their tiles of a round)
-    int row32;                           // 1: 16 channel lanes per pixel, 32-byte rows and swizzle (the space-to-depth stem): one MMA per tap
-    int b_slot, b_rows, staging;         // bytes reserved per weight tile, rows a K-major weight box brings, bytes of an epilogue group's staging slab
+    int lanes;                           // channel lanes per staged pixel: 64, 32 or 16 (128-, 64- or 32-byte rows and swizzle)
+    int direct;                          // 1: at most 32 output channels, stored from registers (no staging)
+    int b_slot, b_rows, staging, slabs;  // bytes reserved per weight tile, rows a K-major weight box brings, bytes and number of an epilogue group's staging slabs
+    int direct_cols;                     // channels the direct stores cover (whole 16-byte vectors)
     int tmem_cols, tma_store, out_f32, ld_out;
     int oH, oW, o_step, o_h0, o_w0;      // direct stores: raster (n, i, j) -> out[((n*oH + i*o_step + o_h0)*oW + j*o_step + o_w0)*ld_out]
     int stats_off;                       // byte offset in shared memory of the epilogue warps' statistics accumulators
@@ -621,6 +623,7 @@ struct HaloP {
 };
 
 constexpr int kHaloMaxIssuers = 4;
+constexpr int kHaloMaxA = 8;             // activation stages: two per issuer (three measured the same or 2 us slower)
 
 // Coordinates of the tiles t0, t0 + D, t0 + 2D, ... of a halo launch, advanced without integer divisions (a division costs
 // a single issuing thread ~150 cycles, and the smallest tiles are only a few hundred cycles of work).
@@ -656,7 +659,7 @@ __device__ unsigned long long g_halo_trace[8][64];
 #endif
 
 struct __align__(8) HCtl {
-    uint64_t full_a[4], empty_a[4];
+    uint64_t full_a[kHaloMaxA], empty_a[kHaloMaxA];
     uint64_t full_b[kMaxStages], empty_b[kMaxStages];
     uint64_t w_full;
     uint64_t acc_full[2 * kHaloMaxIssuers], acc_empty[2 * kHaloMaxIssuers];
@@ -683,9 +686,10 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
     HCtl *ctl = reinterpret_cast<HCtl *>(smem_raw);
     const uint32_t smem_base = smem_u32(smem_raw);
     const uint32_t staging_base = (smem_base + (uint32_t)sizeof(HCtl) + 1023u) & ~1023u;
-    const uint32_t b_base = staging_base + 2u * (uint32_t)p.staging;
+    const uint32_t b_base = staging_base + 2u * (uint32_t)(p.slabs * p.staging);
     // bytes one weight tile brings: a K-major tile only holds the rows (output channels) that exist
-    const uint32_t b_bytes = B_MN ? (uint32_t)((p.BN + 63) / 64) * 8192u : (uint32_t)p.b_rows * (p.row32 ? 32u : 128u);
+    const uint32_t row_bytes = (uint32_t)p.lanes * 2u, b_block = (uint32_t)p.lanes * 128u;   // (an MN-major block: 64 columns x `lanes` rows)
+    const uint32_t b_bytes = B_MN ? (uint32_t)((p.BN + 63) / 64) * b_block : (uint32_t)p.b_rows * row_bytes;
     const uint32_t b_slot = (uint32_t)p.b_slot;
     const uint32_t n_bslots = p.resident ? (uint32_t)(p.taps * p.k_chunks) : (uint32_t)p.stages_b;
     const uint32_t a_base = b_base + n_bslots * b_slot;
@@ -707,7 +711,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
         prefetch_tmap(&tmB);
         if (p.tma_store) prefetch_tmap(&tmC);
     }
-    if (threadIdx.x < p.taps) ctl->tap_aoff[threadIdx.x] = (uint32_t)(p.tap_oh[threadIdx.x] * p.Wp + p.tap_ow[threadIdx.x]) * (p.row32 ? 2u : 8u);
+    if (threadIdx.x < p.taps) ctl->tap_aoff[threadIdx.x] = (uint32_t)(p.tap_oh[threadIdx.x] * p.Wp + p.tap_ow[threadIdx.x]) * (row_bytes >> 4);
     if (warp == 1) {
         tmem_alloc(smem_u32(&ctl->tmem_base), (uint32_t)p.tmem_cols);
         tmem_relinquish();
@@ -747,7 +751,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
                         const uint32_t dst = b_base + (uint32_t)(tap * p.k_chunks + kc) * b_slot;
                         const int wtap = p.tap_wt[tap];
                         if (!B_MN) tma_load_3d(dst, &tmB, bar, kc * kKC, wtap, 0);
-                        else for (int nb = 0; nb < (p.BN + 63) / 64; ++nb) tma_load_3d(dst + (uint32_t)nb * 8192u, &tmB, bar, nb * 64, wtap, kc * kKC);
+                        else for (int nb = 0; nb < (p.BN + 63) / 64; ++nb) tma_load_3d(dst + (uint32_t)nb * b_block, &tmB, bar, nb * 64, wtap, kc * kKC);
                     }
             }
             bool dep_waited = false;             // the activations are the previous kernel's output
@@ -787,7 +791,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
                         const int wtap = p.tap_wt[tap];
                         mbar_arrive_expect_tx(bbar, b_bytes);
                         if (!B_MN) tma_load_3d(dst, &tmB, bbar, kc * kKC, wtap, n0);
-                        else for (int nb = 0; nb < (p.BN + 63) / 64; ++nb) tma_load_3d(dst + (uint32_t)nb * 8192u, &tmB, bbar, n0 + nb * 64, wtap, kc * kKC);
+                        else for (int nb = 0; nb < (p.BN + 63) / 64; ++nb) tma_load_3d(dst + (uint32_t)nb * b_block, &tmB, bbar, n0 + nb * 64, wtap, kc * kKC);
                     }
                 }
                 if (!ok) break;
@@ -813,7 +817,6 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
         const uint32_t leader = lane == 0 ? 1u : 0u;
         const uint32_t idesc = make_idesc_bf16(kBM, p.BN, 0, B_MN ? 1 : 0);
         const uint64_t bstep = B_MN ? 128ull : 2ull;
-        const uint32_t b_lbo = B_MN ? 8192u : 16u;
         int sb_pos = 0, sb_ph = 0;                            // position in this issuer's weight ring
         int s_loc = 0, pha = 0;                               // position in this issuer's A ring
         bool ok = true;
@@ -850,21 +853,17 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
                 tc_fence_after();
                 const int rem = p.c_red - kc * kKC;
                 const int ksteps = rem >= kKC ? 4 : (rem + 15) / 16;
-                const uint64_t abase = make_desc(a_base + (uint32_t)sa * (uint32_t)p.a_alloc, 16u, 1024u);
-                if (p.row32) {
-                    // 32-byte rows: a pixel's 16 lanes are one K step, so a tap is a single MMA on the row-shifted tile
-                    const uint64_t a32 = make_desc_sw32(a_base + (uint32_t)sa * (uint32_t)p.a_alloc, 256u);
-                    uint64_t b32 = make_desc_sw32(b_base, 256u);
-                    const uint64_t b_tap_step = (uint64_t)(b_slot >> 4);
-                    for (int tap = 0; tap < p.taps; ++tap, b32 += b_tap_step) {
-                        umma_bf16_lead(d_tmem, a32 + ctl->tap_aoff[tap], b32, idesc, accumulate, leader);
-                        accumulate = 1u;
-                    }
-                } else if (p.resident) {
+                const uint64_t abase = make_desc_rows(a_base + (uint32_t)sa * (uint32_t)p.a_alloc, row_bytes);
+                if (p.resident) {
                     // every tap is the same A tile read through a descriptor that starts (r*Wp + s) rows further on
-                    uint64_t bd0 = make_desc(b_base + (uint32_t)kc * b_slot, b_lbo, 1024u);
+                    uint64_t bd0 = B_MN ? make_desc(b_base + (uint32_t)kc * b_slot, b_block, 1024u) : make_desc_rows(b_base + (uint32_t)kc * b_slot, row_bytes);
                     const uint64_t b_tap_step = (uint64_t)(((uint32_t)p.k_chunks * b_slot) >> 4);
-                    if (ksteps == 4) {
+                    if (ksteps == 1) {
+                        for (int tap = 0; tap < p.taps; ++tap, bd0 += b_tap_step) {
+                            umma_bf16_lead(d_tmem, abase + ctl->tap_aoff[tap], bd0, idesc, accumulate, leader);
+                            accumulate = 1u;
+                        }
+                    } else if (ksteps == 4) {
                         for (int tap = 0; tap < p.taps; ++tap, bd0 += b_tap_step) {
                             const uint64_t ad0 = abase + ctl->tap_aoff[tap];
 #pragma unroll
@@ -884,7 +883,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
                         if (!ok) break;
                         tc_fence_after();
                         const uint64_t ad0 = abase + ctl->tap_aoff[tap];
-                        const uint64_t bd0 = make_desc(b_base + (uint32_t)sb * b_slot, b_lbo, 1024u);
+                        const uint64_t bd0 = B_MN ? make_desc(b_base + (uint32_t)sb * b_slot, b_block, 1024u) : make_desc_rows(b_base + (uint32_t)sb * b_slot, row_bytes);
 #pragma unroll
                         for (int k = 0; k < 4; ++k)
                             if (k < ksteps) { umma_bf16_lead(d_tmem, ad0 + 2ull * k, bd0 + bstep * k, idesc, accumulate, leader); accumulate = 1u; }
@@ -901,7 +900,11 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
         // ---------------- epilogue: group g (four warps) drains the accumulator buffers of its parity
         const int quarter = warp & 3, group = (warp - 2) >> 2;
         const int gtid = (warp - 2 - group * 4) * 32 + lane;         // 0..127 within the group
-        const uint32_t slab = staging_base + (uint32_t)group * (uint32_t)p.staging;
+        // this thread's raster position: its output row within the tile and its column
+        const int m = quarter * 32 + lane, ri = m / p.Wp, rj = m - ri * p.Wp;
+        const bool on_raster = m < p.nr * p.Wp && rj < p.Q;
+        uint32_t slab = staging_base + (uint32_t)(group * p.slabs) * (uint32_t)p.staging;
+        int sl = 0;
         // statistics: accumulated over the warp's tiles in shared memory, combined at the end
         const uint32_t st_acc = smem_base + (uint32_t)p.stats_off + (uint32_t)(warp - 2) * (uint32_t)p.stats_warp;
         if (STATS && p.stats) {
@@ -925,11 +928,13 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
             if (gtid == 0) HTRACE(4, tc);
             tc_fence_after();
             const uint32_t lane_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * p.BN);
-            const int m = quarter * 32 + lane;                       // raster position of this thread's accumulator row
             if (p.tma_store) {
                 const int n_chunks = (p.BN + 63) / 64;
                 for (int ch = 0; ch < n_chunks; ++ch) {
-                    if (gtid == 0) tma_store_wait_read();            // the slab's previous store has read it
+                    if (gtid == 0) {                                 // the slab's previous store has read it
+                        if (p.slabs == 2) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+                        else tma_store_wait_read();
+                    }
                     if (gtid == 0) HTRACE(5, tc);
                     named_barrier(1 + group, 128);
                     const int groups = min(4, (p.BN - ch * 64) / 16);
@@ -972,17 +977,42 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
                     }
                     if (STATS && p.stats) {
                         // this thread's raster position is a real output pixel iff it lies inside the row and the image
-                        const int ri = m / p.Wp, rj = m - ri * p.Wp;
-                        const uint32_t rows = __ballot_sync(0xffffffffu, m < p.nr * p.Wp && rj < p.Q && p0 + ri < p.P);
+                        const uint32_t rows = __ballot_sync(0xffffffffu, on_raster && p0 + ri < p.P);
                         chunk_stats(slab, quarter * 32, rows, lane, st_acc + (uint32_t)ch * 512u);
                     }
+                    if (p.slabs == 2) { slab = sl ? slab - (uint32_t)p.staging : slab + (uint32_t)p.staging; sl ^= 1; }
                 }
                 continue;
             }
-            // ---- direct stores (fp32 outputs)
-            const int i = m / p.Wp, j = m - i * p.Wp;
-            const bool row_ok = m < p.nr * p.Wp && j < p.Q && p0 + i < p.P;
-            const size_t row_off = ((size_t)(img * p.oH + (p0 + i) * p.o_step + p.o_h0) * p.oW + j * p.o_step + p.o_w0) * (size_t)p.ld_out;
+            // ---- direct stores (fp32 outputs, narrow bf16 outputs)
+            const bool row_ok = on_raster && p0 + ri < p.P;
+            const size_t row_off = ((size_t)(img * p.oH + (p0 + ri) * p.o_step + p.o_h0) * p.oW + rj * p.o_step + p.o_w0) * (size_t)p.ld_out;
+            if (p.direct) {
+                // a pixel's channels are 32 or 64 consecutive bytes: whole sectors from one thread, with no barrier among the warps and
+                // no store to wait for before the next tile (whose staging made a tile cost 0.5 us however little it held)
+                uint32_t v[2][16];
+                tmem_ld16(lane_addr, v[0]);
+                if (p.BN > 16) tmem_ld16(lane_addr + 16u, v[1]);
+                tmem_ld_wait();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&ctl->acc_empty[b]));
+                if (!row_ok) continue;
+                __nv_bfloat16 *o = (__nv_bfloat16 *)p.out + row_off;
+#pragma unroll
+                for (int q8 = 0; q8 < 4; ++q8) {
+                    const uint32_t (&e)[16] = v[q8 >> 1];
+                    const int h8 = (q8 & 1) * 8;
+                    if (q8 * 8 >= p.direct_cols) continue;
+                    __nv_bfloat162 b0 = __floats2bfloat162_rn(__uint_as_float(e[h8 + 0]), __uint_as_float(e[h8 + 1]));
+                    __nv_bfloat162 b1 = __floats2bfloat162_rn(__uint_as_float(e[h8 + 2]), __uint_as_float(e[h8 + 3]));
+                    __nv_bfloat162 b2 = __floats2bfloat162_rn(__uint_as_float(e[h8 + 4]), __uint_as_float(e[h8 + 5]));
+                    __nv_bfloat162 b3 = __floats2bfloat162_rn(__uint_as_float(e[h8 + 6]), __uint_as_float(e[h8 + 7]));
+                    *reinterpret_cast<uint4 *>(o + q8 * 8) = make_uint4(*reinterpret_cast<uint32_t *>(&b0), *reinterpret_cast<uint32_t *>(&b1),
+                                                                        *reinterpret_cast<uint32_t *>(&b2), *reinterpret_cast<uint32_t *>(&b3));
+                }
+                continue;
+            }
             for (int c0 = 0; c0 < p.BN; c0 += 16) {
                 uint32_t v[16];
                 tmem_ld16(lane_addr + (uint32_t)c0, v);
@@ -1328,7 +1358,8 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, const CUtensorMap 
         // The partial tiles sit in L2; what costs time is a chain of dependent loads, so every thread first issues the
         // asynchronous 16-byte copies of its items for ALL splits into the (now idle) stage memory, and only then are the
         // copies summed from shared memory in ascending split order: deterministic, whichever CTA does the work.
-        // In the paired form an item's row varies fastest: its lanes then write consecutive floats of dw (rows are input channels).
+        // (Consecutive items run along a row in both forms: the partial tiles are then read whole sectors at a time. In the paired form
+        // that scatters the writes to dw, but there are as many partial tiles to read as splits: 33 -> 31 us for 46 -> 59 at 56x56.)
         const int rows_real = p.pair ? 2 * p.C : min(128, p.K - k0);
         const int ngrp = pt_ceil_div_dev(p.pair ? p.K : min(acc_cols, p.C - c0), 4);     // float4 groups per row
         const int items = rows_real * ngrp;
@@ -1338,11 +1369,12 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, const CUtensorMap 
         const size_t zstride = (size_t)128 * acc_cols;
         const float *pbase = p.partial + (size_t)blockIdx.x * p.apc * p.splits * zstride;
         const int cap = (int)(((size_t)ring_bytes) / ((size_t)p.splits * 16));   // items the stage memory holds
-        const float inv_items = 1.0f / (float)items, inv_ngrp = 1.0f / (float)ngrp, inv_rows = 1.0f / (float)rows_real;
+        const float inv_items = 1.0f / (float)items, inv_ngrp = 1.0f / (float)ngrp;
         // row of the partial tile and first column of an item
         auto place = [&](int item, int &r, int &col) {
             if (p.pair) {
-                const int gq = fast_div(item, rows_real, inv_rows), rr = item - gq * rows_real;
+                const int rr = fast_div(item, ngrp, inv_ngrp);
+                const int gq = item - rr * ngrp;
                 r = rr >= p.C ? 64 + rr - p.C : rr;
                 col = gq * 4;
             } else {
@@ -1877,16 +1909,21 @@ bool make_act2d_map(const pt_ctx *c, CUtensorMap *tm, const void *base, int C, l
     return map_ok(r, __LINE__);
 }
 
-// bf16 weight shadow as (C, R*S, K) with row pitch ldw: box (64, 1, box_k).
-bool make_weight_map(const pt_ctx *c, CUtensorMap *tm, const void *base, int C, int RS, int K, int ldw, int box_k)
+CUtensorMapSwizzle lanes_swizzle(int lanes)
+{
+    return lanes == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : lanes == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B;
+}
+
+// bf16 weight shadow as (C, R*S, K) with row pitch ldw: box (lanes, 1, box_k).
+bool make_weight_map(const pt_ctx *c, CUtensorMap *tm, const void *base, int C, int RS, int K, int ldw, int box_k, int lanes = kKC)
 {
     if (!c->encode_tiled) return false;
     cuuint64_t dims[3] = {(cuuint64_t)C, (cuuint64_t)RS, (cuuint64_t)K};
     cuuint64_t strides[2] = {(cuuint64_t)ldw * 2, (cuuint64_t)RS * ldw * 2};
-    cuuint32_t box[3] = {(cuuint32_t)kKC, 1, (cuuint32_t)box_k};
+    cuuint32_t box[3] = {(cuuint32_t)lanes, 1, (cuuint32_t)box_k};
     cuuint32_t estr[3] = {1, 1, 1};
     CUresult r = ((EncodeTiledFn)c->encode_tiled)(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), dims, strides, box,
-                                                  estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                                                  estr, CU_TENSOR_MAP_INTERLEAVE_NONE, lanes_swizzle(lanes),
                                                   CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return map_ok(r, __LINE__);
 }
@@ -2038,7 +2075,7 @@ pt_status launch_gemm(pt_ctx *c, const CUtensorMap &tmA, const CUtensorMap &tmB,
 }
 
 // Source activations as a tiled 4-D tensor (C, W, H, N): box 64 channels x box_w x box_h x 1 (the halo tile).
-// `lanes` = 64 (128-byte rows and swizzle) or 16 (32-byte rows and swizzle).
+// `lanes` = 64, 32 or 16 (128-, 64- or 32-byte rows and swizzle).
 // `row_pixels` > 0: pixels between the starts of consecutive rows when that is not W (a padded row).
 bool make_halo_in_map(const pt_ctx *c, CUtensorMap *tm, const void *base, int C, int W, int H, int N, int ld, int box_w, int box_h,
                       int lanes = kKC, int row_pixels = 0)
@@ -2049,7 +2086,7 @@ bool make_halo_in_map(const pt_ctx *c, CUtensorMap *tm, const void *base, int C,
     cuuint64_t strides[3] = {(cuuint64_t)ld * 2, rp * ld * 2, (cuuint64_t)H * rp * ld * 2};
     cuuint32_t box[4] = {(cuuint32_t)lanes, (cuuint32_t)box_w, (cuuint32_t)box_h, 1}, estr[4] = {1, 1, 1, 1};
     CUresult r = ((EncodeTiledFn)c->encode_tiled)(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(base), dims, strides, box,
-                                                  estr, CU_TENSOR_MAP_INTERLEAVE_NONE, lanes == 16 ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_128B,
+                                                  estr, CU_TENSOR_MAP_INTERLEAVE_NONE, lanes_swizzle(lanes),
                                                   CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return map_ok(r, __LINE__);
 }
@@ -2081,8 +2118,11 @@ pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const
     p.n_cols = h.n_cols;
     p.BN = tile_n(h.n_cols, &p.n_tiles);
     p.c_red = h.Cs; p.k_chunks = pt_ceil_div(h.Cs, kKC); p.taps = h.n_taps;
-    p.row32 = h.row32 ? 1 : 0;
-    const int row_bytes = h.row32 ? 32 : 128;
+    // Channel lanes per staged pixel: narrow layers take rows of 64 or 32 bytes. The TMA unit's time is per row, and a row whose tensor
+    // ends in the middle of a sector costs it twice as much in a 128-byte box (4.5 ns for 19 channels) as a whole one (2.3 ns); in a
+    // box of the next width 3.1 ns. The rows also take less shared memory.
+    p.lanes = h.Cs <= 16 ? 16 : h.Cs <= 32 ? 32 : 64;
+    const int row_bytes = p.lanes * 2;
     if (h.row32 && (B_MN || h.Cs != 16)) return PT_ERR_UNSUPPORTED;
     p.lo_h = h.lo_h; p.lo_w = h.lo_w;
     for (int t = 0; t < h.n_taps; ++t) {
@@ -2102,10 +2142,15 @@ pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const
     // read up to BN rows, the rest from whatever follows in shared memory: columns that are never stored
     p.b_rows = p.BN < h.n_cols ? p.BN : pt_ceil_div(h.n_cols, 16) * 16;
     if (p.b_rows > p.BN) p.b_rows = p.BN;
-    const size_t b_bytes = B_MN ? (size_t)pt_ceil_div(p.BN, 64) * 8192 : (size_t)p.b_rows * row_bytes;
+    const size_t b_bytes = B_MN ? (size_t)pt_ceil_div(p.BN, 64) * p.lanes * 128 : (size_t)p.b_rows * row_bytes;
     p.b_slot = (int)b_bytes;
-    // epilogue staging: one slab of the tile's raster rows x 128 bytes per group (direct-store launches use none)
-    p.staging = d->out_f32 ? 0 : (int)pt_align_up((size_t)(p.nr * Wp < 128 ? p.nr * Wp : 128) * 128, 1024);
+    // narrow outputs are stored from registers (the 16-byte vectors of a pixel must be whole: room in the pitch)
+    p.direct_cols = pt_ceil_div(h.n_cols, 16) * 16 <= h.ld_out ? pt_ceil_div(h.n_cols, 16) * 16 : pt_ceil_div(h.n_cols, 8) * 8;
+    p.direct = (!d->out_f32 && !c->stats_mode && p.n_tiles == 1 && p.BN <= 32) ? 1 : 0;
+    // epilogue staging: a slab of the tile's raster rows x 128 bytes per group, two where the launch's other needs leave room (direct-store
+    // launches use none)
+    p.staging = (d->out_f32 || p.direct) ? 0 : (int)pt_align_up((size_t)(p.nr * Wp < 128 ? p.nr * Wp : 128) * 128, 1024);
+    p.slabs = 1;
     p.stats_warp = pt_ceil_div(p.BN, 64) * (int)kStatsChunkBytes;
     const size_t st_smem = c->stats_mode ? (size_t)8 * p.stats_warp : 0;        // statistics accumulators of the eight epilogue warps
     const size_t budget = 227 * 1024 - 2048 - 2 * (size_t)p.staging - a_tail - st_smem;
@@ -2137,11 +2182,13 @@ pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const
         int sa = (int)(left / p.a_alloc);
         p.stages_a = sa > 4 ? 4 : sa;
     } else {
+        // (one stage per issuer leaves its load latency exposed on every tile: 19 -> 19 at 56x56, batch 256, 46 us with 4 stages, 36 with 8)
         int sa = (int)(left / p.a_alloc);
-        p.stages_a = sa > 4 ? 4 : sa;
+        p.stages_a = sa > kHaloMaxA ? kHaloMaxA : sa;
         p.stages_b = 1;
     }
     if (p.stages_a < 2) return PT_ERR_UNSUPPORTED;
+    if (p.staging && p.resident && left >= kHaloMaxA * (size_t)p.a_alloc + 2 * (size_t)p.staging) p.slabs = 2;
     // issuer warps: several only with resident weights; each needs an A stage of its own and an accumulator buffer
     p.n_issuers = 1;
     p.acc_per = 2;
@@ -2157,7 +2204,7 @@ pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const
     p.tmem_cols = pow2_cols(p.n_issuers * p.acc_per * p.BN);
     p.out = out; p.ld_out = h.ld_out; p.out_f32 = d->out_f32;
     p.oH = h.oH; p.oW = h.oW; p.o_step = h.o_step; p.o_h0 = h.o_h0; p.o_w0 = h.o_w0;
-    p.tma_store = d->out_f32 ? 0 : 1;
+    p.tma_store = (d->out_f32 || p.direct) ? 0 : 1;
     p.status = c->d_status;
     CUtensorMap tmA, tmB, tmC;
     memset(&tmC, 0, sizeof(tmC));
@@ -2173,8 +2220,8 @@ pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const
                                                       CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (!map_ok(r, __LINE__)) return PT_ERR_CUDA;
     } else {
-        if (!make_halo_in_map(c, &tmA, h.src, h.Cs, h.Ws, h.Hs, d->N, h.lds, Wp, box_h)) return PT_ERR_CUDA;
-        if (!make_weight_map(c, &tmB, w, d->C, d->R * d->S, d->K, d->ldw, B_MN ? kKC : p.b_rows)) return PT_ERR_CUDA;
+        if (!make_halo_in_map(c, &tmA, h.src, h.Cs, h.Ws, h.Hs, d->N, h.lds, Wp, box_h, p.lanes)) return PT_ERR_CUDA;
+        if (!make_weight_map(c, &tmB, w, d->C, d->R * d->S, d->K, d->ldw, B_MN ? p.lanes : p.b_rows, B_MN ? kKC : p.lanes)) return PT_ERR_CUDA;
     }
     if (p.tma_store) {
         // the output view as a 4-D tensor (channels, raster columns, raster rows, images); strided when o_step > 1
@@ -2189,7 +2236,7 @@ pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const
                                                       CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (!map_ok(r, __LINE__)) return PT_ERR_CUDA;
     }
-    const size_t smem = 2048 + 2 * (size_t)p.staging + (p.resident ? w_all : (size_t)p.stages_b * b_bytes) + (size_t)p.stages_a * p.a_alloc + a_tail +
+    const size_t smem = 2048 + 2 * (size_t)p.slabs * p.staging + (p.resident ? w_all : (size_t)p.stages_b * b_bytes) + (size_t)p.stages_a * p.a_alloc + a_tail +
                         st_smem;
     p.stats_off = (int)(smem - st_smem);
     void (*kernel)(CUtensorMap, CUtensorMap, CUtensorMap, HaloP) =

@@ -208,16 +208,16 @@ __device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t lbo_bytes
     return d;
 }
 
-// The same for the 32-byte swizzle, K-major only: rows of 32 B (16 bf16 along K: exactly one MMA K step), 8-row groups
-// `sbo_bytes` (256 for a dense tile) apart.
-__device__ __forceinline__ uint64_t make_desc_sw32(uint32_t saddr, uint32_t sbo_bytes)
+// K-major tile whose rows are `row_bytes` = 128, 64 or 32 bytes (64, 32 or 16 bf16 along K) with the swizzle of that width.
+__device__ __forceinline__ uint64_t make_desc_rows(uint32_t saddr, uint32_t row_bytes)
 {
+    const uint64_t layout = row_bytes == 128u ? 2ull : row_bytes == 64u ? 4ull : 6ull;      // SWIZZLE_128B / 64B / 32B
     uint64_t d = 0;
     d |= (uint64_t)((saddr & 0x3ffffu) >> 4);
     d |= (uint64_t)1 << 16;
-    d |= (uint64_t)((sbo_bytes >> 4) & 0x3fffu) << 32;
+    d |= (uint64_t)(((8u * row_bytes) >> 4) & 0x3fffu) << 32;
     d |= (uint64_t)1 << 46;
-    d |= (uint64_t)6 << 61;      // SWIZZLE_32B
+    d |= layout << 61;
     return d;
 }
 
