@@ -724,29 +724,30 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
     // the weight producers do not read the previous kernel's output: resident weights are issued first and the wait follows
     // them (below); the producers of streamed weights never need it
     // Warps that load activations wait just before their first activation load, after their set-up (tile walk, ring positions).
-    if (!(warp == 0 || ((warp == 13 || warp == 14 || warp == 15) && !p.resident))) grid_dependency_wait();
+    if (!(warp == 0 || warp >= 13)) grid_dependency_wait();
     grid_launch_dependents();
 
     // Streamed weights with two issuers: two complete pipelines (producer warp, A ring, B ring, issuer warp, accumulators),
-    // one per tile parity. Resident weights: one producer feeds every issuer's A ring.
+    // one per tile parity. Resident weights: every issuer's A ring has a producer warp of its own (a thread issues a box only every
+    // 0.5 us, whatever it holds: one producer for four issuers made that the time of a tile), and they share the weights' loads.
     // With `shared_b` the two pipelines read the same weight stages: the tiles of a round (blockIdx.x + 2r*grid and + (2r+1)*grid)
     // use the same weights, so one stream through the whole ring feeds both issuers, half the bytes and twice the depth.
-    const int n_prod = p.resident ? 1 : NI;
+    const int n_prod = NI;
     const int SB = p.shared_b ? p.stages_b : p.stages_b / n_prod;     // weight stages per weight stream
     // Streamed weights: the activation boxes have a producer warp of their own per pipeline (14, 15), so that the next tile's
     // boxes go out as soon as their stage is free instead of behind the weight loads of the current tile, which wait for the
     // MMAs (the next tile's activations used to be issued only when the current tile was nearly done: ~4 us per tile exposed).
     const bool a_warp = !p.resident && (warp == 14 || (warp == 15 && n_prod == 2));
-    if (warp == 0 || (warp == 13 && n_prod == 2 && !p.shared_b) || a_warp) {
+    if (warp == 0 || (p.resident ? warp >= 13 && warp - 12 < NI : (warp == 13 && n_prod == 2 && !p.shared_b) || a_warp)) {
         if (lane == 0) {
             // ---------------- TMA producer(s)
-            const int pid = (warp == 0 || warp == 14) ? 0 : 1;
+            const int pid = p.resident ? (warp == 0 ? 0 : warp - 12) : (warp == 0 || warp == 14) ? 0 : 1;
             const bool a_role = a_warp || p.resident, b_role = !a_warp && !p.resident;
             if (p.resident) {
                 // n_tiles == 1 here: the whole weight tensor of the layer, tap by tap and chunk by chunk, once
                 const uint32_t bar = smem_u32(&ctl->w_full);
-                mbar_arrive_expect_tx(bar, (uint32_t)(p.taps * p.k_chunks) * b_bytes);
-                for (int tap = 0; tap < p.taps; ++tap)
+                if (pid == 0) mbar_arrive_expect_tx(bar, (uint32_t)(p.taps * p.k_chunks) * b_bytes);
+                for (int tap = pid; tap < p.taps; tap += n_prod)
                     for (int kc = 0; kc < p.k_chunks; ++kc) {
                         const uint32_t dst = b_base + (uint32_t)(tap * p.k_chunks + kc) * b_slot;
                         const int wtap = p.tap_wt[tap];
