@@ -677,7 +677,8 @@ constexpr int kHaloThreads = 512;
 // kernel therefore runs up to four issuer warps, each on its own scheduler: issuer i owns accumulator buffer i and
 // an A ring of its own (a waiter may lag an mbarrier by at most one phase, so issuers cannot share a ring), and takes
 // the tiles i, i + I, i + 2I, ... of the CTA. Weights that stream through a ring keep a single issuer.
-template <bool B_MN, bool STATS>
+// APART: the output pixels are two apart (a variant of its own: one kernel with both epilogues spills).
+template <bool B_MN, bool STATS, bool APART>
 __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid_constant__ CUtensorMap tmA,
                                                                      const __grid_constant__ CUtensorMap tmB,
                                                                      const __grid_constant__ CUtensorMap tmC, const HaloP p)
@@ -929,7 +930,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
             if (gtid == 0) HTRACE(4, tc);
             tc_fence_after();
             const uint32_t lane_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * p.BN);
-            if (p.tma_store) {
+            if (!APART && p.tma_store) {
                 const int n_chunks = (p.BN + 63) / 64;
                 for (int ch = 0; ch < n_chunks; ++ch) {
                     if (gtid == 0) {                                 // the slab's previous store has read it
@@ -987,7 +988,8 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
             }
             // ---- direct stores (fp32 outputs, narrow bf16 outputs)
             const bool row_ok = on_raster && p0 + ri < p.P;
-            const size_t row_off = ((size_t)(img * p.oH + (p0 + ri) * p.o_step + p.o_h0) * p.oW + rj * p.o_step + p.o_w0) * (size_t)p.ld_out;
+            const int pix = (img * p.oH + (p0 + ri) * p.o_step + p.o_h0) * p.oW + rj * p.o_step + p.o_w0;
+            const size_t row_off = (size_t)pix * (size_t)p.ld_out;
             if (p.direct) {
                 // a pixel's channels are 32 or 64 consecutive bytes: whole sectors from one thread, with no barrier among the warps and
                 // no store to wait for before the next tile (whose staging made a tile cost 0.5 us however little it held)
@@ -1014,6 +1016,63 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
                 }
                 continue;
             }
+            if (APART && !p.out_f32) {
+                // bf16 output pixels that are two apart (the parities of a stride-2 data gradient): the warp's 32 raster rows x 64 channels
+                // go through its own 4 KB of shared memory (128-byte swizzle) and leave as whole lines, eight lanes to a pixel. (A 4-D TMA
+                // store of a strided view takes longer: 46 -> 40 us for 103 -> 106 channels at 56x56. Of consecutive pixels it is the
+                // faster one by 1 to 3 us.)
+                const int n_chunks = (p.BN + 63) / 64;
+                const uint32_t wslab = staging_base + (uint32_t)(warp - 2) * 4096u;
+                const uint32_t rows = __ballot_sync(0xffffffffu, row_ok);
+                for (int ch = 0; ch < n_chunks; ++ch) {
+                    const int groups = min(4, (p.BN - ch * 64) / 16);
+                    uint32_t v[4][16];
+#pragma unroll
+                    for (int g = 0; g < 4; ++g)
+                        if (g < groups) tmem_ld16(lane_addr + (uint32_t)(ch * 64 + g * 16), v[g]);
+                    tmem_ld_wait();
+                    if (ch + 1 >= n_chunks) {
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(smem_u32(&ctl->acc_empty[b]));
+                    }
+#pragma unroll
+                    for (int g = 0; g < 4; ++g) {
+                        if (g >= groups) break;
+#pragma unroll
+                        for (int hh = 0; hh < 2; ++hh) {
+                            __nv_bfloat162 b0 = __floats2bfloat162_rn(__uint_as_float(v[g][8 * hh + 0]), __uint_as_float(v[g][8 * hh + 1]));
+                            __nv_bfloat162 b1 = __floats2bfloat162_rn(__uint_as_float(v[g][8 * hh + 2]), __uint_as_float(v[g][8 * hh + 3]));
+                            __nv_bfloat162 b2 = __floats2bfloat162_rn(__uint_as_float(v[g][8 * hh + 4]), __uint_as_float(v[g][8 * hh + 5]));
+                            __nv_bfloat162 b3 = __floats2bfloat162_rn(__uint_as_float(v[g][8 * hh + 6]), __uint_as_float(v[g][8 * hh + 7]));
+                            const uint32_t j = (uint32_t)(g * 2 + hh);
+                            const uint32_t addr = wslab + (uint32_t)lane * 128u + ((j ^ ((uint32_t)lane & 7u)) << 4);
+                            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(*reinterpret_cast<uint32_t *>(&b0)),
+                                         "r"(*reinterpret_cast<uint32_t *>(&b1)), "r"(*reinterpret_cast<uint32_t *>(&b2)),
+                                         "r"(*reinterpret_cast<uint32_t *>(&b3))
+                                         : "memory");
+                        }
+                    }
+                    __syncwarp();
+                    const int pj = lane & 7, col = n0 + ch * 64 + pj * 8;       // this lane's 16-byte piece of every fourth row
+                    const bool col_ok = pj < groups * 2 && col < p.direct_cols;
+                    uint4 t[8];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const uint32_t r = (uint32_t)(i * 4 + (lane >> 3));
+                        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(t[i].x), "=r"(t[i].y), "=r"(t[i].z), "=r"(t[i].w)
+                                     : "r"(wslab + r * 128u + (((uint32_t)pj ^ (r & 7u)) << 4)) : "memory");
+                    }
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const int r = i * 4 + (lane >> 3);
+                        const int px = __shfl_sync(0xffffffffu, pix, r);
+                        if (col_ok && ((rows >> r) & 1u)) *reinterpret_cast<uint4 *>((__nv_bfloat16 *)p.out + (size_t)px * (size_t)p.ld_out + col) = t[i];
+                    }
+                    __syncwarp();
+                }
+                continue;
+            }
             for (int c0 = 0; c0 < p.BN; c0 += 16) {
                 uint32_t v[16];
                 tmem_ld16(lane_addr + (uint32_t)c0, v);
@@ -1026,13 +1085,8 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
                 const int col = n0 + c0;
                 if (!row_ok || col >= p.n_cols) continue;
                 const int nvalid = min(16, p.n_cols - col);
-                if (p.out_f32) {
-                    float *o = (float *)p.out + row_off + col;
-                    for (int e = 0; e < nvalid; ++e) o[e] = __uint_as_float(v[e]);
-                } else {
-                    __nv_bfloat16 *o = (__nv_bfloat16 *)p.out + row_off + col;
-                    for (int e = 0; e < nvalid; ++e) o[e] = __float2bfloat16_rn(__uint_as_float(v[e]));
-                }
+                float *o = (float *)p.out + row_off + col;
+                for (int e = 0; e < nvalid; ++e) o[e] = __uint_as_float(v[e]);
             }
         }
         if (STATS && p.stats) {
@@ -2124,7 +2178,7 @@ pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const
     // box of the next width 3.1 ns. The rows also take less shared memory.
     p.lanes = h.Cs <= 16 ? 16 : h.Cs <= 32 ? 32 : 64;
     const int row_bytes = p.lanes * 2;
-    if (h.row32 && (B_MN || h.Cs != 16)) return PT_ERR_UNSUPPORTED;
+    if ((h.row32 && (B_MN || h.Cs != 16)) || (!B_MN && h.o_step != 1)) return PT_ERR_UNSUPPORTED;
     p.lo_h = h.lo_h; p.lo_w = h.lo_w;
     for (int t = 0; t < h.n_taps; ++t) {
         p.tap_oh[t] = (unsigned char)h.tap_oh[t]; p.tap_ow[t] = (unsigned char)h.tap_ow[t];
@@ -2150,7 +2204,8 @@ pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const
     p.direct = (!d->out_f32 && !c->stats_mode && p.n_tiles == 1 && p.BN <= 32) ? 1 : 0;
     // epilogue staging: a slab of the tile's raster rows x 128 bytes per group, two where the launch's other needs leave room (direct-store
     // launches use none)
-    p.staging = (d->out_f32 || p.direct) ? 0 : (int)pt_align_up((size_t)(p.nr * Wp < 128 ? p.nr * Wp : 128) * 128, 1024);
+    p.tma_store = (d->out_f32 || p.direct || h.o_step != 1) ? 0 : 1;
+    p.staging = (d->out_f32 || p.direct) ? 0 : !p.tma_store ? 4 * 4096 : (int)pt_align_up((size_t)(p.nr * Wp < 128 ? p.nr * Wp : 128) * 128, 1024);
     p.slabs = 1;
     p.stats_warp = pt_ceil_div(p.BN, 64) * (int)kStatsChunkBytes;
     const size_t st_smem = c->stats_mode ? (size_t)8 * p.stats_warp : 0;        // statistics accumulators of the eight epilogue warps
@@ -2189,7 +2244,7 @@ pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const
         p.stages_b = 1;
     }
     if (p.stages_a < 2) return PT_ERR_UNSUPPORTED;
-    if (p.staging && p.resident && left >= kHaloMaxA * (size_t)p.a_alloc + 2 * (size_t)p.staging) p.slabs = 2;
+    if (p.tma_store && p.resident && left >= kHaloMaxA * (size_t)p.a_alloc + 2 * (size_t)p.staging) p.slabs = 2;
     // issuer warps: several only with resident weights; each needs an A stage of its own and an accumulator buffer
     p.n_issuers = 1;
     p.acc_per = 2;
@@ -2205,7 +2260,6 @@ pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const
     p.tmem_cols = pow2_cols(p.n_issuers * p.acc_per * p.BN);
     p.out = out; p.ld_out = h.ld_out; p.out_f32 = d->out_f32;
     p.oH = h.oH; p.oW = h.oW; p.o_step = h.o_step; p.o_h0 = h.o_h0; p.o_w0 = h.o_w0;
-    p.tma_store = (d->out_f32 || p.direct) ? 0 : 1;
     p.status = c->d_status;
     CUtensorMap tmA, tmB, tmC;
     memset(&tmC, 0, sizeof(tmC));
@@ -2241,9 +2295,9 @@ pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const
                         st_smem;
     p.stats_off = (int)(smem - st_smem);
     void (*kernel)(CUtensorMap, CUtensorMap, CUtensorMap, HaloP) =
-        (!B_MN && c->stats_mode) ? conv_halo_kernel<false, true> : conv_halo_kernel<B_MN, false>;
-    const int kid = (!B_MN && c->stats_mode) ? 2 : (B_MN ? 1 : 0);
-    static bool attr_set[3] = {false, false, false};
+        (!B_MN && c->stats_mode) ? conv_halo_kernel<false, true, false> : (B_MN && h.o_step != 1) ? conv_halo_kernel<true, false, true> : conv_halo_kernel<B_MN, false, false>;
+    const int kid = (!B_MN && c->stats_mode) ? 2 : (B_MN && h.o_step != 1) ? 3 : (B_MN ? 1 : 0);
+    static bool attr_set[4] = {false, false, false, false};
     if (!attr_set[kid]) {
         PT_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
         attr_set[kid] = true;
