@@ -2344,9 +2344,10 @@ constexpr size_t kSplitSmemFloor = 116 * 1024;
 // Both kernels cut the work three ways: tiles of dw (channels), groups of taps, and the pixels of the reduction over `splits` CTAs
 // that exchange partial sums at the end. The shape is chosen by a rough time of one CTA (microseconds; the constants are measured):
 //   first load 1.4, then per stage the larger of its MMAs (55 cycles each at N <= 64, N/2 + 8 above) and its bytes at 100 KB/us,
-//   plus 0.12 of waiting and issuing; then the exchange:
-//   none (one split): 1; in a cluster (2..8 splits): 1.8 + bytes of the accumulators at 120 KB/us;
-//   through the workspace: 6 + bytes at 60 KB/us (partial tile to L2, arrival counter, sum: three round trips).
+//   plus 0.25 of waiting and issuing; then the exchange:
+//   none (one split): 1; through the workspace: 5 + bytes of the accumulators at 40 KB/us (partial tile to L2, arrival counter, sum:
+//   three round trips); in a cluster (2..8 splits): 1.5 + the bytes for the other CTAs at 25 KB/us, at 11 KB/us among more than four
+//   (213 -> 242 3x3 at 14x14, 112 KB, eight splits: 27 us as clusters, 23 through the workspace; 8 14x14 64 -> 64, 32 KB: 6.4 and 8.7).
 // A cluster needs its CTAs free at the same time in one GPC: used while the device can hold all of the launch's clusters at once.
 constexpr double kWgSearch = 400.0;      // layers whose tile takes one CTA less than this (us) also choose tap groups and unit size
 
@@ -2354,7 +2355,8 @@ double wg_mma_us(int n) { return (n <= 64 ? 55.0 : n * 0.5 + 8.0) / 1900.0; }
 double wg_exchange_us(int splits, bool cluster, double acc_bytes)
 {
     if (splits <= 1) return 1.0 + acc_bytes / 200e3;
-    return cluster ? 1.8 + acc_bytes / 120e3 : 6.0 + acc_bytes / 60e3;
+    if (!cluster) return 5.0 + acc_bytes / 40e3;
+    return 1.5 + acc_bytes * (splits - 1) / splits / (splits <= 4 ? 25e3 : 11e3);
 }
 
 int wg_max_clusters(const pt_ctx *c, int size);
@@ -2391,7 +2393,6 @@ double wg_pick_splits(const pt_ctx *c, int tiles, int max_s, double acc_bytes, F
         if (tiles > wg_max_clusters(c, k)) continue;
         const double t = main_us(k) + wg_exchange_us(k, true, acc_bytes);
         if (t < best) { best = t; *splits = k; *cluster = 1; }
-        break;                                             // the largest cluster that fits
     }
     return best;
 }
@@ -2413,7 +2414,7 @@ void wgrad_gen_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, pt_wgr
         const int tpc = pt_ceil_div(taps, g), tiles = w->m_tiles * w->n_tiles * pt_ceil_div(taps, tpc);
         if (g > groups0 && (tiles > wgrad_budget(c) || pt_ceil_div(taps, tpc) != g)) continue;
         const double load = ((d->K > 64 ? 16384.0 : 8192.0) + tpc * nb * 8192.0) / 100e3, mma = tpc * 4 * wg_mma_us(w->bn);
-        const double stage = (load > mma ? load : mma) + 0.12;
+        const double stage = (load > mma ? load : mma) + 0.25;
         int s, cl;
         const double t = wg_pick_splits(c, tiles, (int)max_s, (double)tpc * w->bn * 512.0,
                                         [&](int k) { return 1.4 + (double)((npix + 63) / 64 + k - 1) / k * stage; }, &s, &cl);
@@ -2481,7 +2482,7 @@ bool wgrad_rows_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, pt_wg
             for (int g = groups0; g <= pairs; g += groups0) {
                 const int apc = pt_ceil_div(pairs, g), tiles = pt_ceil_div(pairs, apc);
                 if (g > groups0 && (tiles > wgrad_budget(c) || tiles != g)) continue;
-                const double mma = ks * apc * cyc, unit = (load > mma ? load : mma) + 0.12;
+                const double mma = ks * apc * cyc, unit = (load > mma ? load : mma) + 0.25;
                 int s, cl;
                 const double us = wg_pick_splits(c, tiles, units > 3 ? units / 2 : 1, (double)apc * w->acc_cols * 512.0,
                                                  [&](int k) { return 1.4 + pt_ceil_div(units, k) * unit; }, &s, &cl);
@@ -2495,7 +2496,7 @@ bool wgrad_rows_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, pt_wg
             if (large) {
                 int s, cl;
                 wg_pick_splits(c, w->tap_groups, w->units > 3 ? w->units / 2 : 1, (double)w->apc * w->acc_cols * 512.0,
-                               [&](int k) { return 1.4 + pt_ceil_div(w->units, k) * (unit + 0.12); }, &s, &cl);
+                               [&](int k) { return 1.4 + pt_ceil_div(w->units, k) * (unit + 0.25); }, &s, &cl);
                 w->splits = s; w->cluster = cl;
             }
         }
