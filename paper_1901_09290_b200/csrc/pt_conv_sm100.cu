@@ -72,10 +72,13 @@ struct GemmP {
     // output pixel mapping: pixel (n, i, j) of the raster -> out[((n*oH + i*o_step + o_h0)*oW + j*o_step + o_w0)*ld_out]
     int oH, oW, o_step, o_h0, o_w0;
     int ld_out, out_f32;
+    int vec_cols;       // strided bf16 outputs: channels covered by whole 16-byte vectors
     int zero_mask;      // stride-2 dgrad: bit (a*2+b) set => also write zeros to the pixel at parity (a,b) of each 2x2 cell
     int tma_store;      // 1: bf16 output rows are consecutive pixels -> staged in shared memory and written by TMA stores
     int m_tiles;        // ceil(M_total / 128)
     int epi_groups;     // 1..3 groups of four epilogue warps
+    int n_a, n_b;       // producer warps of the activation tiles (two: one per issuer's ring), of streamed weight tiles (1 or 2)
+    int tail_lanes;     // channel lanes the last activation chunk is staged with: 64, 32 or 16 (rows of 128, 64 or 32 bytes)
     int a_tiled;        // 1: 1x1 stride-1 problem, the A operand is a plain 2-D (channels, pixels) tiled map
     int resident;       // 1: every weight tile of the launch stays in shared memory (loaded once); the ring carries A only
     int n_issuers;      // 2 (resident weights only): two MMA issuer warps take alternate tiles, each with half of the ring's stages
@@ -208,8 +211,40 @@ __device__ unsigned int g_chain_seq;
 // tiles. The accumulator has G = 2 or 3 buffers in TMEM and buffer b has its own group of four epilogue warps, so the
 // loads and MMAs of the next tiles overlap the epilogues of the previous ones.
 // STATS: the epilogue also takes the batch-normalisation statistics (a variant of its own: the plain kernels keep their registers).
-template <bool B_MN, bool STATS>
+// n / d for 0 <= n < 2^22 and a divisor known per kernel: float reciprocal plus one correction step (an integer division
+// costs ~40 instructions, and the reduction below does two per 16-byte item).
+__device__ __forceinline__ int fast_div(int n, int d, float inv_d)
+{
+    int q = __float2int_rz(__int2float_rn(n) * inv_d);
+    if ((q + 1) * d <= n) ++q;
+    if (q * d > n) --q;
+    return q;
+}
+
+// Stores a warp's 32 staged rows (128 bytes each, 128-byte swizzle) of `pieces` 16-byte vectors to the pixels `pix` (one per lane) whose bit
+// of `rows` is set: eight lanes to a pixel. (Every lane on the next vector whatever its row: 40.7 -> 44.2 us for 103 -> 106 channels.)
+__device__ __forceinline__ void store_rows_apart(__nv_bfloat16 *out, int ld, uint32_t slab, int col, int pieces, uint32_t rows, int pix, int lane)
+{
+    const int j = lane & 7;
+    uint4 t[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const uint32_t r = (uint32_t)(i * 4 + (lane >> 3));
+        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(t[i].x), "=r"(t[i].y), "=r"(t[i].z), "=r"(t[i].w)
+                     : "r"(slab + r * 128u + (((uint32_t)j ^ (r & 7u)) << 4)) : "memory");
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int r = i * 4 + (lane >> 3);
+        const int px = __shfl_sync(0xffffffffu, pix, r);
+        if (j < pieces && ((rows >> r) & 1u)) *reinterpret_cast<uint4 *>(out + (size_t)px * (size_t)ld + col + j * 8) = t[i];
+    }
+}
+
+// APART: bf16 output pixels two apart (a variant of its own: one kernel with both epilogues spills).
+template <bool B_MN, bool STATS, bool APART>
 __global__ void __launch_bounds__(kGemmThreads, 1) conv_gemm_kernel(const __grid_constant__ CUtensorMap tmA,
+                                                                 const __grid_constant__ CUtensorMap tmT /* last chunk of A */,
                                                                  const __grid_constant__ CUtensorMap tmB,
                                                                  const __grid_constant__ CUtensorMap tmC, const GemmP p)
 {
@@ -230,10 +265,15 @@ __global__ void __launch_bounds__(kGemmThreads, 1) conv_gemm_kernel(const __grid
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int iters = p.taps * p.k_chunks;
     const int total_tiles = p.m_tiles * p.n_tiles;
-    // streamed MN-major weight tiles are one 8 KB box per 64 columns: with several boxes per stage a second producer warp
-    // (warp 15, otherwise idle without resident weights) issues every other one
+    // Producers: warp 0 the activation tiles, warp 14 the weights; streamed MN-major weight tiles are one 8 KB box per 64 columns, every
+    // other one of which warp 15 issues. With two issuers (resident weights) and several chunks per tile warp 14 feeds the second issuer's
+    // ring: a thread issues a box only every 0.3 to 0.5 us (77 -> 19 at 56x56, batch 256: 41.6 -> 29.5 us; with a single chunk per tile
+    // the output side is the longer one and the second producer costs up to 1 us). Halves of an activation or K-major weight tile from
+    // two warps each were measured too: no faster, the deep layers wait for what is in flight.
     const int nb_b = (p.BN + 63) / 64;
-    const bool two_b = B_MN && !p.resident && nb_b > 1;
+    const bool ring2 = p.n_a == 2;
+    const int a_id = warp == 0 ? 0 : (ring2 && warp == 14) ? 1 : -1;
+    const int b_id = warp == 14 ? 0 : (!p.resident && warp == 15 && p.n_b > 1) ? 1 : -1;
 
 #ifdef PT_DEVICE_TRACE
     if (threadIdx.x == 0) {
@@ -243,7 +283,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) conv_gemm_kernel(const __grid
 #endif
     if (threadIdx.x == 0) {
         for (int s = 0; s < p.stages; ++s) {
-            mbar_init(smem_u32(&ctl->full[s]), p.resident ? 1 : (two_b ? 3 : 2));   // the A producer and, with streamed weights, the B producer(s)
+            mbar_init(smem_u32(&ctl->full[s]), (uint32_t)(1 + (p.resident ? 0 : p.n_b)));
             mbar_init(smem_u32(&ctl->empty[s]), 1);
         }
         mbar_init(smem_u32(&ctl->w_full), 1);
@@ -270,22 +310,22 @@ __global__ void __launch_bounds__(kGemmThreads, 1) conv_gemm_kernel(const __grid
     // previous kernel's results here.
     // The activation producer (warp 0) waits just before its first load instead: its set-up (tile coordinates, tap tables: a
     // few hundred cycles of divisions and first-touch parameter reads) then runs while the previous kernel drains.
-    if (!(warp == 0 || warp == 14 || (warp == 15 && two_b))) grid_dependency_wait();
+    if (!(a_id >= 0 || b_id >= 0)) grid_dependency_wait();
     grid_launch_dependents();
 
-    if (warp == 0 || warp == 14 || (warp == 15 && two_b)) {
+    if (a_id >= 0 || b_id >= 0) {
         if (lane == 0) {
-            // ---------------- TMA producers: warp 0 brings the A tile of every stage, warp 14 the B tile (issuing a TMA
-            // instruction costs its thread about 200 cycles, so the two operands are issued side by side)
-            const bool is_a = warp == 0;
-            if (is_a) CTRACE(8);
-            const int bsel = warp == 15 ? 1 : 0, nbp = two_b ? 2 : 1;         // this B producer's boxes: bsel, bsel + nbp, ...
-            const uint32_t my_bytes = is_a ? a_bytes : (two_b ? (uint32_t)((nb_b + 1 - bsel) / 2) * 8192u : b_bytes);
+            // ---------------- TMA producers
+            const bool is_a = a_id >= 0;                     // (warp 14 with two rings: the weights first, then activations)
+            if (warp == 0) CTRACE(8);
+            const uint32_t my_bytes = is_a ? a_bytes : B_MN ? (uint32_t)((nb_b - b_id + p.n_b - 1) / p.n_b) * 8192u : b_bytes;
+            const uint32_t tail_bytes = is_a ? (uint32_t)(kBM * p.tail_lanes * 2) : my_bytes;
             int s = 0, ph = 0, issued = 0;   // stage-ring position, continuous across tiles
-            int s1 = 0, ph1 = 0;             // position in the second issuer's ring
             bool dep_waited = false;         // the activation producer has waited for the previous kernel's results
             const int SR = p.stages / p.n_issuers;
-            if (!is_a && p.resident) {
+            const bool both = is_a && p.n_issuers == 2 && !ring2;      // this producer feeds two rings, a tile each in turn
+            int ring = ring2 && a_id == 1 ? 1 : 0, s1 = 0, ph1 = 0;    // the ring it feeds now; its position in the other one
+            if (b_id == 0 && p.resident) {
                 // n_tiles == 1 here: every weight tile of the launch, once
                 const uint32_t bar = smem_u32(&ctl->w_full);
                 mbar_arrive_expect_tx(bar, (uint32_t)iters * b_bytes);
@@ -297,13 +337,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1) conv_gemm_kernel(const __grid
                         else for (int nb = 0; nb < (p.BN + 63) / 64; ++nb) tma_load_3d(dst + (uint32_t)nb * 8192u, &tmB, bar, nb * 64, wtap, kc * kKC);
                     }
             }
-            int ring = 0;
-            for (int tile = blockIdx.x; tile < total_tiles && !*abort_flag && (is_a || !p.resident); tile += gridDim.x,
-                     ring = p.n_issuers == 2 ? ring ^ 1 : 0) {
-                const int n_tile = tile % p.n_tiles, m_tile = tile / p.n_tiles;
-                const int m0 = m_tile * kBM, n0 = n_tile * p.BN;
-                if (ring) { int t = s; s = s1; s1 = t; t = ph; ph = ph1; ph1 = t; }     // work on the second ring's position
+            // every tile, or with a producer per ring every other one
+            for (int tile = blockIdx.x + ring * (int)gridDim.x; tile < total_tiles && !*abort_flag && (is_a || !p.resident);
+                 tile += (ring2 ? 2 : 1) * (int)gridDim.x) {
                 const int sbase = ring * SR;
+                const int n_tile = tile % p.n_tiles, m_tile = tile / p.n_tiles;
+                const int n0 = n_tile * p.BN;
+                const int m0 = m_tile * kBM;
                 int w0 = 0, h0 = 0, n = 0;
                 if (is_a && !p.a_tiled) {
                     const int q = m0 % p.Qd, t = m0 / p.Qd, pp = t % p.Pd;
@@ -315,39 +355,41 @@ __global__ void __launch_bounds__(kGemmThreads, 1) conv_gemm_kernel(const __grid
                     const int wtap = p.tap_wt[tap];
                     const uint16_t ow = (uint16_t)p.tap_ow[tap], oh = (uint16_t)p.tap_oh[tap];
                     for (int kc = 0; kc < p.k_chunks; ++kc) {
-                        if (is_a && issued == 0) CTRACE(9);
+                        if (warp == 0 && issued == 0) CTRACE(9);
                         ok = mbar_wait(smem_u32(&ctl->empty[sbase + s]), ph ^ 1, abort_flag, p.status, 1);
                         if (!ok) break;
-                        if (is_a && issued == 0) CTRACE(10);
-                        if (is_a) GTRACE(0, issued); else if (warp == 14) GTRACE(2, issued);
+                        if (warp == 0 && issued == 0) CTRACE(10);
+                        if (warp == 0) GTRACE(0, issued); else if (warp == 14) GTRACE(2, issued);
                         const uint32_t bar = smem_u32(&ctl->full[sbase + s]);
                         const uint32_t a_dst = data_base + (uint32_t)(sbase + s) * stage_bytes, b_dst = a_dst + a_bytes;
-                        if (is_a && p.test_skip && issued == 0) {         // test hook: this stage never becomes full
+                        if (warp == 0 && p.test_skip && issued == 0) {    // test hook: this stage never becomes full
                             ++issued;
                             if (++s == SR) { s = 0; ph ^= 1; }
                             continue;
                         }
-                        mbar_arrive_expect_tx(bar, my_bytes);
+                        const bool tail = kc + 1 == p.k_chunks;
+                        mbar_arrive_expect_tx(bar, tail ? tail_bytes : my_bytes);
                         if (is_a && !dep_waited) { CTRACE(1); grid_dependency_wait(); CTRACE(2); dep_waited = true; }
                         if (is_a) {
-                            if (p.a_tiled) tma_load_2d(a_dst, &tmA, bar, kc * kKC, m0);
-                            else tma_load_im2col_4d(a_dst, &tmA, bar, kc * kKC, w0, h0, n, ow, oh);
+                            const CUtensorMap *tm = tail ? &tmT : &tmA;
+                            if (p.a_tiled) tma_load_2d(a_dst, tm, bar, kc * kKC, m0);
+                            else tma_load_im2col_4d(a_dst, tm, bar, kc * kKC, w0, h0, n, ow, oh);
                         } else if (!B_MN) {
                             tma_load_3d(b_dst, &tmB, bar, kc * kKC, wtap, n0);
                         } else {
-                            for (int nb = bsel; nb < nb_b; nb += nbp)
+                            for (int nb = b_id; nb < nb_b; nb += p.n_b)
                                 tma_load_3d(b_dst + (uint32_t)nb * 8192u, &tmB, bar, n0 + nb * 64, wtap, kc * kKC);
                         }
-                        if (is_a) GTRACE(1, issued); else if (warp == 14) GTRACE(3, issued);
-                        if (is_a && issued == 0) CTRACE(3);
+                        if (warp == 0) GTRACE(1, issued); else if (warp == 14) GTRACE(3, issued);
+                        if (warp == 0 && issued == 0) CTRACE(3);
                         ++issued;
                         if (++s == SR) { s = 0; ph ^= 1; }
                     }
                 }
-                if (ring) { int t = s; s = s1; s1 = t; t = ph; ph = ph1; ph1 = t; }
                 if (!ok) break;
+                if (both) { int t = s; s = s1; s1 = t; t = ph; ph = ph1; ph1 = t; ring ^= 1; }
             }
-            if (*abort_flag && is_a) {
+            if (*abort_flag && warp == 0) {
                 // drain: give the copies already issued a bounded time to land before the CTA's smem is released
                 const uint64_t t0 = globaltimer_ns();
                 for (int s2 = 0; s2 < p.stages && issued > 0; ++s2)
@@ -361,7 +403,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) conv_gemm_kernel(const __grid
         const uint32_t leader = lane == 0 ? 1u : 0u;
         const uint32_t idesc = make_idesc_bf16(kBM, p.BN, 0, B_MN ? 1 : 0);
         const uint64_t bstep = B_MN ? 128ull : 2ull;
-        const uint32_t b_lbo = B_MN ? 8192u : 16u;
+        const uint64_t a_desc0 = make_desc_rows(0u, 128u), t_desc0 = make_desc_rows(0u, (uint32_t)p.tail_lanes * 2u);
+        const uint64_t b_desc0 = make_desc(0u, B_MN ? 8192u : 16u, 1024u);
         const int last_steps = (p.c_red - (p.k_chunks - 1) * kKC + 15) / 16;      // k-steps of a tap's last chunk
         const int NI = p.n_issuers, issuer = warp == 1 ? 0 : 1;
         const int SR = p.stages / NI, sbase = issuer * SR;
@@ -388,8 +431,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) conv_gemm_kernel(const __grid
                     const uint32_t b_src = p.resident ? w_base + (uint32_t)(tap * p.k_chunks + kc) * b_slot : a_src + a_bytes;
                     // one descriptor per operand and stage; a k-step only moves the 14-bit start-address field
                     // (units of 16 bytes): +32 B inside a K-major row, +2048 B (16 rows) in an MN-major tile
-                    const uint64_t ad0 = make_desc(a_src, 16u, 1024u);
-                    const uint64_t bd0 = make_desc(b_src, b_lbo, 1024u);
+                    const uint64_t ad0 = (kc + 1 < p.k_chunks ? a_desc0 : t_desc0) | desc_addr(a_src);
+                    const uint64_t bd0 = b_desc0 | desc_addr(b_src);
                     if (kc + 1 < p.k_chunks || last_steps == 4) {
                         umma_bf16_lead(d_tmem, ad0, bd0, idesc, acc, leader);
 #pragma unroll
@@ -433,46 +476,17 @@ __global__ void __launch_bounds__(kGemmThreads, 1) conv_gemm_kernel(const __grid
             // direct stores: this thread's raster pixel and where it lands in the output view
             const int m = m0 + quarter * 32 + lane;
             const bool row_ok = !p.tma_store && m < p.M_total;
-            size_t row_off = 0;
-            int cell_h = 0, cell_w = 0, img = 0;
+            int pix = 0;
             if (row_ok) {
-                const int j = m % p.Qd, t = m / p.Qd, i = t % p.Pd;
-                img = t / p.Pd;
-                cell_h = i * p.o_step;
-                cell_w = j * p.o_step;
-                row_off = ((size_t)(img * p.oH + cell_h + p.o_h0) * p.oW + cell_w + p.o_w0) * (size_t)p.ld_out;
-            }
-            if (!p.tma_store && p.zero_mask && n_tile == 0) {
-                // stride-2 data gradient: the pixels of each 2x2 cell that no tap reaches are zeros. They do not depend on the
-                // accumulator, so the warp writes them (a row at a time, lanes on consecutive 16-byte pieces) while the
-                // main loop is still running
-                for (int r = 0; r < 32; ++r) {
-                    if (!__shfl_sync(0xffffffffu, row_ok ? 1 : 0, r)) continue;
-                    const int ch_ = __shfl_sync(0xffffffffu, cell_h, r), cw_ = __shfl_sync(0xffffffffu, cell_w, r);
-                    const int im_ = __shfl_sync(0xffffffffu, img, r);
-                    for (int ab = 0; ab < 4; ++ab) {
-                        if (!((p.zero_mask >> ab) & 1)) continue;
-                        const int hh = ch_ + (ab >> 1), ww = cw_ + (ab & 1);
-                        if (hh >= p.oH || ww >= p.oW) continue;
-                        const size_t off = ((size_t)(im_ * p.oH + hh) * p.oW + ww) * (size_t)p.ld_out;
-                        if (p.out_f32) {
-                            float *o = (float *)p.out + off;
-                            for (int e = lane; e < p.n_cols; e += 32) o[e] = 0.f;
-                        } else {
-                            __nv_bfloat16 *o = (__nv_bfloat16 *)p.out + off;
-                            const int whole = p.n_cols & ~7;
-                            for (int e = lane * 8; e < whole; e += 256) *reinterpret_cast<uint4 *>(o + e) = make_uint4(0, 0, 0, 0);
-                            if (lane < p.n_cols - whole) o[whole + lane] = __float2bfloat16_rn(0.f);
-                        }
-                    }
-                }
+                const int j = m % p.Qd, t = m / p.Qd, i = t % p.Pd, img = t / p.Pd;
+                pix = (img * p.oH + i * p.o_step + p.o_h0) * p.oW + j * p.o_step + p.o_w0;
             }
             ok = mbar_wait(smem_u32(&ctl->acc_full[b]), aph, abort_flag, p.status, 3);
             if (!ok) break;
             if (quarter == 0) GTRACE(6, tc);
             tc_fence_after();
             const uint32_t lane_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * p.BN);
-            if (p.tma_store) {
+            if (!APART && p.tma_store) {
                 // Each warp stages its 32 rows x 64 channels (4 KB, 128-byte swizzle) and stores it with one TMA store,
                 // which drops the channels past the true count and the rows past the last pixel. Two slabs alternate.
                 const int n_chunks = (p.BN + 63) / 64;
@@ -525,7 +539,45 @@ __global__ void __launch_bounds__(kGemmThreads, 1) conv_gemm_kernel(const __grid
                 if (quarter == 0) GTRACE(7, tc);
                 continue;
             }
-            // ---- direct stores (fp32 outputs, strided stride-2 data-gradient outputs)
+            if (APART) {
+                // ---- strided stride-2 data-gradient outputs: through the warp's staging
+                const uint32_t rows = __ballot_sync(0xffffffffu, row_ok);
+                for (int c0 = 0; c0 < p.BN; c0 += 64) {
+                    const int groups = min(4, (p.BN - c0) / 16);
+                    uint32_t v[4][16];
+#pragma unroll
+                    for (int g = 0; g < 4; ++g)
+                        if (g < groups) tmem_ld16(lane_addr + (uint32_t)(c0 + g * 16), v[g]);
+                    tmem_ld_wait();
+                    if (c0 + 64 >= p.BN) {
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(smem_u32(&ctl->acc_empty[b]));
+                    }
+#pragma unroll
+                    for (int g = 0; g < 4; ++g) {
+                        if (g >= groups) break;
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            __nv_bfloat162 b0 = __floats2bfloat162_rn(__uint_as_float(v[g][8 * h + 0]), __uint_as_float(v[g][8 * h + 1]));
+                            __nv_bfloat162 b1 = __floats2bfloat162_rn(__uint_as_float(v[g][8 * h + 2]), __uint_as_float(v[g][8 * h + 3]));
+                            __nv_bfloat162 b2 = __floats2bfloat162_rn(__uint_as_float(v[g][8 * h + 4]), __uint_as_float(v[g][8 * h + 5]));
+                            __nv_bfloat162 b3 = __floats2bfloat162_rn(__uint_as_float(v[g][8 * h + 6]), __uint_as_float(v[g][8 * h + 7]));
+                            const uint32_t j = (uint32_t)(g * 2 + h);
+                            const uint32_t addr = slab0 + (uint32_t)lane * 128u + ((j ^ ((uint32_t)lane & 7u)) << 4);
+                            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(*reinterpret_cast<uint32_t *>(&b0)),
+                                         "r"(*reinterpret_cast<uint32_t *>(&b1)), "r"(*reinterpret_cast<uint32_t *>(&b2)),
+                                         "r"(*reinterpret_cast<uint32_t *>(&b3))
+                                         : "memory");
+                        }
+                    }
+                    __syncwarp();
+                    store_rows_apart((__nv_bfloat16 *)p.out, p.ld_out, slab0, n0 + c0, min(groups * 2, (p.vec_cols - n0 - c0) >> 3), rows, pix, lane);
+                    __syncwarp();
+                }
+                continue;
+            }
+            // ---- direct stores (fp32 outputs)
             for (int c0 = 0; c0 < p.BN; c0 += 16) {
                 uint32_t v[16];
                 tmem_ld16(lane_addr + (uint32_t)c0, v);
@@ -538,35 +590,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1) conv_gemm_kernel(const __grid
                 const int col = n0 + c0;
                 if (!row_ok || col >= p.n_cols) continue;
                 const int nvalid = min(16, p.n_cols - col);
-                if (p.out_f32) {
-                    float *o = (float *)p.out + row_off + col;
-                    if (nvalid == 16) {
+                float *o = (float *)p.out + (size_t)pix * (size_t)p.ld_out + col;
+                if (nvalid == 16) {
 #pragma unroll
-                        for (int g = 0; g < 4; ++g)
-                            reinterpret_cast<float4 *>(o)[g] = make_float4(__uint_as_float(v[4 * g]), __uint_as_float(v[4 * g + 1]),
-                                                                          __uint_as_float(v[4 * g + 2]), __uint_as_float(v[4 * g + 3]));
-                    } else {
-                        for (int e = 0; e < nvalid; ++e) o[e] = __uint_as_float(v[e]);
-                    }
+                    for (int g = 0; g < 4; ++g)
+                        reinterpret_cast<float4 *>(o)[g] = make_float4(__uint_as_float(v[4 * g]), __uint_as_float(v[4 * g + 1]),
+                                                                      __uint_as_float(v[4 * g + 2]), __uint_as_float(v[4 * g + 3]));
                 } else {
-                    __nv_bfloat16 *o = (__nv_bfloat16 *)p.out + row_off + col;
-#pragma unroll
-                    for (int g = 0; g < 2; ++g) {
-                        if (nvalid >= 8 * (g + 1)) {
-                            uint4 pk;
-                            __nv_bfloat162 b0 = __floats2bfloat162_rn(__uint_as_float(v[8 * g + 0]), __uint_as_float(v[8 * g + 1]));
-                            __nv_bfloat162 b1 = __floats2bfloat162_rn(__uint_as_float(v[8 * g + 2]), __uint_as_float(v[8 * g + 3]));
-                            __nv_bfloat162 b2 = __floats2bfloat162_rn(__uint_as_float(v[8 * g + 4]), __uint_as_float(v[8 * g + 5]));
-                            __nv_bfloat162 b3 = __floats2bfloat162_rn(__uint_as_float(v[8 * g + 6]), __uint_as_float(v[8 * g + 7]));
-                            pk.x = *reinterpret_cast<uint32_t *>(&b0);
-                            pk.y = *reinterpret_cast<uint32_t *>(&b1);
-                            pk.z = *reinterpret_cast<uint32_t *>(&b2);
-                            pk.w = *reinterpret_cast<uint32_t *>(&b3);
-                            *reinterpret_cast<uint4 *>(o + 8 * g) = pk;
-                        } else {
-                            for (int e = 8 * g; e < nvalid; ++e) o[e] = __float2bfloat16_rn(__uint_as_float(v[e]));
-                        }
-                    }
+                    for (int e = 0; e < nvalid; ++e) o[e] = __uint_as_float(v[e]);
                 }
             }
         }
@@ -580,6 +611,44 @@ __global__ void __launch_bounds__(kGemmThreads, 1) conv_gemm_kernel(const __grid
         if (p.tma_store && lane == 0) tma_store_wait_read();     // the staging slabs must outlive the stores' reads
         if (warp == 2) CTRACE(6);
         tc_fence_before();
+    } else if (B_MN && p.zero_mask && warp < 14) {
+        // ---------------- stride-2 data gradient: the pixels of each 2x2 cell that no tap reaches are zeros. They depend on no
+        // accumulator: the warps past the epilogue groups (four or eight) write them, each for 32 of a tile's raster pixels and the
+        // tile's columns, a row's whole 16-byte vectors on consecutive lanes. (Clearing dx in a pass of its own cost 25 of 70 us for
+        // 77 <- 154 channels at 56x56, batch 256; one column tile writing the zeros of all 20 of 38 us for 418 <- 931 at 28x28.)
+        const int z = warp - 2 - 4 * p.epi_groups, quarter = z & 3, nz = 3 - p.epi_groups;
+        const size_t off1 = (size_t)p.ld_out, off2 = (size_t)p.oW * p.ld_out;
+        for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
+            const int n_tile = tile % p.n_tiles, m = tile / p.n_tiles * kBM + quarter * 32 + lane;
+            const int n0 = n_tile * p.BN;
+            int cell = 0, mask = 0;                 // the cell's first pixel, the parities to clear
+            if (m < p.M_total) {
+                const int j = m % p.Qd, t = m / p.Qd, i = t % p.Pd;
+                cell = ((t / p.Pd) * p.oH + 2 * i) * p.oW + 2 * j;
+                mask = p.zero_mask & (2 * i + 1 < p.oH ? 0xf : 0x3) & (2 * j + 1 < p.oW ? 0xf : 0x5);
+            }
+            const int np = p.out_f32 ? min(p.BN, p.n_cols - n0) : min(p.BN, p.vec_cols - n0) >> 3;      // floats or vectors per pixel
+            const float inv_np = 1.0f / (float)np;
+            for (int k = z >> 2; k < np; k += nz) {
+                const int idx = k * 32 + lane, r = fast_div(idx, np, inv_np), e = idx - r * np;
+                const size_t off = (size_t)__shfl_sync(0xffffffffu, cell, r) * (size_t)p.ld_out + (size_t)(n0 + (p.out_f32 ? e : e * 8));
+                const int mk = __shfl_sync(0xffffffffu, mask, r);
+                if (!APART) {
+                    float *o = (float *)p.out + off;
+                    if (mk & 1) o[0] = 0.f;
+                    if (mk & 2) o[off1] = 0.f;
+                    if (mk & 4) o[off2] = 0.f;
+                    if (mk & 8) o[off2 + off1] = 0.f;
+                } else {
+                    __nv_bfloat16 *o = (__nv_bfloat16 *)p.out + off;
+                    const uint4 zero = make_uint4(0, 0, 0, 0);
+                    if (mk & 1) *reinterpret_cast<uint4 *>(o) = zero;
+                    if (mk & 2) *reinterpret_cast<uint4 *>(o + off1) = zero;
+                    if (mk & 4) *reinterpret_cast<uint4 *>(o + off2) = zero;
+                    if (mk & 8) *reinterpret_cast<uint4 *>(o + off2 + off1) = zero;
+                }
+            }
+        }
     }
     __syncthreads();
     if (warp == 0) CTRACE(7);
@@ -818,6 +887,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
         // ---------------- MMA issuer `issuer`: the whole warp walks the loops in lockstep, lane 0 issues
         const uint32_t leader = lane == 0 ? 1u : 0u;
         const uint32_t idesc = make_idesc_bf16(kBM, p.BN, 0, B_MN ? 1 : 0);
+        const uint64_t a_desc0 = make_desc_rows(0u, row_bytes), b_desc0 = B_MN ? make_desc(0u, b_block, 1024u) : make_desc_rows(0u, row_bytes);
         const uint64_t bstep = B_MN ? 128ull : 2ull;
         int sb_pos = 0, sb_ph = 0;                            // position in this issuer's weight ring
         int s_loc = 0, pha = 0;                               // position in this issuer's A ring
@@ -855,10 +925,10 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
                 tc_fence_after();
                 const int rem = p.c_red - kc * kKC;
                 const int ksteps = rem >= kKC ? 4 : (rem + 15) / 16;
-                const uint64_t abase = make_desc_rows(a_base + (uint32_t)sa * (uint32_t)p.a_alloc, row_bytes);
+                const uint64_t abase = a_desc0 | desc_addr(a_base + (uint32_t)sa * (uint32_t)p.a_alloc);
                 if (p.resident) {
                     // every tap is the same A tile read through a descriptor that starts (r*Wp + s) rows further on
-                    uint64_t bd0 = B_MN ? make_desc(b_base + (uint32_t)kc * b_slot, b_block, 1024u) : make_desc_rows(b_base + (uint32_t)kc * b_slot, row_bytes);
+                    uint64_t bd0 = b_desc0 | desc_addr(b_base + (uint32_t)kc * b_slot);
                     const uint64_t b_tap_step = (uint64_t)(((uint32_t)p.k_chunks * b_slot) >> 4);
                     if (ksteps == 1) {
                         for (int tap = 0; tap < p.taps; ++tap, bd0 += b_tap_step) {
@@ -885,7 +955,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
                         if (!ok) break;
                         tc_fence_after();
                         const uint64_t ad0 = abase + ctl->tap_aoff[tap];
-                        const uint64_t bd0 = B_MN ? make_desc(b_base + (uint32_t)sb * b_slot, b_block, 1024u) : make_desc_rows(b_base + (uint32_t)sb * b_slot, row_bytes);
+                        const uint64_t bd0 = b_desc0 | desc_addr(b_base + (uint32_t)sb * b_slot);
 #pragma unroll
                         for (int k = 0; k < 4; ++k)
                             if (k < ksteps) { umma_bf16_lead(d_tmem, ad0 + 2ull * k, bd0 + bstep * k, idesc, accumulate, leader); accumulate = 1u; }
@@ -1018,7 +1088,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
             }
             if (APART && !p.out_f32) {
                 // bf16 output pixels that are two apart (the parities of a stride-2 data gradient): the warp's 32 raster rows x 64 channels
-                // go through its own 4 KB of shared memory (128-byte swizzle) and leave as whole lines, eight lanes to a pixel. (A 4-D TMA
+                // go through its own 4 KB of shared memory (128-byte swizzle) and leave as whole lines. (A 4-D TMA
                 // store of a strided view takes longer: 46 -> 40 us for 103 -> 106 channels at 56x56. Of consecutive pixels it is the
                 // faster one by 1 to 3 us.)
                 const int n_chunks = (p.BN + 63) / 64;
@@ -1054,21 +1124,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
                         }
                     }
                     __syncwarp();
-                    const int pj = lane & 7, col = n0 + ch * 64 + pj * 8;       // this lane's 16-byte piece of every fourth row
-                    const bool col_ok = pj < groups * 2 && col < p.direct_cols;
-                    uint4 t[8];
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const uint32_t r = (uint32_t)(i * 4 + (lane >> 3));
-                        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(t[i].x), "=r"(t[i].y), "=r"(t[i].z), "=r"(t[i].w)
-                                     : "r"(wslab + r * 128u + (((uint32_t)pj ^ (r & 7u)) << 4)) : "memory");
-                    }
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const int r = i * 4 + (lane >> 3);
-                        const int px = __shfl_sync(0xffffffffu, pix, r);
-                        if (col_ok && ((rows >> r) & 1u)) *reinterpret_cast<uint4 *>((__nv_bfloat16 *)p.out + (size_t)px * (size_t)p.ld_out + col) = t[i];
-                    }
+                    store_rows_apart((__nv_bfloat16 *)p.out, p.ld_out, wslab, n0 + ch * 64, min(groups * 2, (p.direct_cols - n0 - ch * 64) >> 3), rows, pix, lane);
                     __syncwarp();
                 }
                 continue;
@@ -1154,16 +1210,6 @@ __device__ unsigned long long g_wg_trace[8][64];
 #else
 #define WTRACE(i) do { } while (0)
 #endif
-// n / d for 0 <= n < 2^22 and a divisor known per kernel: float reciprocal plus one correction step (an integer division
-// costs ~40 instructions, and the reduction below does two per 16-byte item).
-__device__ __forceinline__ int fast_div(int n, int d, float inv_d)
-{
-    int q = __float2int_rz(__int2float_rn(n) * inv_d);
-    if ((q + 1) * d <= n) ++q;
-    if (q * d > n) --q;
-    return q;
-}
-
 __device__ __forceinline__ int pt_ceil_div_dev(int a, int b) { return (a + b - 1) / b; }
 
 // 32 columns (16 where the accumulator ends) of a warp's 32 TMEM lanes; zeros for a CTA that had no work.
@@ -1931,9 +1977,14 @@ typedef CUresult (*EncodeIm2colFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_
                                    const int *, const int *, cuuint32_t, cuuint32_t, const cuuint32_t *, CUtensorMapInterleave,
                                    CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-// bf16 tensor (C, W, H, N) with channel pitch ld: im2col map loading `pixels` x 64 channels.
+CUtensorMapSwizzle lanes_swizzle(int lanes)
+{
+    return lanes == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : lanes == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B;
+}
+
+// bf16 tensor (C, W, H, N) with channel pitch ld: im2col map loading `pixels` x `lanes` channels.
 bool make_im2col_map(const pt_ctx *c, CUtensorMap *tm, const void *base, int C, int W, int H, int N, int ld, int lo_w, int lo_h,
-                     int up_w, int up_h, int stride, int pixels, int row_pixels = 0)
+                     int up_w, int up_h, int stride, int pixels, int row_pixels = 0, int lanes = kKC)
 {
     if (!c->encode_im2col) return false;
     if (lo_w < -128 || lo_h < -128 || up_w < -128 || up_h < -128 || lo_w > 127 || lo_h > 127 || up_w > 127 || up_h > 127) return false;
@@ -1943,30 +1994,25 @@ bool make_im2col_map(const pt_ctx *c, CUtensorMap *tm, const void *base, int C, 
     int lo[2] = {lo_w, lo_h}, up[2] = {up_w, up_h};
     cuuint32_t estr[4] = {1, (cuuint32_t)stride, (cuuint32_t)stride, 1};
     CUresult r = ((EncodeIm2colFn)c->encode_im2col)(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(base), dims, strides, lo,
-                                                    up, (cuuint32_t)kKC, (cuuint32_t)pixels, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                                                    CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                                                    up, (cuuint32_t)lanes, (cuuint32_t)pixels, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                                                    lanes_swizzle(lanes), CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                                                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return map_ok(r, __LINE__);
 }
 
 // bf16 activations as a plain 2-D tensor (channels, pixels) with row pitch ld: box 64 channels x `pixels`.
-bool make_act2d_map(const pt_ctx *c, CUtensorMap *tm, const void *base, int C, long long npix, int ld, int pixels)
+bool make_act2d_map(const pt_ctx *c, CUtensorMap *tm, const void *base, int C, long long npix, int ld, int pixels, int lanes = kKC)
 {
     if (!c->encode_tiled) return false;
     cuuint64_t dims[2] = {(cuuint64_t)C, (cuuint64_t)npix};
     cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
-    cuuint32_t box[2] = {(cuuint32_t)kKC, (cuuint32_t)pixels}, estr[2] = {1, 1};
+    cuuint32_t box[2] = {(cuuint32_t)lanes, (cuuint32_t)pixels}, estr[2] = {1, 1};
     CUresult r = ((CUresult(*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *,
                                const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
                                CUtensorMapL2promotion, CUtensorMapFloatOOBfill))c->encode_tiled)(
         tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-        CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+        lanes_swizzle(lanes), CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return map_ok(r, __LINE__);
-}
-
-CUtensorMapSwizzle lanes_swizzle(int lanes)
-{
-    return lanes == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : lanes == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B;
 }
 
 // bf16 weight shadow as (C, R*S, K) with row pitch ldw: box (lanes, 1, box_k).
@@ -2054,12 +2100,25 @@ bool make_out_map(const pt_ctx *c, CUtensorMap *tm, void *base, int cols, int ro
     return map_ok(r, __LINE__);
 }
 
+// Tensor maps of a GEMM-form launch: activation tiles (of 64 lanes, and of the last chunk's) and weight tiles.
+struct GemmMaps { CUtensorMap a, tail, b; };
+
+// Lanes the last chunk of `c` reduction channels is staged with: the TMA unit's time is per row, and longer where a box is wider than
+// what the tensor has left (128 rows of 13 of 64 lanes 0.62 us, of 16 lanes 0.48; 19 of 64 0.81, of 32 0.62).
+int gemm_tail_lanes(int c)
+{
+    const int rem = c - (pt_ceil_div(c, kKC) - 1) * kKC;
+    return rem <= 16 ? 16 : rem <= 32 ? 32 : 64;
+}
+
 template <bool B_MN>
-pt_status launch_gemm(pt_ctx *c, const CUtensorMap &tmA, const CUtensorMap &tmB, GemmP &p, cudaStream_t st)
+pt_status launch_gemm(pt_ctx *c, const GemmMaps &tm, GemmP &p, cudaStream_t st)
 {
     CUtensorMap tmC;
     memset(&tmC, 0, sizeof(tmC));
     p.tma_store = (!p.out_f32 && p.o_step == 1 && p.zero_mask == 0) ? 1 : 0;
+    const bool apart = !p.out_f32 && !p.tma_store;
+    if (apart && !B_MN) return PT_ERR_UNSUPPORTED;
     if (p.tma_store && !make_out_map(c, &tmC, p.out, p.n_cols, p.M_total, p.ld_out)) return PT_ERR_CUDA;
     const size_t a_bytes = kBM * kKC * 2;
     const size_t b_bytes = B_MN ? (size_t)pt_ceil_div(p.BN, 64) * 8192 : pt_align_up((size_t)p.BN * 128, 1024);
@@ -2070,6 +2129,7 @@ pt_status launch_gemm(pt_ctx *c, const CUtensorMap &tmA, const CUtensorMap &tmB,
     // accumulator buffers = epilogue groups: three when 3 * BN fits the 512 TMEM columns, else two; narrow layers whose
     // CTAs get a single tile need no more than that
     p.epi_groups = 3 * p.BN <= 512 ? 3 : 2;
+    if (p.zero_mask) p.epi_groups = 2;                            // (the warps of the third write the zeros)
     if (per_cta < p.epi_groups) p.epi_groups = per_cta;           // a single tile per CTA: one group, and its staging goes to the ring
     // Small weights (one channel tile, all taps x chunks within 64 KB) stay resident: the ring then carries A tiles only and
     // holds more of them, which is what an activation-bound layer needs to cover the memory latency.
@@ -2104,12 +2164,16 @@ pt_status launch_gemm(pt_ctx *c, const CUtensorMap &tmA, const CUtensorMap &tmB,
         p.stages = p.stages / 2 * 2;
         if (p.stages < 2) { p.n_issuers = 1; p.acc_per = 1; p.stages = 2; }
     }
+    p.n_a = (p.n_issuers == 2 && p.taps * p.k_chunks >= 2) ? 2 : 1;
+    p.n_b = (B_MN && !p.resident && p.BN > 64) ? 2 : 1;
+    p.vec_cols = pt_ceil_div(p.n_cols, 16) * 16 <= p.ld_out ? pt_ceil_div(p.n_cols, 16) * 16 : pt_ceil_div(p.n_cols, 8) * 8;
+    p.tail_lanes = gemm_tail_lanes(p.c_red);
     p.tmem_cols = pow2_cols((p.n_issuers == 2 ? 2 * p.acc_per : p.epi_groups) * p.BN);
     // the statistics variant exists for the forward kernel only
-    void (*kernel)(CUtensorMap, CUtensorMap, CUtensorMap, GemmP) =
-        (!B_MN && c->stats_mode) ? conv_gemm_kernel<false, true> : conv_gemm_kernel<B_MN, false>;
-    const int kid = (!B_MN && c->stats_mode) ? 2 : (B_MN ? 1 : 0);
-    static bool attr_set[3] = {false, false, false};
+    void (*kernel)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, GemmP) =
+        (!B_MN && c->stats_mode) ? conv_gemm_kernel<false, true, false> : apart ? conv_gemm_kernel<true, false, true> : conv_gemm_kernel<B_MN, false, false>;
+    const int kid = (!B_MN && c->stats_mode) ? 2 : apart ? 3 : (B_MN ? 1 : 0);
+    static bool attr_set[4] = {false, false, false, false};
     if (!attr_set[kid]) {
         PT_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
         attr_set[kid] = true;
@@ -2123,7 +2187,7 @@ pt_status launch_gemm(pt_ctx *c, const CUtensorMap &tmA, const CUtensorMap &tmB,
         p.stats = c->stats_out;
     }
     if (c->test_skip == 2) { p.test_skip = 1; c->test_skip = 0; }
-    PT_CUDA_OK(launch_pdl(kernel, dim3((unsigned)grid), dim3(kGemmThreads), smem, st, tmA, tmB, tmC, p));
+    PT_CUDA_OK(launch_pdl(kernel, dim3((unsigned)grid), dim3(kGemmThreads), smem, st, tm.a, tm.tail, tm.b, tmC, p));
     c->launches += 1;
     PT_CUDA_OK(cudaGetLastError());
     return PT_OK;
@@ -2204,7 +2268,11 @@ pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const
     p.direct = (!d->out_f32 && !c->stats_mode && p.n_tiles == 1 && p.BN <= 32) ? 1 : 0;
     // epilogue staging: a slab of the tile's raster rows x 128 bytes per group, two where the launch's other needs leave room (direct-store
     // launches use none)
-    p.tma_store = (d->out_f32 || p.direct || h.o_step != 1) ? 0 : 1;
+    // Outputs two pixels apart leave through the warps' own staging when the launch has the device to itself; launches that share it
+    // have few tiles, and the next tile's work hides the TMA store better (200 channels at 28x28: 24.2 against 25.9 us). Rows of 40 to 48
+    // channels leave two or three of a pixel's eight lanes idle (38 <- 40 at 56x56, batch 256: 50.3 against 52.8).
+    const bool apart = h.o_step != 1 && h.max_ctas == 0 && p.BN > 48;
+    p.tma_store = (d->out_f32 || p.direct || apart) ? 0 : 1;
     p.staging = (d->out_f32 || p.direct) ? 0 : !p.tma_store ? 4 * 4096 : (int)pt_align_up((size_t)(p.nr * Wp < 128 ? p.nr * Wp : 128) * 128, 1024);
     p.slabs = 1;
     p.stats_warp = pt_ceil_div(p.BN, 64) * (int)kStatsChunkBytes;
@@ -2295,8 +2363,8 @@ pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const
                         st_smem;
     p.stats_off = (int)(smem - st_smem);
     void (*kernel)(CUtensorMap, CUtensorMap, CUtensorMap, HaloP) =
-        (!B_MN && c->stats_mode) ? conv_halo_kernel<false, true, false> : (B_MN && h.o_step != 1) ? conv_halo_kernel<true, false, true> : conv_halo_kernel<B_MN, false, false>;
-    const int kid = (!B_MN && c->stats_mode) ? 2 : (B_MN && h.o_step != 1) ? 3 : (B_MN ? 1 : 0);
+        (!B_MN && c->stats_mode) ? conv_halo_kernel<false, true, false> : (B_MN && apart) ? conv_halo_kernel<true, false, true> : conv_halo_kernel<B_MN, false, false>;
+    const int kid = (!B_MN && c->stats_mode) ? 2 : (B_MN && apart) ? 3 : (B_MN ? 1 : 0);
     static bool attr_set[4] = {false, false, false, false};
     if (!attr_set[kid]) {
         PT_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
@@ -2743,9 +2811,9 @@ pt_status dgrad_stride2_halo(pt_ctx *c, const pt_conv_desc *d, int P, int Q, con
         ++n_launch;
     }
     if (n_launch == 0) return PT_ERR_UNSUPPORTED;
-    // a 1x1 filter on tiny images: one image fills less than half of a 128-row tile and the reduction is deep, so the
-    // pixel-linear tiles of the im2col kernel do better
-    if (d->R * d->S == 1 && (d->H / 2) * (d->W / 2) < 64) return PT_ERR_UNSUPPORTED;
+    // a 1x1 filter reads every pixel of dy once and has no halo: the pixel-linear tiles of the GEMM kernel, which also writes the
+    // zeros of the parities without a tap
+    if (d->R * d->S == 1) return PT_ERR_UNSUPPORTED;
     if (any_empty) PT_CUDA_OK(cudaMemsetAsync(dx, 0, (size_t)d->N * d->H * d->W * d->ldx * 2, st));
     // The parity classes write disjoint pixels of dx and read the same inputs: launches 1.. go to the context's helper
     // streams (forked from and joined back to the caller's stream by events) so that their fills and drains overlap.
@@ -2848,7 +2916,7 @@ pt_status pt_sm100_conv(pt_ctx *c, const pt_conv_desc *d, int which, const void 
                         size_t ws_bytes, cudaStream_t st)
 {
     const int P = pt_out_dim(d->H, d->R, d->stride, d->pad), Q = pt_out_dim(d->W, d->S, d->stride, d->pad);
-    CUtensorMap tmA, tmB;
+    GemmMaps tm;
     const StemPlan sp = stem_plan(d);
     if (which == PT_CONV_WGRAD) {
         if (sp.ok) {
@@ -2938,9 +3006,10 @@ pt_status pt_sm100_conv(pt_ctx *c, const pt_conv_desc *d, int which, const void 
         p.oH = sp.P; p.oW = sp.Q; p.o_step = 1; p.o_h0 = 0; p.o_w0 = 0; p.ld_out = d->ldy; p.zero_mask = 0;
         p.tmem_cols = pow2_cols(p.BN);
         const int up_h = (sp.P - 1) - sp.pl - (sp.Hs - 1);
-        if (!make_im2col_map(c, &tmA, xs, 64, sp.Q, sp.Hs, d->N, 16, 0, -sp.pl, 0, up_h, 1, kBM, sp.Wp)) return PT_ERR_CUDA;
-        if (!make_weight_map(c, &tmB, w2, 64, sp.U, d->K, 64, p.BN)) return PT_ERR_CUDA;
-        return launch_gemm<false>(c, tmA, tmB, p, st);
+        if (!make_im2col_map(c, &tm.a, xs, 64, sp.Q, sp.Hs, d->N, 16, 0, -sp.pl, 0, up_h, 1, kBM, sp.Wp)) return PT_ERR_CUDA;
+        tm.tail = tm.a;
+        if (!make_weight_map(c, &tm.b, w2, 64, sp.U, d->K, 64, p.BN)) return PT_ERR_CUDA;
+        return launch_gemm<false>(c, tm, p, st);
     }
     // A halo tile is whole raster rows of ONE image in at most 128 MMA rows: on small maps most of the tile is padding (7x7:
     // 49 useful rows of 128), and the pixel-linear tiles of the im2col kernel do better (7x7, 345 -> 374: 23 us against 30)
@@ -2966,6 +3035,7 @@ pt_status pt_sm100_conv(pt_ctx *c, const pt_conv_desc *d, int which, const void 
         pt_status r = dgrad_stride2_halo(c, d, P, Q, a, b, out, st);
         if (r != PT_ERR_UNSUPPORTED) return r;
     }
+    const int tail = gemm_tail_lanes(which == PT_CONV_FWD ? d->C : d->K);
     if (which == PT_CONV_FWD) {
         // raster = output pixels (P x Q per image); source = x
         p.M_total = d->N * P * Q;
@@ -2982,10 +3052,12 @@ pt_status pt_sm100_conv(pt_ctx *c, const pt_conv_desc *d, int which, const void 
         const int up_w = (Q - 1) * d->stride - d->pad - (d->W - 1), up_h = (P - 1) * d->stride - d->pad - (d->H - 1);
         if (d->R == 1 && d->S == 1 && d->stride == 1 && d->pad == 0) {
             p.a_tiled = 1;
-            if (!make_act2d_map(c, &tmA, a, d->C, (long long)d->N * d->H * d->W, d->ldx, kBM)) return PT_ERR_CUDA;
-        } else if (!make_im2col_map(c, &tmA, a, d->C, d->W, d->H, d->N, d->ldx, -d->pad, -d->pad, up_w, up_h, d->stride, kBM)) return PT_ERR_CUDA;
-        if (!make_weight_map(c, &tmB, b, d->C, d->R * d->S, d->K, d->ldw, p.BN)) return PT_ERR_CUDA;
-        return launch_gemm<false>(c, tmA, tmB, p, st);
+            if (!make_act2d_map(c, &tm.a, a, d->C, (long long)d->N * d->H * d->W, d->ldx, kBM) ||
+                !make_act2d_map(c, &tm.tail, a, d->C, (long long)d->N * d->H * d->W, d->ldx, kBM, tail)) return PT_ERR_CUDA;
+        } else if (!make_im2col_map(c, &tm.a, a, d->C, d->W, d->H, d->N, d->ldx, -d->pad, -d->pad, up_w, up_h, d->stride, kBM) ||
+                   !make_im2col_map(c, &tm.tail, a, d->C, d->W, d->H, d->N, d->ldx, -d->pad, -d->pad, up_w, up_h, d->stride, kBM, 0, tail)) return PT_ERR_CUDA;
+        if (!make_weight_map(c, &tm.b, b, d->C, d->R * d->S, d->K, d->ldw, p.BN)) return PT_ERR_CUDA;
+        return launch_gemm<false>(c, tm, p, st);
     }
     if (which != PT_CONV_DGRAD) return PT_ERR_UNSUPPORTED;
     p.n_cols = d->C;
@@ -2994,7 +3066,7 @@ pt_status pt_sm100_conv(pt_ctx *c, const pt_conv_desc *d, int which, const void 
     p.k_chunks = pt_ceil_div(d->K, kKC);
     p.tmem_cols = pow2_cols(p.BN);
     p.oH = d->H; p.oW = d->W; p.ld_out = d->ldx;
-    if (!make_weight_map(c, &tmB, b, d->C, d->R * d->S, d->K, d->ldw, kKC)) return PT_ERR_CUDA;
+    if (!make_weight_map(c, &tm.b, b, d->C, d->R * d->S, d->K, d->ldw, kKC)) return PT_ERR_CUDA;
     if (d->stride == 1) {
         // raster = input pixels (H x W per image); source = dy with padding R-1-pad and the taps visited flipped:
         // dx[h,w] = sum_{r',s'} dy[h - (R-1-pad) + r', w - (S-1-pad) + s'] * w[R-1-r', S-1-s']
@@ -3011,9 +3083,11 @@ pt_status pt_sm100_conv(pt_ctx *c, const pt_conv_desc *d, int which, const void 
         const int up_w = (d->W - 1) - pw - (Q - 1), up_h = (d->H - 1) - ph - (P - 1);
         if (d->R == 1 && d->S == 1 && d->pad == 0) {
             p.a_tiled = 1;
-            if (!make_act2d_map(c, &tmA, a, d->K, (long long)d->N * P * Q, d->ldy, kBM)) return PT_ERR_CUDA;
-        } else if (!make_im2col_map(c, &tmA, a, d->K, Q, P, d->N, d->ldy, -pw, -ph, up_w, up_h, 1, kBM)) return PT_ERR_CUDA;
-        return launch_gemm<true>(c, tmA, tmB, p, st);
+            if (!make_act2d_map(c, &tm.a, a, d->K, (long long)d->N * P * Q, d->ldy, kBM) ||
+                !make_act2d_map(c, &tm.tail, a, d->K, (long long)d->N * P * Q, d->ldy, kBM, tail)) return PT_ERR_CUDA;
+        } else if (!make_im2col_map(c, &tm.a, a, d->K, Q, P, d->N, d->ldy, -pw, -ph, up_w, up_h, 1, kBM) ||
+                   !make_im2col_map(c, &tm.tail, a, d->K, Q, P, d->N, d->ldy, -pw, -ph, up_w, up_h, 1, kBM, 0, tail)) return PT_ERR_CUDA;
+        return launch_gemm<true>(c, tm, p, st);
     }
     if (d->stride != 2) return PT_ERR_UNSUPPORTED;
     // Stride 2: the input pixels split by the parity (a, b) of (h, w) into four stride-1 problems over dy.
@@ -3057,8 +3131,13 @@ pt_status pt_sm100_conv(pt_ctx *c, const pt_conv_desc *d, int which, const void 
         p.o_step = 2; p.o_h0 = q.a; p.o_w0 = q.b;
         p.zero_mask = (ab == first) ? empty_mask : 0;
         const int up_w = (cols - 1) + min_ow - (Q - 1), up_h = (rows - 1) + min_oh - (P - 1);
-        if (!make_im2col_map(c, &tmA, a, d->K, Q, P, d->N, d->ldy, min_ow, min_oh, up_w, up_h, 1, kBM)) return PT_ERR_CUDA;
-        pt_status s = launch_gemm<true>(c, tmA, tmB, p, st);
+        p.a_tiled = (q.nt == 1 && min_oh == 0 && min_ow == 0 && rows == P && cols == Q) ? 1 : 0;      // dy's pixels in order
+        if (p.a_tiled) {
+            if (!make_act2d_map(c, &tm.a, a, d->K, p.M_total, d->ldy, kBM) || !make_act2d_map(c, &tm.tail, a, d->K, p.M_total, d->ldy, kBM, tail))
+                return PT_ERR_CUDA;
+        } else if (!make_im2col_map(c, &tm.a, a, d->K, Q, P, d->N, d->ldy, min_ow, min_oh, up_w, up_h, 1, kBM) ||
+                   !make_im2col_map(c, &tm.tail, a, d->K, Q, P, d->N, d->ldy, min_ow, min_oh, up_w, up_h, 1, kBM, 0, tail)) return PT_ERR_CUDA;
+        pt_status s = launch_gemm<true>(c, tm, p, st);
         if (s != PT_OK) return s;
     }
     return PT_OK;

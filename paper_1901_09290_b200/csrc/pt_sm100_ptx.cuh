@@ -208,6 +208,9 @@ __device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t lbo_bytes
     return d;
 }
 
+// The start-address field of a descriptor (the rest is the same for every stage of a ring).
+__device__ __forceinline__ uint64_t desc_addr(uint32_t saddr) { return (uint64_t)((saddr & 0x3ffffu) >> 4); }
+
 // K-major tile whose rows are `row_bytes` = 128, 64 or 32 bytes (64, 32 or 16 bf16 along K) with the swizzle of that width.
 __device__ __forceinline__ uint64_t make_desc_rows(uint32_t saddr, uint32_t row_bytes)
 {

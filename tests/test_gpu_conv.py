@@ -262,3 +262,27 @@ def test_weight_gradient_splits_as_a_cluster(N, H, C, K, R, stride):
             assert torch.equal(dw, again)                        # fixed order of the sums
     finally:
         B.pt_set_wgrad_cta_limit(c, 0)
+
+
+# (N, H, W, C, K, R, stride) at the edges of the launch variants: pixel rows of 16, 32 and 64 staged channels and outputs of at most 32
+# (one or several tiles per CTA); last chunks of 16, 17, 32 and 33 channels with a ring per issuer; outputs two pixels apart with one and
+# several column tiles, with and without room for 16-channel vectors, odd heights and widths, parities that no tap reaches
+VARIANTS = [
+    (4, 20, 20, 15, 33, 3, 1), (80, 20, 20, 16, 17, 3, 1), (80, 20, 20, 17, 31, 3, 1), (40, 20, 20, 32, 16, 3, 1), (40, 20, 20, 33, 32, 3, 1),
+    (76, 32, 32, 80, 40, 1, 1), (76, 32, 32, 81, 24, 1, 1), (76, 32, 32, 32, 96, 1, 1), (76, 32, 32, 33, 97, 1, 1),
+    (100, 34, 34, 70, 24, 3, 2), (100, 34, 34, 30, 20, 3, 2), (52, 34, 34, 290, 16, 3, 2),
+    (3, 9, 11, 70, 65, 1, 2), (2, 16, 16, 300, 40, 1, 2), (2, 10, 8, 23, 100, 1, 2), (400, 28, 28, 16, 72, 1, 2),
+]
+
+
+@pytest.mark.parametrize("shape", VARIANTS)
+def test_launch_variants(shape):
+    N, H, Wd, C, K, R, stride = shape
+    x, w, dy, pad = _case(*shape, seed=W.BASE_SEED + 71)
+    y16, dx16, dw, _ = Hh.run_conv_all(N, H, Wd, C, K, R, stride, pad, x, w, dy, algo=2, out_f32=0)
+    y32, dx32, _, _ = Hh.run_conv_all(N, H, Wd, C, K, R, stride, pad, x, w, dy, algo=2, out_f32=1)
+    Hh.check_conv(y16, K, oracle.conv_fwd(x.numpy(), w.numpy(), stride, pad), what="fwd")
+    Hh.check_conv(dx16, C, oracle.conv_dgrad(dy.numpy(), w.numpy(), H, Wd, stride, pad), what="dgrad")
+    Hh.check_conv(dw, C, oracle.conv_wgrad(x.numpy(), dy.numpy(), R, R, stride, pad), what="wgrad")
+    # the same sums, rounded once more
+    assert torch.equal(y16[..., :K], y32[..., :K].to(torch.bfloat16)) and torch.equal(dx16[..., :C], dx32[..., :C].to(torch.bfloat16))
