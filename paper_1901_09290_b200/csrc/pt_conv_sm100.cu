@@ -222,7 +222,7 @@ __device__ __forceinline__ int fast_div(int n, int d, float inv_d)
 }
 
 // Stores a warp's 32 staged rows (128 bytes each, 128-byte swizzle) of `pieces` 16-byte vectors to the pixels `pix` (one per lane) whose bit
-// of `rows` is set: eight lanes to a pixel. (Every lane on the next vector whatever its row: 40.7 -> 44.2 us for 103 -> 106 channels.)
+// of `rows` is set: eight lanes to a pixel. (Every lane on the next vector whatever its row: 33.9 -> 35.9 us for 256 <- 512 channels at 56x56, batch 64.)
 __device__ __forceinline__ void store_rows_apart(__nv_bfloat16 *out, int ld, uint32_t slab, int col, int pieces, uint32_t rows, int pix, int lane)
 {
     const int j = lane & 7;
@@ -746,8 +746,7 @@ constexpr int kHaloThreads = 512;
 // kernel therefore runs up to four issuer warps, each on its own scheduler: issuer i owns accumulator buffer i and
 // an A ring of its own (a waiter may lag an mbarrier by at most one phase, so issuers cannot share a ring), and takes
 // the tiles i, i + I, i + 2I, ... of the CTA. Weights that stream through a ring keep a single issuer.
-// APART: the output pixels are two apart (a variant of its own: one kernel with both epilogues spills).
-template <bool B_MN, bool STATS, bool APART>
+template <bool B_MN, bool STATS>
 __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid_constant__ CUtensorMap tmA,
                                                                      const __grid_constant__ CUtensorMap tmB,
                                                                      const __grid_constant__ CUtensorMap tmC, const HaloP p)
@@ -1000,7 +999,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
             if (gtid == 0) HTRACE(4, tc);
             tc_fence_after();
             const uint32_t lane_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * p.BN);
-            if (!APART && p.tma_store) {
+            if (p.tma_store) {
                 const int n_chunks = (p.BN + 63) / 64;
                 for (int ch = 0; ch < n_chunks; ++ch) {
                     if (gtid == 0) {                                 // the slab's previous store has read it
@@ -1083,49 +1082,6 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
                     __nv_bfloat162 b3 = __floats2bfloat162_rn(__uint_as_float(e[h8 + 6]), __uint_as_float(e[h8 + 7]));
                     *reinterpret_cast<uint4 *>(o + q8 * 8) = make_uint4(*reinterpret_cast<uint32_t *>(&b0), *reinterpret_cast<uint32_t *>(&b1),
                                                                         *reinterpret_cast<uint32_t *>(&b2), *reinterpret_cast<uint32_t *>(&b3));
-                }
-                continue;
-            }
-            if (APART && !p.out_f32) {
-                // bf16 output pixels that are two apart (the parities of a stride-2 data gradient): the warp's 32 raster rows x 64 channels
-                // go through its own 4 KB of shared memory (128-byte swizzle) and leave as whole lines. (A 4-D TMA
-                // store of a strided view takes longer: 46 -> 40 us for 103 -> 106 channels at 56x56. Of consecutive pixels it is the
-                // faster one by 1 to 3 us.)
-                const int n_chunks = (p.BN + 63) / 64;
-                const uint32_t wslab = staging_base + (uint32_t)(warp - 2) * 4096u;
-                const uint32_t rows = __ballot_sync(0xffffffffu, row_ok);
-                for (int ch = 0; ch < n_chunks; ++ch) {
-                    const int groups = min(4, (p.BN - ch * 64) / 16);
-                    uint32_t v[4][16];
-#pragma unroll
-                    for (int g = 0; g < 4; ++g)
-                        if (g < groups) tmem_ld16(lane_addr + (uint32_t)(ch * 64 + g * 16), v[g]);
-                    tmem_ld_wait();
-                    if (ch + 1 >= n_chunks) {
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(smem_u32(&ctl->acc_empty[b]));
-                    }
-#pragma unroll
-                    for (int g = 0; g < 4; ++g) {
-                        if (g >= groups) break;
-#pragma unroll
-                        for (int hh = 0; hh < 2; ++hh) {
-                            __nv_bfloat162 b0 = __floats2bfloat162_rn(__uint_as_float(v[g][8 * hh + 0]), __uint_as_float(v[g][8 * hh + 1]));
-                            __nv_bfloat162 b1 = __floats2bfloat162_rn(__uint_as_float(v[g][8 * hh + 2]), __uint_as_float(v[g][8 * hh + 3]));
-                            __nv_bfloat162 b2 = __floats2bfloat162_rn(__uint_as_float(v[g][8 * hh + 4]), __uint_as_float(v[g][8 * hh + 5]));
-                            __nv_bfloat162 b3 = __floats2bfloat162_rn(__uint_as_float(v[g][8 * hh + 6]), __uint_as_float(v[g][8 * hh + 7]));
-                            const uint32_t j = (uint32_t)(g * 2 + hh);
-                            const uint32_t addr = wslab + (uint32_t)lane * 128u + ((j ^ ((uint32_t)lane & 7u)) << 4);
-                            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(*reinterpret_cast<uint32_t *>(&b0)),
-                                         "r"(*reinterpret_cast<uint32_t *>(&b1)), "r"(*reinterpret_cast<uint32_t *>(&b2)),
-                                         "r"(*reinterpret_cast<uint32_t *>(&b3))
-                                         : "memory");
-                        }
-                    }
-                    __syncwarp();
-                    store_rows_apart((__nv_bfloat16 *)p.out, p.ld_out, wslab, n0 + ch * 64, min(groups * 2, (p.direct_cols - n0 - ch * 64) >> 3), rows, pix, lane);
-                    __syncwarp();
                 }
                 continue;
             }
@@ -2242,7 +2198,7 @@ pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const
     // box of the next width 3.1 ns. The rows also take less shared memory.
     p.lanes = h.Cs <= 16 ? 16 : h.Cs <= 32 ? 32 : 64;
     const int row_bytes = p.lanes * 2;
-    if ((h.row32 && (B_MN || h.Cs != 16)) || (!B_MN && h.o_step != 1)) return PT_ERR_UNSUPPORTED;
+    if (h.row32 && (B_MN || h.Cs != 16)) return PT_ERR_UNSUPPORTED;
     p.lo_h = h.lo_h; p.lo_w = h.lo_w;
     for (int t = 0; t < h.n_taps; ++t) {
         p.tap_oh[t] = (unsigned char)h.tap_oh[t]; p.tap_ow[t] = (unsigned char)h.tap_ow[t];
@@ -2268,12 +2224,8 @@ pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const
     p.direct = (!d->out_f32 && !c->stats_mode && p.n_tiles == 1 && p.BN <= 32) ? 1 : 0;
     // epilogue staging: a slab of the tile's raster rows x 128 bytes per group, two where the launch's other needs leave room (direct-store
     // launches use none)
-    // Outputs two pixels apart leave through the warps' own staging when the launch has the device to itself; launches that share it
-    // have few tiles, and the next tile's work hides the TMA store better (200 channels at 28x28: 24.2 against 25.9 us). Rows of 40 to 48
-    // channels leave two or three of a pixel's eight lanes idle (38 <- 40 at 56x56, batch 256: 50.3 against 52.8).
-    const bool apart = h.o_step != 1 && h.max_ctas == 0 && p.BN > 48;
-    p.tma_store = (d->out_f32 || p.direct || apart) ? 0 : 1;
-    p.staging = (d->out_f32 || p.direct) ? 0 : !p.tma_store ? 4 * 4096 : (int)pt_align_up((size_t)(p.nr * Wp < 128 ? p.nr * Wp : 128) * 128, 1024);
+    p.tma_store = (d->out_f32 || p.direct) ? 0 : 1;
+    p.staging = !p.tma_store ? 0 : (int)pt_align_up((size_t)(p.nr * Wp < 128 ? p.nr * Wp : 128) * 128, 1024);
     p.slabs = 1;
     p.stats_warp = pt_ceil_div(p.BN, 64) * (int)kStatsChunkBytes;
     const size_t st_smem = c->stats_mode ? (size_t)8 * p.stats_warp : 0;        // statistics accumulators of the eight epilogue warps
@@ -2363,9 +2315,9 @@ pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const
                         st_smem;
     p.stats_off = (int)(smem - st_smem);
     void (*kernel)(CUtensorMap, CUtensorMap, CUtensorMap, HaloP) =
-        (!B_MN && c->stats_mode) ? conv_halo_kernel<false, true, false> : (B_MN && apart) ? conv_halo_kernel<true, false, true> : conv_halo_kernel<B_MN, false, false>;
-    const int kid = (!B_MN && c->stats_mode) ? 2 : (B_MN && apart) ? 3 : (B_MN ? 1 : 0);
-    static bool attr_set[4] = {false, false, false, false};
+        (!B_MN && c->stats_mode) ? conv_halo_kernel<false, true> : conv_halo_kernel<B_MN, false>;
+    const int kid = (!B_MN && c->stats_mode) ? 2 : (B_MN ? 1 : 0);
+    static bool attr_set[3] = {false, false, false};
     if (!attr_set[kid]) {
         PT_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
         attr_set[kid] = true;
@@ -2815,7 +2767,7 @@ pt_status dgrad_stride2_halo(pt_ctx *c, const pt_conv_desc *d, int P, int Q, con
         h.lo_h = min_oh; h.lo_w = min_ow;
         h.n_cols = d->C; h.ld_out = d->ldx;
         h.oH = d->H; h.oW = d->W; h.o_step = 2; h.o_h0 = pa; h.o_w0 = pb;
-        if (h.Q + h.span_w - 1 > 128) return PT_ERR_UNSUPPORTED;
+        if (h.Q + h.span_w - 1 > 128) return PT_ERR_UNSUPPORTED;      // (so a tile has a row)
         ++n_launch;
     }
     if (n_launch == 0) return PT_ERR_UNSUPPORTED;
@@ -2833,19 +2785,36 @@ pt_status dgrad_stride2_halo(pt_ctx *c, const pt_conv_desc *d, int P, int Q, con
         if (!ok) { (void)cudaGetLastError(); return PT_ERR_CUDA; }
     }
     if (n_launch > 1) {
-        // each parity launch would fill the device on its own and they would run one after the other, each paying its start
-        // and drain; sharing the SMs in proportion to their taps lets them run side by side
-        // (measured: 28x28 <- 14x14, 200 channels: 40.7 -> 26.0 us; with three or more tiles per CTA it no longer pays)
-        int taps_total = 0;
-        for (int i = 0; i < n_launch; ++i) taps_total += hs[i].n_taps;
-        const int wp = hs[0].Q + 1, nr = 128 / wp < hs[0].P ? 128 / wp : hs[0].P;
-        int n_tiles;
-        (void)tile_n(d->C, &n_tiles);
-        const bool few_tiles = nr > 0 && d->N * pt_ceil_div(hs[0].P, nr) * n_tiles <= 2 * c->sm_count;
-        for (int i = 0; i < n_launch && few_tiles; ++i) {
-            hs[i].max_ctas = c->sm_count * hs[i].n_taps / taps_total;
-            if (hs[i].max_ctas < 8) hs[i].max_ctas = 8;
+        // Each parity launch would fill the device on its own and they would run one after the other, each paying its start and drain:
+        // they get shares of the SMs on which they run side by side and end together. A tile takes its taps' matrix work (0.066 us per
+        // 64 x 64 channels and tap) and 0.22 us; the shares are the smallest that finish all of their tiles, in whole rounds, within
+        // the shortest time for which they fit. 103 -> 106 at 56x56, batch 64: 40.6 -> 23.3 us; 64 -> 64, batch 256 49 -> 30;
+        // 11 -> 21 at 32x32, batch 128 15.6 -> 8.9; 200 -> 200 at 28x28, batch 64 40.7 -> 24.5.
+        int n_tiles, tiles[4], share[4];
+        const int bn = tile_n(d->C, &n_tiles);
+        double cost[4], lo = 0.0, hi = 0.0;
+        for (int i = 0; i < n_launch; ++i) {
+            const int wp = hs[i].Q + hs[i].span_w - 1, nr = 128 / wp < hs[i].P ? 128 / wp : hs[i].P;
+            tiles[i] = d->N * pt_ceil_div(hs[i].P, nr) * n_tiles;
+            cost[i] = 0.066 * hs[i].n_taps * pt_ceil_div(d->K, kKC) * (bn > 64 ? bn / 64.0 : 1.0) + 0.22;
+            if (tiles[i] * cost[i] > hi) hi = tiles[i] * cost[i];
         }
+        const auto fits = [&](double t) {
+            int sum = 0;
+            for (int i = 0; i < n_launch; ++i) {
+                const int rounds = (int)(t / cost[i] + 1e-6);
+                share[i] = rounds < 1 ? tiles[i] + c->sm_count : pt_ceil_div(tiles[i], rounds);
+                sum += share[i];
+            }
+            return sum <= c->sm_count;
+        };
+        while (!fits(hi)) hi *= 2.0;                  // (one CTA per launch fits)
+        for (int it = 0; it < 24; ++it) {
+            const double mid = 0.5 * (lo + hi);
+            if (fits(mid)) hi = mid; else lo = mid;
+        }
+        (void)fits(hi);
+        for (int i = 0; i < n_launch; ++i) hs[i].max_ctas = share[i];
     }
     if (n_launch > 1) PT_CUDA_OK(cudaEventRecord(c->fork_ev, st));
     pt_status first = PT_OK;
