@@ -1145,11 +1145,13 @@ struct WgradP {
     int ksteps;             // 16-pixel MMA steps per unit: ceil(nr * Wp / 16)
     int nb_a;               // 64-channel dy boxes per stage (1 when K <= 64)
     int lo_span;            // R - 1: extra rows of the x halo box
-    int pair;               // row-block form, C <= 64: the M side of an MMA is TWO taps x 64 input channels of the x tile
-                            // (the second tap is the first one shifted: the operand's 64-element block stride is that shift)
-                            // and the N side is the output channels; accumulator lanes = (tap, c), columns = k
+    int pair;               // row-block form: the M side of an MMA is two taps x 64 or four taps x 32 channel lanes of the x tile (a
+                            // tap is another one shifted: the operand's block stride is that shift) and the N side is the output
+                            // channels; accumulator lanes = (tap, c), columns = k
+    int lanes, dy_lanes;    // row-block form: channel lanes per staged pixel of x and of dy (rows of 128 or 64 bytes)
+    int acc_row;            // 32 lanes: accumulators per filter row, ceil(S / 4): each holds four neighbouring taps
     int cluster;            // 1: the splits of a tile are one thread-block cluster and meet in shared memory (no workspace)
-    int apc;                // accumulators per CTA (= tpc, or tpc / 2 in the paired form)
+    int apc;                // accumulators per CTA (= tpc in the generic form)
     int acc_cols;           // columns of one accumulator (= BN, or the padded K in the paired form)
     unsigned a_box, b_box;  // bytes reserved per dy box and per x box (multiples of 1024)
     unsigned data_bytes;    // shared memory behind the control block: the stages, and what the exchange of the splits may use
@@ -1167,6 +1169,14 @@ __device__ unsigned long long g_wg_trace[8][64];
 #define WTRACE(i) do { } while (0)
 #endif
 __device__ __forceinline__ int pt_ceil_div_dev(int a, int b) { return (a + b - 1) / b; }
+
+// Row-block form: the tap that the `g`-th group of lanes of accumulator `acc` (of all of the layer's) holds; `taps` where there is none.
+__device__ __forceinline__ int wgrad_tap(const WgradP &p, int acc, int g)
+{
+    if (p.lanes == 64) return min(2 * acc + g, p.taps);
+    const int r = acc / p.acc_row, s = (acc - r * p.acc_row) * 4 + g;
+    return s < p.S ? r * p.S + s : p.taps;
+}
 
 // 32 columns (16 where the accumulator ends) of a warp's 32 TMEM lanes; zeros for a CTA that had no work.
 __device__ __forceinline__ void wgrad_load32(uint32_t taddr, bool second, bool any, uint32_t (&v)[32])
@@ -1208,9 +1218,8 @@ __device__ __forceinline__ void wgrad_cluster_sum(const WgradP &p, Ctl *ctl, uin
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int S = p.splits, nch = pt_ceil_div_dev(acc_cols, 32);
-    // quarters of the 128 lanes that hold something: output channels below K; in the paired form channel lanes below C of both taps
-    const int nq = p.pair ? (p.C > 32 ? 4 : 2) : min(4, pt_ceil_div_dev(p.K - k0, 32));
-    const int qstep = p.pair && p.C <= 32 ? 2 : 1;
+    // quarters of the 128 lanes that hold something: output channels below K; in the row-block form the taps that exist
+    const int nq = !p.pair ? min(4, pt_ceil_div_dev(p.K - k0, 32)) : p.lanes == 32 ? min(4, p.S) : 4;
     const int slots = n_acc * nch * nq, mine = pt_ceil_div_dev(slots, S);              // slot u: owner u % S, its (u / S)-th
     const int cap = (int)(ring_bytes / ((uint32_t)S * 4096u));                         // slots an owner can receive at a time
     const bool any = iters > 0 && !*(volatile int *)&ctl->abort_flag;
@@ -1219,10 +1228,10 @@ __device__ __forceinline__ void wgrad_cluster_sum(const WgradP &p, Ctl *ctl, uin
         const int n = min(cap, mine - base);
         if (warp >= 1) {
             const int quarter = warp & 3, wset = (warp >= 2 && warp < 6) ? 0 : 1;
-            if (quarter % qstep == 0 && quarter / qstep < nq) {
+            if (quarter < nq) {
                 const uint32_t lane_addr = tmem_base + ((uint32_t)(quarter * 32) << 16);
                 for (int ci = wset; ci < n_acc * nch; ci += 2) {
-                    const int u = ci * nq + quarter / qstep, pos = u / S - base;
+                    const int u = ci * nq + quarter, pos = u / S - base;
                     if (pos < 0 || pos >= n) continue;
                     const int tt = ci / nch, cc = (ci - tt * nch) * 32;
                     uint32_t v[32];
@@ -1241,7 +1250,7 @@ __device__ __forceinline__ void wgrad_cluster_sum(const WgradP &p, Ctl *ctl, uin
         for (int i = threadIdx.x; i < n * 256; i += kThreads) {
             const int pos = i >> 8, u = (base + pos) * S + split;
             if (u >= slots) break;
-            const int ci = u / nq, quarter = (u - ci * nq) * qstep, tt = ci / nch, cc = (ci - tt * nch) * 32;
+            const int ci = u / nq, quarter = u - ci * nq, tt = ci / nch, cc = (ci - tt * nch) * 32;
             const int r = p.pair ? i & 31 : (i >> 3) & 31, j = p.pair ? (i >> 5) & 7 : i & 7;
             const int row = quarter * 32 + r, col = cc + j * 4;
             const uint32_t a = data_base + (uint32_t)pos * (uint32_t)S * 4096u + (uint32_t)r * 128u + ((uint32_t)(j ^ (r & 7)) << 4);
@@ -1252,8 +1261,8 @@ __device__ __forceinline__ void wgrad_cluster_sum(const WgradP &p, Ctl *ctl, uin
                 sum.x += t.x; sum.y += t.y; sum.z += t.z; sum.w += t.w;
             }
             if (p.pair) {
-                const int tap = tap0 + 2 * tt + (row >> 6), c = row & 63;
-                if (c < p.C && tap < tap0 + ntap) {
+                const int tap = wgrad_tap(p, tap0 + tt, row / p.lanes), c = row & (p.lanes - 1);
+                if (c < p.C && tap < p.taps) {
                     const float v4[4] = {sum.x, sum.y, sum.z, sum.w};
 #pragma unroll
                     for (int e = 0; e < 4; ++e)
@@ -1268,7 +1277,8 @@ __device__ __forceinline__ void wgrad_cluster_sum(const WgradP &p, Ctl *ctl, uin
 
 // Everything after the main loop of a weight-gradient kernel: the accumulators leave TMEM (directly to dw, or as this
 // split's partial tile), the splits of a tile meet, and every CTA sums its share of the tile over the splits.
-// `ring_bytes` of shared memory at `data_base` are free by then and serve as staging.
+// `ring_bytes` of shared memory at `data_base` are free by then and serve as staging. `tap0` is the CTA's first tap (generic form) or
+// accumulator (row-block form).
 __device__ __forceinline__ void wgrad_finish(const WgradP &p, const CUtensorMap &tmP, Ctl *ctl, uint32_t data_base, uint32_t tmem_base,
                                              int ntap, int tap0, int k0, int c0, int split, int iters, uint32_t ring_bytes, int n_acc, int acc_cols)
 {
@@ -1293,7 +1303,7 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, const CUtensorMap 
                 // ---- (1) this CTA's fp32 partial tile goes to the workspace through swizzled staging + TMA stores (the rows that
                 // hold something: not the output channels past K, in the paired form not the channel lanes past C)
                 const int gtid = (warp - 1) * 32 + lane;
-                const bool rows_used = p.pair ? (quarter & 1) * 32 < p.C : k0 + quarter * 32 < p.K;
+                const bool rows_used = !p.pair ? k0 + quarter * 32 < p.K : p.lanes == 64 || quarter < p.S;
                 int sl = 0, ci = 0;
                 for (int tt = 0; tt < n_acc && rows_used; ++tt)
                 for (int cc = 0; cc < acc_cols; cc += 32, ++ci) {
@@ -1342,14 +1352,14 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, const CUtensorMap 
                 named_barrier(1, 256);
                 if (warp == 2) WTRACE(5);
             } else if (p.pair) {
-                // lanes are (tap of the pair, input channel), columns are output channels: for one column a warp's lanes
+                // lanes are (tap of the accumulator, input channel), columns are output channels: for one column a warp's lanes
                 // write consecutive floats of dw
-                const int l = quarter * 32 + lane, c = l & 63;
+                const int l = quarter * 32 + lane, c = l & (p.lanes - 1);
                 int ci = 0;
                 for (int tt = 0; tt < n_acc; ++tt)
                 for (int cc = 0; cc < acc_cols; cc += 16, ++ci) {
                     if ((ci & 1) != wset) continue;
-                    const int tap = tap0 + 2 * tt + (l >> 6);
+                    const int tap = wgrad_tap(p, tap0 + tt, l / p.lanes);
                     uint32_t v[16];
                     if (iters > 0) {
                         tmem_ld16(lane_addr + (uint32_t)(tt * acc_cols + cc), v);
@@ -1358,7 +1368,7 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, const CUtensorMap 
 #pragma unroll
                         for (int e = 0; e < 16; ++e) v[e] = 0u;
                     }
-                    if (c >= p.C || tap >= tap0 + ntap) continue;
+                    if (c >= p.C || tap >= p.taps) continue;
 #pragma unroll
                     for (int e = 0; e < 16; ++e)
                         if (cc + e < p.K) p.out[((size_t)(cc + e) * p.taps + tap) * p.C + c] = __uint_as_float(v[e]);
@@ -1417,7 +1427,7 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, const CUtensorMap 
         // copies summed from shared memory in ascending split order: deterministic, whichever CTA does the work.
         // (Consecutive items run along a row in both forms: the partial tiles are then read whole sectors at a time. In the paired form
         // that scatters the writes to dw, but there are as many partial tiles to read as splits: 33 -> 31 us for 46 -> 59 at 56x56.)
-        const int rows_real = p.pair ? 2 * p.C : min(128, p.K - k0);
+        const int rows_real = !p.pair ? min(128, p.K - k0) : (p.lanes == 32 ? min(4, p.S) : 2) * p.C;
         const int ngrp = pt_ceil_div_dev(p.pair ? p.K : min(acc_cols, p.C - c0), 4);     // float4 groups per row
         const int items = rows_real * ngrp;
         const int total = n_acc * items;
@@ -1426,13 +1436,14 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, const CUtensorMap 
         const size_t zstride = (size_t)128 * acc_cols;
         const float *pbase = p.partial + (size_t)blockIdx.x * p.apc * p.splits * zstride;
         const int cap = (int)(((size_t)ring_bytes) / ((size_t)p.splits * 16));   // items the stage memory holds
-        const float inv_items = 1.0f / (float)items, inv_ngrp = 1.0f / (float)ngrp;
+        const float inv_items = 1.0f / (float)items, inv_ngrp = 1.0f / (float)ngrp, inv_c = 1.0f / (float)p.C;
         // row of the partial tile and first column of an item
         auto place = [&](int item, int &r, int &col) {
             if (p.pair) {
                 const int rr = fast_div(item, ngrp, inv_ngrp);
                 const int gq = item - rr * ngrp;
-                r = rr >= p.C ? 64 + rr - p.C : rr;
+                const int g = fast_div(rr, p.C, inv_c);
+                r = g * p.lanes + rr - g * p.C;
                 col = gq * 4;
             } else {
                 r = fast_div(item, ngrp, inv_ngrp);
@@ -1464,9 +1475,9 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, const CUtensorMap 
                     sum.x += t.x; sum.y += t.y; sum.z += t.z; sum.w += t.w;
                 }
                 if (p.pair) {
-                    // row = (tap of the pair, input channel), columns = output channels
-                    const int tap = tap0 + 2 * tt + (r >> 6), c = r & 63;
-                    if (c < p.C && tap < tap0 + ntap) {
+                    // row = (tap of the accumulator, input channel), columns = output channels
+                    const int tap = wgrad_tap(p, tap0 + tt, r / p.lanes), c = r & (p.lanes - 1);
+                    if (c < p.C && tap < p.taps) {
                         const float v4[4] = {sum.x, sum.y, sum.z, sum.w};
 #pragma unroll
                         for (int e = 0; e < 4; ++e)
@@ -1656,16 +1667,18 @@ __global__ void __launch_bounds__(kThreads) conv_wgrad_kernel(const __grid_const
 // Row-block form of the weight gradient for stride-1 filters with several taps and at most 64 input channels. A stage is
 // one unit = `nr` output rows of one image: dy as a box of nr rows x Wp columns (the columns past Q and the rows past P
 // are zero-filled by the TMA unit) and x as the halo box of nr + R - 1 rows x Wp columns starting at (-pad, -pad) of the
-// unit, both with one 128-byte swizzle row per pixel. Pixel m = i * Wp + j of the dy box pairs with pixel
+// unit, both with one swizzle row per pixel. Pixel m = i * Wp + j of the dy box pairs with pixel
 // m + r * Wp + s of the x box for tap (r, s), so every tap reads the SAME staged x tile through an operand descriptor
 // whose start is shifted by r * Wp + s rows: x crosses the memory system once per unit instead of once per tap. Where
 // j + s runs past the row the dy factor is a zero column. Rows past the boxes (up to the 16-pixel step) are zeroed once
 // and never written again.
-//   The x tile is the M side of the MMA and carries TWO taps: M rows 0..63 are the 64 channel lanes at the first tap's
-// shift, rows 64..127 the same lanes at the second tap's shift (the descriptor's 64-element block stride is the
-// difference of the shifts). The N side is dy's output channels. An accumulator therefore holds dw^T of a pair of taps:
-// lanes = (tap, c), columns = k -- half the MMAs of the one-tap-per-accumulator form, and none of the 128 rows wasted
-// when K is small.
+//   The x tile is the M side of the MMA and carries several taps. With 33 to 64 channels a pixel is a 128-byte row and M rows 0..63 are
+// its 64 lanes at the first tap's shift, rows 64..127 the same lanes at the second tap's (the descriptor's block stride is the difference
+// of the shifts). With at most 32 channels it is a 64-byte row and the four 32-lane blocks are the four neighbouring taps s, s + 1, ..
+// of a filter row (block stride one pixel; past S they are not stored). The N side is dy's output channels. An accumulator therefore
+// holds dw^T of two or four taps: lanes = (tap, c), columns = k -- a half or a third of the MMAs of the one-tap-per-accumulator form
+// for a 3x3 filter. The MMAs (29 ns each however narrow) and the TMA unit's time per row bound the narrow layers, and a 64-byte
+// row that ends inside a sector takes it 3.1 ns instead of 4.5.
 __global__ void __launch_bounds__(kThreads) conv_wgrad_rows_kernel(const __grid_constant__ CUtensorMap tmDy,
                                                                    const __grid_constant__ CUtensorMap tmX,
                                                                    const __grid_constant__ CUtensorMap tmP, const WgradP p)
@@ -1683,15 +1696,15 @@ __global__ void __launch_bounds__(kThreads) conv_wgrad_rows_kernel(const __grid_
     int bx = blockIdx.x;
     const int n_tile = bx % p.n_tiles; bx /= p.n_tiles;
     const int m_tile = bx % p.m_tiles; bx /= p.m_tiles;
-    const int tap0 = bx * p.tpc;
-    const int ntap = min(p.tpc, p.taps - tap0);
+    const int acc0 = bx * p.apc;                                      // this CTA's accumulators: acc0 .. acc0 + n_acc - 1
     const int split = blockIdx.y;
     const int k0 = m_tile * 128, c0 = n_tile * p.BN;
     const int u_beg = split * p.units_per_split;
     const int u_end = min(p.units, u_beg + p.units_per_split);
     const int iters = u_end > u_beg ? u_end - u_beg : 0;
-    const int n_acc = (ntap + 1) / 2;                                 // accumulators: one per pair of taps
-    const int NI = n_acc < 4 ? n_acc : 4;                             // MMA issuer warps in use: pairs i, i + NI, ...
+    const int n_acc = min(p.apc, (p.lanes == 64 ? (p.taps + 1) / 2 : p.taps / p.S * p.acc_row) - acc0);
+    const int NI = n_acc < 4 ? n_acc : 4;                             // MMA issuer warps in use: accumulators i, i + NI, ...
+    const uint32_t x_row = (uint32_t)p.lanes * 2u, dy_row = (uint32_t)p.dy_lanes * 2u;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < p.stages; ++s) {
@@ -1706,7 +1719,7 @@ __global__ void __launch_bounds__(kThreads) conv_wgrad_rows_kernel(const __grid_
     }
     // the rows between the end of a box and the end of the last 16-pixel step are read by the MMAs (times zero) and must be finite
     {
-        const uint32_t a_used = (uint32_t)(p.nr * p.Wp) * 128u, b_used = (uint32_t)((p.nr + p.lo_span) * p.Wp) * 128u;
+        const uint32_t a_used = (uint32_t)(p.nr * p.Wp) * dy_row, b_used = (uint32_t)((p.nr + p.lo_span) * p.Wp) * x_row;
         const uint32_t a_rest = (p.a_box - a_used) / 16u, b_rest = (p.b_box - b_used) / 16u;
         const uint32_t per_stage = (uint32_t)p.nb_a * a_rest + nb_b * b_rest;
         for (uint32_t i = threadIdx.x; i < (uint32_t)p.stages * per_stage; i += kThreads) {
@@ -1737,8 +1750,8 @@ __global__ void __launch_bounds__(kThreads) conv_wgrad_rows_kernel(const __grid_
             // ---------------- producers: warp 0 brings the dy boxes of every unit, warp 2 the x halo boxes
             const bool is_dy = warp == 0;
             const int n_dy = p.nb_a;
-            const uint32_t my_bytes = is_dy ? (uint32_t)(n_dy * p.nr * p.Wp) * 128u
-                                            : nb_b * (uint32_t)((p.nr + p.lo_span) * p.Wp) * 128u;
+            const uint32_t my_bytes = is_dy ? (uint32_t)(n_dy * p.nr * p.Wp) * dy_row
+                                            : nb_b * (uint32_t)((p.nr + p.lo_span) * p.Wp) * x_row;
             int n = u_beg / p.RB, rb = u_beg - n * p.RB;
             int s = 0, ph = 0, issued = 0;
             grid_dependency_wait();
@@ -1772,20 +1785,19 @@ __global__ void __launch_bounds__(kThreads) conv_wgrad_rows_kernel(const __grid_
         // ---------------- MMA issuer `issuer`: the warp walks the loop in lockstep, lane 0 issues
         const uint32_t leader = lane == 0 ? 1u : 0u;
         const uint32_t idesc = make_idesc_bf16(128, p.acc_cols, 1, 1);
-        // this issuer's pairs (at most four: 16 accumulators of 32 columns fill the tensor memory): byte offset of the
-        // first tap's rows in the x tile and the distance to the second tap's rows
-        uint32_t tap_shift[4] = {0u, 0u, 0u, 0u}, tap_lbo[4] = {128u, 128u, 128u, 128u};
+        // this issuer's accumulators (at most four: 16 of 32 columns fill the tensor memory): byte offset of the first tap's rows in
+        // the x tile and the distance to the next tap's rows
+        uint32_t tap_shift[4] = {0u, 0u, 0u, 0u}, tap_lbo[4] = {x_row, x_row, x_row, x_row};
         int n_mine = 0;
         for (int a = issuer; a < n_acc && n_mine < 4; a += NI, ++n_mine) {
-            const int t0 = tap0 + 2 * a, r0 = t0 / p.S, sh0 = r0 * p.Wp + (t0 - r0 * p.S);
-            int sh1 = sh0 + 1;                                        // an odd last tap: the upper 64 lanes are not stored
-            if (2 * a + 1 < ntap) {
+            const int t0 = wgrad_tap(p, acc0 + a, 0), r0 = t0 / p.S, sh0 = r0 * p.Wp + (t0 - r0 * p.S);
+            tap_shift[n_mine] = (uint32_t)sh0 * x_row;
+            if (p.lanes == 64 && t0 + 1 < p.taps) {                   // (an odd last tap: the upper 64 lanes are not stored)
                 const int r1 = (t0 + 1) / p.S;
-                sh1 = r1 * p.Wp + (t0 + 1 - r1 * p.S);
+                tap_lbo[n_mine] = (uint32_t)(r1 * p.Wp + (t0 + 1 - r1 * p.S) - sh0) * x_row;
             }
-            tap_shift[n_mine] = (uint32_t)sh0 * 128u;
-            tap_lbo[n_mine] = (uint32_t)(sh1 - sh0) * 128u;
         }
+        const uint64_t x_step = x_row, dy_step = dy_row;              // 16 pixels further on, in units of 16 bytes
         bool ok = true;
         int s = 0, ph = 0;
         for (int it = 0; it < iters && ok; ++it) {
@@ -1794,15 +1806,15 @@ __global__ void __launch_bounds__(kThreads) conv_wgrad_rows_kernel(const __grid_
             if (it == 0 && warp == 1) WTRACE(1);
             tc_fence_after();
             const uint32_t a_src = data_base + (uint32_t)s * stage_bytes, b_src = a_src + a_bytes;
-            const uint64_t dyd = make_desc(a_src, p.a_box, 1024u);
+            const uint64_t dyd = make_desc_mn(a_src, p.a_box, dy_row);
             const uint32_t acc = it != 0 ? 1u : 0u;
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 if (j >= n_mine) break;
-                const uint64_t xd = make_desc(b_src + tap_shift[j], tap_lbo[j], 1024u);
+                const uint64_t xd = make_desc_mn(b_src + tap_shift[j], tap_lbo[j], x_row);
                 const uint32_t d_tmem = tmem_base + (uint32_t)((issuer + j * NI) * p.acc_cols);
                 umma_bf16_lead(d_tmem, xd, dyd, idesc, acc, leader);
-                for (int k = 1; k < p.ksteps; ++k) umma_bf16_lead(d_tmem, xd + 128ull * k, dyd + 128ull * k, idesc, 1u, leader);
+                for (int k = 1; k < p.ksteps; ++k) umma_bf16_lead(d_tmem, xd + x_step * k, dyd + dy_step * k, idesc, 1u, leader);
             }
             umma_commit_lead(smem_u32(&ctl->empty[s]), leader);
             if (++s == p.stages) { s = 0; ph ^= 1; }
@@ -1810,7 +1822,7 @@ __global__ void __launch_bounds__(kThreads) conv_wgrad_rows_kernel(const __grid_
         if (ok) umma_commit_lead(smem_u32(&ctl->accum), leader);
         if (warp == 1) WTRACE(2);
     }
-    wgrad_finish(p, tmP, ctl, data_base, tmem_base, ntap, tap0, k0, c0, split, iters, p.data_bytes, n_acc, p.acc_cols);
+    wgrad_finish(p, tmP, ctl, data_base, tmem_base, 0, acc0, k0, c0, split, iters, p.data_bytes, n_acc, p.acc_cols);
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem_base, (uint32_t)p.tmem_cols);
@@ -2472,7 +2484,11 @@ bool wgrad_rows_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, pt_wg
     if (d->C > 64 || w->acc_cols > 256) return false;
     w->bn = tile_n(d->C, &w->n_tiles);
     w->m_tiles = 1;
-    const int pairs = pt_ceil_div(taps, 2);
+    w->lanes = d->C <= 32 ? 32 : 64;
+    w->dy_lanes = d->K <= 32 ? 32 : 64;
+    const size_t x_row = w->lanes * 2, dy_row = w->dy_lanes * 2;
+    const int span = w->lanes == 64 ? d->S : pt_ceil_div(d->S, 4) * 4;                       // columns of shifts the operands reach
+    const int pairs = w->lanes == 64 ? pt_ceil_div(taps, 2) : d->R * pt_ceil_div(d->S, 4);   // accumulators: of two or four taps
     int t = 512 / w->acc_cols;
     if (t > 16) t = 16;                                   // four issuer warps x four accumulators
     if (t > pairs) t = pairs;
@@ -2486,8 +2502,8 @@ bool wgrad_rows_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, pt_wg
     for (int pass = 0; pass < 2 && !large; ++pass) {
         for (int nr = 1; nr <= P && nr + d->R - 1 <= 256; ++nr) {
             const int ks = pt_ceil_div(nr * w->Wp, 16);
-            const size_t a_box = (size_t)ks * 2048;
-            const size_t b_box = pt_align_up(((size_t)(d->R - 1) * w->Wp + d->S + (size_t)ks * 16) * 128, 1024);
+            const size_t a_box = (size_t)ks * 16 * dy_row;
+            const size_t b_box = pt_align_up(((size_t)(d->R - 1) * w->Wp + span + (size_t)ks * 16) * x_row, 1024);
             const size_t stage = w->nb_a * a_box + b_box;
             const int st = (int)((220 * 1024 - 2048) / stage);
             if (st < 2) break;
@@ -2496,7 +2512,7 @@ bool wgrad_rows_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, pt_wg
                 w->nr = nr; w->ksteps = ks; w->a_box = (unsigned)a_box; w->b_box = (unsigned)b_box;
                 w->stages = st > kMaxStages ? kMaxStages : st;
                 w->stage_bytes = stage; w->RB = rb; w->units = units;
-                w->apc = apc; w->tpc = 2 * apc; w->tap_groups = pt_ceil_div(taps, w->tpc);
+                w->apc = apc; w->tap_groups = pt_ceil_div(pairs, apc);
                 w->splits = s; w->cluster = cl;
             };
             const double load = (double)(w->nb_a * nr + nr + d->R - 1) * w->Wp * 128.0 / 100e3;
@@ -2716,10 +2732,11 @@ pt_status run_wgrad_rows(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const p
     p.nr = wr.nr; p.Wp = wr.Wp; p.RB = wr.RB; p.units = wr.units; p.units_per_split = wr.units_per_split;
     p.ksteps = wr.ksteps; p.nb_a = wr.nb_a; p.lo_span = d->R - 1; p.a_box = wr.a_box; p.b_box = wr.b_box;
     p.stages = wr.stages;
+    p.lanes = wr.lanes; p.dy_lanes = wr.dy_lanes; p.acc_row = pt_ceil_div(d->S, 4);
     const int gx = p.n_tiles * p.m_tiles * p.tap_groups;
     // dy: box of nr rows x Wp columns (Wp > Q: the extra columns are out of bounds and read as zeros); x: the halo box
-    if (!make_halo_in_map(c, &tmA, dy, d->K, Q, P, d->N, d->ldy, wr.Wp, wr.nr)) return PT_ERR_UNSUPPORTED;
-    if (!make_halo_in_map(c, &tmX, x, d->C, d->W, d->H, d->N, d->ldx, wr.Wp, wr.nr + d->R - 1, kKC, x_row_pixels)) return PT_ERR_UNSUPPORTED;
+    if (!make_halo_in_map(c, &tmA, dy, d->K, Q, P, d->N, d->ldy, wr.Wp, wr.nr, wr.dy_lanes)) return PT_ERR_UNSUPPORTED;
+    if (!make_halo_in_map(c, &tmX, x, d->C, d->W, d->H, d->N, d->ldx, wr.Wp, wr.nr + d->R - 1, wr.lanes, x_row_pixels)) return PT_ERR_UNSUPPORTED;
     dim3 grid((unsigned)gx, (unsigned)p.splits);
     const size_t smem = (p.splits > 1 && wr.smem < kSplitSmemFloor) ? kSplitSmemFloor : wr.smem;
     p.data_bytes = (unsigned)(smem - 2048);

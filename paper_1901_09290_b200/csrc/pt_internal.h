@@ -50,6 +50,7 @@ struct pt_wgrad_plan {
     int splits, cluster;            // CTAs that share a tile's pixels; 1: they are one thread-block cluster
     // row-block form
     int nr, Wp, RB, units, units_per_split, ksteps, nb_a, stages;
+    int lanes, dy_lanes;            // channel lanes per staged pixel of x (64: two taps per accumulator, 32: four) and of dy
     unsigned a_box, b_box;
     size_t stage_bytes, smem;
 };

@@ -224,6 +224,19 @@ __device__ __forceinline__ uint64_t make_desc_rows(uint32_t saddr, uint32_t row_
     return d;
 }
 
+// MN-major operand in blocks of 64 or 32 elements (rows of 128 or 64 bytes along M or N, one row per k, the swizzle of that width):
+// `lbo_bytes` between blocks, groups of eight k rows dense.
+__device__ __forceinline__ uint64_t make_desc_mn(uint32_t saddr, uint32_t lbo_bytes, uint32_t row_bytes)
+{
+    uint64_t d = 0;
+    d |= (uint64_t)((saddr & 0x3ffffu) >> 4);
+    d |= (uint64_t)((lbo_bytes >> 4) & 0x3fffu) << 16;
+    d |= (uint64_t)((8u * row_bytes) >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (row_bytes == 128u ? 2ull : 4ull) << 61;
+    return d;
+}
+
 // Instruction descriptor: bf16 x bf16 -> fp32, M x N tile, operand majors (0 = K-major, 1 = MN-major).
 __host__ __device__ __forceinline__ uint32_t make_idesc_bf16(int M, int N, int a_mn, int b_mn)
 {
