@@ -2515,7 +2515,7 @@ bool wgrad_rows_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, pt_wg
                 w->apc = apc; w->tap_groups = pt_ceil_div(pairs, apc);
                 w->splits = s; w->cluster = cl;
             };
-            const double load = (double)(w->nb_a * nr + nr + d->R - 1) * w->Wp * 128.0 / 100e3;
+            const double load = (double)(w->nb_a * nr + nr + d->R - 1) * w->Wp * 2.4e-3;      // the TMA unit, by the row
             if (pass == 0) {
                 const double traffic = (double)(w->nb_a * nr + nr + d->R - 1) * rb / P, steps = (double)ks * 16 * rb / ((double)P * w->Wp);
                 if (traffic * steps >= best_cost) continue;
