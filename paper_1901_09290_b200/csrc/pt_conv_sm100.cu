@@ -1149,6 +1149,7 @@ struct WgradP {
                             // tap is another one shifted: the operand's block stride is that shift) and the N side is the output
                             // channels; accumulator lanes = (tap, c), columns = k
     int lanes, dy_lanes;    // row-block form: channel lanes per staged pixel of x and of dy (rows of 128 or 64 bytes)
+    int lane_shift;         // log2 of `lanes`
     int acc_row;            // 32 lanes: accumulators per filter row, ceil(S / 4): each holds four neighbouring taps
     int cluster;            // 1: the splits of a tile are one thread-block cluster and meet in shared memory (no workspace)
     int apc;                // accumulators per CTA (= tpc in the generic form)
@@ -1174,7 +1175,7 @@ __device__ __forceinline__ int pt_ceil_div_dev(int a, int b) { return (a + b - 1
 __device__ __forceinline__ int wgrad_tap(const WgradP &p, int acc, int g)
 {
     if (p.lanes == 64) return min(2 * acc + g, p.taps);
-    const int r = acc / p.acc_row, s = (acc - r * p.acc_row) * 4 + g;
+    const int r = p.acc_row == 1 ? acc : acc / p.acc_row, s = (acc - r * p.acc_row) * 4 + g;
     return s < p.S ? r * p.S + s : p.taps;
 }
 
@@ -1261,7 +1262,7 @@ __device__ __forceinline__ void wgrad_cluster_sum(const WgradP &p, Ctl *ctl, uin
                 sum.x += t.x; sum.y += t.y; sum.z += t.z; sum.w += t.w;
             }
             if (p.pair) {
-                const int tap = wgrad_tap(p, tap0 + tt, row / p.lanes), c = row & (p.lanes - 1);
+                const int tap = wgrad_tap(p, tap0 + tt, row >> p.lane_shift), c = row & (p.lanes - 1);
                 if (c < p.C && tap < p.taps) {
                     const float v4[4] = {sum.x, sum.y, sum.z, sum.w};
 #pragma unroll
@@ -1359,7 +1360,7 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, const CUtensorMap 
                 for (int tt = 0; tt < n_acc; ++tt)
                 for (int cc = 0; cc < acc_cols; cc += 16, ++ci) {
                     if ((ci & 1) != wset) continue;
-                    const int tap = wgrad_tap(p, tap0 + tt, l / p.lanes);
+                    const int tap = wgrad_tap(p, tap0 + tt, l >> p.lane_shift);
                     uint32_t v[16];
                     if (iters > 0) {
                         tmem_ld16(lane_addr + (uint32_t)(tt * acc_cols + cc), v);
@@ -1436,14 +1437,14 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, const CUtensorMap 
         const size_t zstride = (size_t)128 * acc_cols;
         const float *pbase = p.partial + (size_t)blockIdx.x * p.apc * p.splits * zstride;
         const int cap = (int)(((size_t)ring_bytes) / ((size_t)p.splits * 16));   // items the stage memory holds
-        const float inv_items = 1.0f / (float)items, inv_ngrp = 1.0f / (float)ngrp, inv_c = 1.0f / (float)p.C;
+        const float inv_items = 1.0f / (float)items, inv_ngrp = 1.0f / (float)ngrp;
         // row of the partial tile and first column of an item
         auto place = [&](int item, int &r, int &col) {
             if (p.pair) {
                 const int rr = fast_div(item, ngrp, inv_ngrp);
                 const int gq = item - rr * ngrp;
-                const int g = fast_div(rr, p.C, inv_c);
-                r = g * p.lanes + rr - g * p.C;
+                const int g = (rr >= p.C ? 1 : 0) + (rr >= 2 * p.C ? 1 : 0) + (rr >= 3 * p.C ? 1 : 0);
+                r = (g << p.lane_shift) + rr - g * p.C;
                 col = gq * 4;
             } else {
                 r = fast_div(item, ngrp, inv_ngrp);
@@ -1476,7 +1477,7 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, const CUtensorMap 
                 }
                 if (p.pair) {
                     // row = (tap of the accumulator, input channel), columns = output channels
-                    const int tap = wgrad_tap(p, tap0 + tt, r / p.lanes), c = r & (p.lanes - 1);
+                    const int tap = wgrad_tap(p, tap0 + tt, r >> p.lane_shift), c = r & (p.lanes - 1);
                     if (c < p.C && tap < p.taps) {
                         const float v4[4] = {sum.x, sum.y, sum.z, sum.w};
 #pragma unroll
@@ -1503,7 +1504,7 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, const CUtensorMap 
     }
 }
 
-__global__ void __launch_bounds__(kThreads) conv_wgrad_kernel(const __grid_constant__ CUtensorMap tmDy,
+__global__ void __launch_bounds__(kThreads, 1) conv_wgrad_kernel(const __grid_constant__ CUtensorMap tmDy,
                                                               const __grid_constant__ CUtensorMap tmX,
                                                               const __grid_constant__ CUtensorMap tmP, const WgradP p)
 {
@@ -1679,7 +1680,7 @@ __global__ void __launch_bounds__(kThreads) conv_wgrad_kernel(const __grid_const
 // holds dw^T of two or four taps: lanes = (tap, c), columns = k -- a half or a third of the MMAs of the one-tap-per-accumulator form
 // for a 3x3 filter. The MMAs (29 ns each however narrow) and the TMA unit's time per row bound the narrow layers, and a 64-byte
 // row that ends inside a sector takes it 3.1 ns instead of 4.5.
-__global__ void __launch_bounds__(kThreads) conv_wgrad_rows_kernel(const __grid_constant__ CUtensorMap tmDy,
+__global__ void __launch_bounds__(kThreads, 1) conv_wgrad_rows_kernel(const __grid_constant__ CUtensorMap tmDy,
                                                                    const __grid_constant__ CUtensorMap tmX,
                                                                    const __grid_constant__ CUtensorMap tmP, const WgradP p)
 {
@@ -2732,7 +2733,7 @@ pt_status run_wgrad_rows(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const p
     p.nr = wr.nr; p.Wp = wr.Wp; p.RB = wr.RB; p.units = wr.units; p.units_per_split = wr.units_per_split;
     p.ksteps = wr.ksteps; p.nb_a = wr.nb_a; p.lo_span = d->R - 1; p.a_box = wr.a_box; p.b_box = wr.b_box;
     p.stages = wr.stages;
-    p.lanes = wr.lanes; p.dy_lanes = wr.dy_lanes; p.acc_row = pt_ceil_div(d->S, 4);
+    p.lanes = wr.lanes; p.dy_lanes = wr.dy_lanes; p.acc_row = pt_ceil_div(d->S, 4); p.lane_shift = wr.lanes == 64 ? 6 : 5;
     const int gx = p.n_tiles * p.m_tiles * p.tap_groups;
     // dy: box of nr rows x Wp columns (Wp > Q: the extra columns are out of bounds and read as zeros); x: the halo box
     if (!make_halo_in_map(c, &tmA, dy, d->K, Q, P, d->N, d->ldy, wr.Wp, wr.nr, wr.dy_lanes)) return PT_ERR_UNSUPPORTED;
