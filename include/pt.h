@@ -87,7 +87,8 @@ uint64_t pt_launch_count(const pt_ctx *ctx);
  * The CTAs of a split launch wait (bounded) for one another and occupy an SM each, so all of them must be able to be on
  * the device at once: a caller that keeps weight-gradient launches in flight on S streams sets a limit L with
  * S * L <= the SM count. Beyond that the launches may starve each other until a wait expires (PT_ERR_TIMEOUT at the next
- * pt_poll_device_status; nothing hangs). */
+ * pt_poll_device_status; nothing hangs). A limit of at most half of the SMs also tells pt_conv_dgrad that such launches run
+ * beside it: it then leaves SMs free for them (results unchanged). */
 pt_status pt_set_wgrad_cta_limit(pt_ctx *ctx, int max_ctas);
 
 /* ------------------------------------------------------------------------------------------
