@@ -401,6 +401,8 @@ class TrainStep:
             self.conv_fwd(li, main)
         first_of = {d: f for f, d in br}
         join_after = None
+        if not wgrad:
+            self.ctx.set_wgrad_cta_limit(0)      # nothing runs beside the data gradients: all SMs are theirs
         wi = 0
         for li in range(n - 1, -1, -1):
             # dy_l exists once the data gradients above layer l are done: the weight gradient of layer l starts there, next
@@ -426,6 +428,8 @@ class TrainStep:
             if join_after == li:
                 main.wait_stream(aux)            # the gradient of the block's input sums both branches
                 join_after = None
+        if not wgrad:
+            self.ctx.set_wgrad_cta_limit(self.wgrad_ctas)
         if gather_join is not None:
             main.wait_stream(gather_join[1])
         for w in forked:
