@@ -180,16 +180,19 @@ class TrainStep:
         self.h_reg = torch.zeros(1, dtype=torch.float64).pin_memory()
 
     def _wgrad_work(self, li: int) -> float:
-        """Rough device time (us on one SM) of a layer's weight gradient: the larger of its MMA count at 55+ cycles each
-        and its tensor bytes at the ~35 GB/s one SM pulls; only ratios between layers are used."""
+        """Rough device time (us on one SM) of a layer's weight gradient: the largest of its MMA count at 55+ cycles each,
+        its tensor bytes at the ~35 GB/s one SM pulls and, for the row-block kernel, its staged pixel rows at 2.4 ns each; only
+        ratios between layers are used."""
         l = self.net.layers[li]
         px = self.N * l.P * l.P
         taps = l.R * l.R
+        t_rows = 0.0
         if l.stride == 2 and l.C <= 4:                       # space-to-depth stem: (R+1)/2 vertical taps of 64 lanes, two per MMA
             mmas = px / 16 * (((l.R + 1) // 2 + 1) // 2)
             cyc = 55
-        elif l.stride == 1 and l.C <= 64:                    # row-block kernel: two taps per MMA, N = K
-            mmas = px / 16 * ((taps + 1) // 2)
+        elif l.stride == 1 and l.C <= 64:                    # row-block kernel: two taps per MMA (four of a row), N = K
+            mmas = px / 16 * (l.R * -(-l.R // 4) if l.C <= 32 else (taps + 1) // 2)
+            t_rows = px * (1 + -(-W.pad16(l.K) // 64) + (l.R - 1) / 3) * 2.4e-3
             cyc = max(55, W.pad16(l.K) // 2 + 8)
         else:
             bn = min(256, W.pad16(l.C))
@@ -197,7 +200,7 @@ class TrainStep:
             cyc = max(55, bn // 2 + 8)
         t_mma = mmas * cyc / 1.9e3
         t_mem = (self.N * l.H * l.H * W.pad16(l.C) + px * W.pad16(l.K)) * 2 / 35e3
-        return max(t_mma, t_mem)
+        return max(t_mma, t_mem, t_rows)
 
     def _wgrad_limits(self) -> Dict[int, int]:
         """CTA limit of every weight-gradient launch. The launches go round-robin to three streams in reverse layer order,
