@@ -2754,7 +2754,7 @@ pt_status run_wgrad_rows(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const p
 // Stride-2 data gradient of a bf16 dx with even H and W: the input pixels split by the parity (a, b) of (h, w) into four
 // stride-1 correlations over dy (pixel h = 2i + a receives tap r iff a + pad - r is even, from dy row i + (a + pad - r)/2).
 // Each parity with taps is one halo-kernel launch that TMA-stores into the strided view of dx holding that parity; if some
-// parity has no tap (1x1 stride 2), dx is cleared first. Returns PT_ERR_UNSUPPORTED for shapes the halo kernel declines
+// parity has no tap, dx is cleared first (1x1 filters go to the GEMM kernel, which writes those zeros itself). Returns PT_ERR_UNSUPPORTED for shapes the halo kernel declines
 // (nothing has been launched then).
 pt_status dgrad_stride2_halo(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const void *dy, const void *w, void *dx, cudaStream_t st)
 {
