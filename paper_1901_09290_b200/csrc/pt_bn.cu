@@ -81,6 +81,7 @@ __device__ __forceinline__ uint4 lds128(uint32_t a)
 //                           free of the cancellation a large mean would cause in sum(x^2) - sum(x)^2/M).        in: x
 // PASS 1 (backward reduce): a0 = sum(dz), a1 = sum(dz * xhat), dz = dy where y > 0 (ReLU) else 0.               in: x, dy (, y)
 // PASS 2 (forward apply):   out = relu(x*scale + shift + residual), scale = gamma*invstd, shift = beta - mean*scale.  in: x (, residual)
+//                           The pivot comes from the row pass 0 left: out may be x itself, whose pixel 0 another block may have written.
 // PASS 3 (backward apply):  out2 = dz; out = gamma*invstd * (dz - dbeta/M - xhat*dgamma/M).                     in: x, dy (, y)
 // A reduce pass leaves `parts` rows [2][ld] of partial sums. Pad lanes (channel >= C) of the outputs are written as zeros.
 struct BnArgs {
@@ -90,6 +91,7 @@ struct BnArgs {
     float *rmean, *rvar;                    // moving statistics (pass 2, optional)
     float *dgamma, *dbeta;                  // written by pass 3
     float *partial;                         // rows of partial sums: written by the reduce passes, read by the apply passes
+    float *pivots;                          // the channels' pivots: written by pass 0, read by pass 2 (p.pivot)
     uint4 *out, *out2;
     unsigned int *status;
 };
@@ -165,6 +167,7 @@ bn_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUten
             const int c = c0 + e;
             tab[e] = c < p.C ? (PASS == 0 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(g.in[0])[c]) : g.mean[c]) : 0.f;
             tab[64 + e] = (PASS == 1 && c < p.C) ? g.invstd[c] : 0.f;
+            if (PASS == 0 && part == 0 && c < p.C) g.pivots[c] = tab[e];
         }
     } else {
         // fp64 sums of the slab's columns of the partial rows: thread (quad of columns, slice) adds its rows in ascending order, eight
@@ -206,7 +209,7 @@ bn_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUten
                     const double M = (double)p.M, d = s0 / M;
                     double var = s1 / M - d * d;
                     if (var < 0.0) var = 0.0;
-                    const double mean = (p.pivot ? (double)__bfloat162float(reinterpret_cast<const __nv_bfloat16 *>(g.in[0])[c]) : 0.0) + d;
+                    const double mean = (p.pivot ? (double)g.pivots[c] : 0.0) + d;
                     const float fm = (float)mean, fi = (float)(1.0 / sqrt(var + (double)p.eps));
                     k0 = g.gamma[c] * fi;
                     k1 = g.beta[c] - fm * k0;
@@ -421,7 +424,7 @@ extern "C" size_t pt_bn_workspace_bytes(const pt_ctx *c, const pt_bn_desc *d)
 {
     BnP p;
     if (bn_params(c, d, &p) != PT_OK) return 0;
-    return (size_t)p.parts * 2 * p.ld * sizeof(float);           // the reduce pass's rows of partial sums
+    return ((size_t)p.parts * 2 + 1) * p.ld * sizeof(float);     // the reduce pass's rows of partial sums, the forward pass's pivots
 }
 
 static bool aligned16(const void *q) { return ((uintptr_t)q & 15) == 0; }
@@ -441,7 +444,7 @@ extern "C" pt_status pt_bn_relu_fwd(pt_ctx *c, const pt_bn_desc *d, const void *
     BnArgs g{};
     g.in[0] = (const uint4 *)x; g.in[1] = (const uint4 *)residual;
     g.gamma = gamma; g.beta = beta; g.mean = save_mean; g.invstd = save_invstd; g.rmean = running_mean; g.rvar = running_var;
-    g.partial = (float *)ws; g.out = (uint4 *)y; g.status = c->d_status;
+    g.partial = (float *)ws; g.pivots = g.partial + (size_t)p.parts * 2 * p.ld; g.out = (uint4 *)y; g.status = c->d_status;
     r = launch_bn<0>(c, p, g, 1, st);
     if (r != PT_OK) return r;
     p.rows = p.parts; p.pivot = 1;

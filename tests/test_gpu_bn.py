@@ -110,3 +110,40 @@ def test_bn_is_run_to_run_identical_and_validates():
 def test_bn_relu_at_the_edges_of_the_channel_slabs(shape):
     test_bn_relu_forward_and_backward(shape, True, True)
     test_bn_relu_forward_and_backward(shape, False, True)
+
+
+def test_forward_in_place_when_its_blocks_start_late():
+    """y may be x: no block may read of x what another one has already overwritten. A weight gradient on another stream holds more than
+    half of the SMs meanwhile, so that blocks of the apply pass start after the first ones have finished."""
+    c = Hh.ctx()
+    N, H, C = 64, 28, 371                                    # six channel slabs of 24 blocks each
+    ld = W.pad16(C)
+    gen = torch.Generator(device="cuda").manual_seed(W.BASE_SEED + 577)
+    x = torch.zeros((N, H, H, ld), dtype=torch.bfloat16, device="cuda")
+    x[..., :C] = torch.randn((N, H, H, C), generator=gen, device="cuda") * 3.0 + 0.5
+    g, b = torch.rand(C, generator=gen, device="cuda") + 0.5, torch.rand(C, generator=gen, device="cuda") - 0.5
+    d = B.make_bn_desc(N, H, H, C, ld)
+    ws = torch.empty(B.pt_bn_workspace_bytes(c, d), dtype=torch.uint8, device="cuda")
+    stats = [torch.empty(C, device="cuda") for _ in range(4)]
+    y = torch.empty_like(x)
+    B.pt_bn_relu_fwd(c, d, x, None, g, b, None, None, stats[0], stats[1], y, ws)
+    wN, wH, wC = 128, 56, 256                                # about a millisecond on the SMs it may use
+    wd = B.make_conv_desc(wN, wH, wH, wC, wC, 3, 3, 1, 1)
+    wx = torch.randn((wN, wH, wH, wC), generator=gen, device="cuda").to(torch.bfloat16)
+    dw = torch.empty((wC, 3, 3, wC), device="cuda")
+    side = torch.cuda.Stream()
+    try:
+        B.pt_set_wgrad_cta_limit(c, 100)
+        assert B.pt_conv_wgrad_ctas(c, wd)[0] > 74
+        wws = Hh.conv_ws(wd, B.PT_CONV_WGRAD)
+        B.pt_conv_wgrad(c, wd, wx, wx, dw, wws)              # (loads the kernel: the launch below starts at once)
+        z = x.clone()
+        torch.cuda.synchronize()
+        B.pt_conv_wgrad(c, wd, wx, wx, dw, wws, stream=side)
+        torch.cuda._sleep(200000)                            # (a tenth of a millisecond: the weight gradient has its SMs by then)
+        B.pt_bn_relu_fwd(c, d, z, None, g, b, None, None, stats[2], stats[3], z, ws)
+        torch.cuda.synchronize()
+        c.poll()
+    finally:
+        B.pt_set_wgrad_cta_limit(c, 0)
+    assert torch.equal(z, y) and torch.equal(stats[0], stats[2]) and torch.equal(stats[1], stats[3])
