@@ -32,12 +32,13 @@ struct BnP {
     int slabs, sv;          // channel slabs, vectors of a slab
     int ppb;                // pixel rows the consumer threads cover at a time
     int consumers;          // consumer threads: sv * ppb rounded up to whole warps
-    int parts;              // blocks that share a slab's pixels = rows of partial sums of a reduce pass
+    int parts;              // blocks that share a slab's pixels
     int pix;                // pixels per chunk
     long long chunks;
     int stages, n_in;       // ring depth; input tensors of the pass
     int reverse;            // walk the chunks from the last to the first
     int rows, rows_vec;     // apply passes: rows of partial sums to finish; 1 = they may be read 16 bytes at a time
+    int pairs;              // 1: every row is followed by one of what its rounding left (a reduce pass's rows; not a convolution's)
     int pivot;              // the forward sums are about the channel's value at pixel 0 (else about 0)
     float eps, momentum;
     int relu;
@@ -83,7 +84,9 @@ __device__ __forceinline__ uint4 lds128(uint32_t a)
 // PASS 2 (forward apply):   out = relu(x*scale + shift + residual), scale = gamma*invstd, shift = beta - mean*scale.  in: x (, residual)
 //                           The pivot comes from the row pass 0 left: out may be x itself, whose pixel 0 another block may have written.
 // PASS 3 (backward apply):  out2 = dz; out = gamma*invstd * (dz - dbeta/M - xhat*dgamma/M).                     in: x, dy (, y)
-// A reduce pass leaves `parts` rows [2][ld] of partial sums. Pad lanes (channel >= C) of the outputs are written as zeros.
+// A reduce pass leaves two rows [2][ld] of partial sums per part: the sums, and what their rounding to fp32 left. A thread adds a chunk's few rows in fp32 and the chunks'
+// sums after that, a block its threads' in fp64: one fp32 chain per thread over all of its rows stagnates on the small terms of the
+// squares (1/std off by 2.7e-7 at 256x56x56x64, now 3e-8: the rounding of the result). Pad lanes (channel >= C) of the outputs are written as zeros.
 struct BnArgs {
     const uint4 *in[3];
     const float *gamma, *beta;
@@ -177,26 +180,27 @@ bn_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUten
         const int q = t % quads, z = t / quads, half = q >= quads / 2 ? 1 : 0, cq = (q - half * (quads / 2)) * 4;
         if (z < slices) {
             double acc[4] = {0.0, 0.0, 0.0, 0.0};
+            float lo[4] = {0.f, 0.f, 0.f, 0.f};                                  // the roundings' rows: fp32 is plenty for their sum
             if (c0 + cq < p.ld) {
+                const int pitch = p.pairs ? 4 * p.ld : 2 * p.ld;
                 const float *src = g.partial + (size_t)half * p.ld + c0 + cq;
-                for (int r = z; r < p.rows; r += 8 * slices) {
-                    float4 v[8];
+                const auto row = [&](int rr, int off) {
+                    const float *a = src + (size_t)rr * pitch + off;
+                    return rr >= p.rows ? make_float4(0.f, 0.f, 0.f, 0.f) : p.rows_vec ? *reinterpret_cast<const float4 *>(a) : make_float4(a[0], a[1], a[2], a[3]);
+                };
+                for (int r = z; r < p.rows; r += (p.pairs ? 4 : 8) * slices) {
+                    float4 v[8];                                                 // eight rows, or four and what their rounding left
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) v[u] = p.pairs ? row(r + (u & 3) * slices, u < 4 ? 0 : 2 * p.ld) : row(r + u * slices, 0);
 #pragma unroll
                     for (int u = 0; u < 8; ++u) {
-                        const int rr = r + u * slices;
-                        v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-                        if (rr < p.rows) {
-                            const float *a = src + (size_t)rr * 2 * p.ld;
-                            if (p.rows_vec) v[u] = *reinterpret_cast<const float4 *>(a);
-                            else v[u] = make_float4(a[0], a[1], a[2], a[3]);
-                        }
+                        if (u >= 4 && p.pairs) { lo[0] += v[u].x; lo[1] += v[u].y; lo[2] += v[u].z; lo[3] += v[u].w; }
+                        else { acc[0] += (double)v[u].x; acc[1] += (double)v[u].y; acc[2] += (double)v[u].z; acc[3] += (double)v[u].w; }
                     }
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) { acc[0] += (double)v[u].x; acc[1] += (double)v[u].y; acc[2] += (double)v[u].z; acc[3] += (double)v[u].w; }
                 }
             }
 #pragma unroll
-            for (int e = 0; e < 4; ++e) sl[(size_t)z * (quads * 4) + q * 4 + e] = acc[e];
+            for (int e = 0; e < 4; ++e) sl[(size_t)z * (quads * 4) + q * 4 + e] = acc[e] + (double)lo[e];
         }
         sm100::named_barrier(1, p.consumers);
         for (int e = t; e < cols; e += p.consumers) {
@@ -240,7 +244,7 @@ bn_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUten
     const bool masked = BWD && p.n_in > 2;
     const bool has_aux = p.n_in > 1;
     // per-channel constants of the thread's vector (0 past the true channel count) and, for the outputs, the bits to keep
-    float k0[8], k1[8], k2[PASS == 3 ? 8 : 1], k3[PASS == 3 ? 8 : 1], a0[REDUCE ? 8 : 1], a1[REDUCE ? 8 : 1];
+    float k0[8], k1[8], k2[PASS == 3 ? 8 : 1], k3[PASS == 3 ? 8 : 1], t0[REDUCE ? 8 : 1], t1[REDUCE ? 8 : 1];
     unsigned keep[REDUCE ? 1 : 4];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
@@ -248,7 +252,7 @@ bn_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUten
         k0[j] = tab[e];
         k1[j] = tab[64 + e];
         if (PASS == 3) { k2[j] = tab[128 + e]; k3[j] = tab[192 + e]; }
-        if (REDUCE) a0[j] = a1[j] = 0.f;
+        if (REDUCE) t0[j] = t1[j] = 0.f;
         if (!REDUCE && (j & 1) == 0) keep[j >> 1] = (c0 + e < p.C ? 0xffffu : 0u) | (c0 + e + 1 < p.C ? 0xffff0000u : 0u);
     }
     const __nv_bfloat162 zero2 = __floats2bfloat162_rn(0.f, 0.f);
@@ -261,6 +265,10 @@ bn_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUten
         if (active) {
             const uint32_t base = ring + (uint32_t)s * stage_bytes + (uint32_t)cv * 16u;
             const size_t row0 = (size_t)p0 * p.LV + v0 + cv;
+            float a0[REDUCE ? 8 : 1], a1[REDUCE ? 8 : 1];                        // the chunk's sums
+            if (REDUCE)
+#pragma unroll
+                for (int j = 0; j < 8; ++j) a0[j] = a1[j] = 0.f;
 #pragma unroll 2
             for (int r = pr; r < n; r += p.ppb) {
                 const uint32_t at = base + (uint32_t)r * pitch;
@@ -309,34 +317,52 @@ bn_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUten
                     }
                 }
             }
+            if (REDUCE)
+#pragma unroll
+                for (int j = 0; j < 8; ++j) { t0[j] += a0[j]; t1[j] += a1[j]; }
         }
         __syncwarp();
         if (lane == 0) sm100::mbar_arrive(sm100::smem_u32(&ctl->empty[s]));
         if (++s == p.stages) { s = 0; ph ^= 1; }
     }
     if (!REDUCE) return;
-    // the slab's part of one row of partial sums. The ring is idle by then (every chunk has been consumed) and takes the threads'
-    // sums, 16 per thread at a pitch of 17 words; the 16 x sv values are then added over the ppb pixel rows by all threads, in
+    // the slab's part of two rows of partial sums. The ring is idle by then (every chunk has been consumed) and takes the threads'
+    // sums, 16 per thread at a pitch of 17 words; the 16 x sv values are then added in fp64 over the ppb pixel rows by all threads, in
     // `pieces` groups of rows, and the groups by one thread per value: a fixed order
-    float *red = reinterpret_cast<float *>(smem + kBnData), *red2 = red + p.consumers * 17;
+    float *red = reinterpret_cast<float *>(smem + kBnData);
+    double *red2 = reinterpret_cast<double *>(red + p.consumers * 17);           // (consumers is a multiple of 32)
     sm100::named_barrier(1, p.consumers);
     if (pr < p.ppb)
 #pragma unroll
-        for (int j = 0; j < 8; ++j) { red[t * 17 + j] = active ? a0[j] : 0.f; red[t * 17 + 8 + j] = active ? (PASS == 1 ? a1[j] * k1[j] : a1[j]) : 0.f; }
+        for (int j = 0; j < 8; ++j) { red[t * 17 + j] = active ? t0[j] : 0.f; red[t * 17 + 8 + j] = active ? t1[j] : 0.f; }
     sm100::named_barrier(1, p.consumers);
     const int vals = p.sv * 16, pieces = p.consumers / vals;                     // (at least 2: a slab has at most 128 values)
     const int piece = t / vals, v = t - piece * vals, half = v >= cols ? 1 : 0, c = v - half * cols;
     if (piece < pieces) {
         const float *src = red + (c >> 3) * 17 + half * 8 + (c & 7);
-        float sum = 0.f;
-        for (int r = piece; r < p.ppb; r += pieces) sum += src[r * p.sv * 17];
-        red2[piece * vals + v] = sum;
+        // (two rows at a time in fp32: half of the conversions to fp64, and what that rounds is lost among the many pairs)
+        double acc[2] = {0.0, 0.0};
+        const int step = pieces * p.sv * 17;
+        src += piece * p.sv * 17;
+        for (int r = piece; r < p.ppb; r += 8 * pieces, src += 8 * step) {
+            float u[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) u[i] = r + i * pieces < p.ppb ? src[i * step] : 0.f;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[i & 1] += (double)(u[2 * i] + u[2 * i + 1]);
+        }
+        red2[piece * vals + v] = acc[0] + acc[1];
     }
     sm100::named_barrier(1, p.consumers);
     if (piece == 0 && c0 + c < p.ld) {
-        float sum = 0.f;
+        double sum = 0.0;
+#pragma unroll 4
         for (int k = 0; k < pieces; ++k) sum += red2[k * vals + v];
-        g.partial[((size_t)part * 2 + half) * p.ld + c0 + c] = sum;
+        if (PASS == 1 && half) sum *= (double)tab[64 + c];                       // sum(dz * (x - mean)) -> sum(dz * xhat)
+        const float hi = (float)sum;
+        float *o = g.partial + ((size_t)part * 4 + half) * p.ld + c0 + c;
+        *o = hi;
+        o[2 * p.ld] = isfinite(hi) ? (float)(sum - (double)hi) : 0.f;
     }
 }
 
@@ -399,7 +425,7 @@ pt_status launch_bn(pt_ctx *c, BnP p, const BnArgs &g, int n_in, cudaStream_t st
     p.reverse = PASS >= 2 ? 1 : 0;
     p.rows_vec = ((uintptr_t)g.partial & 15) == 0 ? 1 : 0;
     size_t smem = kBnData + (size_t)p.stages * stage;
-    const size_t red = kBnData + ((size_t)p.consumers * 17 + kBnThreads) * sizeof(float);
+    const size_t red = kBnData + (size_t)p.consumers * 17 * sizeof(float) + kBnThreads * sizeof(double);
     if (PASS < 2 && smem < red) smem = red;
     if (PASS >= 2) smem += (size_t)p.consumers * 4 * sizeof(double);             // the fp64 slices of the partial rows' sums
     static bool attr_set = false;
@@ -424,7 +450,7 @@ extern "C" size_t pt_bn_workspace_bytes(const pt_ctx *c, const pt_bn_desc *d)
 {
     BnP p;
     if (bn_params(c, d, &p) != PT_OK) return 0;
-    return ((size_t)p.parts * 2 + 1) * p.ld * sizeof(float);     // the reduce pass's rows of partial sums, the forward pass's pivots
+    return ((size_t)p.parts * 4 + 1) * p.ld * sizeof(float);     // the reduce pass's rows of partial sums, the forward pass's pivots
 }
 
 static bool aligned16(const void *q) { return ((uintptr_t)q & 15) == 0; }
@@ -444,10 +470,10 @@ extern "C" pt_status pt_bn_relu_fwd(pt_ctx *c, const pt_bn_desc *d, const void *
     BnArgs g{};
     g.in[0] = (const uint4 *)x; g.in[1] = (const uint4 *)residual;
     g.gamma = gamma; g.beta = beta; g.mean = save_mean; g.invstd = save_invstd; g.rmean = running_mean; g.rvar = running_var;
-    g.partial = (float *)ws; g.pivots = g.partial + (size_t)p.parts * 2 * p.ld; g.out = (uint4 *)y; g.status = c->d_status;
+    g.partial = (float *)ws; g.pivots = g.partial + (size_t)p.parts * 4 * p.ld; g.out = (uint4 *)y; g.status = c->d_status;
     r = launch_bn<0>(c, p, g, 1, st);
     if (r != PT_OK) return r;
-    p.rows = p.parts; p.pivot = 1;
+    p.rows = p.parts; p.pairs = 1; p.pivot = 1;
     r = launch_bn<2>(c, p, g, residual ? 2 : 1, st);
     if (r != PT_OK) return r;
     PT_CUDA_OK(cudaGetLastError());
@@ -473,7 +499,7 @@ extern "C" pt_status pt_bn_relu_bwd(pt_ctx *c, const pt_bn_desc *d, const void *
     g.partial = (float *)ws; g.out = (uint4 *)dx; g.out2 = (uint4 *)dresidual; g.status = c->d_status;
     r = launch_bn<1>(c, p, g, n_in, st);
     if (r != PT_OK) return r;
-    p.rows = p.parts;
+    p.rows = p.parts; p.pairs = 1;
     r = launch_bn<3>(c, p, g, n_in, st);
     if (r != PT_OK) return r;
     PT_CUDA_OK(cudaGetLastError());

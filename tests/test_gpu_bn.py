@@ -147,3 +147,34 @@ def test_forward_in_place_when_its_blocks_start_late():
     finally:
         B.pt_set_wgrad_cta_limit(c, 0)
     assert torch.equal(z, y) and torch.equal(stats[0], stats[2]) and torch.equal(stats[1], stats[3])
+
+
+# Batch statistics and parameter gradients against 64-bit sums of the same bf16 values: they carry little more than their own rounding to
+# fp32. Rounding is at most 2^-24 relative, 2^-24/sqrt(3) = 3.4e-8 rms for the worst place in a binade; the sums may add a third of that.
+# dgamma is a sum of terms of both signs, about sqrt(M) times smaller than their absolute sum: what the fp32 products and a chunk's few
+# fp32 additions leave (2^-25 per term, independent) is 2^-25 of the norm, and four times that is allowed.
+# (pixels and channels: many rows per thread; six slabs; 32 slabs of four blocks each)
+@pytest.mark.parametrize("shape", [(256, 56, 56, 64), (64, 28, 28, 371), (16, 7, 7, 2000)])
+def test_bn_sums_keep_their_precision(shape):
+    N, H, Wd, C = shape
+    c, ld = Hh.ctx(), W.pad8(C)
+    gen = torch.Generator(device="cuda").manual_seed(W.BASE_SEED + C)
+    x, dy = (torch.zeros((N, H, Wd, ld), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    x[..., :C] = torch.randn((N, H, Wd, C), generator=gen, device="cuda") + 0.25
+    dy[..., :C] = torch.randn((N, H, Wd, C), generator=gen, device="cuda")
+    d = B.make_bn_desc(N, H, Wd, C, ld, relu=False)
+    ws = torch.empty(B.pt_bn_workspace_bytes(c, d), dtype=torch.uint8, device="cuda")
+    one, zero = torch.ones(C, device="cuda"), torch.zeros(C, device="cuda")
+    mean, inv, dg, db = (torch.empty(C, device="cuda") for _ in range(4))
+    out = torch.empty_like(x)
+    B.pt_bn_relu_fwd(c, d, x, None, one, zero, None, None, mean, inv, out, ws)
+    B.pt_bn_relu_bwd(c, d, x, None, dy, one, mean, inv, out, None, dg, db, ws)
+    torch.cuda.synchronize()
+    xd, dd = x[..., :C].double(), dy[..., :C].double()
+    var, m64 = torch.var_mean(xd, (0, 1, 2), unbiased=False)
+    i64 = (var + float(np.float32(1e-5))).rsqrt()
+    rel = lambda got, ref: float((got.double() - ref).norm() / ref.norm())
+    assert rel(inv, i64) <= 4.5e-8
+    assert float(((mean.double() - m64) / var.sqrt()).square().mean().sqrt()) <= 4.5e-8
+    assert rel(db, dd.sum((0, 1, 2))) <= 4.5e-8
+    assert rel(dg, (dd * ((xd - mean.double()) * inv.double())).sum((0, 1, 2))) <= 1.2e-7
