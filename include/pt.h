@@ -131,7 +131,8 @@ pt_status pt_conv_fwd(pt_ctx *ctx, const pt_conv_desc *d, const void *x, const v
 /* The same forward convolution (bf16 output, tcgen05 kernels only: PT_ERR_UNSUPPORTED otherwise) that also takes the
  * statistics the batch normalisation after it needs (Sec. 2.1: the normalisation layers are bound by memory bandwidth because
  * they read their input several times): the epilogue adds, per output channel, the sum and the sum of squares of the bf16
- * values it stores -- from the tile that is still in shared memory -- and the CTAs leave them as rows. stats receives *n_parts (host, out)
+ * values it stores -- from the tile that is still in shared memory -- and the CTAs leave them as rows (one each, or two: the
+ * sums rounded to fp32 and what the rounding left). stats receives *n_parts (host, out)
  * rows of [2][ldy] floats (row r: sums, then sums of squares; columns >= K are zero); pt_bn_relu_fwd_stats combines them in a
  * fixed order. stats must hold pt_conv_fwd_stats_bytes(ctx, d) bytes (an upper bound that does not depend on which kernel
  * serves the layer); PT_ERR_WORKSPACE if it is smaller than this launch needs. Run-to-run identical. */

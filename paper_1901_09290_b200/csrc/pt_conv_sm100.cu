@@ -87,6 +87,7 @@ struct GemmP {
     int test_skip;      // test hook (pt_test_skip_next_arrive): the A producer leaves out the first stage of its first tile
     int stats_off;      // byte offset in shared memory of the epilogue warps' statistics accumulators (stats != nullptr)
     int stats_warp;     // bytes of one warp's accumulators: 512 per 64-channel chunk of the tile
+    int stats_lo;       // 1: two rows of sums per row of CTAs
     float *stats;       // optional: rows [2][ld_out] of floats, one per n_tiles CTAs: per output channel, sum and sum of squares of
                         // the bf16 values they stored (the batch-normalisation statistics of the layer that follows)
     void *out;
@@ -125,6 +126,8 @@ constexpr uint32_t kSlabs = 2;                          // staging slabs per epi
 // accumulated in the warp's own shared-memory slots (acc: 128 floats per chunk of the tile, four per lane); stats_store_cta
 // combines the warps of a CTA at the end. Feature normalisation (Sec. 2.1) reads its input twice; taking the sums here,
 // from the tile that is still in shared memory, removes the first of the two passes.
+// Fewer rows than this and the rounding of a CTA's sums (2^-25 over the square root of their number) shows in 1/std: 16x7x7x2000 has 18.
+constexpr int kStatsFewRows = 64;
 constexpr uint32_t kStatsChunkBytes = 128u * 4u;              // per 64-channel chunk: 32 lanes x (sum, sum of squares) x two channels
 
 __device__ __forceinline__ void chunk_stats(uint32_t slab, int row0, uint32_t rows, int lane, uint32_t acc)
@@ -165,28 +168,34 @@ __device__ __forceinline__ void stats_clear(uint32_t acc0, int lane, int n_chunk
             asm volatile("st.shared.v4.f32 [%0], {%1, %1, %1, %1};" ::"r"(acc0 + (uint32_t)ch * 512u + (uint32_t)lane * 16u), "f"(0.f) : "memory");
 }
 
-// The sums of a CTA's epilogue warps (accumulators of `stride` bytes each, from `acc0` on) are added in the order of the warps and
-// leave for a row of partial sums, [2][ld] floats. A CTA's tiles all have the same output channels n0 .. (its grid is a multiple of
+// The sums of a CTA's epilogue warps (accumulators of `stride` bytes each, from `acc0` on) are added in the order of the warps, in fp64
+// (two warps at a time in fp32: half of the conversions), and leave for a row of partial sums, [2][ld] floats, or for two (`lo`): the sums rounded, and what the rounding left. A CTA's tiles all have the same output channels n0 .. (its grid is a multiple of
 // the number of channel tiles), so that it writes once, and the CTAs of a row, one per channel tile, write disjoint columns; the
 // last one also writes the zeros up to ld. `tid` of `nthr` epilogue threads; a barrier of theirs comes before the call. (One row
 // per epilogue warp made up to 1776 rows, a few megabytes, for the normalisation to add up.)
-__device__ __forceinline__ void stats_store_cta(uint32_t acc0, uint32_t stride, int n_warps, int tid, int nthr, float *dst, int ld, int n_cols,
+__device__ __forceinline__ void stats_store_cta(uint32_t acc0, uint32_t stride, int n_warps, int tid, int nthr, float *dst, int ld, int lo, int n_cols,
                                                 int n0, int n_end)
 {
     for (int c = n0 + tid; c < n_end; c += nthr) {
-        float s0 = 0.f, s1 = 0.f;
+        double s0 = 0.0, s1 = 0.0;
         if (c < n_cols) {
             // a chunk is 64 channels: lane (c % 64) / 2 keeps (sum, sum of squares) of its two channels
             const int e = c - n0;
             const uint32_t a = acc0 + (uint32_t)(e >> 6) * 512u + (uint32_t)((e & 63) >> 1) * 16u + (uint32_t)(e & 1) * 8u;
-            for (int w = 0; w < n_warps; ++w) {
-                float u0, u1;
+            for (int w = 0; w < n_warps; w += 2) {               // (four, eight or twelve warps)
+                float u0, u1, v0, v1;
                 asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(u0), "=f"(u1) : "r"(a + (uint32_t)w * stride) : "memory");
-                s0 += u0; s1 += u1;
+                asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v0), "=f"(v1) : "r"(a + (uint32_t)(w + 1) * stride) : "memory");
+                s0 += (double)(u0 + v0); s1 += (double)(u1 + v1);
             }
         }
-        dst[c] = s0;
-        dst[ld + c] = s1;
+        const float h0 = (float)s0, h1 = (float)s1;
+        dst[c] = h0;
+        dst[ld + c] = h1;
+        if (lo) {
+            dst[2 * ld + c] = isfinite(h0) ? (float)(s0 - (double)h0) : 0.f;
+            dst[3 * ld + c] = isfinite(h1) ? (float)(s1 - (double)h1) : 0.f;
+        }
     }
 }
 
@@ -605,7 +614,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) conv_gemm_kernel(const __grid
             named_barrier(1, 128 * G);
             const int nt = (int)blockIdx.x % p.n_tiles;
             stats_store_cta(smem_base + (uint32_t)p.stats_off, (uint32_t)p.stats_warp, 4 * G, (int)threadIdx.x - 64, 128 * G,
-                            p.stats + (size_t)(blockIdx.x / p.n_tiles) * 2 * p.ld_out, p.ld_out, p.n_cols, nt * p.BN,
+                            p.stats + (size_t)(blockIdx.x / p.n_tiles) * (1 + p.stats_lo) * 2 * p.ld_out, p.ld_out, p.stats_lo, p.n_cols, nt * p.BN,
                             nt + 1 < p.n_tiles ? (nt + 1) * p.BN : p.ld_out);
         }
         if (p.tma_store && lane == 0) tma_store_wait_read();     // the staging slabs must outlive the stores' reads
@@ -684,6 +693,7 @@ struct HaloP {
     int oH, oW, o_step, o_h0, o_w0;      // direct stores: raster (n, i, j) -> out[((n*oH + i*o_step + o_h0)*oW + j*o_step + o_w0)*ld_out]
     int stats_off;                       // byte offset in shared memory of the epilogue warps' statistics accumulators
     int stats_warp;                      // bytes of one warp's accumulators: 512 per 64-channel chunk of the tile
+    int stats_lo;                        // 1: two rows of sums per row of CTAs
     float *stats;                        // optional: rows [2][ld_out], one per n_tiles CTAs: sums and sums of squares of the stored bf16
     void *out;
     unsigned int *status;
@@ -1105,7 +1115,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
             named_barrier(3, 256);
             const int nt = (int)blockIdx.x % p.n_tiles;
             stats_store_cta(smem_base + (uint32_t)p.stats_off, (uint32_t)p.stats_warp, 8, (int)threadIdx.x - 64, 256,
-                            p.stats + (size_t)(blockIdx.x / p.n_tiles) * 2 * p.ld_out, p.ld_out, p.n_cols, nt * p.BN,
+                            p.stats + (size_t)(blockIdx.x / p.n_tiles) * (1 + p.stats_lo) * 2 * p.ld_out, p.ld_out, p.stats_lo, p.n_cols, nt * p.BN,
                             nt + 1 < p.n_tiles ? (nt + 1) * p.BN : p.ld_out);
         }
         if (p.tma_store && gtid == 0) tma_store_wait_read();
@@ -2151,7 +2161,8 @@ pt_status launch_gemm(pt_ctx *c, const GemmMaps &tm, GemmP &p, cudaStream_t st)
     if (c->stats_mode) {
         if (!p.tma_store) return PT_ERR_UNSUPPORTED;
         if (grid > p.n_tiles) grid = grid / p.n_tiles * p.n_tiles;     // every CTA keeps one channel tile
-        c->stats_parts = grid / p.n_tiles;
+        p.stats_lo = grid / p.n_tiles < kStatsFewRows ? 1 : 0;
+        c->stats_parts = grid / p.n_tiles * (1 + p.stats_lo);
         if ((size_t)c->stats_parts * 2 * p.ld_out * sizeof(float) > c->stats_cap) return PT_ERR_WORKSPACE;
         p.stats = c->stats_out;
     }
@@ -2353,7 +2364,8 @@ pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const
     if (c->stats_mode) {
         if (!p.tma_store || B_MN) return PT_ERR_UNSUPPORTED;
         if (grid > p.n_tiles) grid = grid / p.n_tiles * p.n_tiles;     // every CTA keeps one channel tile
-        c->stats_parts = grid / p.n_tiles;
+        p.stats_lo = grid / p.n_tiles < kStatsFewRows ? 1 : 0;
+        c->stats_parts = grid / p.n_tiles * (1 + p.stats_lo);
         if ((size_t)c->stats_parts * 2 * p.ld_out * sizeof(float) > c->stats_cap) return PT_ERR_WORKSPACE;
         p.stats = c->stats_out;
     }

@@ -153,3 +153,29 @@ def test_every_layer_of_the_bench_workload_at_full_size():
         assert np.allclose(st[1, :l.K], s1, rtol=2e-5), l.name
         assert np.all(st[:, l.K:] == 0), l.name
         del x, w, y, y2, stats
+
+
+# Statistics taken by the convolution against 64-bit sums of the bf16 values it stored: the fp32 sums of a warp and the rounding of the result
+# (at most 2^-24/sqrt(3) = 3.4e-8 rms) are all that may show, whether few CTAs leave rows (18 at 7x7x2000) or one per SM
+@pytest.mark.parametrize("shape", [(16, 7, 300, 2000), (64, 14, 128, 512), (128, 16, 21, 24)])
+def test_statistics_keep_their_precision(shape):
+    N, H, C, K = shape
+    c = Hh.ctx()
+    gen = torch.Generator(device="cuda").manual_seed(W.BASE_SEED + K)
+    d = B.make_conv_desc(N, H, H, C, K, 1, 1, 1, 0)
+    x = torch.randn((N, H, H, d.ldx), generator=gen, device="cuda").clamp_(min=0).to(torch.bfloat16)
+    w = (torch.randn((K, 1, 1, d.ldw), generator=gen, device="cuda") * (2.0 / C) ** 0.5).to(torch.bfloat16)
+    y, a = (torch.zeros((N, H, H, d.ldy), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    stats = torch.empty(B.pt_conv_fwd_stats_bytes(c, d) // 4, device="cuda")
+    bn = B.make_bn_desc(N, H, H, K, d.ldy)
+    mean, inv = (torch.empty(K, device="cuda") for _ in range(2))
+    parts = B.pt_conv_fwd_stats(c, d, x, w, y, stats, None)
+    B.pt_bn_relu_fwd_stats(c, bn, y, None, torch.ones(K, device="cuda"), torch.zeros(K, device="cuda"), None, None, mean, inv, a, stats, parts)
+    var, m64 = torch.var_mean(y[..., :K].double(), (0, 1, 2), unbiased=False)
+    ref = (var + float(np.float32(1e-5))).rsqrt()
+    err = float((inv.double() - ref).norm() / ref.norm())
+    assert err <= 4.5e-8, err
+    rows = stats[:parts * 2 * d.ldy].view(parts, 2, d.ldy)[..., :K].double().sum(0)
+    y64 = y[..., :K].double()
+    # a warp's fp32 sum of squares: 2^-25 per addition, tens of additions, averaged over the warps of the grid
+    assert float((rows[1] / y64.square().sum((0, 1, 2)) - 1).abs().max()) <= 2.5e-8 * 4
