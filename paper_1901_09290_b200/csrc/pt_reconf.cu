@@ -116,7 +116,8 @@ __device__ __forceinline__ void bad_map_entry(unsigned int *status, unsigned int
 template <int U, int NS>
 __device__ __forceinline__ void gather_lines(const GatherJob &J, int line, int n, const int (&ol)[U], const int (&co)[4], int c)
 {
-    // 32-bit element offsets throughout (the host checks that both tensors have fewer than 2^31 elements at their pitches)
+    // 32-bit element offsets (the host checks that the old tensors have fewer than 2^31 elements at their pitch, and the new w and v are
+    // dense and no larger), except for the new shadow, whose pitch is the caller's choice
     float w[U][NS], v[U][NS];
     unsigned short h[U][NS];
     const unsigned short *ob = reinterpret_cast<const unsigned short *>(J.owb);
@@ -139,7 +140,7 @@ __device__ __forceinline__ void gather_lines(const GatherJob &J, int line, int n
             const unsigned dst = (unsigned)(line + u) * (unsigned)J.Cn + (unsigned)(c + 32 * j);
             J.nw[dst] = w[u][j];
             if (J.nv) J.nv[dst] = v[u][j];
-            if (nb) nb[(unsigned)(line + u) * (unsigned)J.ldwn + (unsigned)(c + 32 * j)] = h[u][j];
+            if (nb) nb[(size_t)(line + u) * (size_t)J.ldwn + (unsigned)(c + 32 * j)] = h[u][j];
         }
 }
 

@@ -270,3 +270,23 @@ def test_new_graph_larger_than_the_plan_is_reported_and_reads_nothing_out_of_ran
     assert np.array_equal(dn.w[0][:90].cpu().numpy(), ref)
     # layer 1 reads space 1: its extra input channel kept the guard
     assert torch.all(dn.w[1][:, :, :, 90] == guard)
+
+
+def test_new_shadow_with_a_pitch_past_32_bit_offsets():
+    """The pitch of the new shadow is the caller's choice: line 32 at a pitch of 2^27 starts 2^32 elements in."""
+    c, K, C, ldw = Hh.ctx(), 33, 8, 1 << 27
+    gen = torch.Generator(device="cuda").manual_seed(W.BASE_SEED)
+    w = torch.randn((K, C), generator=gen, device="cuda") + 3.0
+    old = B.make_layer(w, None, torch.zeros_like(w), w.to(torch.bfloat16), K, C, 1, C, True, True, *(torch.zeros(n, device="cuda") for n in (K, C)),
+                       *(torch.zeros(n, dtype=torch.uint8, device="cuda") for n in (K, C)))
+    shadow = torch.empty((K - 1) * ldw + C, dtype=torch.bfloat16, device="cuda")
+    nw, nv = torch.empty_like(w), torch.empty_like(w)
+    new = B.make_layer(nw, None, nv, shadow, K, C, 1, ldw, True, True, None, None, None, None)
+    g_old = B.GraphHandle([C, K], [True, True], [old], [(0, 1)])
+    n2o = torch.empty(C + K, dtype=torch.int32, device="cuda")
+    assert B.pt_reconfigure_plan(c, g_old, n2o) == [C, K]
+    B.pt_reconfigure(c, g_old, n2o, B.GraphHandle([C, K], [True, True], [new], [(0, 1)]))
+    torch.cuda.synchronize()
+    c.poll()
+    got = torch.stack([shadow[k * ldw:k * ldw + C] for k in range(K)])
+    assert torch.equal(nw, w) and torch.equal(got, w.to(torch.bfloat16))
