@@ -2766,7 +2766,7 @@ pt_status run_wgrad_rows(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const p
 // Stride-2 data gradient of a bf16 dx with even H and W: the input pixels split by the parity (a, b) of (h, w) into four
 // stride-1 correlations over dy (pixel h = 2i + a receives tap r iff a + pad - r is even, from dy row i + (a + pad - r)/2).
 // Each parity with taps is one halo-kernel launch that TMA-stores into the strided view of dx holding that parity; if some
-// parity has no tap, dx is cleared first (1x1 filters go to the GEMM kernel, which writes those zeros itself). Returns PT_ERR_UNSUPPORTED for shapes the halo kernel declines
+// parity has no tap, dx is cleared first (1x1 filters without padding go to the GEMM kernel, which writes those zeros itself). Returns PT_ERR_UNSUPPORTED for shapes the halo kernel declines
 // (nothing has been launched then).
 pt_status dgrad_stride2_halo(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const void *dy, const void *w, void *dx, cudaStream_t st)
 {
@@ -2806,8 +2806,9 @@ pt_status dgrad_stride2_halo(pt_ctx *c, const pt_conv_desc *d, int P, int Q, con
     }
     if (n_launch == 0) return PT_ERR_UNSUPPORTED;
     // a 1x1 filter reads every pixel of dy once and has no halo: the pixel-linear tiles of the GEMM kernel, which also writes the
-    // zeros of the parities without a tap
-    if (d->R * d->S == 1) return PT_ERR_UNSUPPORTED;
+    // zeros of the parities without a tap. It anchors them at parity (0, 0), which the tap of a filter with padding 1 does not reach:
+    // that one stays here, unless the maps are so small that a tile is mostly padding
+    if (d->R * d->S == 1 && ((d->pad & 1) == 0 || (d->H / 2) * (d->W / 2) < 64)) return PT_ERR_UNSUPPORTED;
     if (any_empty) PT_CUDA_OK(cudaMemsetAsync(dx, 0, (size_t)d->N * d->H * d->W * d->ldx * 2, st));
     // The parity classes write disjoint pixels of dx and read the same inputs: launches 1.. go to the context's helper
     // streams (forked from and joined back to the caller's stream by events) so that their fills and drains overlap.

@@ -286,3 +286,16 @@ def test_launch_variants(shape):
     Hh.check_conv(dw, C, oracle.conv_wgrad(x.numpy(), dy.numpy(), R, R, stride, pad), what="wgrad")
     # the same sums, rounded once more
     assert torch.equal(y16[..., :K], y32[..., :K].to(torch.bfloat16)) and torch.equal(dx16[..., :C], dx32[..., :C].to(torch.bfloat16))
+
+
+# a 1x1 filter of stride 2 with padding 1 reaches the odd pixels only: the pixels of parity (0, 0) are among the zeros
+@pytest.mark.parametrize("N,H,W_,C,K", [(2, 16, 16, 40, 24), (3, 18, 32, 130, 70)])
+def test_data_gradient_of_a_padded_1x1_at_stride_2(N, H, W_, C, K):
+    c = Hh.ctx()
+    w, dy = W.bf16_round(W.gen_weight(K, 1, 1, C, W.BASE_SEED + 81)), W.gen_dy(N, H // 2 + 1, W_ // 2 + 1, K, W.BASE_SEED + 82)
+    d = B.make_conv_desc(N, H, W_, C, K, 1, 1, 2, 1, algo=2)
+    dx = Hh.out_buffer((N, H, W_), C, d.ldx, False)
+    B.pt_conv_dgrad(c, d, Hh.to_dev_padded(dy, d.ldy), Hh.to_dev_padded(w, d.ldw), dx, None)
+    torch.cuda.synchronize()
+    c.poll()
+    Hh.check_conv(dx, C, oracle.conv_dgrad(dy.numpy(), w.numpy(), H, W_, 2, 1), what="dgrad")
