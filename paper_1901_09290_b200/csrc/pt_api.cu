@@ -109,12 +109,16 @@ extern "C" pt_status pt_test_set_wait_limit(pt_ctx *c, uint32_t milliseconds)
 {
     if (!c) return PT_ERR_INVALID_ARG;
     PT_CUDA_OK(cudaSetDevice(c->device));
-    return pt_sm100_set_wait_limit_ns(milliseconds ? (unsigned long long)milliseconds * 1000000ull : 2000000000ull, nullptr);
+    const unsigned long long ns = milliseconds ? (unsigned long long)milliseconds * 1000000ull : 2000000000ull;
+    PT_CUDA_OK(cudaDeviceSynchronize());
+    pt_status s = pt_sm100_set_wait_limit_ns(ns);
+    if (s == PT_OK) s = pt_bn_set_wait_limit_ns(ns);
+    return s == PT_OK ? pt_gate_set_wait_limit_ns(ns) : s;
 }
 
 extern "C" pt_status pt_test_skip_next_arrive(pt_ctx *c, int32_t which)
 {
-    if (!c || which < 0 || which > 2) return PT_ERR_INVALID_ARG;
+    if (!c || which < 0 || which > 5) return PT_ERR_INVALID_ARG;
     c->test_skip = which;
     return PT_OK;
 }

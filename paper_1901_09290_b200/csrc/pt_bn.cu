@@ -42,6 +42,7 @@ struct BnP {
     int pivot;              // the forward sums are about the channel's value at pixel 0 (else about 0)
     float eps, momentum;
     int relu;
+    int test_skip;          // test hook (pt_test_skip_next_arrive): the producers leave out their first stage
 };
 
 struct __align__(8) BnCtl {
@@ -133,10 +134,14 @@ bn_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUten
     sm100::grid_launch_dependents();
     if (warp == cons_warps) {
         if (lane == 0) {
-            int s = 0, ph = 0;
-            for (long long i = part; i < p.chunks; i += p.parts) {
+            int s = 0, ph = 0, issued = 0;
+            for (long long i = part; i < p.chunks; i += p.parts, ++issued) {
                 const long long ch = p.reverse ? p.chunks - 1 - i : i, p0 = ch * p.pix;
                 if (!sm100::mbar_wait(sm100::smem_u32(&ctl->empty[s]), ph ^ 1, abort_flag, g.status, 60)) break;
+                if (p.test_skip && issued == 0) {                                // test hook: this stage never becomes full
+                    if (++s == p.stages) { s = 0; ph ^= 1; }
+                    continue;
+                }
                 const uint32_t bar = sm100::smem_u32(&ctl->full[s]), dst = ring + (uint32_t)s * stage_bytes;
                 if (p.slabs == 1) {                                              // whole rows: consecutive bytes
                     const uint32_t bytes = (uint32_t)(p.M - p0 < p.pix ? p.M - p0 : p.pix) * (uint32_t)p.ld * 2u;
@@ -152,12 +157,7 @@ bn_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUten
                 }
                 if (++s == p.stages) { s = 0; ph ^= 1; }
             }
-            if (*abort_flag) {       // bounded drain of the copies in flight before the shared memory is released
-                const uint64_t t0 = sm100::globaltimer_ns();
-                for (int k = 0; k < p.stages; ++k)
-                    while (!sm100::mbar_try_wait(sm100::smem_u32(&ctl->full[k]), 0) && !sm100::mbar_try_wait(sm100::smem_u32(&ctl->full[k]), 1) &&
-                           sm100::globaltimer_ns() - t0 < 20000000ull) {}
-            }
+            if (*abort_flag) sm100::drain_ring(sm100::smem_u32(&ctl->full[0]), p.stages, issued);
         }
         return;
     }
@@ -433,6 +433,7 @@ pt_status launch_bn(pt_ctx *c, BnP p, const BnArgs &g, int n_in, cudaStream_t st
         PT_CUDA_OK(cudaFuncSetAttribute(bn_kernel<PASS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
         attr_set = true;
     }
+    if (c->test_skip == 3) { p.test_skip = 1; c->test_skip = 0; }
     CUtensorMap tm[3];
     memset(tm, 0, sizeof(tm));
     if (p.slabs > 1)
@@ -445,6 +446,12 @@ pt_status launch_bn(pt_ctx *c, BnP p, const BnArgs &g, int n_in, cudaStream_t st
 }
 
 }  // namespace
+
+pt_status pt_bn_set_wait_limit_ns(unsigned long long ns)
+{
+    PT_CUDA_OK(cudaMemcpyToSymbol(sm100::g_wait_limit_ns, &ns, sizeof(ns)));
+    return PT_OK;
+}
 
 extern "C" size_t pt_bn_workspace_bytes(const pt_ctx *c, const pt_bn_desc *d)
 {

@@ -62,6 +62,7 @@ struct GateP {
     int n_in;                   // channels of the rows picked from
     int n_sel, c_out;           // selection length; channels of the output that exist
     unsigned long long chunks;
+    int test_skip;              // test hook (pt_test_skip_next_arrive): the producers leave out their first stage
 };
 constexpr int kGateStages = 3;
 constexpr int kGateBlock = 256;                  // most consumer threads of a block of the staged form
@@ -107,17 +108,22 @@ __global__ void __launch_bounds__(kGateBlock + 32, kGatePerSm) gate_kernel(const
     __syncthreads();
     if (tid >= nthr) {
         if (lane == 0) {
-            int s = 0, ph = 0;
-            for (long long ch = blockIdx.x; ch < (long long)p.chunks; ch += gridDim.x) {
+            int s = 0, ph = 0, issued = 0;
+            for (long long ch = blockIdx.x; ch < (long long)p.chunks; ch += gridDim.x, ++issued) {
                 const long long p0 = ch * p.pix;
                 const uint32_t n = (uint32_t)(p.npix - p0 < p.pix ? p.npix - p0 : p.pix);
                 if (!sm100::mbar_wait(sm100::smem_u32(&ctl->empty[s]), ph ^ 1, abort_flag, status, 43)) break;
+                if (p.test_skip && issued == 0) {                        // test hook: this stage never becomes full
+                    if (++s == kGateStages) { s = 0; ph ^= 1; }
+                    continue;
+                }
                 const uint32_t bar = sm100::smem_u32(&ctl->full[s]), dst = ring + (uint32_t)s * stage_bytes;
                 sm100::mbar_arrive_expect_tx(bar, n * (in_row + node_row));
                 sm100::bulk_load(dst, in + (size_t)p0 * p.in_ld, n * in_row, bar);
                 if (SCATTER && node_row) sm100::bulk_load(dst + (uint32_t)p.pix * in_row, node + (size_t)p0 * p.node_ld, n * node_row, bar);
                 if (++s == kGateStages) { s = 0; ph ^= 1; }
             }
+            if (*abort_flag) sm100::drain_ring(sm100::smem_u32(&ctl->full[0]), kGateStages, issued);
         }
         __syncwarp();
     } else {
@@ -182,12 +188,6 @@ __global__ void __launch_bounds__(kGateBlock + 32, kGatePerSm) gate_kernel(const
             if (lane == 0) sm100::mbar_arrive(sm100::smem_u32(&ctl->empty[s]));
             if (++s == kGateStages) { s = 0; ph ^= 1; }
         }
-    }
-    if (tid == nthr && *abort_flag) {            // bounded drain of the copies still in flight before the shared memory is released
-        const uint64_t t0 = sm100::globaltimer_ns();
-        for (int k = 0; k < kGateStages; ++k)
-            while (!sm100::mbar_try_wait(sm100::smem_u32(&ctl->full[k]), 0) && !sm100::mbar_try_wait(sm100::smem_u32(&ctl->full[k]), 1) &&
-                   sm100::globaltimer_ns() - t0 < 20000000ull) {}
     }
 }
 
@@ -292,6 +292,7 @@ template <bool SCATTER, bool RELU>
 pt_status gate_launch(pt_ctx *ctx, GateP p, const void *in, const int *idx, const void *node, void *out, cudaStream_t st)
 {
     const size_t row = (size_t)(p.in_ld + p.node_ld) * 2;
+    if (ctx->test_skip == 4) { p.test_skip = 1; ctx->test_skip = 0; }
     p.pix = (int)(kGateChunk / row);
     if (p.pix < 1) p.pix = 1;
     // small tensors: chunks no larger than what gives every SM one
@@ -316,6 +317,12 @@ pt_status gate_launch(pt_ctx *ctx, GateP p, const void *in, const int *idx, cons
 }
 
 }  // namespace
+
+pt_status pt_gate_set_wait_limit_ns(unsigned long long ns)
+{
+    PT_CUDA_OK(cudaMemcpyToSymbol(sm100::g_wait_limit_ns, &ns, sizeof(ns)));
+    return PT_OK;
+}
 
 extern "C" pt_status pt_dense_channel_list(pt_ctx *ctx, const uint8_t *zero_flags, int32_t n, int32_t *idx, int32_t *count, void *stream)
 {

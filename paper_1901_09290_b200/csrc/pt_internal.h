@@ -94,7 +94,8 @@ struct pt_ctx {
     int stats_parts = 0;
     float *stats_out = nullptr;
     size_t stats_cap = 0;
-    int test_skip = 0;                  // pt_test_skip_next_arrive: 1 = next split weight gradient, 2 = next fwd/dgrad GEMM-form launch
+    int test_skip = 0;                  // pt_test_skip_next_arrive: 1 = next split weight gradient, 2 = next fwd/dgrad GEMM-form launch,
+                                        // 3 = next batch-norm pass, 4 = next staged gate, 5 = next halo-form launch
     // Plans of recent weight-gradient descriptors: choosing one walks a few hundred candidates (about 10 us), a call must not.
     struct WgradSlot {
         pt_conv_desc d;
@@ -154,4 +155,6 @@ pt_status pt_sm100_conv(pt_ctx *ctx, const pt_conv_desc *d, int which, const voi
                         void *ws, size_t ws_bytes, cudaStream_t st);
 size_t pt_sm100_conv_workspace(const pt_ctx *ctx, const pt_conv_desc *d, int which);
 int pt_sm100_wgrad_ctas(const pt_ctx *ctx, const pt_conv_desc *d, int *waits);
-pt_status pt_sm100_set_wait_limit_ns(unsigned long long ns, cudaStream_t st);
+pt_status pt_sm100_set_wait_limit_ns(unsigned long long ns);
+pt_status pt_bn_set_wait_limit_ns(unsigned long long ns);
+pt_status pt_gate_set_wait_limit_ns(unsigned long long ns);

@@ -51,8 +51,9 @@ __device__ __forceinline__ void record_timeout(unsigned int *status, unsigned in
     if (atomicCAS(&status[0], 0u, 1u) == 0u) status[1] = where;
 }
 
-// Limit of every bounded device-side wait, in nanoseconds (2 s unless pt_test_set_wait_limit changed it). It is read only
-// on the slow path of a wait (after 256 failed polls), never by a wait that succeeds at once.
+// Limit of every bounded device-side wait, in nanoseconds (2 s unless pt_test_set_wait_limit changed it; every file that includes this
+// has its own, which that call sets through the file's pt_*_set_wait_limit_ns). It is read only on the slow path of a wait (after
+// 256 failed polls), never by a wait that succeeds at once.
 __device__ unsigned long long g_wait_limit_ns = 2000000000ull;
 
 // Waits for the phase with the given parity to complete, for at most g_wait_limit_ns. On expiry it
@@ -75,6 +76,17 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
         }
     }
     return true;
+}
+
+// The end of a producer whose CTA gives up: waits, for at most 20 ms in all, until the copies it has issued into a ring have landed, so
+// that none writes shared memory that another CTA owns by then. `full` is the ring's first full barrier (the others follow it), `issued`
+// the number of its stages this thread has filled since the start: use i of the ring is stage i % stages, phase (i / stages) & 1.
+// (A barrier is always in one of its two phases, and a wait for the other one succeeds at once: the phase must be the stage's own.)
+__device__ __forceinline__ void drain_ring(uint32_t full, int stages, int issued)
+{
+    const uint64_t t0 = globaltimer_ns();
+    for (int i = issued > stages ? issued - stages : 0; i < issued; ++i)
+        while (!mbar_try_wait(full + 8u * (uint32_t)(i % stages), (uint32_t)(i / stages) & 1u) && globaltimer_ns() - t0 < 20000000ull) {}
 }
 
 // ---------------------------------------------------------------- TMA loads (no multicast anywhere)

@@ -97,3 +97,71 @@ def test_pipeline_barrier_wait_runs_out_and_the_context_recovers():
         torch.cuda.synchronize()
         ctx.poll()
         Hh.check_conv(yo, K, ref, what="fwd after a time-out")
+
+
+def test_halo_pipeline_wait_runs_out_and_the_context_recovers():
+    ctx = Hh.ctx()
+    N, H, C, K, R = 8, 16, 72, 40, 3                            # two chunks per tile, a producer warp per ring
+    x, w, dy = _inputs(N, H, C, K, R, W.BASE_SEED + 65)
+    d = B.make_conv_desc(N, H, H, C, K, R, R, 1, 1, algo=2)
+    xd, wd = Hh.to_dev_padded(x, d.ldx), Hh.to_dev_padded(w, d.ldw)
+    y = torch.zeros((N, H, H, d.ldy), dtype=torch.bfloat16, device="cuda")
+
+    def launch():
+        B.pt_test_skip_next_arrive(ctx, 5)
+        B.pt_conv_fwd(ctx, d, xd, wd, y, None)
+
+    _expect_timeout(ctx, launch)
+    ref = oracle.conv_fwd(x.numpy(), w.numpy(), 1, 1)
+    for _ in range(3):
+        yo = Hh.out_buffer((N, H, H), K, d.ldy, False)
+        B.pt_conv_fwd(ctx, d, xd, wd, yo, None)
+        torch.cuda.synchronize()
+        ctx.poll()
+        Hh.check_conv(yo, K, ref, what="fwd after a time-out")
+
+
+@pytest.mark.parametrize("C", [24, 371])                        # whole rows by bulk copies; channel slabs by TMA boxes
+def test_batch_norm_wait_runs_out_and_the_context_recovers(C):
+    ctx = Hh.ctx()
+    N, H, ld = 32, 28, W.pad8(C)
+    gen = torch.Generator(device="cuda").manual_seed(W.BASE_SEED + 66)
+    x = torch.randn((N, H, H, ld), generator=gen, device="cuda").to(torch.bfloat16)
+    g, b, sm, si = torch.ones(C, device="cuda"), torch.zeros(C, device="cuda"), torch.empty(C, device="cuda"), torch.empty(C, device="cuda")
+    y, again = torch.zeros_like(x), torch.zeros_like(x)
+    d = B.make_bn_desc(N, H, H, C, ld)
+    ws = torch.empty(B.pt_bn_workspace_bytes(ctx, d), dtype=torch.uint8, device="cuda")
+    run = lambda out: B.pt_bn_relu_fwd(ctx, d, x, None, g, b, None, None, sm, si, out, ws)
+    run(y)
+
+    def launch():
+        B.pt_test_skip_next_arrive(ctx, 3)
+        run(again)
+
+    _expect_timeout(ctx, launch)
+    for _ in range(3):
+        run(again)
+        torch.cuda.synchronize()
+        ctx.poll()
+        assert torch.equal(y, again)
+
+
+def test_channel_gate_wait_runs_out_and_the_context_recovers():
+    ctx = Hh.ctx()
+    npix, C, S = 50000, 222, 211
+    gen = torch.Generator(device="cuda").manual_seed(W.BASE_SEED + 67)
+    ld, lds = W.pad8(C), W.pad8(S)
+    node = torch.randn((npix, ld), generator=gen, device="cuda").to(torch.bfloat16)
+    idx = torch.randperm(C, generator=gen, device="cuda")[:S].to(torch.int32)
+    out = torch.zeros((npix, lds), dtype=torch.bfloat16, device="cuda")
+
+    def launch():
+        B.pt_test_skip_next_arrive(ctx, 4)
+        B.pt_channel_gather(ctx, node, ld, C, idx, S, out, lds, npix)
+
+    _expect_timeout(ctx, launch)
+    for _ in range(3):
+        B.pt_channel_gather(ctx, node, ld, C, idx, S, out, lds, npix)
+        torch.cuda.synchronize()
+        ctx.poll()
+        assert torch.equal(out[:, :S], node[:, idx.long()])
