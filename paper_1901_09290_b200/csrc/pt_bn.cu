@@ -428,10 +428,9 @@ pt_status launch_bn(pt_ctx *c, BnP p, const BnArgs &g, int n_in, cudaStream_t st
     const size_t red = kBnData + (size_t)p.consumers * 17 * sizeof(float) + kBnThreads * sizeof(double);
     if (PASS < 2 && smem < red) smem = red;
     if (PASS >= 2) smem += (size_t)p.consumers * 4 * sizeof(double);             // the fp64 slices of the partial rows' sums
-    static bool attr_set = false;
-    if (!attr_set) {
+    if (!(c->attr_done & (kAttrBn << PASS))) {
         PT_CUDA_OK(cudaFuncSetAttribute(bn_kernel<PASS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
-        attr_set = true;
+        c->attr_done |= kAttrBn << PASS;
     }
     if (c->test_skip == 3) { p.test_skip = 1; c->test_skip = 0; }
     CUtensorMap tm[3];

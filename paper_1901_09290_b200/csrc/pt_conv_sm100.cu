@@ -2143,10 +2143,9 @@ pt_status launch_gemm(pt_ctx *c, const GemmMaps &tm, GemmP &p, cudaStream_t st)
     void (*kernel)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, GemmP) =
         (!B_MN && c->stats_mode) ? conv_gemm_kernel<false, true, false> : apart ? conv_gemm_kernel<true, false, true> : conv_gemm_kernel<B_MN, false, false>;
     const int kid = (!B_MN && c->stats_mode) ? 2 : apart ? 3 : (B_MN ? 1 : 0);
-    static bool attr_set[4] = {false, false, false, false};
-    if (!attr_set[kid]) {
+    if (!(c->attr_done & (kAttrGemm << kid))) {
         PT_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-        attr_set[kid] = true;
+        c->attr_done |= kAttrGemm << kid;
     }
     int grid = total_tiles < c->sm_count ? total_tiles : c->sm_count;
     if (c->stats_mode) {
@@ -2332,10 +2331,9 @@ pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const
     void (*kernel)(CUtensorMap, CUtensorMap, CUtensorMap, HaloP) =
         (!B_MN && c->stats_mode) ? conv_halo_kernel<false, true> : conv_halo_kernel<B_MN, false>;
     const int kid = (!B_MN && c->stats_mode) ? 2 : (B_MN ? 1 : 0);
-    static bool attr_set[3] = {false, false, false};
-    if (!attr_set[kid]) {
+    if (!(c->attr_done & (kAttrHalo << kid))) {
         PT_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-        attr_set[kid] = true;
+        c->attr_done |= kAttrHalo << kid;
     }
     const int total_tiles = p.N * p.row_tiles * p.n_tiles;
     int grid = total_tiles < c->sm_count ? total_tiles : c->sm_count;
@@ -2623,13 +2621,12 @@ cudaError_t launch_wgrad(void (*kernel)(CUtensorMap, CUtensorMap, CUtensorMap, W
     return cudaLaunchKernelEx(&cfg, kernel, a, b, q, p);
 }
 
-pt_status wgrad_attr()
+pt_status wgrad_attr(const pt_ctx *c)
 {
-    static bool attr_set = false;
-    if (!attr_set) {
+    if (!(c->attr_done & kAttrWgrad)) {
         PT_CUDA_OK(cudaFuncSetAttribute(conv_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
         PT_CUDA_OK(cudaFuncSetAttribute(conv_wgrad_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
-        attr_set = true;
+        c->attr_done |= kAttrWgrad;
     }
     return PT_OK;
 }
@@ -2639,7 +2636,10 @@ int wg_max_clusters(const pt_ctx *c, int size)
 {
     if (size < 2 || size > 8) return 0;
     if (c->max_clusters[size] == 0) {
-        int n = 0;
+        // (a workspace query may come while another device is the current one)
+        int n = 0, cur = c->device;
+        (void)cudaGetDevice(&cur);
+        if (cur != c->device) (void)cudaSetDevice(c->device);
         cudaLaunchConfig_t cfg;
         memset(&cfg, 0, sizeof(cfg));
         cfg.gridDim = dim3(1, (unsigned)size); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = 220 * 1024;
@@ -2647,10 +2647,11 @@ int wg_max_clusters(const pt_ctx *c, int size)
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = (unsigned)size; attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr; cfg.numAttrs = 1;
-        if (wgrad_attr() != PT_OK || cudaOccupancyMaxActiveClusters(&n, conv_wgrad_kernel, &cfg) != cudaSuccess || n < 1) {
+        if (wgrad_attr(c) != PT_OK || cudaOccupancyMaxActiveClusters(&n, conv_wgrad_kernel, &cfg) != cudaSuccess || n < 1) {
             (void)cudaGetLastError();
             n = -1;
         }
+        if (cur != c->device) (void)cudaSetDevice(cur);
         c->max_clusters[size] = n;
     }
     return c->max_clusters[size] < 0 ? 0 : c->max_clusters[size];
@@ -2684,7 +2685,7 @@ pt_status wgrad_common(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const pt_
         c->sync_next += 2 * gx;
         if (!make_partial_map(c, tmP, ws, w.acc_cols, (size_t)gx * w.apc * w.splits * 128)) return PT_ERR_CUDA;
     }
-    return wgrad_attr();
+    return wgrad_attr(c);
 }
 
 // Launches the weight-gradient kernel for a problem whose x operand is described by `tmX` (64 pixels x 64 channels boxes).

@@ -303,10 +303,10 @@ pt_status gate_launch(pt_ctx *ctx, GateP p, const void *in, const int *idx, cons
     const int pairs = p.out_ld / 2;
     const int threads = pairs >= kGateBlock ? kGateBlock : pt_ceil_div(kGateBlock / pairs * pairs, 32) * 32;
     const size_t smem = 128 + pt_align_up((size_t)p.out_ld * 2, 128) + kGateStages * (size_t)p.pix * row;
-    static bool attr_set = false;
-    if (!attr_set) {
+    const unsigned attr = kAttrGate << (SCATTER ? RELU ? 2 : 1 : 0);
+    if (!(ctx->attr_done & attr)) {
         PT_CUDA_OK(cudaFuncSetAttribute(gate_kernel<SCATTER, RELU>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-        attr_set = true;
+        ctx->attr_done |= attr;
     }
     const unsigned long long cap = (unsigned long long)ctx->sm_count * kGatePerSm;
     gate_kernel<SCATTER, RELU><<<(unsigned)(p.chunks < cap ? p.chunks : cap), threads + 32, smem, st>>>(

@@ -4,6 +4,7 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 #include <string.h>
+#include <atomic>
 #include <mutex>
 #include <vector>
 
@@ -43,6 +44,11 @@ struct pt_group_slot {
     size_t ws[10];                  // offsets of the workspace's parts
 };
 
+// Kernels whose opt-in to more than 48 KB of dynamic shared memory a context has set (pt_ctx::attr_done). The attribute belongs to a
+// device, so it is remembered per context and not per process; setting it twice does no harm.
+enum : unsigned { kAttrGemm = 1u << 0 /* four variants */, kAttrHalo = 1u << 4 /* three */, kAttrWgrad = 1u << 7, kAttrBn = 1u << 8 /* four */,
+                  kAttrGate = 1u << 12 /* three */ };
+
 // Launch shape of a weight gradient. rows = 1: the row-block kernel (stride-1 filters with at most 64 input channels).
 struct pt_wgrad_plan {
     int rows;
@@ -58,6 +64,7 @@ struct pt_wgrad_plan {
 struct pt_ctx {
     int device = 0;
     int sm_count = 0;
+    mutable std::atomic<unsigned> attr_done{0};
     int cc_major = 0, cc_minor = 0;
     unsigned int *d_status = nullptr;   // 4 words, device
     unsigned int *h_status = nullptr;   // 4 words, pinned host
