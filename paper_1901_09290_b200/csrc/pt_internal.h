@@ -41,7 +41,7 @@ struct pt_group_slot {
     unsigned n_chunks = 0, n_jobs = 0;
     bool small = false;
     std::vector<int> first_chunk;
-    size_t ws[10];                  // offsets of the workspace's parts
+    size_t ws[11];                  // offsets of the workspace's parts
 };
 
 // Kernels whose opt-in to more than 48 KB of dynamic shared memory a context has set (pt_ctx::attr_done). The attribute belongs to a

@@ -44,7 +44,7 @@ struct Chunk { int layer, line0, nlines, cg, lc, nsub, pad0, pad1; };
 // kind 0: 32 output-channel groups from `start` (four per warp); kind 1: 32 input-channel groups from `start` (x 8 slices of the chunks)
 struct FinishJob { int layer, kind, start, pad; };
 
-struct WsLayout { size_t linesum, colpart, linemax, colmax, inv_out, inv_in, gmax_out, gmax_in, job_reg, total; };
+struct WsLayout { size_t linesum, colpart, linemax, colmax, inv_out, inv_in, gmax_out, gmax_in, job_reg, ticket, total; };
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
@@ -86,6 +86,7 @@ struct GroupP {
     float *linesum, *colpart;
     unsigned *linemax, *colmax, *gmax_out, *gmax_in;
     double *job_reg;
+    unsigned *ticket;           // arrivals of the finish launch's blocks; cleared by the sweep in front of it
     pt_sgd_hparams hp;
     float thr;
     int split;                  // blocks that share a chunk (the plain update)
@@ -250,6 +251,7 @@ __global__ void __launch_bounds__(kThreads) group_kernel(const GroupP p)
     // producers do not wait for their predecessor (weights are never written by a kernel that releases its dependents early),
     // and a convolution may well be the next launch of the stream.
     if (!UPD) pdl_trigger();
+    if (SUM && blockIdx.x == 0 && threadIdx.x == 0) *p.ticket = 0u;
     if (L.vec) chunk_body<UPD, SUM, MAX, FLAG, 4, true>(p, L, ch, sub, s_col, s_colm);
     else if (ch.nsub == 4) chunk_body<UPD, SUM, MAX, FLAG, 4, false>(p, L, ch, sub, s_col, s_colm);
     else if (ch.nsub == 3) chunk_body<UPD, SUM, MAX, FLAG, 3, false>(p, L, ch, sub, s_col, s_colm);
@@ -276,7 +278,7 @@ __global__ void __launch_bounds__(kThreads) group_kernel(const GroupP p)
 
 // ---- finish
 template <bool SUM, bool MAX, bool FLAG>
-__global__ void __launch_bounds__(kThreads) finish_kernel(const GroupP p, const FinishJob *__restrict__ jobs, unsigned *ticket, double *reg_out)
+__global__ void __launch_bounds__(kThreads) finish_kernel(const GroupP p, const FinishJob *__restrict__ jobs, double *reg_out)
 {
     __shared__ double s_red[kWarps];
     __shared__ float s_ps[kWarps][32];
@@ -364,8 +366,7 @@ __global__ void __launch_bounds__(kThreads) finish_kernel(const GroupP p, const 
         for (int w = 0; w < kWarps; ++w) tot += s_red[w];
         p.job_reg[blockIdx.x] = tot;
         __threadfence();
-        s_last = atomicAdd(ticket, 1u) == gridDim.x - 1u ? 1u : 0u;
-        if (s_last) *ticket = 0u;
+        s_last = atomicAdd(p.ticket, 1u) == gridDim.x - 1u ? 1u : 0u;
     }
     __syncthreads();
     if (!s_last) return;
@@ -489,6 +490,7 @@ pt_status build_tables(const pt_layer *layers, int n, Tables *t)
     w.gmax_out = o; o = pt_align_up(o + (size_t)k_off * 4, 256);
     w.gmax_in = o;  o = pt_align_up(o + (size_t)c_off * 4, 256);
     w.job_reg = o;  o = pt_align_up(o + t->jobs.size() * 8, 256);
+    w.ticket = o;   o += 256;
     w.total = o;
     return PT_OK;
 }
@@ -556,16 +558,14 @@ pt_status bind(pt_ctx *c, const pt_layer *layers, int n, bool detect, void *ws, 
     p.inv_out = (float *)(a + w.inv_out); p.inv_in = (float *)(a + w.inv_in);
     p.gmax_out = (unsigned *)(a + w.gmax_out); p.gmax_in = (unsigned *)(a + w.gmax_in);
     p.job_reg = (double *)(a + w.job_reg);
+    p.ticket = (unsigned *)(a + w.ticket);
     return PT_OK;
 }
 
 template <bool SUM, bool MAX, bool FLAG>
 pt_status launch_finish(pt_ctx *c, const Bound &b, double *reg_out, cudaStream_t st)
 {
-    // a self-resetting ticket from the context's ring of zero-initialised counters
-    if (c->sync_next + 1 > 16384) c->sync_next = 0;
-    unsigned *ticket = c->d_sync + c->sync_next++;
-    PT_CUDA_OK(pt_launch_pdl(finish_kernel<SUM, MAX, FLAG>, dim3(b.slot->n_jobs), dim3(kThreads), 0, st, b.p, b.dj, ticket, reg_out));
+    PT_CUDA_OK(pt_launch_pdl(finish_kernel<SUM, MAX, FLAG>, dim3(b.slot->n_jobs), dim3(kThreads), 0, st, b.p, b.dj, reg_out));
     c->launches += 1;
     return PT_OK;
 }

@@ -277,8 +277,8 @@ def test_new_shadow_with_a_pitch_past_32_bit_offsets():
     c, K, C, ldw = Hh.ctx(), 33, 8, 1 << 27
     gen = torch.Generator(device="cuda").manual_seed(W.BASE_SEED)
     w = torch.randn((K, C), generator=gen, device="cuda") + 3.0
-    old = B.make_layer(w, None, torch.zeros_like(w), w.to(torch.bfloat16), K, C, 1, C, True, True, *(torch.zeros(n, device="cuda") for n in (K, C)),
-                       *(torch.zeros(n, dtype=torch.uint8, device="cuda") for n in (K, C)))
+    v, wb, zo, zi = torch.zeros_like(w), w.to(torch.bfloat16), *(torch.zeros(n, dtype=torch.uint8, device="cuda") for n in (K, C))
+    old = B.make_layer(w, None, v, wb, K, C, 1, C, True, True, None, None, zo, zi)
     shadow = torch.empty((K - 1) * ldw + C, dtype=torch.bfloat16, device="cuda")
     nw, nv = torch.empty_like(w), torch.empty_like(w)
     new = B.make_layer(nw, None, nv, shadow, K, C, 1, ldw, True, True, None, None, None, None)

@@ -165,3 +165,38 @@ def test_channel_gate_wait_runs_out_and_the_context_recovers():
         torch.cuda.synchronize()
         ctx.poll()
         assert torch.equal(out[:, :S], node[:, idx.long()])
+
+
+def test_regulariser_value_does_not_depend_on_an_unpolled_time_out():
+    """A weight gradient that gave up leaves its arrival counters behind until the status is polled: nothing else may count with them,
+    however many launches have gone round the ring of counters meanwhile."""
+    ctx = B.Context(0)                                          # a ring of its own
+    N, H, C, K, R = 8, 16, 16, 32, 3
+    x, w, dy = _inputs(N, H, C, K, R, W.BASE_SEED + 68)
+    d = B.make_conv_desc(N, H, H, C, K, R, R, 1, 1, algo=2)
+    xd, dyd = Hh.to_dev_padded(x, d.ldx), Hh.to_dev_padded(dy, d.ldy)
+    dw = torch.zeros((K, R, R, C), device="cuda")
+    ws = torch.empty(B.pt_conv_workspace_bytes(ctx, d, B.PT_CONV_WGRAD), dtype=torch.uint8, device="cuda")
+    wt, sq_o, sq_i = w.cuda().contiguous(), torch.zeros(K, device="cuda"), torch.zeros(C, device="cuda")
+    v = torch.zeros_like(wt)
+    arr = B.layer_array([B.make_layer(wt, dw, v, None, K, C, R * R, d.ldw, True, True, sq_o, sq_i, None, None)])
+    lws = torch.empty(max(256, B.pt_group_lasso_workspace_bytes(ctx, arr)), dtype=torch.uint8, device="cuda")
+    reg = torch.zeros(1, dtype=torch.float64, device="cuda")
+    B.pt_test_set_wait_limit(ctx, LIMIT_MS)
+    try:
+        B.pt_test_skip_next_arrive(ctx, 1)
+        B.pt_conv_wgrad(ctx, d, xd, dyd, dw, ws)
+        torch.cuda.synchronize()
+        bad = torch.zeros((), dtype=torch.int64, device="cuda")
+        B.pt_group_lasso_norms(ctx, arr, reg, lws)
+        ref = reg.clone()
+        for _ in range(16500):                                  # (the ring has 16384 counters)
+            reg.fill_(-1.0)
+            B.pt_group_lasso_norms(ctx, arr, reg, lws)
+            bad += (reg != ref).sum()
+        assert int(bad) == 0
+        with pytest.raises(B.PtError):
+            ctx.poll()
+    finally:
+        B.pt_test_set_wait_limit(ctx, 0)
+        ctx.close()
