@@ -379,7 +379,8 @@ pt_status pt_reconfigure_plan(pt_ctx *ctx, const pt_graph *g, int32_t *new2old, 
 /* The same in two calls, for a caller that has more work to enqueue behind the plan: the first enqueues it and returns, the second
  * waits for the counts of the context's last plan (n_spaces as in its graph; stream: the one it was enqueued on). A training loop that
  * expects the sizes it allocated for can enqueue the gather and the whole step between the two and check the counts afterwards: the
- * GPU does not idle while the host wakes up. PT_ERR_INVALID_ARG if no plan was enqueued or n_spaces differs. */
+ * GPU does not idle while the host wakes up. PT_ERR_INVALID_ARG if no plan was enqueued or n_spaces differs, and for a plan enqueued
+ * while one on another stream is still running (the counts are the context's); PT_ERR_UNSUPPORTED on a stream that is being captured. */
 pt_status pt_reconfigure_plan_enqueue(pt_ctx *ctx, const pt_graph *g, int32_t *new2old, void *stream);
 pt_status pt_reconfigure_plan_wait(pt_ctx *ctx, int32_t n_spaces, int32_t *new_sizes /*host*/, void *stream);
 

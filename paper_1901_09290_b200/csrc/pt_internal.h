@@ -91,6 +91,7 @@ struct pt_ctx {
     int32_t *h_counts = nullptr;        // pinned, for pt_reconfigure_plan: [0] = flag the kernel raises, [16..] = counts
     unsigned int plan_seq = 0;          // sequence number of the last plan's flag
     int plan_spaces = 0;                // number of spaces of the last plan
+    void *plan_stream = nullptr;        // the stream it was enqueued on
     unsigned int *d_sync = nullptr;     // zero-initialised, self-resetting arrival counters of the split weight gradient
     unsigned int sync_next = 0;         // ring position in d_sync
     uint64_t launches = 0;

@@ -216,6 +216,12 @@ extern "C" pt_status pt_reconfigure_plan_enqueue(pt_ctx *c, const pt_graph *g, i
     pt_status s = check_graph(g);
     if (s != PT_OK) return s;
     if (g->n_spaces > 65536) return PT_ERR_UNSUPPORTED;
+    // The counts, their flag and its sequence number are the context's: a captured launch would raise the flag of its capture again on
+    // every replay, and a plan on another stream could overwrite the counts of one that is still running.
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    PT_CUDA_OK(cudaStreamIsCapturing((cudaStream_t)stream, &cap));
+    if (cap != cudaStreamCaptureStatusNone) return PT_ERR_UNSUPPORTED;
+    if (c->plan_spaces && c->plan_stream != stream && *(volatile unsigned int *)c->h_counts != c->plan_seq) return PT_ERR_INVALID_ARG;
     std::vector<SpaceDev> sp(g->n_spaces);
     std::vector<MemberDev> mem;
     long long off = 0;
@@ -264,6 +270,7 @@ extern "C" pt_status pt_reconfigure_plan_enqueue(pt_ctx *c, const pt_graph *g, i
     c->launches += 1;
     PT_CUDA_OK(cudaGetLastError());
     c->plan_spaces = g->n_spaces;
+    c->plan_stream = stream;
     return PT_OK;
 }
 

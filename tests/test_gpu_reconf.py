@@ -290,3 +290,48 @@ def test_new_shadow_with_a_pitch_past_32_bit_offsets():
     c.poll()
     got = torch.stack([shadow[k * ldw:k * ldw + C] for k in range(K)])
     assert torch.equal(nw, w) and torch.equal(got, w.to(torch.bfloat16))
+
+
+def _two_spaces(c, K=40, C=24):
+    gen = torch.Generator(device="cuda").manual_seed(W.BASE_SEED + 91)
+    w, v = torch.randn((K, C), generator=gen, device="cuda") + 3.0, torch.zeros((K, C), device="cuda")
+    zo, zi = torch.zeros(K, dtype=torch.uint8, device="cuda"), torch.zeros(C, dtype=torch.uint8, device="cuda")
+    zo[:7] = 1
+    layer = B.make_layer(w, None, v, None, K, C, 1, C, True, True, None, None, zo, zi)
+    return B.GraphHandle([C, K], [True, False], [layer], [(0, 1)]), torch.empty(C + K, dtype=torch.int32, device="cuda"), (w, v, zo, zi)
+
+
+def test_plan_in_two_calls_and_its_errors():
+    c = B.Context(0)
+    g, n2o, keep = _two_spaces(c)
+    one = B.GraphHandle([24], [True], [], [])
+    with pytest.raises(B.PtError) as e:                              # no plan yet
+        B.pt_reconfigure_plan_wait(c, g)
+    assert e.value.status == 1
+    B.pt_reconfigure_plan_enqueue(c, g, n2o)
+    with pytest.raises(B.PtError) as e:                              # a graph of another number of spaces
+        B.pt_reconfigure_plan_wait(c, one)
+    assert e.value.status == 1
+    assert B.pt_reconfigure_plan_wait(c, g) == [24, 33]
+    assert n2o.cpu().tolist() == list(range(24)) + list(range(7, 40)) + [-1] * 7
+    # a second plan on another stream: refused while the first is still running, fine afterwards
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    torch.cuda._sleep(20000000)                                      # (about 10 ms)
+    B.pt_reconfigure_plan_enqueue(c, g, n2o)
+    other = torch.empty_like(n2o)
+    with pytest.raises(B.PtError) as e:
+        B.pt_reconfigure_plan_enqueue(c, g, other, stream=side)
+    assert e.value.status == 1
+    assert B.pt_reconfigure_plan_wait(c, g) == [24, 33]
+    B.pt_reconfigure_plan_enqueue(c, g, other, stream=side)
+    assert B.pt_reconfigure_plan_wait(c, g, stream=side) == [24, 33] and torch.equal(other, n2o)
+    # under capture
+    gr = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(gr):
+        other.fill_(0)
+        with pytest.raises(B.PtError) as e:
+            B.pt_reconfigure_plan_enqueue(c, g, n2o)
+    assert e.value.status == 2                                       # PT_ERR_UNSUPPORTED
+    assert B.pt_reconfigure_plan(c, g, n2o) == [24, 33]
+    c.close()
