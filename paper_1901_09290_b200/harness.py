@@ -293,6 +293,18 @@ class TrainStep:
         if sizes != self.counts:
             raise RuntimeError(f"reconfiguration plan returned {sizes}, expected {self.counts}")
 
+    def _check_plan_ahead(self, stream=None):
+        """The sizes of a plan behind which work was enqueued. Where they disagree that work has run on a map that does not fit: it is
+        waited for and the status it left is cleared, so that the error says it all and the context is as usable as before."""
+        sizes = B.pt_reconfigure_plan_wait(self.ctx, self.md.graph(), stream)
+        if sizes != self.counts:
+            torch.cuda.synchronize()
+            try:
+                self.ctx.poll()
+            except B.PtError:
+                pass
+        self._check_sizes(sizes)
+
     def gather(self, first: int = 0, count: Optional[int] = None, stream=None):
         """The compaction gather of layers [first, first + count) into the pruned model."""
         n = len(self.net.layers)
@@ -482,9 +494,12 @@ class TrainStep:
         return self.graph
 
     def step(self, stream=None, before_train=None):
-        # With the gather inside the graph (in two parts, beside the first layers) nothing of the step needs the host before the sizes are
-        # checked: the whole step is enqueued first, so that the GPU goes from the plan to the gather without waiting for the host to
-        # wake up and launch a graph of ~180 nodes (60 to 90 us of the step). A plan that disagrees raises as before.
+        """One step. A plan whose sizes are not the ones the step was built for raises RuntimeError. With the gather inside the graph the
+        training part has been enqueued by then: the pruned model (weights, momenta, gradients), the layers' outputs and the regulariser
+        value are undefined until the next step gathers them anew; the dense model is untouched. In a data-parallel run neither the
+        exchange of the gradients nor the update has been started."""
+        # Nothing of the step needs the host before the sizes are checked: the whole step is enqueued first, so that the GPU goes from the
+        # plan to the gather without waiting for the host to wake up and launch a graph of ~180 nodes (60 to 90 us of the step).
         ahead = getattr(self, "graph", None) is not None and getattr(self, "_graph_has_gather", False)
         if ahead:
             B.pt_find_zero_groups(self.ctx, self.md.arr, 1e-4, False, self.md.ws, stream)
@@ -495,11 +510,11 @@ class TrainStep:
             torch.cuda.current_stream().wait_event(before_train)     # e.g. the image batch has reached the stem's input
         if getattr(self, "graph", None) is not None:
             self.graph.replay()
+            if ahead:                        # (the GPU is busy with the graph meanwhile; before the other ranks see the gradients)
+                self._check_plan_ahead(stream)
             if not self._graph_has_update:
                 allreduce_mean(self.mp.g_flat, self.world)       # the one exchange of a data-parallel step
                 self.lasso(stream)
-            if ahead:
-                self._check_sizes(B.pt_reconfigure_plan_wait(self.ctx, self.md.graph(), stream))
         else:
             self.train(stream)
 

@@ -335,3 +335,41 @@ def test_plan_in_two_calls_and_its_errors():
     assert e.value.status == 2                                       # PT_ERR_UNSUPPORTED
     assert B.pt_reconfigure_plan(c, g, n2o) == [24, 33]
     c.close()
+
+
+@pytest.mark.parametrize("world", [1, 2])
+def test_step_with_a_plan_that_disagrees(world, monkeypatch):
+    """The step enqueues its graph before it checks the plan's sizes: a model that has grown another live channel raises, nothing is
+    exchanged with other ranks, no status stays behind, and the next step of the right model gives what the first one gave."""
+    from paper_1901_09290_b200 import harness
+    exchanged = []
+    monkeypatch.setattr(harness, "allreduce_mean", lambda flat, n: exchanged.append(n))
+    c = B.Context(0)
+    net = W.resnet32()
+    counts = W.random_keep(net, 3, 0.4, 0.9)
+    kept = W.choose_kept(net, counts, 3)
+    ts = harness.TrainStep(c, net, counts, kept, 8, 3, world=world)
+    ts.step()
+    torch.cuda.synchronize()
+    ts.build_graph()
+    ts.step()
+    torch.cuda.synchronize()
+    c.poll()
+    ref, n_ex = [t.clone() for t in ts.mp.w], len(exchanged)
+    s = next(i for i in range(len(net.space_sizes)) if not net.space_fixed[i] and counts[i] < net.space_sizes[i])
+    dead = int(np.setdiff1d(np.arange(net.space_sizes[s]), kept[s])[0])
+    li = next(i for i, l in enumerate(net.layers) if l.out_space == s)
+    row = ts.md.w[li][dead].clone()
+    ts.md.w[li][dead] = 1.0
+    with pytest.raises(RuntimeError, match="reconfiguration plan"):
+        ts.step()
+    assert len(exchanged) == n_ex
+    torch.cuda.synchronize()
+    c.poll()
+    ts.md.w[li][dead] = row
+    ts.step()
+    torch.cuda.synchronize()
+    c.poll()
+    assert len(exchanged) == (n_ex + 1 if world > 1 else 0)
+    assert all(torch.equal(a, b) for a, b in zip(ts.mp.w, ref))
+    c.close()
