@@ -2565,21 +2565,19 @@ bool wgrad_rows_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, pt_wg
 // The plan of a descriptor at the context's CTA limit. rows_only: only a row-block plan is asked for (its `rows` is 0 if there is none).
 pt_wgrad_plan wgrad_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, bool rows_only = false)
 {
-    pt_conv_desc key = *d;
-    key.ldw = key.out_f32 = 0; key.algo = rows_only ? 1 : 0;
-    const int limit = wgrad_budget(c);
-    unsigned h = 2166136261u;
-    for (size_t i = 0; i < sizeof(key) / 4; ++i) h = (h ^ (unsigned)reinterpret_cast<const int32_t *>(&key)[i]) * 16777619u;
-    h = (h ^ (unsigned)limit) * 16777619u;
+    pt_ctx::WgradKey key{*d, wgrad_budget(c), P, Q};
+    static_assert(sizeof(key) == sizeof(pt_conv_desc) + 12, "the key is compared and hashed as words");
+    key.d.ldw = key.d.out_f32 = 0; key.d.algo = rows_only ? 1 : 0;
     std::lock_guard<std::mutex> lock(c->wgrad_mutex);
-    pt_ctx::WgradSlot &slot = c->wgrad_slot[(h >> 8) & 127];
-    if (slot.valid && slot.limit == limit && slot.P == P && slot.Q == Q && memcmp(&slot.d, &key, sizeof(key)) == 0) return slot.plan;
+    const auto known = c->wgrad_plans.find(key);
+    if (known != c->wgrad_plans.end()) return known->second;
     pt_wgrad_plan w;
     if (!wgrad_rows_plan(c, d, P, Q, &w)) {
         w.rows = 0;
         if (!rows_only) wgrad_gen_plan(c, d, P, Q, &w);
     }
-    slot.d = key; slot.limit = limit; slot.P = P; slot.Q = Q; slot.plan = w; slot.valid = true;
+    if (c->wgrad_plans.size() >= pt_ctx::kWgradPlans) c->wgrad_plans.clear();
+    c->wgrad_plans.emplace(key, w);
     return w;
 }
 

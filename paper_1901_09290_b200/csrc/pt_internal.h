@@ -6,6 +6,7 @@
 #include <string.h>
 #include <atomic>
 #include <mutex>
+#include <unordered_map>
 #include <vector>
 
 #include "../../include/pt.h"
@@ -104,14 +105,22 @@ struct pt_ctx {
     size_t stats_cap = 0;
     int test_skip = 0;                  // pt_test_skip_next_arrive: 1 = next split weight gradient, 2 = next fwd/dgrad GEMM-form launch,
                                         // 3 = next batch-norm pass, 4 = next staged gate, 5 = next halo-form launch
-    // Plans of recent weight-gradient descriptors: choosing one walks a few hundred candidates (about 10 us), a call must not.
-    struct WgradSlot {
+    // Plans of the weight-gradient descriptors met so far: choosing one walks a few hundred candidates (about 10 us), a call must not.
+    // A network has about fifty, each at a few CTA limits; past kWgradPlans the table starts again.
+    struct WgradKey {
         pt_conv_desc d;
         int limit, P, Q;
-        bool valid = false;
-        pt_wgrad_plan plan;
+        bool operator==(const WgradKey &o) const { return memcmp(this, &o, sizeof(o)) == 0; }
     };
-    mutable WgradSlot wgrad_slot[128];
+    struct WgradHash {
+        size_t operator()(const WgradKey &k) const {
+            uint64_t h = 1469598103934665603ull;
+            for (size_t i = 0; i < sizeof(k) / 4; ++i) h = (h ^ reinterpret_cast<const uint32_t *>(&k)[i]) * 1099511628211ull;
+            return (size_t)(h ^ (h >> 32));
+        }
+    };
+    static constexpr size_t kWgradPlans = 2048;
+    mutable std::unordered_map<WgradKey, pt_wgrad_plan, WgradHash> wgrad_plans;
     mutable std::mutex wgrad_mutex;
     mutable int max_clusters[9] = {0};  // co-resident weight-gradient clusters of 2..8 CTAs (0: not asked yet)
     // Helper streams for independent launches inside one call (the parity classes of a stride-2 data gradient): the caller's

@@ -299,3 +299,28 @@ def test_data_gradient_of_a_padded_1x1_at_stride_2(N, H, W_, C, K):
     torch.cuda.synchronize()
     c.poll()
     Hh.check_conv(dx, C, oracle.conv_dgrad(dy.numpy(), w.numpy(), H, W_, 2, 1), what="dgrad")
+
+
+def test_a_round_of_many_layers_costs_the_host_no_more_per_call_than_one_layer():
+    """The launch shape of a weight gradient is chosen once per descriptor: going round the layers of a network must not choose it again."""
+    import time
+    c = B.Context(0)
+    # small maps and batches, where every candidate is weighed
+    descs = [B.make_conv_desc(N, H, H, C, K, 3, 3, 1, 1) for N in (2, 3, 4, 6, 8) for H in (14, 28, 32) for C in (20, 31, 48, 64) for K in (17, 60, 128)]
+    for d in descs:
+        B.pt_conv_workspace_bytes(c, d, B.PT_CONV_WGRAD)
+
+    def per_call(ds):
+        best = 1e9
+        for _ in range(5):
+            t0 = time.perf_counter()
+            for d in ds:
+                B.pt_conv_workspace_bytes(c, d, B.PT_CONV_WGRAD)
+            best = min(best, (time.perf_counter() - t0) / len(ds))
+        return best
+
+    many, one = per_call(descs), per_call([descs[-1]] * len(descs))
+    c.close()
+    assert len(descs) == 180
+    # (with 128 places of one plan each, the round took 2.4 times as long per call as the repeated layer)
+    assert many < 1.6 * one, (many, one)
