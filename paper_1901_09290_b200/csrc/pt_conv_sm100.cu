@@ -2589,6 +2589,26 @@ size_t wgrad_partial_bytes(const pt_wgrad_plan &w)
     return (size_t)w.n_tiles * w.m_tiles * w.tap_groups * w.apc * w.splits * 128 * w.acc_cols * sizeof(float);
 }
 
+// What a caller is asked for: the most that a launch shape of this descriptor needs at the context's CTA limit, so that a workspace sized
+// at one limit serves every smaller one too, whatever shape is chosen there (a smaller limit may well choose more splits, through the
+// workspace, where a larger one takes a few in a cluster).
+size_t wgrad_workspace_bound(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, const pt_wgrad_plan &w)
+{
+    const int taps = d->R * d->S, budget = wgrad_budget(c);
+    // what is dealt out in groups (taps, or accumulators of two or four taps), as few as fit one CTA at most, and the most splits
+    const int parts = !w.rows ? taps : w.lanes == 64 ? pt_ceil_div(taps, 2) : d->R * pt_ceil_div(d->S, 4);
+    const int most = !w.rows ? wgrad_taps_per_cta(taps, w.bn) : 512 / w.acc_cols < 16 ? 512 / w.acc_cols : 16;
+    const long long units = (long long)d->N * P, max_s = !w.rows ? ((long long)d->N * P * Q + 255) / 256 : units > 3 ? units / 2 : 1;
+    long long tiles128 = 0;                                // 128 x acc_cols tiles of fp32
+    for (int g = pt_ceil_div(parts, most < parts ? most : parts); g <= parts; ++g) {
+        const int per = pt_ceil_div(parts, g), tiles = w.n_tiles * w.m_tiles * pt_ceil_div(parts, per);
+        long long s = budget / tiles;
+        if (s > max_s) s = max_s;
+        if (s >= 2 && tiles * s * per > tiles128) tiles128 = tiles * s * per;
+    }
+    return (size_t)tiles128 * 128 * w.acc_cols * sizeof(float);
+}
+
 // The splits' fp32 partial tiles as a 2-D tensor (BN columns, rows): box 32 x 32, 128-byte swizzle.
 bool make_partial_map(const pt_ctx *c, CUtensorMap *tm, void *ws, int bn, size_t rows)
 {
@@ -2907,12 +2927,13 @@ size_t pt_sm100_conv_workspace(const pt_ctx *c, const pt_conv_desc *d, int which
     if (sp.ok && which == PT_CONV_FWD) return sp.xs_bytes + pt_align_up(sp.w2_elems * 2, 1024);
     if (sp.ok && which == PT_CONV_WGRAD) {
         const pt_conv_desc v = stem_virtual_desc(d, sp), vr = stem_rows_desc(d, sp);
-        const size_t pa = wgrad_partial_bytes(wgrad_plan(c, &v, sp.P, sp.Q)), pb = wgrad_partial_bytes(wgrad_plan(c, &vr, sp.P, sp.Q, true));
+        const pt_wgrad_plan wa = wgrad_plan(c, &v, sp.P, sp.Q), wb = wgrad_plan(c, &vr, sp.P, sp.Q, true);
+        const size_t pa = wgrad_workspace_bound(c, &v, sp.P, sp.Q, wa), pb = wb.rows ? wgrad_workspace_bound(c, &vr, sp.P, sp.Q, wb) : 0;
         return sp.xs_bytes + pt_align_up(sp.w2_elems * 4, 1024) + (pa > pb ? pa : pb);
     }
     if (which != PT_CONV_WGRAD) return 0;
     const int P = pt_out_dim(d->H, d->R, d->stride, d->pad), Q = pt_out_dim(d->W, d->S, d->stride, d->pad);
-    return wgrad_partial_bytes(wgrad_plan(c, d, P, Q));
+    return wgrad_workspace_bound(c, d, P, Q, wgrad_plan(c, d, P, Q));
 }
 
 pt_status pt_sm100_conv(pt_ctx *c, const pt_conv_desc *d, int which, const void *a, const void *b, void *out, void *ws,

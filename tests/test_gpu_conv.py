@@ -324,3 +324,33 @@ def test_a_round_of_many_layers_costs_the_host_no_more_per_call_than_one_layer()
     assert len(descs) == 180
     # (with 128 places of one plan each, the round took 2.4 times as long per call as the repeated layer)
     assert many < 1.6 * one, (many, one)
+
+
+def test_a_workspace_sized_at_one_cta_limit_serves_every_smaller_one():
+    c = B.Context(0)
+    for N, H, C, K, R, stride in [(9, 56, 41, 9, 3, 1), (6, 32, 3, 60, 3, 1), (14, 7, 30, 503, 3, 1), (24, 28, 18, 228, 3, 2), (64, 112, 3, 55, 7, 2),
+                                  (4, 16, 300, 200, 1, 1), (11, 28, 1373, 458, 1, 1), (2, 9, 64, 256, 3, 1)]:
+        d = B.make_conv_desc(N, H, H, C, K, R, R, stride, R // 2, ldx=8 if C <= 4 else None)
+        need = []
+        for limit in [0] + list(range(147, 0, -1)):
+            B.pt_set_wgrad_cta_limit(c, limit)
+            need.append(B.pt_conv_workspace_bytes(c, d, B.PT_CONV_WGRAD))
+        assert all(a >= b for a, b in zip(need, need[1:])), (N, H, C, K, R)
+    # the workspace of the largest limit, at every limit: what a launch uses stays inside it
+    N, H, C, K = 9, 56, 41, 9
+    d = B.make_conv_desc(N, H, H, C, K, 3, 3, 1, 1)
+    x, _, dy, _ = _case(N, H, H, C, K, 3, 1, W.BASE_SEED + 83)
+    xd, dyd = Hh.to_dev_padded(x, d.ldx), Hh.to_dev_padded(dy, d.ldy)
+    B.pt_set_wgrad_cta_limit(c, 0)
+    n = B.pt_conv_workspace_bytes(c, d, B.PT_CONV_WGRAD)
+    buf = torch.full((n + 4096,), 77, dtype=torch.uint8, device="cuda")
+    ref = oracle.conv_wgrad(x.numpy(), dy.numpy(), 3, 3, 1, 1)
+    for limit in (0, 140, 110, 74, 49, 36, 24, 12, 6, 2, 1):
+        B.pt_set_wgrad_cta_limit(c, limit)
+        dw = torch.empty((K, 3, 3, C), device="cuda")
+        B.pt_conv_wgrad(c, d, xd, dyd, dw, buf[:n])
+        torch.cuda.synchronize()
+        c.poll()
+        Hh.check_conv(dw, C, ref, what=f"wgrad at limit {limit}")
+        assert torch.all(buf[n:] == 77)
+    c.close()
