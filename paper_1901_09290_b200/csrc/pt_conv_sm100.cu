@@ -2396,7 +2396,7 @@ constexpr size_t kSplitSmemFloor = 116 * 1024;
 //   three round trips); in a cluster (2..8 splits): 1.5 + the bytes for the other CTAs at 25 KB/us, at 11 KB/us among more than four
 //   (213 -> 242 3x3 at 14x14, 112 KB, eight splits: 27 us as clusters, 23 through the workspace; 8 14x14 64 -> 64, 32 KB: 6.4 and 8.7).
 // A cluster needs its CTAs free at the same time in one GPC: used while the device can hold all of the launch's clusters at once.
-constexpr double kWgSearch = 400.0;      // layers whose tile takes one CTA less than this (us) also choose tap groups and unit size
+constexpr double kWgSearch = 400.0;      // generic kernel: layers whose tile takes one CTA less than this (us) also choose tap groups
 
 double wg_mma_us(int n) { return (n <= 64 ? 55.0 : n * 0.5 + 8.0) / 1900.0; }
 double wg_exchange_us(int splits, bool cluster, double acc_bytes)
@@ -2502,56 +2502,37 @@ bool wgrad_rows_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, pt_wg
     const int groups0 = pt_ceil_div(pairs, t);
     w->nb_a = pt_ceil_div(w->acc_cols, 64);
     const double cyc = wg_mma_us(w->acc_cols);
-    // Rows per unit. Large layers: the least traffic per useful row (dy rows + x halo rows, the last unit of an image padded) times
-    // the MMA steps spent per useful pixel. Small ones: with the tap groups and the splits, by the estimated time.
-    double best_cost = 1e30, best_us = 1e30;
-    bool large = false;
-    for (int pass = 0; pass < 2 && !large; ++pass) {
-        for (int nr = 1; nr <= P && nr + d->R - 1 <= 256; ++nr) {
-            const int ks = pt_ceil_div(nr * w->Wp, 16);
-            const size_t a_box = (size_t)ks * 16 * dy_row;
-            const size_t b_box = pt_align_up(((size_t)(d->R - 1) * w->Wp + span + (size_t)ks * 16) * x_row, 1024);
-            const size_t stage = w->nb_a * a_box + b_box;
-            const int st = (int)((220 * 1024 - 2048) / stage);
-            if (st < 2) break;
-            const int rb = pt_ceil_div(P, nr), units = d->N * rb;
-            auto take = [&](int apc, int s, int cl) {
-                w->nr = nr; w->ksteps = ks; w->a_box = (unsigned)a_box; w->b_box = (unsigned)b_box;
-                w->stages = st > kMaxStages ? kMaxStages : st;
-                w->stage_bytes = stage; w->RB = rb; w->units = units;
-                w->apc = apc; w->tap_groups = pt_ceil_div(pairs, apc);
-                w->splits = s; w->cluster = cl;
-            };
-            const double load = (double)(w->nb_a * nr + nr + d->R - 1) * w->Wp * 2.4e-3;      // the TMA unit, by the row
-            if (pass == 0) {
-                const double traffic = (double)(w->nb_a * nr + nr + d->R - 1) * rb / P, steps = (double)ks * 16 * rb / ((double)P * w->Wp);
-                if (traffic * steps >= best_cost) continue;
-                best_cost = traffic * steps;
-                take(pt_ceil_div(pairs, groups0), 1, 0);
-                continue;
-            }
-            for (int g = groups0; g <= pairs; g += groups0) {
-                const int apc = pt_ceil_div(pairs, g), tiles = pt_ceil_div(pairs, apc);
-                if (g > groups0 && (tiles > wgrad_budget(c) || tiles != g)) continue;
-                const double mma = ks * apc * cyc, unit = (load > mma ? load : mma) + 0.25;
-                int s, cl;
-                const double us = wg_pick_splits(c, tiles, units > 3 ? units / 2 : 1, (double)apc * w->acc_cols * 512.0,
-                                                 [&](int k) { return 1.4 + pt_ceil_div(units, k) * unit; }, &s, &cl);
-                if (us < best_us) { best_us = us; take(apc, s, cl); }
-            }
-        }
-        if (w->nr == 0) return false;
-        if (pass == 0) {
-            const double unit = w->ksteps * w->apc * cyc;
-            large = unit * w->units > kWgSearch;
-            if (large) {
-                int s, cl;
-                wg_pick_splits(c, w->tap_groups, w->units > 3 ? w->units / 2 : 1, (double)w->apc * w->acc_cols * 512.0,
-                               [&](int k) { return 1.4 + pt_ceil_div(w->units, k) * (unit + 0.25); }, &s, &cl);
-                w->splits = s; w->cluster = cl;
-            }
+    // Rows per unit, tap groups and splits, by the estimated time: a unit takes the longer of its matrix instructions and its staged rows.
+    // (Large layers took the unit with the least traffic and MMA steps per useful pixel instead, and no account of the rows: units of a
+    // single row, or so large that the splits came out uneven. 10 -> 22 1x1 at 32x32, batch 253: 23.8 -> 15.4 us; 9 -> 13 at 37x37, batch
+    // 58: 16.8 -> 13.4; 60 -> 29 at 56x56, batch 53: 23.8 -> 22.6; others the same.)
+    double best_us = 1e30;
+    for (int nr = 1; nr <= P && nr + d->R - 1 <= 256; ++nr) {
+        const int ks = pt_ceil_div(nr * w->Wp, 16);
+        const size_t a_box = (size_t)ks * 16 * dy_row;
+        const size_t b_box = pt_align_up(((size_t)(d->R - 1) * w->Wp + span + (size_t)ks * 16) * x_row, 1024);
+        const size_t stage = w->nb_a * a_box + b_box;
+        const int st = (int)((220 * 1024 - 2048) / stage);
+        if (st < 2) break;
+        const int rb = pt_ceil_div(P, nr), units = d->N * rb;
+        const double load = (double)(w->nb_a * nr + nr + d->R - 1) * w->Wp * 2.4e-3;      // the TMA unit, by the row
+        for (int g = groups0; g <= pairs; g += groups0) {
+            const int apc = pt_ceil_div(pairs, g), tiles = pt_ceil_div(pairs, apc);
+            if (g > groups0 && (tiles > wgrad_budget(c) || tiles != g)) continue;
+            const double mma = ks * apc * cyc, unit = (load > mma ? load : mma) + 0.25;
+            int s, cl;
+            const double us = wg_pick_splits(c, tiles, units > 3 ? units / 2 : 1, (double)apc * w->acc_cols * 512.0,
+                                             [&](int k) { return 1.4 + pt_ceil_div(units, k) * unit; }, &s, &cl);
+            if (us >= best_us) continue;
+            best_us = us;
+            w->nr = nr; w->ksteps = ks; w->a_box = (unsigned)a_box; w->b_box = (unsigned)b_box;
+            w->stages = st > kMaxStages ? kMaxStages : st;
+            w->stage_bytes = stage; w->RB = rb; w->units = units;
+            w->apc = apc; w->tap_groups = tiles;
+            w->splits = s; w->cluster = cl;
         }
     }
+    if (w->nr == 0) return false;
     w->units_per_split = pt_ceil_div(w->units, w->splits);
     w->splits = pt_ceil_div(w->units, w->units_per_split);
     if (w->splits < 2) w->cluster = 0;
