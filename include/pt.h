@@ -84,7 +84,7 @@ uint64_t pt_launch_count(const pt_ctx *ctx);
  * (Eq. 4) splits its reduction over the output pixels across CTAs, and the weight gradients of different layers are
  * independent of each other: launches that leave SMs free can run side by side on several streams, which amortises their
  * fixed cost (pipeline fill, partial-tile exchange). The setting changes the workspace pt_conv_workspace_bytes reports for
- * PT_CONV_WGRAD, so set it before sizing workspaces; it has no effect on results beyond the summation order of the splits
+ * PT_CONV_WGRAD (one sized at a limit serves every smaller limit), so set it before sizing workspaces; it has no effect on results beyond the summation order of the splits
  * (still fixed for a given setting). PT_ERR_INVALID_ARG if max_ctas is negative.
  * The CTAs of a split launch wait (bounded) for one another and occupy an SM each, so all of them must be able to be on
  * the device at once: a caller that keeps weight-gradient launches in flight on S streams sets a limit L with
@@ -112,8 +112,8 @@ enum { PT_CONV_FWD = 0, PT_CONV_DGRAD = 1, PT_CONV_WGRAD = 2 };
 /* Bytes of caller-provided workspace the given pass needs for this descriptor (0 = none). */
 size_t pt_conv_workspace_bytes(const pt_ctx *ctx, const pt_conv_desc *d, int which);
 /* CTAs pt_conv_wgrad launches for this descriptor at the context's current limit (pt_set_wgrad_cta_limit): tiles x splits,
- * splits being the largest count that keeps the product within the limit (at least 1: a descriptor with more tiles than
- * the limit runs unsplit). *waits (optional) = 1 if those CTAs wait for one another (splits > 1), which is what the
+ * splits being at most what keeps the product within the limit (1 for a descriptor with more tiles than the limit), fewer
+ * where the exchange between them would cost more than they save. *waits (optional) = 1 if those CTAs wait for one another (splits > 1), which is what the
  * co-residency rule of pt_set_wgrad_cta_limit is about. Lets a caller choose per-launch limits that waste no SMs.
  * 0 if the tcgen05 kernels do not take the descriptor. */
 int32_t pt_conv_wgrad_ctas(const pt_ctx *ctx, const pt_conv_desc *d, int32_t *waits);
@@ -121,7 +121,7 @@ int32_t pt_conv_wgrad_ctas(const pt_ctx *ctx, const pt_conv_desc *d, int32_t *wa
 /* Stream order: the three calls below are ordinary stream work. Their kernels are launched with programmatic stream
  * serialization and read the WEIGHTS before waiting for the preceding kernel of the stream; that is invisible to callers
  * because only kernels that release their dependents early (griddepcontrol.launch_dependents before their last store) can be
- * overtaken: of this library's kernels the convolutions and the read-only sweeps of the lasso step do that, and none of them
+ * overtaken: of this library's kernels the convolutions, the batch norms and the read-only sweeps and the finish of the lasso step do that, and none of them
  * writes weights (the update of pt_group_lasso_sgd_step and the gather of pt_reconfigure complete before their successors
  * start). A caller's own kernel that writes w and releases its dependents early must be followed by an event or another
  * kernel before a convolution reads w. */
@@ -212,7 +212,7 @@ typedef struct {
 /* Bytes of workspace both calls need for this descriptor (partial sums of the reduction blocks). */
 size_t pt_bn_workspace_bytes(const pt_ctx *ctx, const pt_bn_desc *d);
 
-/* y = relu(gamma*xhat + beta + residual). residual may be NULL. running_mean / running_var: both NULL (not kept) or both
+/* y = relu(gamma*xhat + beta + residual). residual may be NULL; y may be x or residual. running_mean / running_var: both NULL (not kept) or both
  * given (updated in place). save_mean, save_invstd (C floats each) receive the batch statistics the backward pass needs.
  * PT_ERR_INVALID_ARG for bad sizes, pitches, alignment or missing pointers; PT_ERR_UNSUPPORTED for ld > 2048;
  * PT_ERR_WORKSPACE if ws is too small. */
@@ -222,7 +222,7 @@ pt_status pt_bn_relu_fwd(pt_ctx *ctx, const pt_bn_desc *d, const void *x, const 
 
 /* The same forward pass without its reduction over x: the batch statistics come from the rows of partial sums the producing
  * convolution left (pt_conv_fwd_stats: stats, n_parts; the sums are those of the stored bf16 values, exactly what the
- * reduction pass of pt_bn_relu_fwd would read). Two launches instead of three, one pass over x instead of two; no workspace. */
+ * reduction pass of pt_bn_relu_fwd would read). One launch instead of two, one pass over x instead of two; no workspace. */
 pt_status pt_bn_relu_fwd_stats(pt_ctx *ctx, const pt_bn_desc *d, const void *x, const void *residual, const float *gamma,
                                const float *beta, float *running_mean, float *running_var, float *save_mean, float *save_invstd,
                                void *y, const float *stats, int32_t n_parts, void *stream);

@@ -9,7 +9,7 @@
 //   conv_wgrad_kernel  weight gradient: both operands MN-major, reduction over pixels split across CTAs, partial tiles
 //                      summed in-kernel in a fixed order.
 //   conv_wgrad_rows_kernel  weight gradient of stride-1 layers with at most 64 input channels: row blocks of x staged
-//                      once, taps as row-shifted descriptors, two taps per MMA on the M side; same finish phase.
+//                      once, taps as row-shifted descriptors, two or four taps per MMA on the M side; same finish phase.
 //   stem_* kernels     space-to-depth layout kernels of the few-channel stride-2 stem.
 // Ragged channel counts are handled by the TMA unit (true extents in the tensor maps: zero-fill on load, clipping on
 // store) and by skipping the 16-wide k-steps past the last valid channel.
@@ -17,7 +17,9 @@
 // tcgen05.mma, more than a narrow MMA takes to run, so operands are loaded by several producer warps and, where
 // independent accumulators exist, MMAs are issued by up to four warps, each with its own ring and TMEM buffers.
 // The kernels are launched with programmatic stream serialization (griddepcontrol.wait after the prologue).
-// Every wait is bounded; on expiry the CTA records PT_DEV_TIMEOUT in the status word, drains its copies and exits.
+// Every wait on a barrier or a counter is bounded; on expiry the CTA records PT_DEV_TIMEOUT in the status word, drains its copies and
+// exits. (The cluster barriers of the weight gradients' exchange have no limit: every thread of every CTA reaches them, aborting ones
+// too.)
 #include "pt_internal.h"
 #include "pt_sm100_ptx.cuh"
 #include <cudaTypedefs.h>
@@ -25,22 +27,6 @@
 using namespace sm100;
 
 namespace {
-// Launch with programmatic stream serialization: the kernel may be scheduled while the previous kernel of the stream is
-// still draining, so its prologue (barrier setup, TMEM allocation, descriptor prefetch) and the launch latency overlap that
-// kernel's tail. Every kernel launched this way executes griddepcontrol.wait before its first global-memory access.
-template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args)
-{
-    cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-
 // A tensor-map encode that the driver refused is kept, with its line, for pt_last_cuda_error.
 bool map_ok(CUresult r, int line)
 {
@@ -1227,8 +1213,8 @@ __device__ __forceinline__ void wgrad_store4(float *dst, const float4 &v, int nv
 // here it is two cluster barriers and the bytes (about 2.5 us). At most eight splits: what a portable cluster can be.
 // Every thread of every CTA of the cluster calls this, with the same trip counts, and aborting CTAs too (they hand on zeros; dw is
 // then undefined and the time-out already recorded): the barriers always complete.
-__device__ __forceinline__ void wgrad_cluster_sum(const WgradP &p, Ctl *ctl, uint32_t data_base, uint32_t tmem_base, int ntap, int tap0, int k0,
-                                                  int c0, int split, int iters, uint32_t ring_bytes, int n_acc, int acc_cols)
+__device__ __forceinline__ void wgrad_cluster_sum(const WgradP &p, Ctl *ctl, uint32_t data_base, uint32_t tmem_base, int tap0, int k0, int c0,
+                                                  int split, int iters, uint32_t ring_bytes, int n_acc, int acc_cols)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int S = p.splits, nch = pt_ceil_div_dev(acc_cols, 32);
@@ -1294,7 +1280,7 @@ __device__ __forceinline__ void wgrad_cluster_sum(const WgradP &p, Ctl *ctl, uin
 // `ring_bytes` of shared memory at `data_base` are free by then and serve as staging. `tap0` is the CTA's first tap (generic form) or
 // accumulator (row-block form).
 __device__ __forceinline__ void wgrad_finish(const WgradP &p, const CUtensorMap &tmP, Ctl *ctl, uint32_t data_base, uint32_t tmem_base,
-                                             int ntap, int tap0, int k0, int c0, int split, int iters, uint32_t ring_bytes, int n_acc, int acc_cols)
+                                             int tap0, int k0, int c0, int split, int iters, uint32_t ring_bytes, int n_acc, int acc_cols)
 {
     volatile int *abort_flag = &ctl->abort_flag;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1307,9 +1293,6 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, const CUtensorMap 
         if (warp == 2) WTRACE(3);
         tc_fence_after();
         if (ok) {
-            const int k = k0 + quarter * 32 + lane;
-            const bool row_ok = k < p.K;
-            (void)row_ok;
             const uint32_t lane_addr = tmem_base + ((uint32_t)(quarter * 32) << 16);
             if (p.cluster) {
                 // the exchange is below: every thread of the cluster takes part in its barriers
@@ -1428,7 +1411,7 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, const CUtensorMap 
         tc_fence_before();
     }
     if (p.cluster) {
-        wgrad_cluster_sum(p, ctl, data_base, tmem_base, ntap, tap0, k0, c0, split, iters, ring_bytes, n_acc, acc_cols);
+        wgrad_cluster_sum(p, ctl, data_base, tmem_base, tap0, k0, c0, split, iters, ring_bytes, n_acc, acc_cols);
         return;
     }
     __syncthreads();
@@ -1665,7 +1648,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_wgrad_kernel(const __grid_co
         if (ok) umma_commit_lead(smem_u32(&ctl->accum), leader);
         if (warp == 1) WTRACE(2);
     }
-    wgrad_finish(p, tmP, ctl, data_base, tmem_base, ntap, tap0, k0, c0, split, iters, p.data_bytes, ntap, p.BN);
+    wgrad_finish(p, tmP, ctl, data_base, tmem_base, tap0, k0, c0, split, iters, p.data_bytes, ntap, p.BN);
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem_base, (uint32_t)p.tmem_cols);
@@ -1824,7 +1807,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_wgrad_rows_kernel(const __gr
         if (ok) umma_commit_lead(smem_u32(&ctl->accum), leader);
         if (warp == 1) WTRACE(2);
     }
-    wgrad_finish(p, tmP, ctl, data_base, tmem_base, 0, acc0, k0, c0, split, iters, p.data_bytes, n_acc, p.acc_cols);
+    wgrad_finish(p, tmP, ctl, data_base, tmem_base, acc0, k0, c0, split, iters, p.data_bytes, n_acc, p.acc_cols);
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem_base, (uint32_t)p.tmem_cols);
@@ -2157,7 +2140,7 @@ pt_status launch_gemm(pt_ctx *c, const GemmMaps &tm, GemmP &p, cudaStream_t st)
         p.stats = c->stats_out;
     }
     if (c->test_skip == 2) { p.test_skip = 1; c->test_skip = 0; }
-    PT_CUDA_OK(launch_pdl(kernel, dim3((unsigned)grid), dim3(kGemmThreads), smem, st, tm.a, tm.tail, tm.b, tmC, p));
+    PT_CUDA_OK(pt_launch_pdl(kernel, dim3((unsigned)grid), dim3(kGemmThreads), smem, st, tm.a, tm.tail, tm.b, tmC, p));
     c->launches += 1;
     PT_CUDA_OK(cudaGetLastError());
     return PT_OK;
@@ -2359,7 +2342,7 @@ pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const
         p.stats = c->stats_out;
     }
     if (c->test_skip == 5) { p.test_skip = 1; c->test_skip = 0; }
-    PT_CUDA_OK(launch_pdl(kernel, dim3((unsigned)grid), dim3(kHaloThreads), smem, st, tmA, tmB, tmC, p));
+    PT_CUDA_OK(pt_launch_pdl(kernel, dim3((unsigned)grid), dim3(kHaloThreads), smem, st, tmA, tmB, tmC, p));
     c->launches += 1;
     PT_CUDA_OK(cudaGetLastError());
     return PT_OK;

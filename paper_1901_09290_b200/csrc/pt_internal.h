@@ -140,8 +140,10 @@ static inline int pt_out_dim(int H, int R, int stride, int pad) {
 }
 
 // Launch with programmatic stream serialization: the kernel may be scheduled while the previous kernel of the stream is still
-// draining, so that its launch latency and prologue overlap that kernel's tail. Every kernel launched this way executes
-// griddepcontrol.wait before it touches anything a predecessor wrote, and before it releases its own dependents.
+// draining, so that its launch latency and prologue overlap that kernel's tail. In a kernel launched this way every thread executes
+// griddepcontrol.wait before it touches anything a predecessor wrote, and all but the producers before they release its dependents. Those
+// wait later, right before their first load, or not at all where what they load has been complete for longer: weights, which no kernel
+// that releases its dependents early writes, and the inputs of a batch-norm apply pass, whose predecessor reads them too.
 template <typename... KArgs, typename... Args>
 cudaError_t pt_launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args)
 {

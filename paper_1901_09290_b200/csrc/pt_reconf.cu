@@ -258,15 +258,9 @@ extern "C" pt_status pt_reconfigure_plan_enqueue(pt_ctx *c, const pt_graph *g, i
     volatile unsigned int *flag = (volatile unsigned int *)c->h_counts;
     volatile int32_t *counts = (volatile int32_t *)c->h_counts + 16;
     const unsigned int seq = ++c->plan_seq;
-    cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3((unsigned)g->n_spaces); cfg.blockDim = dim3(1024); cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    PT_CUDA_OK(cudaLaunchKernelEx(&cfg, keep_scan_kernel, (const SpaceDev *)dev, (const MemberDev *)(dev + sb), new2old,
-                                  (volatile int32_t *)counts, (volatile unsigned int *)flag, seq, c->d_status + 2));
+    PT_CUDA_OK(pt_launch_pdl(keep_scan_kernel, dim3((unsigned)g->n_spaces), dim3(1024), 0, st, (const SpaceDev *)dev,
+                             (const MemberDev *)(dev + sb), new2old, (volatile int32_t *)counts, (volatile unsigned int *)flag, seq,
+                             c->d_status + 2));
     c->launches += 1;
     PT_CUDA_OK(cudaGetLastError());
     c->plan_spaces = g->n_spaces;
