@@ -2,8 +2,10 @@
 #include "pt_internal.h"
 #include <stdio.h>
 
-static const size_t kArenaBytes = 5u << 20;     // 5 MiB of tables: ten slots of 512 KiB
-static const size_t kSlotBytes = 512u << 10;
+// Ten slots for tables. 1.25 MiB hold what a chunk list of column groups needs for every model whose list of whole lines fitted 512 KiB
+// (a layer of many output and few input channels takes up to 2.3 times the bytes).
+static const size_t kSlotBytes = 1280u << 10;
+static const size_t kArenaBytes = 10 * kSlotBytes;
 static const size_t kSyncWords = 16384;         // arrival counters of the split weight gradients
 
 static thread_local char g_last_cuda[384] = "";

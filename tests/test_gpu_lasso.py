@@ -329,3 +329,36 @@ def test_conv_right_behind_the_update_reads_the_new_weights():
         w_now = dm.wb[li][..., :l.C].float().cpu().numpy()
         ref = oracle.conv_fwd(x.numpy(), w_now, 1, l.pad)
         Hh.check_conv(y, l.K, ref, what=f"iteration {it}")
+
+
+def test_a_model_of_a_thousand_layers_fits_the_tables():
+    """The tables of the step, the detection and the gather: 920 bytes a layer here, where lists of whole lines took 344."""
+    c, n, K, C = B.Context(0), 1000, 1024, 32
+    gen = torch.Generator(device="cuda").manual_seed(W.BASE_SEED + 95)
+    w = torch.empty((n, K, C), device="cuda").normal_(0, 0.1, generator=gen)
+    g, v, so, si = torch.zeros_like(w), torch.zeros_like(w), torch.zeros((n, K), device="cuda"), torch.zeros((n, C), device="cuda")
+    zo, zi = torch.zeros((n, K), dtype=torch.uint8, device="cuda"), torch.zeros((n, C), dtype=torch.uint8, device="cuda")
+    w[:, 5] = 0.0
+    layers = [B.make_layer(w[i], g[i], v[i], None, K, C, 1, C, True, True, so[i], si[i], zo[i], zi[i]) for i in range(n)]
+    arr = B.layer_array(layers)
+    ws = torch.empty(B.pt_group_lasso_workspace_bytes(c, arr), dtype=torch.uint8, device="cuda")
+    B.pt_group_lasso_norms(c, arr, None, ws)
+    B.pt_find_zero_groups(c, arr, 1e-4, False, ws)
+    torch.cuda.synchronize()
+    c.poll()
+    assert torch.allclose(so.double(), w.double().square().sum(2), rtol=1e-5) and torch.allclose(si.double(), w.double().square().sum(1), rtol=1e-5)
+    assert int(zo.sum()) == n and bool((zo[:, 5] == 1).all()) and int(zi.sum()) == 0
+    # the gather of all of them into models without the dead channel
+    sizes, links = [C] + [K] * n, [(0, i + 1) for i in range(n)]
+    fixed = [True] + [False] * n
+    old = B.GraphHandle(sizes, fixed, layers, links)
+    n2o = torch.empty(sum(sizes), dtype=torch.int32, device="cuda")
+    assert B.pt_reconfigure_plan(c, old, n2o) == [C] + [K - 1] * n
+    nw, nv = torch.zeros((n, K - 1, C), device="cuda"), torch.zeros((n, K - 1, C), device="cuda")
+    new = B.GraphHandle([C] + [K - 1] * n, fixed, [B.make_layer(nw[i], None, nv[i], None, K - 1, C, 1, C, True, True, None, None, None, None)
+                                                   for i in range(n)], links)
+    B.pt_reconfigure(c, old, n2o, new)
+    torch.cuda.synchronize()
+    c.poll()
+    assert torch.equal(nw[:, :5], w[:, :5]) and torch.equal(nw[:, 5:], w[:, 6:])
+    c.close()
