@@ -89,9 +89,13 @@ uint64_t pt_launch_count(const pt_ctx *ctx);
  * The CTAs of a split launch wait (bounded) for one another and occupy an SM each, so all of them must be able to be on
  * the device at once: a caller that keeps weight-gradient launches in flight on S streams sets a limit L with
  * S * L <= the SM count. Beyond that the launches may starve each other until a wait expires (PT_ERR_TIMEOUT at the next
- * pt_poll_device_status; nothing hangs). A limit of at most half of the SMs also tells pt_conv_dgrad that such launches run
- * beside it: it then leaves SMs free for them (results unchanged). */
+ * pt_poll_device_status; nothing hangs). */
 pt_status pt_set_wgrad_cta_limit(pt_ctx *ctx, int max_ctas);
+/* The same for the data gradients of stride-1 filters with several taps; 0 (the default) is all SMs. Their CTAs are persistent with a
+ * fixed share of the work: beside weight gradients on other streams, those that find their SM taken start when the others are done, and
+ * a launch takes two rounds. A caller who keeps weight gradients in flight leaves them SMs this way (three fifths for the data gradients
+ * measured best in the steps of two networks). No effect on results. PT_ERR_INVALID_ARG if max_ctas is negative. */
+pt_status pt_set_dgrad_cta_limit(pt_ctx *ctx, int max_ctas);
 
 /* ------------------------------------------------------------------------------------------
  * Convolutions (paper Sec. 2.1: convolution layers dominate training time; Eq. 4: weight gradient).

@@ -83,6 +83,7 @@ EXPORTS = {
     "pt_test_set_wait_limit": (c_int32, [c_void_p, ctypes.c_uint32]),
     "pt_test_skip_next_arrive": (c_int32, [c_void_p, c_int32]),
     "pt_set_wgrad_cta_limit": (c_int32, [c_void_p, c_int32]),
+    "pt_set_dgrad_cta_limit": (c_int32, [c_void_p, c_int32]),
     "pt_conv_wgrad_ctas": (c_int32, [c_void_p, POINTER(pt_conv_desc), POINTER(c_int32)]),
     "pt_conv_workspace_bytes": (c_size_t, [c_void_p, POINTER(pt_conv_desc), c_int32]),
     "pt_conv_fwd": (c_int32, [c_void_p, POINTER(pt_conv_desc), c_void_p, c_void_p, c_void_p, c_void_p, c_size_t, c_void_p]),
@@ -197,6 +198,9 @@ class Context:
     def set_wgrad_cta_limit(self, max_ctas: int):
         _check(lib().pt_set_wgrad_cta_limit(self.handle, int(max_ctas)), "pt_set_wgrad_cta_limit")
 
+    def set_dgrad_cta_limit(self, max_ctas: int):
+        _check(lib().pt_set_dgrad_cta_limit(self.handle, int(max_ctas)), "pt_set_dgrad_cta_limit")
+
     def poll(self, stream=None):
         _check(lib().pt_poll_device_status(self.handle, _stream(stream)), "pt_poll_device_status")
 
@@ -216,6 +220,10 @@ def pt_test_skip_next_arrive(ctx: Context, which: int):
 
 def pt_set_wgrad_cta_limit(ctx: Context, max_ctas: int):
     ctx.set_wgrad_cta_limit(max_ctas)
+
+
+def pt_set_dgrad_cta_limit(ctx: Context, max_ctas: int):
+    ctx.set_dgrad_cta_limit(max_ctas)
 
 
 def pt_conv_workspace_bytes(ctx: Context, d: pt_conv_desc, which: int) -> int:

@@ -107,6 +107,13 @@ extern "C" pt_status pt_set_wgrad_cta_limit(pt_ctx *c, int max_ctas)
     return PT_OK;
 }
 
+extern "C" pt_status pt_set_dgrad_cta_limit(pt_ctx *c, int max_ctas)
+{
+    if (!c || max_ctas < 0) return PT_ERR_INVALID_ARG;
+    c->dgrad_ctas = max_ctas;
+    return PT_OK;
+}
+
 extern "C" pt_status pt_test_set_wait_limit(pt_ctx *c, uint32_t milliseconds)
 {
     if (!c) return PT_ERR_INVALID_ARG;

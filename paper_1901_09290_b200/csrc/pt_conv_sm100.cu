@@ -2328,10 +2328,8 @@ pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const
         const int want = c->sm_count * 2 / 3, rounds = total_tiles <= 2 * want ? 2 : pt_ceil_div(total_tiles, want);
         grid = pt_ceil_div(total_tiles, rounds);
     }
-    // A limit on the weight gradients' CTAs says that they run beside other kernels: the data gradients, persistent with a fixed share of
-    // the tiles per CTA, then leave them two fifths of the SMs. On all SMs, the CTAs that find theirs taken only start when the others
-    // are done and every launch takes two rounds (ResNet-32's step 630 -> 612 us, ResNet-50's at keep 0.60 2645 -> 2625).
-    if (B_MN && h.o_step == 1 && c->wgrad_ctas > 0 && 2 * c->wgrad_ctas <= c->sm_count && grid > c->sm_count * 3 / 5) grid = c->sm_count * 3 / 5;
+    // (the parities of a stride-2 data gradient share the SMs among themselves)
+    if (B_MN && h.o_step == 1 && c->dgrad_ctas > 0 && grid > c->dgrad_ctas) grid = c->dgrad_ctas;
     if (h.max_ctas > 0 && grid > h.max_ctas) grid = h.max_ctas;
     if (c->stats_mode) {
         if (!p.tma_store || B_MN) return PT_ERR_UNSUPPORTED;

@@ -354,3 +354,39 @@ def test_a_workspace_sized_at_one_cta_limit_serves_every_smaller_one():
         Hh.check_conv(dw, C, ref, what=f"wgrad at limit {limit}")
         assert torch.all(buf[n:] == 77)
     c.close()
+
+
+def test_a_limit_on_the_weight_gradients_leaves_the_data_gradients_alone():
+    """Only the data gradients' own limit makes their launches smaller; neither changes a result."""
+    c = B.Context(0)
+    N, H, C = 64, 56, 64
+    gen = torch.Generator(device="cuda").manual_seed(W.BASE_SEED + 84)
+    d = B.make_conv_desc(N, H, H, C, C, 3, 3, 1, 1)
+    dy = torch.randn((N, H, H, C), generator=gen, device="cuda").to(torch.bfloat16)
+    w = torch.randn((C, 3, 3, C), generator=gen, device="cuda").to(torch.bfloat16)
+
+    def run(wgrad_limit, dgrad_limit):
+        B.pt_set_wgrad_cta_limit(c, wgrad_limit)
+        if dgrad_limit:
+            B.pt_set_dgrad_cta_limit(c, dgrad_limit)
+        dx = torch.empty_like(dy)
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        best = 1e9
+        for _ in range(5):
+            a.record()
+            for _ in range(40):
+                B.pt_conv_dgrad(c, d, dy, w, dx, None)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b))
+        return dx, best
+
+    run(0, 0)
+    dx0, t0 = run(0, 0)
+    dx1, t1 = run(49, 0)
+    assert torch.equal(dx0, dx1) and t1 < 1.1 * t0, (t0, t1)
+    dx2, t2 = run(49, 74)
+    assert torch.equal(dx0, dx2) and t2 > 1.3 * t0, (t0, t2)      # (half of the SMs: about twice the time)
+    with pytest.raises(B.PtError):
+        B.pt_set_dgrad_cta_limit(c, -1)
+    c.close()
