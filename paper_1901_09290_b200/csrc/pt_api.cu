@@ -2,10 +2,11 @@
 #include "pt_internal.h"
 #include <stdio.h>
 
-// Ten slots for tables. 1.25 MiB hold what a chunk list of column groups needs for every model whose list of whole lines fitted 512 KiB
-// (a layer of many output and few input channels takes up to 2.3 times the bytes).
-static const size_t kSlotBytes = 1280u << 10;
-static const size_t kArenaBytes = 10 * kSlotBytes;
+static const size_t kArenaBytes = 5u << 20;     // 5 MiB of tables: ten slots of 512 KiB
+static const size_t kSlotBytes = 512u << 10;
+// A larger table gets memory of its own, of this size: it holds what a chunk list of column groups needs for every model whose list of
+// whole lines fitted 512 KiB (a layer of many output and few input channels takes up to 2.3 times the bytes).
+static const size_t kLargeSlotBytes = 1280u << 10;
 static const size_t kSyncWords = 16384;         // arrival counters of the split weight gradients
 
 static thread_local char g_last_cuda[384] = "";
@@ -31,6 +32,16 @@ extern "C" const char *pt_status_string(pt_status s)
     case PT_ERR_ARCH: return "PT_ERR_ARCH";
     }
     return "PT_ERR_UNKNOWN";
+}
+
+static std::vector<pt_region *> pt_regions(pt_ctx *c)
+{
+    std::vector<pt_region *> r;
+    for (pt_group_slot &s : c->lasso_tab) r.push_back(&s.reg);
+    for (pt_group_slot &s : c->detect_tab) r.push_back(&s.reg);
+    r.push_back(&c->graph_tab);
+    for (pt_ctx::GatherSlot &s : c->gather_slot) r.push_back(&s.reg);
+    return r;
 }
 
 extern "C" pt_status pt_create(pt_ctx **out, int device)
@@ -60,10 +71,10 @@ extern "C" pt_status pt_create(pt_ctx **out, int device)
     // pinned memory comes back from an earlier context with what it held: a flag left there must not look like this context's first plan
     memset(c->h_counts, 0, (65536 + 16) * sizeof(int32_t));
     size_t off = 0;
-    for (int i = 0; i < 3; ++i) { c->lasso_tab[i].reg.off = off; c->lasso_tab[i].reg.cap = kSlotBytes; off += kSlotBytes; }
-    for (int i = 0; i < 2; ++i) { c->detect_tab[i].reg.off = off; c->detect_tab[i].reg.cap = kSlotBytes; off += kSlotBytes; }
-    c->graph_tab.off = off;  c->graph_tab.cap = kSlotBytes; off += kSlotBytes;
-    for (int i = 0; i < 4; ++i) { c->gather_slot[i].reg.off = off; c->gather_slot[i].reg.cap = kSlotBytes; off += kSlotBytes; }
+    for (pt_region *r : pt_regions(c)) {
+        r->dev = c->d_arena + off; r->host = c->h_stage + off; r->cap = kSlotBytes;
+        off += kSlotBytes;
+    }
     // Driver entry points for tensor-map encoding, looked up at run time so the library loads without libcuda.
     cudaDriverEntryPointQueryResult qr;
     void *fn = nullptr;
@@ -89,6 +100,10 @@ extern "C" pt_status pt_destroy(pt_ctx *c)
     if (c->fork_ev) cudaEventDestroy(c->fork_ev);
     if (c->d_status) cudaFree(c->d_status);
     if (c->h_status) cudaFreeHost(c->h_status);
+    for (pt_region *r : pt_regions(c)) {
+        if (r->large_dev) cudaFree(r->large_dev);
+        if (r->large_host) cudaFreeHost(r->large_host);
+    }
     if (c->d_arena) cudaFree(c->d_arena);
     if (c->h_stage) cudaFreeHost(c->h_stage);
     if (c->h_counts) cudaFreeHost(c->h_counts);
@@ -155,15 +170,25 @@ extern "C" pt_status pt_poll_device_status(pt_ctx *c, void *stream)
 
 pt_status pt_upload_table(pt_ctx *c, pt_region *reg, const void *host, size_t bytes, cudaStream_t st, char **dev)
 {
-    if (bytes > reg->cap) return PT_ERR_UNSUPPORTED;
-    *dev = c->d_arena + reg->off;
+    if (bytes > reg->cap) {
+        // (what a captured graph may hold of the smaller slot stays where it is)
+        if (bytes > kLargeSlotBytes) return PT_ERR_UNSUPPORTED;
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        PT_CUDA_OK(cudaStreamIsCapturing(st, &cap));
+        if (cap != cudaStreamCaptureStatusNone) return PT_ERR_UNSUPPORTED;
+        if (!reg->large_dev) PT_CUDA_OK(cudaMalloc(&reg->large_dev, kLargeSlotBytes));
+        if (!reg->large_host) PT_CUDA_OK(cudaMallocHost(&reg->large_host, kLargeSlotBytes));
+        reg->dev = reg->large_dev; reg->host = reg->large_host; reg->cap = kLargeSlotBytes;
+        reg->valid = false;
+    }
+    *dev = reg->dev;
     if (reg->valid && reg->key.size() == bytes && memcmp(reg->key.data(), host, bytes) == 0) return PT_OK;
     if (c->upload_pending) {                       // the staging buffer may still be the source of a copy
         PT_CUDA_OK(cudaEventSynchronize(c->upload_done));
         c->upload_pending = false;
     }
-    memcpy(c->h_stage + reg->off, host, bytes);
-    PT_CUDA_OK(cudaMemcpyAsync(c->d_arena + reg->off, c->h_stage + reg->off, bytes, cudaMemcpyHostToDevice, st));
+    memcpy(reg->host, host, bytes);
+    PT_CUDA_OK(cudaMemcpyAsync(reg->dev, reg->host, bytes, cudaMemcpyHostToDevice, st));
     PT_CUDA_OK(cudaEventRecord(c->upload_done, st));
     c->upload_pending = true;
     reg->key.assign((const char *)host, (const char *)host + bytes);

@@ -28,8 +28,10 @@ void pt_note_cuda_error(cudaError_t e, const char *call, const char *file, int l
 // keep-set scan (self-resetting), [3] spare.
 enum { PT_DEV_OK = 0, PT_DEV_TIMEOUT = 1, PT_DEV_BAD_INDEX = 2 };
 
-struct pt_region {              // one cached table in the arena
-    size_t off = 0, cap = 0;    // byte range inside the arena
+struct pt_region {              // one cached table: a slot of the arena, or memory of its own for a larger one
+    char *dev = nullptr, *host = nullptr;               // where it is on the device and its pinned staging
+    size_t cap = 0;
+    char *large_dev = nullptr, *large_host = nullptr;
     std::vector<char> key;      // host bytes the current device copy was built from
     bool valid = false;
 };

@@ -546,9 +546,9 @@ pt_status bind(pt_ctx *c, const pt_layer *layers, int n, bool detect, void *ws, 
     memcpy(&w, s->ws, sizeof(w));
     if (!ws || ws_bytes < w.total || ((uintptr_t)ws & 255)) return PT_ERR_WORKSPACE;
     b->slot = s;
-    b->dl = (const LayerDev *)(c->d_arena + s->reg.off);
-    b->dc = (const Chunk *)(c->d_arena + s->reg.off + s->chunks_off);
-    b->dj = (const FinishJob *)(c->d_arena + s->reg.off + s->jobs_off);
+    b->dl = (const LayerDev *)s->reg.dev;
+    b->dc = (const Chunk *)(s->reg.dev + s->chunks_off);
+    b->dj = (const FinishJob *)(s->reg.dev + s->jobs_off);
     char *a = (char *)ws;
     GroupP &p = b->p;
     memset(&p, 0, sizeof(p));

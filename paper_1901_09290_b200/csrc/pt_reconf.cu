@@ -326,7 +326,7 @@ extern "C" pt_status pt_reconfigure(pt_ctx *c, const pt_graph *og, const int32_t
     for (int i = 0; i < 4; ++i) {
         pt_ctx::GatherSlot &gs = c->gather_slot[i];
         if (!(gs.reg.valid && gs.chunks && args == gs.args)) continue;
-        const char *dev = c->d_arena + gs.reg.off;
+        const char *dev = gs.reg.dev;
         gather_kernel<<<gs.chunks, kGThreads, 0, st>>>((const GatherJob *)dev, (const GatherChunk *)(dev + gs.jobs_bytes), c->d_status);
         c->launches += 1;
         PT_CUDA_OK(cudaGetLastError());
