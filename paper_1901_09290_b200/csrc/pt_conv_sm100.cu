@@ -316,7 +316,6 @@ __global__ void __launch_bounds__(kGemmThreads, 1) conv_gemm_kernel(const __grid
             const uint32_t my_bytes = is_a ? a_bytes : B_MN ? (uint32_t)((nb_b - b_id + p.n_b - 1) / p.n_b) * 8192u : b_bytes;
             const uint32_t tail_bytes = is_a ? (uint32_t)(kBM * p.tail_lanes * 2) : my_bytes;
             int s = 0, ph = 0, issued = 0;   // stage-ring position, continuous across tiles; stages filled
-            int other = 0;                   // of them in the ring that it does not feed now
             bool dep_waited = false;         // the activation producer has waited for the previous kernel's results
             const int SR = p.stages / p.n_issuers;
             const bool both = is_a && p.n_issuers == 2 && !ring2;      // this producer feeds two rings, a tile each in turn
@@ -383,12 +382,15 @@ __global__ void __launch_bounds__(kGemmThreads, 1) conv_gemm_kernel(const __grid
                     }
                 }
                 if (!ok) break;
-                if (both) { int t = s; s = s1; s1 = t; t = ph; ph = ph1; ph1 = t; ring ^= 1; other = issued - other; }
+                if (both) { int t = s; s = s1; s1 = t; t = ph; ph = ph1; ph1 = t; ring ^= 1; }
             }
             if (*abort_flag) {       // the copies this thread issued: stages of one ring or of both, resident weights
                 if (b_id == 0 && p.resident) drain_ring(smem_u32(&ctl->w_full), 1, 1);
-                drain_ring(smem_u32(&ctl->full[ring * SR]), SR, issued - other);
-                if (both) drain_ring(smem_u32(&ctl->full[(ring ^ 1) * SR]), SR, other);
+                // (a producer of two rings fills a tile's stages in each in turn: how many of them each got follows from their number)
+                const int tiles = issued / iters, rest = issued - tiles * iters;
+                const int first = both ? (tiles + 1) / 2 * iters + (tiles & 1 ? 0 : rest) : issued;
+                drain_ring(smem_u32(&ctl->full[(both ? 0 : ring) * SR]), SR, first);
+                if (both) drain_ring(smem_u32(&ctl->full[SR]), SR, issued - first);
             }
         }
     } else if (warp == 1 || (warp == 15 && p.n_issuers == 2)) {
@@ -829,6 +831,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
             int ring = pid % NI, base_pos = 0, base_ph = 0;
             const int kdiv = p.k_chunks / SR, kmod = p.k_chunks - kdiv * SR;
             int sb_pos = 0, sb_ph = 0;                         // position in this pipeline's weight ring
+            const int skip_a = p.test_skip;
             int issued_a = 0, issued_b = 0;                    // stages filled (a producer of activations feeds one ring)
             for (int tile = blockIdx.x + pid * (int)gridDim.x; tile < total_tiles && !*abort_flag; tile += n_prod * (int)gridDim.x, tc += n_prod) {
                 const int img = tw.img, p0 = tw.rt * p.nr;
@@ -845,7 +848,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
                         HTRACE(0, tc);
                         mbar_arrive_expect_tx(bar, (uint32_t)p.a_box_bytes);
                         if (!dep_waited) { grid_dependency_wait(); dep_waited = true; }
-                        if (!(p.test_skip && issued_a == 0))   // (test hook: the first stage never becomes full)
+                        if (issued_a >= skip_a)                // (test hook: the first stage never becomes full)
                             tma_load_4d(a_base + (uint32_t)sa * (uint32_t)p.a_alloc, &tmA, bar, kc * kKC, p.lo_w, p0 + p.lo_h, img);
                         ++issued_a;
                     }
