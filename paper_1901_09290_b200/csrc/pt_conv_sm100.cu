@@ -2039,6 +2039,11 @@ int pick_stages(size_t stage_bytes, int iters, size_t reserved, size_t *smem, si
 // Channel extent of an output tensor map: the channel count rounded up to a whole 32-byte sector where the pitch has room
 // for it (the pad lanes there receive zeros). A row whose last sector is only partly written costs a read-modify-write in
 // the memory system: measured 35 us against 20 us for 56x56x209..216 channels at pitch 224.
+// The operands of a weight gradient are loaded with the same extent: their channels are rows and columns of the result, so that whatever
+// a pad lane holds (a NaN too) stays in sums that are not stored, and the TMA unit's time for a row that ends inside a box depends on
+// where (ns per row with several issuing threads, box of 64 lanes: 64 channels 0.73, 57 to 63 1.03, 48 to 56 1.4 to 1.5, 41 to 47 1.6,
+// 33 to 40 3.4; of 32 lanes: 32 0.53, 25 to 31 1.0, 17 to 24 1.5). Weight gradients of 106 -> 103 3x3 at 28x28, batch 64 27.2 -> 24.1 us,
+// at 56x56 and stride 2 28.3 -> 25.2; 30 -> 33 at 56x56 22.8 -> 20.8; the 7x7 stem 3 -> 19, batch 256 156.9 -> 145.3.
 int store_cols(int cols, int ld)
 {
     const int up = pt_ceil_div(cols, 16) * 16;
@@ -2687,7 +2692,7 @@ pt_status run_wgrad(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const pt_wgr
     if (!c->encode_tiled) return PT_ERR_CUDA;
     CUtensorMap tmA;
     {
-        cuuint64_t dims[2] = {(cuuint64_t)d->K, (cuuint64_t)p.npix};
+        cuuint64_t dims[2] = {(cuuint64_t)store_cols(d->K, d->ldy), (cuuint64_t)p.npix};
         cuuint64_t strides[1] = {(cuuint64_t)d->ldy * 2};
         cuuint32_t box[2] = {64, 64}, estr[2] = {1, 1};
         CUresult r = ((EncodeTiledFn)c->encode_tiled)(&tmA, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(dy), dims, strides, box,
@@ -2728,8 +2733,9 @@ pt_status run_wgrad_rows(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const p
     p.lanes = wr.lanes; p.dy_lanes = wr.dy_lanes; p.acc_row = pt_ceil_div(d->S, 4); p.lane_shift = wr.lanes == 64 ? 6 : 5;
     const int gx = p.n_tiles * p.m_tiles * p.tap_groups;
     // dy: box of nr rows x Wp columns (Wp > Q: the extra columns are out of bounds and read as zeros); x: the halo box
-    if (!make_halo_in_map(c, &tmA, dy, d->K, Q, P, d->N, d->ldy, wr.Wp, wr.nr, wr.dy_lanes)) return PT_ERR_UNSUPPORTED;
-    if (!make_halo_in_map(c, &tmX, x, d->C, d->W, d->H, d->N, d->ldx, wr.Wp, wr.nr + d->R - 1, wr.lanes, x_row_pixels)) return PT_ERR_UNSUPPORTED;
+    if (!make_halo_in_map(c, &tmA, dy, store_cols(d->K, d->ldy), Q, P, d->N, d->ldy, wr.Wp, wr.nr, wr.dy_lanes)) return PT_ERR_UNSUPPORTED;
+    if (!make_halo_in_map(c, &tmX, x, x_row_pixels > 0 ? d->C : store_cols(d->C, d->ldx), d->W, d->H, d->N, d->ldx, wr.Wp, wr.nr + d->R - 1, wr.lanes, x_row_pixels))
+        return PT_ERR_UNSUPPORTED;
     dim3 grid((unsigned)gx, (unsigned)p.splits);
     const size_t smem = (p.splits > 1 && wr.smem < kSplitSmemFloor) ? kSplitSmemFloor : wr.smem;
     p.data_bytes = (unsigned)(smem - 2048);
@@ -2948,8 +2954,8 @@ pt_status pt_sm100_conv(pt_ctx *c, const pt_conv_desc *d, int which, const void 
         const int up_w = (Q - 1) * d->stride - d->pad - (d->W - 1), up_h = (P - 1) * d->stride - d->pad - (d->H - 1);
         const bool plain = d->R == 1 && d->S == 1 && d->stride == 1 && d->pad == 0;     // pixels of x and dy coincide
         if (plain) {
-            if (!make_act2d_map(c, &tmX, a, d->C, (long long)d->N * d->H * d->W, d->ldx, 64)) return PT_ERR_CUDA;
-        } else if (!make_im2col_map(c, &tmX, a, d->C, d->W, d->H, d->N, d->ldx, -d->pad, -d->pad, up_w, up_h, d->stride, 64)) return PT_ERR_CUDA;
+            if (!make_act2d_map(c, &tmX, a, store_cols(d->C, d->ldx), (long long)d->N * d->H * d->W, d->ldx, 64)) return PT_ERR_CUDA;
+        } else if (!make_im2col_map(c, &tmX, a, store_cols(d->C, d->ldx), d->W, d->H, d->N, d->ldx, -d->pad, -d->pad, up_w, up_h, d->stride, 64)) return PT_ERR_CUDA;
         return run_wgrad(c, d, P, Q, w, d->stride, -d->pad, -d->pad, tmX, b, (float *)out, ws, ws_bytes, st, plain);
     }
 

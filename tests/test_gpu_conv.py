@@ -154,6 +154,21 @@ def test_pad_lanes_up_to_a_multiple_of_16_are_zero(shape):
     assert torch.all(y[..., K:] == 0) and torch.all(dx[..., C:] == 0)
 
 
+# (N, H, W, C, K, R, stride, extra pitch of x, of dy): the weight gradient loads pad lanes (here NaN) up to a multiple of 16 channels where
+# the pitch has them, up to a multiple of 8 where not; both kernels, the space-to-depth stem
+@pytest.mark.parametrize("shape", [(3, 12, 12, 19, 33, 3, 1, 8, 8), (3, 12, 12, 33, 19, 3, 1, 0, 16), (2, 14, 14, 70, 103, 3, 1, 8, 0),
+                                   (2, 16, 16, 106, 41, 3, 2, 16, 32), (2, 10, 10, 130, 300, 1, 1, 24, 8), (2, 32, 32, 3, 19, 7, 2, 0, 8)])
+def test_weight_gradient_of_nan_pad_lanes(shape):
+    N, H, Wd, C, K, R, stride, ex, ey = shape
+    x, w, dy, pad = _case(N, H, Wd, C, K, R, stride, seed=W.BASE_SEED + 29)
+    d = B.make_conv_desc(N, H, Wd, C, K, R, R, stride, pad, W.pad8(C) + ex, W.pad8(K) + ey, W.pad8(C), 0, 2)
+    dw = torch.full((K, R, R, C), 7680.0, device="cuda")
+    B.pt_conv_wgrad(Hh.ctx(), d, Hh.to_dev_padded(x, d.ldx), Hh.to_dev_padded(dy, d.ldy), dw, Hh.conv_ws(d, B.PT_CONV_WGRAD))
+    torch.cuda.synchronize()
+    Hh.ctx().poll()
+    Hh.check_conv(dw, C, oracle.conv_wgrad(x.numpy(), dy.numpy(), R, R, stride, pad), what="wgrad")
+
+
 def test_wgrad_is_run_to_run_identical():
     N, H, C, K, R = 4, 14, 27, 19, 3
     x, w, dy, pad = _case(N, H, H, C, K, R, 1, W.BASE_SEED + 5)
