@@ -1160,8 +1160,8 @@ struct WgradP {
     unsigned data_bytes;    // shared memory behind the control block: the stages, and what the exchange of the splits may use
     float *out;             // dw
     int test_skip;          // test hook (pt_test_skip_next_arrive): split 0 does not announce its partial tile
-    float *partial;         // splits > 1: workspace [blockIdx.x][tap in group][split][128][BN] fp32
-    unsigned int *sync;     // splits > 1: two zeroed counters per blockIdx.x (arrived, reduced); left zero again at exit
+    float *partial;         // splits > 1: workspace [blockIdx.x][split], room for the accumulators of 128 x acc_cols floats (WgradShare)
+    unsigned int *sync;     // splits > 1: two zeroed counters per blockIdx.x (arrived, seen by); left zero again at exit
     unsigned int *status;
 };
 
@@ -1278,11 +1278,40 @@ __device__ __forceinline__ void wgrad_cluster_sum(const WgradP &p, Ctl *ctl, uin
     }
 }
 
+// A split's partial sums of a tile in the workspace: 16-byte pieces [accumulator][four columns][row], the rows and columns that are part of
+// dw only (not the output channels past K; in the paired form not the channel lanes past C), so that a warp, whose lanes hold a row each
+// when they read the tensor memory, stores 512 consecutive bytes at a time, and a CTA's share of the sum is one run of every
+// split's pieces. (As 32 x 32 boxes through staging and TMA stores the 172 KB of three accumulators of 112 columns took 4.1 us to store,
+// and 4.4 us to read back and sum; 2.2 and 2.9 this way. 418 -> 111 1x1 at 28x28, batch 64 21.8 -> 20.5 us a launch, 69 -> 418 19.8 -> 16.9,
+// 8 -> 14 3x3 at 32x32, batch 128 16.6 -> 14.1; at a limit of 49 CTAs 112 -> 111 3x3/2 at 56x56 54.4 -> 50.8.)
+struct WgradShare {
+    int lanes_used, rows, quads;
+    __device__ __forceinline__ WgradShare(const WgradP &p, int k0, int c0, int acc_cols)
+    {
+        const int groups = !p.pair ? 1 : p.lanes == 32 ? min(4, p.S) : 2;       // taps of an accumulator
+        rows = !p.pair ? min(128, p.K - k0) : groups * p.C;
+        lanes_used = !p.pair ? rows : groups << p.lane_shift;
+        quads = pt_ceil_div_dev(p.pair ? p.K : min(acc_cols, p.C - c0), 4);
+    }
+    // the row of a TMEM lane; -1: none
+    __device__ __forceinline__ int row(const WgradP &p, int l) const
+    {
+        if (!p.pair) return l < rows ? l : -1;
+        const int g = l >> p.lane_shift, c = l & (p.lanes - 1);
+        return l < lanes_used && c < p.C ? g * p.C + c : -1;
+    }
+    // where a split's pieces start, in floats (room for whole accumulators)
+    __device__ __forceinline__ size_t split_off(const WgradP &p, int split, int acc_cols) const
+    {
+        return ((size_t)blockIdx.x * p.splits + split) * (size_t)p.apc * 128 * acc_cols;
+    }
+};
+
 // Everything after the main loop of a weight-gradient kernel: the accumulators leave TMEM (directly to dw, or as this
 // split's partial tile), the splits of a tile meet, and every CTA sums its share of the tile over the splits.
 // `ring_bytes` of shared memory at `data_base` are free by then and serve as staging. `tap0` is the CTA's first tap (generic form) or
 // accumulator (row-block form).
-__device__ __forceinline__ void wgrad_finish(const WgradP &p, const CUtensorMap &tmP, Ctl *ctl, uint32_t data_base, uint32_t tmem_base,
+__device__ __forceinline__ void wgrad_finish(const WgradP &p, Ctl *ctl, uint32_t data_base, uint32_t tmem_base,
                                              int tap0, int k0, int c0, int split, int iters, uint32_t ring_bytes, int n_acc, int acc_cols)
 {
     volatile int *abort_flag = &ctl->abort_flag;
@@ -1300,41 +1329,31 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, const CUtensorMap 
             if (p.cluster) {
                 // the exchange is below: every thread of the cluster takes part in its barriers
             } else if (p.splits > 1) {
-                // ---- (1) this CTA's fp32 partial tile goes to the workspace through swizzled staging + TMA stores (the rows that
-                // hold something: not the output channels past K, in the paired form not the channel lanes past C)
+                // ---- (1) this CTA's partial sums go to the workspace straight from the registers (WgradShare: a lane's 16 bytes lie beside
+                // its neighbour's, 512 bytes a store)
+                const WgradShare sh(p, k0, c0, acc_cols);
                 const int gtid = (warp - 1) * 32 + lane;
-                const bool rows_used = !p.pair ? k0 + quarter * 32 < p.K : p.lanes == 64 || quarter < p.S;
-                int sl = 0, ci = 0;
-                for (int tt = 0; tt < n_acc && rows_used; ++tt)
+                const int row = sh.row(p, quarter * 32 + lane);
+                float *const dst = p.partial + sh.split_off(p, split, acc_cols);
+                int ci = 0;
+                for (int tt = 0; tt < n_acc && quarter * 32 < sh.lanes_used; ++tt)
                 for (int cc = 0; cc < acc_cols; cc += 32, ++ci) {
                     if ((ci & 1) != wset) continue;
-                    sl ^= 1;
-                    const uint32_t slab = data_base + (uint32_t)((wset * 4 + quarter) * 2 + sl) * 4096u;
-                    if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
-                    __syncwarp();
                     uint32_t v[32];
                     wgrad_load32(lane_addr + (uint32_t)(tt * acc_cols + cc), cc + 16 < acc_cols, iters > 0, v);
+                    float4 *const d4 = reinterpret_cast<float4 *>(dst) + (size_t)(tt * sh.quads + cc / 4) * sh.rows + row;
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const uint32_t addr = slab + (uint32_t)lane * 128u + (((uint32_t)j ^ ((uint32_t)lane & 7u)) << 4);
-                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v[4 * j]), "r"(v[4 * j + 1]), "r"(v[4 * j + 2]),
-                                     "r"(v[4 * j + 3])
-                                     : "memory");
-                    }
-                    fence_proxy_async();
-                    __syncwarp();
-                    if (lane == 0) {
-                        tma_store_2d(&tmP, slab, cc, (((int)blockIdx.x * p.apc + tt) * p.splits + split) * 128 + quarter * 32);
-                        tma_store_commit();
-                    }
+                    for (int j = 0; j < 8; ++j)
+                        if (row >= 0 && cc / 4 + j < sh.quads)
+                            __stcg(d4 + (size_t)j * sh.rows, make_float4(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1]),
+                                                                         __uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3])));
                 }
-                if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");      // the writes have completed
-                __threadfence();
                 if (warp == 2) WTRACE(4);
                 named_barrier(1, 256);
                 // ---- (2) every split CTA of this tile is resident (the grid is at most one CTA per SM): wait for all of them
                 unsigned int *arrived = p.sync + 2 * blockIdx.x;
                 if (gtid == 0) {
+                    __threadfence();                             // the CTA's stores (ordered before this by the barrier), then its arrival
                     // (test hook: split 0 stays silent, so that every split of the tile runs into the bounded wait below)
                     if (!(p.test_skip && split == 0)) atomicAdd(arrived, 1u);
                     const uint64_t t0 = globaltimer_ns();
@@ -1347,6 +1366,11 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, const CUtensorMap 
                             *abort_flag = 1;
                             break;
                         }
+                    }
+                    // the last CTA to see that all have arrived clears the counters (nobody looks at them again)
+                    if (seen >= (unsigned)p.splits && atomicAdd(arrived + 1, 1u) == (unsigned)p.splits - 1u) {
+                        arrived[0] = 0u;
+                        arrived[1] = 0u;
                     }
                 }
                 named_barrier(1, 256);
@@ -1419,65 +1443,46 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, const CUtensorMap 
     }
     __syncthreads();
     if (p.splits > 1 && !*abort_flag) {
-        // ---- (3) all threads: this CTA sums its share of the tile's elements over the splits
-        __threadfence();
-        // Work items are (tap, row, 4-column group) of the real rows of the CTA's tiles, dealt out evenly to the split CTAs.
-        // The partial tiles sit in L2; what costs time is a chain of dependent loads, so every thread first issues the
-        // asynchronous 16-byte copies of its items for ALL splits into the (now idle) stage memory, and only then are the
-        // copies summed from shared memory in ascending split order: deterministic, whichever CTA does the work.
-        // (Consecutive items run along a row in both forms: the partial tiles are then read whole sectors at a time. In the paired form
-        // that scatters the writes to dw, but there are as many partial tiles to read as splits: 33 -> 31 us for 46 -> 59 at 56x56.)
-        const int rows_real = !p.pair ? min(128, p.K - k0) : (p.lanes == 32 ? min(4, p.S) : 2) * p.C;
-        const int ngrp = pt_ceil_div_dev(p.pair ? p.K : min(acc_cols, p.C - c0), 4);     // float4 groups per row
-        const int items = rows_real * ngrp;
-        const int total = n_acc * items;
-        const int per_cta = (total + p.splits - 1) / p.splits;
+        // ---- (3) all threads: this CTA sums its share of the tile's 16-byte pieces over the splits. The partial sums sit in L2 and what costs
+        // time is a chain of dependent loads, so the asynchronous copies of the whole share, a run of every split's pieces, go out first, into
+        // the (now idle) stage memory; the copies are then summed from there in ascending split order: deterministic, whichever CTA
+        // does the work.
+        const WgradShare sh(p, k0, c0, acc_cols);
+        const int total = n_acc * sh.quads * sh.rows, per_cta = (total + p.splits - 1) / p.splits;
         const int it_beg = split * per_cta, it_end = min(total, it_beg + per_cta);
-        const size_t zstride = (size_t)128 * acc_cols;
-        const float *pbase = p.partial + (size_t)blockIdx.x * p.apc * p.splits * zstride;
-        const int cap = (int)(((size_t)ring_bytes) / ((size_t)p.splits * 16));   // items the stage memory holds
-        const float inv_items = 1.0f / (float)items, inv_ngrp = 1.0f / (float)ngrp;
-        // row of the partial tile and first column of an item
-        auto place = [&](int item, int &r, int &col) {
-            if (p.pair) {
-                const int rr = fast_div(item, ngrp, inv_ngrp);
-                const int gq = item - rr * ngrp;
-                const int g = (rr >= p.C ? 1 : 0) + (rr >= 2 * p.C ? 1 : 0) + (rr >= 3 * p.C ? 1 : 0);
-                r = (g << p.lane_shift) + rr - g * p.C;
-                col = gq * 4;
-            } else {
-                r = fast_div(item, ngrp, inv_ngrp);
-                col = (item - r * ngrp) * 4;
-            }
-        };
+        const float4 *const pbase = reinterpret_cast<const float4 *>(p.partial + sh.split_off(p, 0, acc_cols));
+        const size_t zstride = (size_t)p.apc * acc_cols * 32;                    // in pieces
+        const int cap = (int)(ring_bytes / ((uint32_t)p.splits * 16u));         // pieces the stage memory holds
+        const float inv_rows = 1.0f / (float)sh.rows, inv_quads = 1.0f / (float)sh.quads;
         for (int c_beg = it_beg; c_beg < it_end; c_beg += cap) {
             const int n_chunk = min(cap, it_end - c_beg);
-            for (int i = threadIdx.x; i < n_chunk; i += kThreads) {
-                const int idx = c_beg + i, tt = fast_div(idx, items, inv_items), item = idx - tt * items;
-                int r, col;
-                place(item, r, col);
-                const float *src = pbase + (size_t)tt * p.splits * zstride + (size_t)r * acc_cols + col;
-                uint32_t dst = data_base + (uint32_t)i * 16u;
-                for (int z = 0; z < p.splits; ++z, src += zstride, dst += (uint32_t)n_chunk * 16u)
-                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+            // copies are dealt out evenly: piece i of split z, i fastest
+            int z = threadIdx.x / n_chunk, i = threadIdx.x - z * n_chunk;
+            const int dz = kThreads / n_chunk, di = kThreads - dz * n_chunk;
+            while (z < p.splits) {
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
+                             ::"r"(data_base + (uint32_t)(z * n_chunk + i) * 16u), "l"(pbase + (size_t)z * zstride + c_beg + i) : "memory");
+                z += dz; i += di;
+                if (i >= n_chunk) { i -= n_chunk; ++z; }
             }
             asm volatile("cp.async.wait_all;" ::: "memory");
             __syncthreads();
-            for (int i = threadIdx.x; i < n_chunk; i += kThreads) {
-                const int idx = c_beg + i, tt = fast_div(idx, items, inv_items), item = idx - tt * items;
-                int r, col;
-                place(item, r, col);
+            for (int k = threadIdx.x; k < n_chunk; k += kThreads) {
                 float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
-                uint32_t a = data_base + (uint32_t)i * 16u;
-                for (int z = 0; z < p.splits; ++z, a += (uint32_t)n_chunk * 16u) {
+                uint32_t a = data_base + (uint32_t)k * 16u;
+#pragma unroll 4
+                for (int y = 0; y < p.splits; ++y, a += (uint32_t)n_chunk * 16u) {
                     float4 t;
                     asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(t.x), "=f"(t.y), "=f"(t.z), "=f"(t.w) : "r"(a) : "memory");
                     sum.x += t.x; sum.y += t.y; sum.z += t.z; sum.w += t.w;
                 }
+                const int piece = c_beg + k, tq = fast_div(piece, sh.rows, inv_rows), row = piece - tq * sh.rows;
+                const int tt = fast_div(tq, sh.quads, inv_quads), col = (tq - tt * sh.quads) * 4;
                 if (p.pair) {
-                    // row = (tap of the accumulator, input channel), columns = output channels
-                    const int tap = wgrad_tap(p, tap0 + tt, r >> p.lane_shift), c = r & (p.lanes - 1);
-                    if (c < p.C && tap < p.taps) {
+                    // row = (tap of the accumulator, input channel), columns = output channels: consecutive threads, consecutive floats
+                    const int g = (row >= p.C ? 1 : 0) + (row >= 2 * p.C ? 1 : 0) + (row >= 3 * p.C ? 1 : 0);
+                    const int tap = wgrad_tap(p, tap0 + tt, g), c = row - g * p.C;
+                    if (tap < p.taps) {
                         const float v4[4] = {sum.x, sum.y, sum.z, sum.w};
 #pragma unroll
                         for (int e = 0; e < 4; ++e)
@@ -1485,27 +1490,16 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, const CUtensorMap 
                     }
                     continue;
                 }
-                wgrad_store4(p.out + ((size_t)(k0 + r) * p.taps + tap0 + tt) * p.C + c0 + col, sum, min(4, p.C - (c0 + col)));
+                wgrad_store4(p.out + ((size_t)(k0 + row) * p.taps + tap0 + tt) * p.C + c0 + col, sum, min(4, p.C - (c0 + col)));
             }
             __syncthreads();
         }
-        __syncthreads();
         if (threadIdx.x == 0) WTRACE(6);
-        if (threadIdx.x == 0) {
-            unsigned int *arrived = p.sync + 2 * blockIdx.x, *reduced = arrived + 1;
-            __threadfence();
-            if (atomicAdd(reduced, 1u) == (unsigned)p.splits - 1u) {          // last one out clears the counters
-                *arrived = 0u;
-                *reduced = 0u;
-                __threadfence();
-            }
-        }
     }
 }
 
 __global__ void __launch_bounds__(kThreads, 1) conv_wgrad_kernel(const __grid_constant__ CUtensorMap tmDy,
-                                                              const __grid_constant__ CUtensorMap tmX,
-                                                              const __grid_constant__ CUtensorMap tmP, const WgradP p)
+                                                              const __grid_constant__ CUtensorMap tmX, const WgradP p)
 {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     Ctl *ctl = reinterpret_cast<Ctl *>(smem_raw);
@@ -1651,7 +1645,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_wgrad_kernel(const __grid_co
         if (ok) umma_commit_lead(smem_u32(&ctl->accum), leader);
         if (warp == 1) WTRACE(2);
     }
-    wgrad_finish(p, tmP, ctl, data_base, tmem_base, tap0, k0, c0, split, iters, p.data_bytes, ntap, p.BN);
+    wgrad_finish(p, ctl, data_base, tmem_base, tap0, k0, c0, split, iters, p.data_bytes, ntap, p.BN);
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem_base, (uint32_t)p.tmem_cols);
@@ -1674,8 +1668,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_wgrad_kernel(const __grid_co
 // for a 3x3 filter. The MMAs (29 ns each however narrow) and the TMA unit's time per row bound the narrow layers, and a 64-byte
 // row that ends inside a sector takes it 3.1 ns instead of 4.5.
 __global__ void __launch_bounds__(kThreads, 1) conv_wgrad_rows_kernel(const __grid_constant__ CUtensorMap tmDy,
-                                                                   const __grid_constant__ CUtensorMap tmX,
-                                                                   const __grid_constant__ CUtensorMap tmP, const WgradP p)
+                                                                   const __grid_constant__ CUtensorMap tmX, const WgradP p)
 {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     Ctl *ctl = reinterpret_cast<Ctl *>(smem_raw);
@@ -1810,7 +1803,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_wgrad_rows_kernel(const __gr
         if (ok) umma_commit_lead(smem_u32(&ctl->accum), leader);
         if (warp == 1) WTRACE(2);
     }
-    wgrad_finish(p, tmP, ctl, data_base, tmem_base, acc0, k0, c0, split, iters, p.data_bytes, n_acc, p.acc_cols);
+    wgrad_finish(p, ctl, data_base, tmem_base, acc0, k0, c0, split, iters, p.data_bytes, n_acc, p.acc_cols);
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem_base, (uint32_t)p.tmem_cols);
@@ -2579,23 +2572,11 @@ size_t wgrad_workspace_bound(const pt_ctx *c, const pt_conv_desc *d, int P, int 
     return (size_t)tiles128 * 128 * w.acc_cols * sizeof(float);
 }
 
-// The splits' fp32 partial tiles as a 2-D tensor (BN columns, rows): box 32 x 32, 128-byte swizzle.
-bool make_partial_map(const pt_ctx *c, CUtensorMap *tm, void *ws, int bn, size_t rows)
-{
-    if (!c->encode_tiled) return false;
-    cuuint64_t dims[2] = {(cuuint64_t)bn, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {(cuuint64_t)bn * 4};
-    cuuint32_t box[2] = {32, 32}, estr[2] = {1, 1};
-    CUresult r = ((EncodeTiledFn)c->encode_tiled)(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, ws, dims, strides, box, estr,
-                                                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                                                  CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return map_ok(r, __LINE__);
-}
-
 // Launch of a weight-gradient kernel: with programmatic stream serialization and, where the splits of a tile meet in shared memory,
 // as clusters of `cluster` CTAs along y.
-cudaError_t launch_wgrad(void (*kernel)(CUtensorMap, CUtensorMap, CUtensorMap, WgradP), dim3 grid, int cluster, size_t smem, cudaStream_t st,
-                         const CUtensorMap &a, const CUtensorMap &b, const CUtensorMap &q, const WgradP &p)
+template <typename XMaps>
+cudaError_t launch_wgrad(void (*kernel)(CUtensorMap, XMaps, WgradP), dim3 grid, int cluster, size_t smem, cudaStream_t st,
+                         const CUtensorMap &a, const XMaps &b, const WgradP &p)
 {
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
@@ -2606,7 +2587,7 @@ cudaError_t launch_wgrad(void (*kernel)(CUtensorMap, CUtensorMap, CUtensorMap, W
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = 1; attr[1].val.clusterDim.y = (unsigned)cluster; attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr; cfg.numAttrs = cluster > 1 ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, kernel, a, b, q, p);
+    return cudaLaunchKernelEx(&cfg, kernel, a, b, p);
 }
 
 pt_status wgrad_attr(const pt_ctx *c)
@@ -2646,8 +2627,7 @@ int wg_max_clusters(const pt_ctx *c, int size)
 }
 
 // What both forms have in common: tiles, splits and where the partial tiles go.
-pt_status wgrad_common(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const pt_wgrad_plan &w, float *out, void *ws, size_t ws_bytes, WgradP *p,
-                       CUtensorMap *tmP)
+pt_status wgrad_common(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const pt_wgrad_plan &w, float *out, void *ws, size_t ws_bytes, WgradP *p)
 {
     memset(p, 0, sizeof(*p));
     p->K = d->K; p->C = d->C; p->taps = d->R * d->S; p->S = d->S;
@@ -2659,7 +2639,6 @@ pt_status wgrad_common(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const pt_
     p->tmem_cols = pow2_cols(w.apc * w.acc_cols);
     p->status = c->d_status;
     p->out = out;
-    memset(tmP, 0, sizeof(*tmP));
     if (c->test_skip == 1 && p->splits > 1) { p->test_skip = 1; p->cluster = 0; c->test_skip = 0; }
     if (p->splits > 1 && !p->cluster) {
         const int gx = p->n_tiles * p->m_tiles * p->tap_groups;
@@ -2671,7 +2650,6 @@ pt_status wgrad_common(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const pt_
         if (c->sync_next + 2 * gx > 16384) c->sync_next = 0;
         p->sync = c->d_sync + c->sync_next;
         c->sync_next += 2 * gx;
-        if (!make_partial_map(c, tmP, ws, w.acc_cols, (size_t)gx * w.apc * w.splits * 128)) return PT_ERR_CUDA;
     }
     return wgrad_attr(c);
 }
@@ -2681,8 +2659,7 @@ pt_status run_wgrad(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const pt_wgr
                     const void *dy, float *out, void *ws, size_t ws_bytes, cudaStream_t st, bool x_tiled = false)
 {
     WgradP p;
-    CUtensorMap tmP;
-    const pt_status r0 = wgrad_common(c, d, P, Q, w, out, ws, ws_bytes, &p, &tmP);
+    const pt_status r0 = wgrad_common(c, d, P, Q, w, out, ws, ws_bytes, &p);
     if (r0 != PT_OK) return r0;
     p.x_tiled = x_tiled ? 1 : 0;
     p.pix_per_split = pt_ceil_div(pt_ceil_div(p.npix, p.splits), 64) * 64;
@@ -2707,7 +2684,7 @@ pt_status run_wgrad(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const pt_wgr
     if (p.splits > 1 && smem < kSplitSmemFloor) smem = kSplitSmemFloor;
     dim3 grid((unsigned)gx, (unsigned)p.splits);
     p.data_bytes = (unsigned)(smem - 2048);
-    PT_CUDA_OK(launch_wgrad(conv_wgrad_kernel, grid, p.cluster ? p.splits : 1, smem, st, tmA, tmX, tmP, p));
+    PT_CUDA_OK(launch_wgrad(conv_wgrad_kernel, grid, p.cluster ? p.splits : 1, smem, st, tmA, tmX, p));
     c->launches += 1;
     PT_CUDA_OK(cudaGetLastError());
     return PT_OK;
@@ -2721,8 +2698,8 @@ pt_status run_wgrad_rows(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const p
 {
     if (!c->encode_tiled) return PT_ERR_CUDA;
     WgradP p;
-    CUtensorMap tmP, tmA, tmX;
-    const pt_status r0 = wgrad_common(c, d, P, Q, wr, out, ws, ws_bytes, &p, &tmP);
+    CUtensorMap tmA, tmX;
+    const pt_status r0 = wgrad_common(c, d, P, Q, wr, out, ws, ws_bytes, &p);
     if (r0 != PT_OK) return r0;
     p.pair = 1;
     p.stride = 1; p.lo_h = -d->pad; p.lo_w = -d->pad;
@@ -2739,7 +2716,7 @@ pt_status run_wgrad_rows(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const p
     dim3 grid((unsigned)gx, (unsigned)p.splits);
     const size_t smem = (p.splits > 1 && wr.smem < kSplitSmemFloor) ? kSplitSmemFloor : wr.smem;
     p.data_bytes = (unsigned)(smem - 2048);
-    PT_CUDA_OK(launch_wgrad(conv_wgrad_rows_kernel, grid, p.cluster ? p.splits : 1, smem, st, tmA, tmX, tmP, p));
+    PT_CUDA_OK(launch_wgrad(conv_wgrad_rows_kernel, grid, p.cluster ? p.splits : 1, smem, st, tmA, tmX, p));
     c->launches += 1;
     PT_CUDA_OK(cudaGetLastError());
     return PT_OK;
