@@ -1130,6 +1130,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
 //   With more than one split every CTA TMA-stores its fp32 partial tile to the workspace, announces it on a counter,
 //   waits (bounded) until all splits of its tile have arrived, and then sums its share of the tile's rows over the
 //   splits in ascending order: deterministic, and no second kernel.
+constexpr int kMaxRow = 8;  // filter rows and columns of the filter-row form
 struct WgradP {
     int K, C, taps;         // true channel counts, number of taps (R*S)
     int BN, n_tiles;        // input-channel tile
@@ -1153,6 +1154,13 @@ struct WgradP {
     int lanes, dy_lanes;    // row-block form: channel lanes per staged pixel of x and of dy (rows of 128 or 64 bytes)
     int lane_shift;         // log2 of `lanes`
     int acc_row;            // 32 lanes: accumulators per filter row, ceil(S / 4): each holds four neighbouring taps
+    // filter-row form: the taps of one filter row share a unit; a tap is plane tap_plane[s] of the unit's x rows (stride 2: the columns of
+    // either parity are a plane each), tap_shift[s] pixels on
+    int planes;
+    int plane_lo[2];                                    // first column of a unit's rows in either plane
+    unsigned char tap_plane[kMaxRow], tap_shift[kMaxRow];
+    unsigned char row_par[kMaxRow];                     // filter row -> parity of the x rows it reads
+    signed char row_off[kMaxRow];                       //               and their offset from the output row
     int cluster;            // 1: the splits of a tile are one thread-block cluster and meet in shared memory (no workspace)
     int apc;                // accumulators per CTA (= tpc in the generic form)
     int acc_cols;           // columns of one accumulator (= BN, or the padded K in the paired form)
@@ -1810,6 +1818,145 @@ __global__ void __launch_bounds__(kThreads, 1) conv_wgrad_rows_kernel(const __gr
     }
 }
 
+// Filter-row form of the weight gradient: filters of several columns at stride 1 (where the row-block form does not apply: more than 64
+// input channels) or 2. A CTA has one filter row: a unit is `nr` output rows of one image, dy as a box of nr x Wp pixels (columns past Q
+// and rows past P zero-filled) and the x rows that filter row reads, as a box of the same size; at stride 2 the columns of either parity
+// are a box each (every other pixel: a tensor map of its own). The taps of the row are the same staged pixels one pixel apart, read
+// through descriptors that start that many 128-byte rows further on, and have an accumulator each. Against the generic kernel, which loads a
+// 64-pixel x tile per tap and reloads dy for every two taps or so: 33 KB instead of 72 KB per 64 pixels and three taps at stride 1
+// (106 -> 103 channels, 48 against 72 at stride 2). What an SM can pull from L2, 130 to 140 GB/s, bounded that kernel; this one's matrix
+// instructions (N = 112: 60 cycles) take as long as its loads.
+struct TapMaps { CUtensorMap m[4]; };        // x: [row parity * 2 + column parity]; at stride 1 the first only
+
+__global__ void __launch_bounds__(kThreads, 1) conv_wgrad_taps_kernel(const __grid_constant__ CUtensorMap tmDy, const __grid_constant__ TapMaps tmX, const WgradP p)
+{
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    Ctl *ctl = reinterpret_cast<Ctl *>(smem_raw);
+    const uint32_t smem_base = smem_u32(smem_raw);
+    const uint32_t data_base = (smem_base + (uint32_t)sizeof(Ctl) + 1023u) & ~1023u;
+    const uint32_t nb_b = (uint32_t)((p.BN + 63) / 64), x_boxes = (uint32_t)p.planes * nb_b;
+    const uint32_t a_bytes = (uint32_t)p.nb_a * p.a_box, stage_bytes = a_bytes + x_boxes * p.b_box;
+    volatile int *abort_flag = &ctl->abort_flag;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int bx = blockIdx.x;
+    const int n_tile = bx % p.n_tiles; bx /= p.n_tiles;
+    const int m_tile = bx % p.m_tiles; bx /= p.m_tiles;
+    const int r = bx;                                                 // this CTA's filter row
+    const int split = blockIdx.y;
+    const int k0 = m_tile * 128, c0 = n_tile * p.BN;
+    const int u_beg = split * p.units_per_split;
+    const int u_end = min(p.units, u_beg + p.units_per_split);
+    const int iters = u_end > u_beg ? u_end - u_beg : 0;
+    const uint32_t box_bytes = (uint32_t)(p.nr * p.Wp) * 128u;
+    // blocks of 64 channels that exist: what an accumulator's other rows and columns hold is not stored, so they are not loaded
+    const int n_dy = min(p.nb_a, pt_ceil_div_dev(p.K - k0, 64)), n_xb = min((int)nb_b, pt_ceil_div_dev(p.C - c0, 64)), n_x = p.planes * n_xb;
+    const int NXP = n_x < 4 ? n_x : 4;                                // x producer warps in use
+    const int NI = p.S < 4 ? p.S : 4;                                 // MMA issuer warps in use: taps i, i + NI, ... of the row
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < p.stages; ++s) {
+            mbar_init(smem_u32(&ctl->full[s]), 1u + (uint32_t)NXP);
+            mbar_init(smem_u32(&ctl->empty[s]), (uint32_t)NI);
+        }
+        mbar_init(smem_u32(&ctl->accum), (uint32_t)NI);
+        ctl->abort_flag = 0;
+        fence_mbar_init();
+        prefetch_tmap(&tmDy);
+        prefetch_tmap(&tmX.m[p.row_par[r] * 2]);
+        if (p.planes > 1) prefetch_tmap(&tmX.m[p.row_par[r] * 2 + 1]);
+    }
+    // rows past the end of a box, up to the last 16-pixel step and the largest shift: dy zeros, x times zero and must be finite
+    {
+        const uint32_t a_rest = (p.a_box - box_bytes) / 16u, b_rest = (p.b_box - box_bytes) / 16u;
+        const uint32_t a_all = (uint32_t)p.nb_a * a_rest, per_stage = a_all + x_boxes * b_rest;
+        for (uint32_t i = threadIdx.x; i < (uint32_t)p.stages * per_stage; i += kThreads) {
+            const uint32_t st = i / per_stage, o = i - st * per_stage;
+            const uint32_t at = o < a_all ? o / a_rest * p.a_box + o % a_rest * 16u : a_bytes + (o - a_all) / b_rest * p.b_box + (o - a_all) % b_rest * 16u;
+            asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(data_base + st * stage_bytes + at + box_bytes), "r"(0u) : "memory");
+        }
+    }
+    fence_proxy_async();
+    if (warp == 1) {
+        tmem_alloc(smem_u32(&ctl->tmem_base), (uint32_t)p.tmem_cols);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = ctl->tmem_base;
+    const int issuer = warp == 1 ? 0 : warp - 5;                      // warps 6, 7, 8 -> issuers 1, 2, 3
+    // nothing above touches global memory; the producer threads wait after their set-up
+    if (!((warp == 0 || (warp >= 2 && warp < 2 + NXP)) && lane == 0)) grid_dependency_wait();
+    grid_launch_dependents();
+    if (threadIdx.x == 0) WTRACE(0);
+
+    if (warp == 0 || (warp >= 2 && warp < 2 + NXP)) {
+        if (lane == 0) {
+            // ---------------- producers: warp 0 brings the dy boxes of every unit, warp 2 + j the x boxes j, j + 4, ...
+            const bool is_dy = warp == 0;
+            const int xp = warp - 2;
+            const uint32_t my_bytes = (uint32_t)(is_dy ? n_dy : (n_x - xp + 3) / 4) * box_bytes;
+            const int row0 = p.row_off[r];
+            int n = u_beg / p.RB, rb = u_beg - n * p.RB;
+            int s = 0, ph = 0, issued = 0;
+            grid_dependency_wait();
+            for (int it = 0; it < iters; ++it) {
+                if (!mbar_wait(smem_u32(&ctl->empty[s]), ph ^ 1, abort_flag, p.status, 4)) break;
+                const uint32_t bar = smem_u32(&ctl->full[s]);
+                const uint32_t a_dst = data_base + (uint32_t)s * stage_bytes, b_dst = a_dst + a_bytes;
+                mbar_arrive_expect_tx(bar, my_bytes);
+                const int p0 = rb * p.nr;
+                if (is_dy) {
+                    for (int b = 0; b < n_dy; ++b) tma_load_4d(a_dst + (uint32_t)b * p.a_box, &tmDy, bar, k0 + b * 64, 0, p0, n);
+                } else {
+                    for (int j = xp; j < n_x; j += 4) {
+                        const int pl = j >= n_xb ? 1 : 0, b = j - pl * n_xb;
+                        tma_load_4d(b_dst + ((uint32_t)pl * nb_b + (uint32_t)b) * p.b_box, &tmX.m[p.row_par[r] * 2 + pl], bar, c0 + b * 64, p.plane_lo[pl],
+                                    p0 + row0, n);
+                    }
+                }
+                if (++rb == p.RB) { rb = 0; ++n; }
+                issued = it + 1;
+                if (++s == p.stages) { s = 0; ph ^= 1; }
+            }
+            if (*abort_flag) drain_ring(smem_u32(&ctl->full[0]), p.stages, issued);
+        }
+        __syncwarp();
+    }
+    if (warp == 1 || (warp >= 6 && issuer < NI)) {
+        // ---------------- MMA issuer `issuer`: the warp walks the loop in lockstep, lane 0 issues
+        const uint32_t leader = lane == 0 ? 1u : 0u;
+        const uint32_t idesc = make_idesc_bf16(128, p.BN, 1, 1);
+        bool ok = true;
+        int s = 0, ph = 0;
+        for (int it = 0; it < iters && ok; ++it) {
+            ok = mbar_wait(smem_u32(&ctl->full[s]), ph, abort_flag, p.status, 5);
+            if (!ok) break;
+            if (it == 0 && warp == 1) WTRACE(1);
+            tc_fence_after();
+            const uint32_t a_src = data_base + (uint32_t)s * stage_bytes, b_src = a_src + a_bytes;
+            const uint64_t ad = make_desc(a_src, p.a_box, 1024u);
+            const uint32_t acc = it != 0 ? 1u : 0u;
+            for (int t = issuer; t < p.S; t += NI) {
+                const uint64_t bd = make_desc(b_src + (uint32_t)p.tap_plane[t] * nb_b * p.b_box + (uint32_t)p.tap_shift[t] * 128u, p.b_box, 1024u);
+                const uint32_t d_tmem = tmem_base + (uint32_t)(t * p.BN);
+                umma_bf16_lead(d_tmem, ad, bd, idesc, acc, leader);
+                for (int k = 1; k < p.ksteps; ++k) umma_bf16_lead(d_tmem, ad + 128ull * k, bd + 128ull * k, idesc, 1u, leader);
+            }
+            umma_commit_lead(smem_u32(&ctl->empty[s]), leader);
+            if (++s == p.stages) { s = 0; ph ^= 1; }
+        }
+        if (ok) umma_commit_lead(smem_u32(&ctl->accum), leader);
+        if (warp == 1) WTRACE(2);
+    }
+    wgrad_finish(p, ctl, data_base, tmem_base, r * p.S, k0, c0, split, iters, p.data_bytes, p.S, p.BN);
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem_base, (uint32_t)p.tmem_cols);
+    }
+}
+
 // ------------------------------------------------------------------------------------------ few-channel stride-2 stem
 // A stride-2 convolution over very few input channels (the 7x7 / 3-channel network stem) is rewritten as a stride-1
 // convolution over a space-to-depth copy of the input: xs[n][i][j + pl][(a,b,c)] = x[n][2i+a][2j+b][c], 16 bf16 per pixel,
@@ -2164,6 +2311,21 @@ bool make_halo_in_map(const pt_ctx *c, CUtensorMap *tm, const void *base, int C,
     return map_ok(r, __LINE__);
 }
 
+// The pixels (a + i * stride, b + j * stride) of bf16 activations as a tiled 4-D tensor (C, columns j, rows i, N): box 64 channels x box_w x
+// box_h x 1.
+bool make_plane_map(const pt_ctx *c, CUtensorMap *tm, const void *base, int C, int W, int H, int N, int ld, int stride, int a, int b, int box_w, int box_h)
+{
+    if (!c->encode_tiled || box_w > 256 || box_h > 256 || a >= H || b >= W) return false;
+    const char *first = (const char *)base + ((size_t)a * W + b) * ld * 2;
+    cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)pt_ceil_div(W - b, stride), (cuuint64_t)pt_ceil_div(H - a, stride), (cuuint64_t)N};
+    cuuint64_t strides[3] = {(cuuint64_t)stride * ld * 2, (cuuint64_t)stride * W * ld * 2, (cuuint64_t)H * W * ld * 2};
+    cuuint32_t box[4] = {(cuuint32_t)kKC, (cuuint32_t)box_w, (cuuint32_t)box_h, 1}, estr[4] = {1, 1, 1, 1};
+    CUresult r = ((EncodeTiledFn)c->encode_tiled)(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<char *>(first), dims, strides, box, estr,
+                                                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                                                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return map_ok(r, __LINE__);
+}
+
 // One launch of the halo kernel: a stride-1 correlation of `src` with a list of taps, written to a (possibly strided)
 // view of the output.
 struct HaloSpec {
@@ -2370,22 +2532,30 @@ void halo_spec_stride1(const pt_conv_desc *d, HaloSpec *h, const void *src, int 
 constexpr size_t kSplitSmemFloor = 116 * 1024;
 
 // ---- launch shape of a weight gradient
-// Both kernels cut the work three ways: tiles of dw (channels), groups of taps, and the pixels of the reduction over `splits` CTAs
+// The kernels cut the work three ways: tiles of dw (channels), groups of taps, and the pixels of the reduction over `splits` CTAs
 // that exchange partial sums at the end. The shape is chosen by a rough time of one CTA (microseconds; the constants are measured):
-//   first load 1.4, then per stage the larger of its MMAs (55 cycles each at N <= 64, N/2 + 8 above) and its bytes at 100 KB/us,
-//   plus 0.25 of waiting and issuing; then the exchange:
-//   none (one split): 1; through the workspace: 5 + bytes of the accumulators at 40 KB/us (partial tile to L2, arrival counter, sum:
-//   three round trips); in a cluster (2..8 splits): 1.5 + the bytes for the other CTAs at 25 KB/us, at 11 KB/us among more than four
-//   (213 -> 242 3x3 at 14x14, 112 KB, eight splits: 27 us as clusters, 23 through the workspace; 8 14x14 64 -> 64, 32 KB: 6.4 and 8.7).
+//   first load 1.4, then per stage the longer of its matrix instructions and its staged rows, and what waiting and issuing add; then the
+//   exchange of the sums that are part of dw: none (one split) 1 + bytes at 17 KB/us (transposed 4 bytes at a time); through the workspace
+//   4 + bytes at 33 KB/us (stores, arrival counter, sum: three round trips), slower by what all CTAs exchange over 35 MB; in a cluster (2..8 splits) 2.6 + bytes at 20 KB/us (25 for two).
+//   (512 -> 128 1x1 at 7x7, batch 16, 131 KB: workspace 7.9, clusters of two and four 9.9 and 9.2; 64 -> 256 at 14x14, batch 8, 32 KB: 4.5
+//   and 3.9; 13 -> 27 3x3 at 16x16, batch 8, 16 KB: 4.3 and 2.9.)
 // A cluster needs its CTAs free at the same time in one GPC: used while the device can hold all of the launch's clusters at once.
-constexpr double kWgSearch = 400.0;      // generic kernel: layers whose tile takes one CTA less than this (us) also choose tap groups
+constexpr double kWgSearch = 400.0;      // generic kernel: layers whose tile takes one CTA less than this (us) also choose tap groups,
+constexpr double kWgNarrow = 40.0;       // less than this: tile widths
 
-double wg_mma_us(int n) { return (n <= 64 ? 55.0 : n * 0.5 + 8.0) / 1900.0; }
-double wg_exchange_us(int splits, bool cluster, double acc_bytes)
+// One MMA of M = 128, K = 16: cycles by its columns, and what one issuing warp needs where no other issues beside it.
+double wg_mma_us(int n, bool several) { const double c = n <= 32 ? 40.0 : n <= 128 ? 32.0 + n * 0.25 : n * 0.5; return (several || c > 75.0 ? c : 75.0) / 1920.0; }
+double wg_exchange_us(int tiles, int splits, bool cluster, double bytes)
 {
-    if (splits <= 1) return 1.0 + acc_bytes / 200e3;
-    if (!cluster) return 5.0 + acc_bytes / 40e3;
-    return 1.5 + acc_bytes * (splits - 1) / splits / (splits <= 4 ? 25e3 : 11e3);
+    if (splits <= 1) return 1.0 + bytes / 17e3;
+    return cluster ? 2.6 + bytes / (splits == 2 ? 25e3 : 20e3) : 4.0 + bytes / 33e3 * (1.0 + bytes * splits * tiles / 35e6);
+}
+// Nanoseconds the TMA unit takes per staged row of `cols` channels in boxes of 64 or 32 (see store_cols), all boxes together.
+double wg_row_ns(int cols, int lanes = 64)
+{
+    if (lanes == 32) return cols == 32 ? 0.55 : cols > 16 && cols <= 24 ? 1.5 : 1.05;
+    const int rest = cols & 63;
+    return (cols >> 6) * 0.95 + (rest == 0 ? 0.0 : rest <= 32 ? 1.05 : rest <= 40 ? 3.4 : rest <= 56 ? 1.45 : 1.05);
 }
 
 int wg_max_clusters(const pt_ctx *c, int size);
@@ -2410,50 +2580,69 @@ int wgrad_budget(const pt_ctx *c) { return (c->wgrad_ctas > 0 && c->wgrad_ctas <
 // Splits of a launch with `tiles` CTAs per split, at most `max_s`: all the budget holds through the workspace, or up to eight as
 // clusters, whichever is estimated faster; `main_us(s)` is the main loop with s splits.
 template <typename F>
-double wg_pick_splits(const pt_ctx *c, int tiles, int max_s, double acc_bytes, F main_us, int *splits, int *cluster)
+double wg_pick_splits(const pt_ctx *c, int tiles, int max_s, double bytes, F main_us, int *splits, int *cluster)
 {
     int s = wgrad_budget(c) / tiles;                       // at most one CTA per SM, one wave
     if (s > max_s) s = max_s;
     if (s > 512) s = 512;
     if (s < 1) s = 1;
-    double best = main_us(s) + wg_exchange_us(s, false, acc_bytes);
+    double best = main_us(s) + wg_exchange_us(tiles, s, false, bytes);
     *splits = s; *cluster = 0;
     for (int k = s < 8 ? s : 8; k >= 2; --k) {
         if (tiles > wg_max_clusters(c, k)) continue;
-        const double t = main_us(k) + wg_exchange_us(k, true, acc_bytes);
+        const double t = main_us(k) + wg_exchange_us(tiles, k, true, bytes);
         if (t < best) { best = t; *splits = k; *cluster = 1; }
     }
     return best;
 }
 
-// The generic kernel: 64 pixels per stage.
-void wgrad_gen_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, pt_wgrad_plan *w)
+// Tile widths of the generic kernel: tile_n's, and for small layers a half and a quarter of it (a narrow accumulator is sooner exchanged, and
+// more CTAs share the work). False past the last.
+bool wgrad_gen_bn(const pt_conv_desc *d, int option, int *bn, int *n_tiles)
+{
+    *bn = tile_n(d->C, n_tiles);
+    if (option == 0) return true;
+    if (option > 2 || *bn >> option < 48) return false;
+    *n_tiles <<= option;
+    *bn = pt_ceil_div(pt_ceil_div(d->C, *n_tiles), 16) * 16;
+    return (*n_tiles - 1) * *bn < d->C;
+}
+long long wgrad_gen_splits(const pt_conv_desc *d, int P, int Q) { return ((long long)d->N * P * Q + 127) / 128; }     // two 64-pixel stages each
+
+// The generic kernel: 64 pixels per stage. Returns the estimated time.
+double wgrad_gen_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, pt_wgrad_plan *w)
 {
     memset(w, 0, sizeof(*w));
     const int taps = d->R * d->S;
-    w->bn = tile_n(d->C, &w->n_tiles);
     w->m_tiles = pt_ceil_div(d->K, 128);
-    w->acc_cols = w->bn;
-    const long long npix = (long long)d->N * P * Q;
-    long long max_s = (npix + 255) / 256;                  // at least four 64-pixel stages per split
+    const long long stages = ((long long)d->N * P * Q + 63) / 64;
+    long long max_s = wgrad_gen_splits(d, P, Q);
     if (max_s > 512) max_s = 512;
-    const int nb = pt_ceil_div(w->bn, 64), base = wgrad_taps_per_cta(taps, w->bn), groups0 = pt_ceil_div(taps, base);
+    const double dy_ns = wg_row_ns(d->K > 128 ? 128 : store_cols(d->K, d->ldy)), rows = d->K > 128 ? 128 : d->K;
     double best = 1e30;
-    for (int g = groups0; g <= taps; g += groups0) {
-        const int tpc = pt_ceil_div(taps, g), tiles = w->m_tiles * w->n_tiles * pt_ceil_div(taps, tpc);
-        if (g > groups0 && (tiles > wgrad_budget(c) || pt_ceil_div(taps, tpc) != g)) continue;
-        const double load = ((d->K > 64 ? 16384.0 : 8192.0) + tpc * nb * 8192.0) / 100e3, mma = tpc * 4 * wg_mma_us(w->bn);
-        const double stage = (load > mma ? load : mma) + 0.25;
-        int s, cl;
-        const double t = wg_pick_splits(c, tiles, (int)max_s, (double)tpc * w->bn * 512.0,
-                                        [&](int k) { return 1.4 + (double)((npix + 63) / 64 + k - 1) / k * stage; }, &s, &cl);
-        if (t < best) {
-            best = t;
-            w->tpc = w->apc = tpc; w->tap_groups = pt_ceil_div(taps, tpc);
-            w->splits = s; w->cluster = cl;
+    int bn, n_tiles;
+    for (int o = 0; wgrad_gen_bn(d, o, &bn, &n_tiles); ++o) {
+        const int base = wgrad_taps_per_cta(taps, bn), groups0 = pt_ceil_div(taps, base);
+        const double x_ns = wg_row_ns(n_tiles > 1 ? bn : store_cols(d->C, d->ldx)) * (d->stride > 1 ? 1.08 : 1.0);     // (im2col boxes two pixels apart)
+        double stage = 0.0;
+        for (int g = groups0; g <= taps; g += groups0) {
+            const int tpc = pt_ceil_div(taps, g), tiles = w->m_tiles * n_tiles * pt_ceil_div(taps, tpc);
+            if ((o > 0 || g > groups0) && (2 * tiles > wgrad_budget(c) || pt_ceil_div(taps, tpc) != g)) continue;
+            const double load = 64e-3 * (dy_ns + tpc * x_ns), mma = tpc * 4 * wg_mma_us(bn, tpc > 1);
+            stage = load > mma ? load : mma;
+            int s, cl;
+            const double t = wg_pick_splits(c, tiles, (int)max_s, tpc * bn * rows * 4.0, [&](int k) { return 1.4 + (double)((stages + k - 1) / k) * stage; }, &s, &cl);
+            if (t < best) {
+                best = t;
+                w->bn = w->acc_cols = bn; w->n_tiles = n_tiles;
+                w->tpc = w->apc = tpc; w->tap_groups = pt_ceil_div(taps, tpc);
+                w->splits = s; w->cluster = cl;
+            }
+            if ((double)stages * stage > kWgSearch) break;              // large: the fewest groups read the least
         }
-        if ((double)((npix + 63) / 64) * stage > kWgSearch) break;      // large: the fewest groups read the least
+        if ((double)stages * stage > kWgNarrow) break;
     }
+    return best;
 }
 
 // The row-block kernel (stride-1 filters with at most 64 input channels); false where the generic kernel is used.
@@ -2483,7 +2672,8 @@ bool wgrad_rows_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, pt_wg
     if (t > pairs) t = pairs;
     const int groups0 = pt_ceil_div(pairs, t);
     w->nb_a = pt_ceil_div(w->acc_cols, 64);
-    const double cyc = wg_mma_us(w->acc_cols);
+    const double dy_ns = wg_row_ns(store_cols(d->K, d->ldy), w->dy_lanes), x_ns = wg_row_ns(store_cols(d->C, d->ldx), w->lanes);
+    const double rows_used = (w->lanes == 64 ? 2 : d->S < 4 ? d->S : 4) * d->C;              // of an accumulator
     // Rows per unit, tap groups and splits, by the estimated time: a unit takes the longer of its matrix instructions and its staged rows.
     // (Large layers took the unit with the least traffic and MMA steps per useful pixel instead, and no account of the rows: units of a
     // single row, or so large that the splits came out uneven. 10 -> 22 1x1 at 32x32, batch 253: 23.8 -> 15.4 us; 9 -> 13 at 37x37, batch
@@ -2497,13 +2687,13 @@ bool wgrad_rows_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, pt_wg
         const int st = (int)((220 * 1024 - 2048) / stage);
         if (st < 2) break;
         const int rb = pt_ceil_div(P, nr), units = d->N * rb;
-        const double load = (double)(w->nb_a * nr + nr + d->R - 1) * w->Wp * 2.4e-3;      // the TMA unit, by the row
+        const double load = (dy_ns * nr + x_ns * (nr + d->R - 1)) * w->Wp * 1e-3;         // the TMA unit, by the row
         for (int g = groups0; g <= pairs; g += groups0) {
             const int apc = pt_ceil_div(pairs, g), tiles = pt_ceil_div(pairs, apc);
             if (g > groups0 && (tiles > wgrad_budget(c) || tiles != g)) continue;
-            const double mma = ks * apc * cyc, unit = (load > mma ? load : mma) + 0.25;
+            const double mma = ks * apc * wg_mma_us(w->acc_cols, apc > 1), unit = (load > mma ? load : mma) + 0.15;
             int s, cl;
-            const double us = wg_pick_splits(c, tiles, units > 3 ? units / 2 : 1, (double)apc * w->acc_cols * 512.0,
+            const double us = wg_pick_splits(c, tiles, units > 3 ? units / 2 : 1, apc * rows_used * d->K * 4.0,
                                              [&](int k) { return 1.4 + pt_ceil_div(units, k) * unit; }, &s, &cl);
             if (us >= best_us) continue;
             best_us = us;
@@ -2525,6 +2715,70 @@ bool wgrad_rows_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, pt_wg
     return true;
 }
 
+// Columns of an accumulator, and tiles of them, of the filter-row form: S accumulators fit the tensor memory.
+int wgrad_taps_bn(const pt_conv_desc *d, int *n_tiles)
+{
+    int top = 512 / d->S / 16 * 16;
+    if (top > 256) top = 256;
+    *n_tiles = pt_ceil_div(d->C, top);
+    return pt_ceil_div(pt_ceil_div(d->C, *n_tiles), 16) * 16;
+}
+
+bool wgrad_taps_ok(const pt_conv_desc *d)
+{
+    return d->S >= 2 && d->S <= kMaxRow && d->R <= kMaxRow && (d->stride == 1 || d->stride == 2) && d->pad <= 64 && d->H >= d->stride && d->W >= d->stride;
+}
+
+// The filter-row kernel; false where it does not apply.
+double wgrad_taps_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, pt_wgrad_plan *w)
+{
+    memset(w, 0, sizeof(*w));
+    if (!wgrad_taps_ok(d) || P < 1 || Q < 1) return 1e30;
+    w->planes = d->stride;
+    const int shift = d->stride == 1 ? d->S - 1 : d->S / 2;             // the largest one (at stride 2 and an even S it may be one less)
+    w->Wp = Q + shift;
+    if (w->Wp > 256) return 1e30;
+    w->bn = w->acc_cols = wgrad_taps_bn(d, &w->n_tiles);
+    if (w->n_tiles > 1) return 1e30;          // (dy would be loaded again: no fewer bytes, 147 -> 186 to 213 -> 242 3x3 at 14x14 no faster per SM)
+    w->m_tiles = pt_ceil_div(d->K, 128);
+    w->nb_a = d->K > 64 ? 2 : 1;
+    w->tpc = w->apc = d->S; w->tap_groups = d->R;
+    const int nb = pt_ceil_div(w->bn, 64), tiles = w->n_tiles * w->m_tiles * d->R;
+    const double cyc = wg_mma_us(w->bn, true);
+    const double dy_ns = wg_row_ns(d->K > 128 ? 128 : store_cols(d->K, d->ldy)), x_ns = wg_row_ns(w->n_tiles > 1 ? w->bn : store_cols(d->C, d->ldx));
+    double best = 1e30;
+    for (int nr = 1; nr <= P && nr <= 256; ++nr) {
+        const int ks = pt_ceil_div(nr * w->Wp, 16);
+        const size_t a_box = (size_t)ks * 2048, b_box = pt_align_up((size_t)(ks * 16 + shift) * 128, 1024);
+        const size_t stage = w->nb_a * a_box + (size_t)w->planes * nb * b_box;
+        int st = (int)((220 * 1024 - 2048) / stage);
+        if (st < 3) break;
+        if (st > kMaxStages) st = kMaxStages;
+        const int rb = pt_ceil_div(P, nr), units = d->N * rb;
+        // a unit takes the longest of its matrix instructions, its staged rows and a load's latency over the stages in flight
+        const double mma = ks * d->S * cyc, load = (dy_ns + w->planes * x_ns) * nr * w->Wp * 1e-3, lat = 1.4 / (st - 1);
+        double unit = mma > load ? mma : load;
+        unit = (unit > lat ? unit : lat) + 0.08;
+        int s, cl;
+        const double us = wg_pick_splits(c, tiles, units > 3 ? units / 2 : 1, w->apc * w->bn * (d->K > 128 ? 128 : d->K) * 4.0,
+                                         [&](int k) { return 1.4 + pt_ceil_div(units, k) * unit; }, &s, &cl);
+        if (us >= best) continue;
+        best = us;
+        w->nr = nr; w->ksteps = ks; w->a_box = (unsigned)a_box; w->b_box = (unsigned)b_box;
+        w->stages = st; w->stage_bytes = stage; w->RB = rb; w->units = units;
+        w->splits = s; w->cluster = cl;
+    }
+    if (w->nr == 0) return 1e30;
+    w->units_per_split = pt_ceil_div(w->units, w->splits);
+    w->splits = pt_ceil_div(w->units, w->units_per_split);
+    if (w->splits < 2) w->cluster = 0;
+    if (w->stages > w->units_per_split && w->units_per_split >= 2) w->stages = w->units_per_split;
+    w->smem = 2048 + (size_t)w->stages * w->stage_bytes;
+    if (w->smem < 2048 + 8 * 2 * 4096) w->smem = 2048 + 8 * 2 * 4096;    // the epilogue's staging slabs reuse the ring
+    w->filter_row = 1;
+    return best;
+}
+
 // The plan of a descriptor at the context's CTA limit. rows_only: only a row-block plan is asked for (its `rows` is 0 if there is none).
 pt_wgrad_plan wgrad_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, bool rows_only = false)
 {
@@ -2537,7 +2791,13 @@ pt_wgrad_plan wgrad_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, b
     pt_wgrad_plan w;
     if (!wgrad_rows_plan(c, d, P, Q, &w)) {
         w.rows = 0;
-        if (!rows_only) wgrad_gen_plan(c, d, P, Q, &w);
+        if (!rows_only) {
+            pt_wgrad_plan g;
+            // (measured against estimated times at all SMs and at 49: within 10 % of each other, so that near a tie either may be the faster;
+            // 106 -> 103 3x3 at 28x28, batch 64 22.9 us generic, 21.8 by filter rows, 49.5 and 34.6 at 49; 128 -> 128 at 32x32 25.7 and 28.2,
+            // 54.1 and 46.5; 147 -> 186 at 14x14 19.7 and 22.1, 44.5 and 32.1)
+            if (0.98 * wgrad_gen_plan(c, d, P, Q, &g) <= wgrad_taps_plan(c, d, P, Q, &w)) w = g;
+        }
     }
     if (c->wgrad_plans.size() >= pt_ctx::kWgradPlans) c->wgrad_plans.clear();
     c->wgrad_plans.emplace(key, w);
@@ -2558,18 +2818,35 @@ size_t wgrad_partial_bytes(const pt_wgrad_plan &w)
 size_t wgrad_workspace_bound(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, const pt_wgrad_plan &w)
 {
     const int taps = d->R * d->S, budget = wgrad_budget(c);
-    // what is dealt out in groups (taps, or accumulators of two or four taps), as few as fit one CTA at most, and the most splits
-    const int parts = !w.rows ? taps : w.lanes == 64 ? pt_ceil_div(taps, 2) : d->R * pt_ceil_div(d->S, 4);
-    const int most = !w.rows ? wgrad_taps_per_cta(taps, w.bn) : 512 / w.acc_cols < 16 ? 512 / w.acc_cols : 16;
-    const long long units = (long long)d->N * P, max_s = !w.rows ? ((long long)d->N * P * Q + 255) / 256 : units > 3 ? units / 2 : 1;
-    long long tiles128 = 0;                                // 128 x acc_cols tiles of fp32
-    for (int g = pt_ceil_div(parts, most < parts ? most : parts); g <= parts; ++g) {
-        const int per = pt_ceil_div(parts, g), tiles = w.n_tiles * w.m_tiles * pt_ceil_div(parts, per);
-        long long s = budget / tiles;
-        if (s > max_s) s = max_s;
-        if (s >= 2 && tiles * s * per > tiles128) tiles128 = tiles * s * per;
+    // `parts` (taps, or accumulators of two or four taps) dealt out in groups, as few as fit one CTA (`most`) at most, each with `tiles1` tiles of
+    // `cols` columns, and the most splits: floats
+    const auto floats = [&](int parts, int most, int g_step, int tiles1, int cols, long long max_s) {
+        long long tiles128 = 0;                            // 128 x cols tiles
+        for (int g = pt_ceil_div(parts, most < parts ? most : parts); g <= parts; g += g_step) {
+            const int per = pt_ceil_div(parts, g), tiles = tiles1 * pt_ceil_div(parts, per);
+            long long s = budget / tiles;
+            if (s > max_s) s = max_s;
+            if (s >= 2 && tiles * s * per > tiles128) tiles128 = tiles * s * per;
+        }
+        return tiles128 * 128 * cols;
+    };
+    const long long units = (long long)d->N * P, unit_s = units > 3 ? units / 2 : 1;
+    if (w.rows)
+        return (size_t)floats(w.lanes == 64 ? pt_ceil_div(taps, 2) : d->R * pt_ceil_div(d->S, 4), 512 / w.acc_cols < 16 ? 512 / w.acc_cols : 16, 1,
+                              w.n_tiles * w.m_tiles, w.acc_cols, unit_s) * sizeof(float);
+    int bn, n_tiles;
+    const int m_tiles = pt_ceil_div(d->K, 128);
+    long long most = 0;
+    for (int o = 0; wgrad_gen_bn(d, o, &bn, &n_tiles); ++o) {
+        const long long t = floats(taps, wgrad_taps_per_cta(taps, bn), 1, n_tiles * m_tiles, bn, wgrad_gen_splits(d, P, Q));
+        if (t > most) most = t;
     }
-    return (size_t)tiles128 * 128 * w.acc_cols * sizeof(float);
+    const int bt = wgrad_taps_bn(d, &n_tiles);
+    if (wgrad_taps_ok(d) && n_tiles == 1) {                // (either form may be the choice of a smaller limit)
+        const long long t = floats(taps, d->S, taps, n_tiles * m_tiles, bt, unit_s);
+        if (t > most) most = t;
+    }
+    return (size_t)most * sizeof(float);
 }
 
 // Launch of a weight-gradient kernel: with programmatic stream serialization and, where the splits of a tile meet in shared memory,
@@ -2595,6 +2872,7 @@ pt_status wgrad_attr(const pt_ctx *c)
     if (!(c->attr_done & kAttrWgrad)) {
         PT_CUDA_OK(cudaFuncSetAttribute(conv_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
         PT_CUDA_OK(cudaFuncSetAttribute(conv_wgrad_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
+        PT_CUDA_OK(cudaFuncSetAttribute(conv_wgrad_taps_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
         c->attr_done |= kAttrWgrad;
     }
     return PT_OK;
@@ -2717,6 +2995,45 @@ pt_status run_wgrad_rows(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const p
     const size_t smem = (p.splits > 1 && wr.smem < kSplitSmemFloor) ? kSplitSmemFloor : wr.smem;
     p.data_bytes = (unsigned)(smem - 2048);
     PT_CUDA_OK(launch_wgrad(conv_wgrad_rows_kernel, grid, p.cluster ? p.splits : 1, smem, st, tmA, tmX, p));
+    c->launches += 1;
+    PT_CUDA_OK(cudaGetLastError());
+    return PT_OK;
+}
+
+// Launches the filter-row weight-gradient kernel.
+pt_status run_wgrad_taps(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const pt_wgrad_plan &wt, const void *x, const void *dy, float *out, void *ws,
+                         size_t ws_bytes, cudaStream_t st)
+{
+    if (!c->encode_tiled) return PT_ERR_CUDA;
+    WgradP p;
+    CUtensorMap tmA;
+    TapMaps tmX;
+    memset(&tmX, 0, sizeof(tmX));
+    const pt_status r0 = wgrad_common(c, d, P, Q, wt, out, ws, ws_bytes, &p);
+    if (r0 != PT_OK) return r0;
+    p.nr = wt.nr; p.Wp = wt.Wp; p.RB = wt.RB; p.units = wt.units; p.units_per_split = wt.units_per_split;
+    p.ksteps = wt.ksteps; p.nb_a = wt.nb_a; p.a_box = wt.a_box; p.b_box = wt.b_box; p.stages = wt.stages; p.planes = wt.planes;
+    // tap column s reads pixel stride * j + s - pad of output column j: plane (s - pad) mod stride, column j + floor((s - pad) / stride) of it
+    const int sh = d->stride - 1;                                     // (stride 1 or 2: shifts and masks)
+    p.plane_lo[0] = p.plane_lo[1] = 1 << 20;
+    for (int s = 0; s < d->S; ++s) {
+        const int pl = (s - d->pad) & sh, off = (s - d->pad) >> sh;
+        p.tap_plane[s] = (unsigned char)pl;
+        if (off < p.plane_lo[pl]) p.plane_lo[pl] = off;
+    }
+    for (int s = 0; s < d->S; ++s) p.tap_shift[s] = (unsigned char)(((s - d->pad) >> sh) - p.plane_lo[p.tap_plane[s]]);
+    for (int r = 0; r < d->R; ++r) {
+        p.row_par[r] = (unsigned char)((r - d->pad) & sh);
+        p.row_off[r] = (signed char)((r - d->pad) >> sh);
+    }
+    if (!make_halo_in_map(c, &tmA, dy, store_cols(d->K, d->ldy), Q, P, d->N, d->ldy, wt.Wp, wt.nr)) return PT_ERR_UNSUPPORTED;
+    for (int a = 0; a < d->stride; ++a)
+        for (int b = 0; b < d->stride; ++b)
+            if (!make_plane_map(c, &tmX.m[a * 2 + b], x, store_cols(d->C, d->ldx), d->W, d->H, d->N, d->ldx, d->stride, a, b, wt.Wp, wt.nr)) return PT_ERR_UNSUPPORTED;
+    dim3 grid((unsigned)(p.n_tiles * p.m_tiles * p.tap_groups), (unsigned)p.splits);
+    const size_t smem = (p.splits > 1 && wt.smem < kSplitSmemFloor) ? kSplitSmemFloor : wt.smem;
+    p.data_bytes = (unsigned)(smem - 2048);
+    PT_CUDA_OK(launch_wgrad(conv_wgrad_taps_kernel, grid, p.cluster ? p.splits : 1, smem, st, tmA, tmX, p));
     c->launches += 1;
     PT_CUDA_OK(cudaGetLastError());
     return PT_OK;
@@ -2924,6 +3241,11 @@ pt_status pt_sm100_conv(pt_ctx *c, const pt_conv_desc *d, int which, const void 
         pt_wgrad_plan w = wgrad_plan(c, d, P, Q);
         if (w.rows) {
             const pt_status r = run_wgrad_rows(c, d, P, Q, w, a, b, (float *)out, ws, ws_bytes, st);
+            if (r != PT_ERR_UNSUPPORTED) return r;
+            wgrad_gen_plan(c, d, P, Q, &w);
+        }
+        if (w.filter_row) {
+            const pt_status r = run_wgrad_taps(c, d, P, Q, w, a, b, (float *)out, ws, ws_bytes, st);
             if (r != PT_ERR_UNSUPPORTED) return r;
             wgrad_gen_plan(c, d, P, Q, &w);
         }

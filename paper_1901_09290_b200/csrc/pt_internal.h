@@ -62,6 +62,7 @@ struct pt_wgrad_plan {
     int lanes, dy_lanes;            // channel lanes per staged pixel of x (64: two taps per accumulator, 32: four) and of dy
     unsigned a_box, b_box;
     size_t stage_bytes, smem;
+    int filter_row, planes;         // filter-row form (nr, Wp, RB, units, ksteps, nb_a, stages, boxes as above); x boxes per unit and block
 };
 
 struct pt_ctx {

@@ -169,6 +169,33 @@ def test_weight_gradient_of_nan_pad_lanes(shape):
     Hh.check_conv(dw, C, oracle.conv_wgrad(x.numpy(), dy.numpy(), R, R, stride, pad), what="wgrad")
 
 
+# (N, H, W, C, K, R, S, stride, pad) of the filter-row form of the weight gradient: one and two blocks of channels on either side and just
+# past them, units that leave rows over, both parities (odd and even sizes, no padding, more padding than the filter), filters of 2, 4, 5 and
+# 8 columns, other than square, a wide image, a single output row
+@pytest.mark.parametrize("shape", [(5, 14, 14, 65, 64, 3, 3, 1, 1), (4, 28, 28, 106, 129, 3, 3, 1, 1), (3, 13, 9, 160, 40, 3, 3, 1, 0), (2, 6, 100, 70, 20, 3, 3, 1, 1),
+                                   (4, 28, 28, 106, 103, 3, 3, 2, 1), (3, 15, 17, 20, 70, 3, 3, 2, 1), (3, 15, 16, 33, 65, 3, 3, 2, 0), (2, 17, 12, 90, 30, 5, 5, 2, 2),
+                                   (3, 12, 12, 66, 50, 2, 2, 2, 0), (3, 16, 16, 60, 130, 4, 4, 2, 3), (2, 24, 24, 64, 40, 8, 8, 2, 3), (2, 9, 20, 100, 24, 1, 5, 1, 2),
+                                   (2, 3, 30, 80, 64, 3, 3, 1, 0), (64, 14, 14, 77, 77, 3, 3, 1, 1), (64, 28, 28, 38, 38, 3, 3, 2, 1)])
+def test_filter_row_weight_gradient(shape):
+    N, H, Wd, C, K, R, S, stride, pad = shape
+    x = W.gen_act(N, H, Wd, C, W.BASE_SEED + 43)
+    P, Q = (H + 2 * pad - R) // stride + 1, (Wd + 2 * pad - S) // stride + 1
+    dy = W.gen_dy(N, P, Q, K, W.BASE_SEED + 44)
+    ref = oracle.conv_wgrad(x.numpy(), dy.numpy(), R, S, stride, pad)
+    c = B.Context(0)
+    d = B.make_conv_desc(N, H, Wd, C, K, R, S, stride, pad, W.pad8(C), W.pad16(K), W.pad8(C), 0, 2)
+    xd, dyd = Hh.to_dev_padded(x, d.ldx), Hh.to_dev_padded(dy, d.ldy)
+    for limit in (0, 49, 3):                                    # (all SMs, a share of them, one CTA per filter row)
+        B.pt_set_wgrad_cta_limit(c, limit)
+        ws = torch.empty(max(16, B.pt_conv_workspace_bytes(c, d, B.PT_CONV_WGRAD)), dtype=torch.uint8, device="cuda")
+        dw = torch.full((K, R, S, C), 7680.0, device="cuda")
+        B.pt_conv_wgrad(c, d, xd, dyd, dw, ws)
+        torch.cuda.synchronize()
+        c.poll()
+        Hh.check_conv(dw, C, ref, what=f"wgrad at limit {limit}")
+    c.close()
+
+
 def test_wgrad_is_run_to_run_identical():
     N, H, C, K, R = 4, 14, 27, 19, 3
     x, w, dy, pad = _case(N, H, H, C, K, R, 1, W.BASE_SEED + 5)
