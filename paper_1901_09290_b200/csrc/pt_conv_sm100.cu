@@ -1992,6 +1992,306 @@ StemPlan stem_plan(const pt_conv_desc *d)
     return s;
 }
 
+// Forward pass of a few-channel stride-2 stem straight from the image (U >= 2; 64 to 128 output columns, at most 128 channels, bf16 out).
+// A CTA has a run of consecutive output rows. Two teams of four warps turn each pair of image rows into one space-to-depth row in shared
+// memory (every one of them once: the next output row needs one new one of its U), in a ring of rows of 32-byte positions with the
+// swizzle of that width; an output row is then U x V matrix instructions on those rows (tap (u, v) starts at row u, v positions on) with the
+// weights, laid out once per CTA, resident. Four issuers take output rows in turn (one needs 1.6 us for the 16 instructions, waits and
+// commits of a row; two issuers 54.7 us for the launch), a group of epilogue warps every other one.
+// Through a space-to-depth copy in memory it was two launches more (11 and 2 us at batch 64) and four staged rows per output row: 3 -> 55
+// 7x7/2 at 224x224, batch 64 53.7 -> 37.5 us, 3 -> 19 at batch 256 153 -> 110. Bound by the matrix instructions' reads of shared memory
+// (6 KB each, 16 a row: 0.4 us of the 0.6 to 0.7 a row takes) and by the stores.
+constexpr int kStemAhead = 3;                                     // rows a converting thread has on their way (2 and 3: 38.8 and 37.5 us)
+constexpr int kStemRing = 16, kStemSlot = 4352;                     // rows in the ring (a power of two); bytes of one: up to 131 positions of 32
+constexpr int kStemIssuers = 4, kStemThreads = (kStemIssuers + 16) * 32;        // issuers, eight epilogue warps, two teams of four converting warps
+
+struct StemP {
+    int N, H, W, C, K, R, S, ldw;
+    int P, Q, Hs, Ws, Wp, pl, off, U, V;
+    int BN, rows, rows_per_cta;         // output rows in all (N * P) and of a CTA
+    int tmem_cols, acc_per;
+    int stats_off, stats_warp, stats_lo, ld_out;
+    float *stats;
+    const __nv_bfloat16 *x, *w;
+    unsigned int *status;
+};
+
+struct __align__(8) StemCtl {
+    uint64_t full[kStemRing], empty[kStemRing];
+    uint64_t acc_full[2 * kStemIssuers], acc_empty[2 * kStemIssuers];
+    uint32_t tmem_base;
+    int abort_flag;
+};
+
+// The output rows of a CTA image by image: first row, number of rows, position of the first space-to-depth row in the CTA's sequence.
+struct StemWalk {
+    int n, p0, len, q0, left;
+    __device__ __forceinline__ void init(const StemP &p)
+    {
+        const int g0 = (int)blockIdx.x * p.rows_per_cta;
+        left = min(p.rows_per_cta, p.rows - g0);
+        n = g0 / p.P; p0 = g0 - n * p.P;
+        len = min(left, p.P - p0); q0 = 0;
+    }
+    __device__ __forceinline__ void next(const StemP &p)
+    {
+        left -= len; q0 += len + p.U - 1;
+        ++n; p0 = 0; len = min(left, p.P);
+    }
+};
+
+// One position of a space-to-depth row: the four channels of four pixels of the image, zeros outside (i: the row, jp: the position), and
+// the 16 lanes they make, pixel by pixel.
+__device__ __forceinline__ void stem_load(const StemP &p, int n, int i, int jp, uint2 (&px)[4])
+{
+    const int j = jp - p.pl;
+    const bool in = i >= 0 && i < p.Hs && j >= 0 && j < p.Ws;
+#pragma unroll
+    for (int ab = 0; ab < 4; ++ab)
+        px[ab] = in ? __ldg(reinterpret_cast<const uint2 *>(p.x + ((size_t)(n * p.H + 2 * i + (ab >> 1)) * p.W + 2 * j + (ab & 1)) * 8)) : make_uint2(0, 0);
+}
+__device__ __forceinline__ void stem_pack(int C, const uint2 (&px)[4], uint4 &lo, uint4 &hi)
+{
+    hi = make_uint4(0, 0, 0, 0);
+    if (C == 3) {
+        lo = make_uint4(px[0].x, (px[0].y & 0xffffu) | (px[1].x << 16), (px[1].x >> 16) | (px[1].y << 16), px[2].x);
+        hi.x = (px[2].y & 0xffffu) | (px[3].x << 16);
+        hi.y = (px[3].x >> 16) | (px[3].y << 16);
+    } else if (C == 4) {
+        lo = make_uint4(px[0].x, px[0].y, px[1].x, px[1].y);
+        hi = make_uint4(px[2].x, px[2].y, px[3].x, px[3].y);
+    } else if (C == 2) {
+        lo = make_uint4(px[0].x, px[1].x, px[2].x, px[3].x);
+    } else {
+        lo = make_uint4((px[0].x & 0xffffu) | (px[1].x << 16), (px[2].x & 0xffffu) | (px[3].x << 16), 0u, 0u);
+    }
+}
+__device__ __forceinline__ void st_shared_v4(uint32_t addr, const uint4 &v)
+{
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+}
+
+template <bool STATS>
+__global__ void __launch_bounds__(kStemThreads, 1) conv_stem_kernel(const __grid_constant__ CUtensorMap tmC, const StemP p)
+{
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    StemCtl *ctl = reinterpret_cast<StemCtl *>(smem_raw);
+    const uint32_t smem_base = smem_u32(smem_raw);
+    const uint32_t staging_base = (smem_base + (uint32_t)sizeof(StemCtl) + 1023u) & ~1023u;
+    const uint32_t ring_base = staging_base + 8u * kSlabs * 4096u, w_base = ring_base + (uint32_t)(kStemRing * kStemSlot);
+    const uint32_t w_tile = (uint32_t)p.BN * 32u;
+    volatile int *abort_flag = &ctl->abort_flag;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kStemRing; ++s) { mbar_init(smem_u32(&ctl->full[s]), 4); mbar_init(smem_u32(&ctl->empty[s]), kStemIssuers); }
+        for (int b = 0; b < 2 * kStemIssuers; ++b) { mbar_init(smem_u32(&ctl->acc_full[b]), 1); mbar_init(smem_u32(&ctl->acc_empty[b]), 4); }
+        ctl->abort_flag = 0;
+        fence_mbar_init();
+        prefetch_tmap(&tmC);
+    }
+    if (warp == 0) {
+        tmem_alloc(smem_u32(&ctl->tmem_base), (uint32_t)p.tmem_cols);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = ctl->tmem_base;
+    if (warp < kStemIssuers + 8) {
+        // The weights as [tap (u, v)][output channel][16 lanes], K-major rows of 32 bytes, laid out like the positions: lane (a*2+b)*C + c
+        // is filter position (2u + a - off, 2v + b - off), zeros outside the filter and past K. The converting warps are at work on the
+        // image meanwhile. (Weights are not written by a kernel that releases its dependents early.)
+        const unsigned short *w = reinterpret_cast<const unsigned short *>(p.w);
+        for (int i = threadIdx.x; i < p.U * p.V * p.BN; i += (kStemIssuers + 8) * 32) {
+            const int t = i / p.BN, k = i - t * p.BN, u = t / p.V, v = t - u * p.V;
+            uint2 px[4];
+#pragma unroll
+            for (int ab = 0; ab < 4; ++ab) {
+                const int r = 2 * u + (ab >> 1) - p.off, s = 2 * v + (ab & 1) - p.off;
+                px[ab] = k < p.K && r >= 0 && r < p.R && s >= 0 && s < p.S ? __ldg(reinterpret_cast<const uint2 *>(w + ((size_t)(k * p.R + r) * p.S + s) * p.ldw))
+                                                                           : make_uint2(0, 0);
+            }
+            uint4 lo, hi;
+            stem_pack(p.C, px, lo, hi);
+            const uint32_t row = w_base + (uint32_t)t * w_tile + (uint32_t)k * 32u, x = (row >> 3) & 16u;
+            st_shared_v4(row + x, lo);
+            st_shared_v4(row + (16u ^ x), hi);
+        }
+        fence_proxy_async();
+        named_barrier(2, (kStemIssuers + 8) * 32);
+        grid_dependency_wait();                                       // (the converting warps wait before their first load)
+    }
+    grid_launch_dependents();
+    StemWalk sw;
+    sw.init(p);
+
+    if (warp < kStemIssuers) {
+        // ---------------- MMA issuers: output rows warp, warp + kStemIssuers, ... of the CTA; the warp walks the loop in lockstep, lane 0 issues
+        const uint32_t leader = lane == 0 ? 1u : 0u;
+        const uint32_t idesc = make_idesc_bf16(128, p.BN, 0, 0);
+        const uint64_t desc0 = make_desc_rows(0u, 32u);
+        bool ok = true;
+        int nt = 0, row0 = 0;                                        // rows this issuer has started; the segment's first row in the CTA's count
+        for (; sw.left > 0 && ok; row0 += sw.len, sw.next(p)) {
+            int rel = sw.q0;                                         // ring rows of the segment that this issuer has released
+            const int end = sw.q0 + sw.len + p.U - 1;
+            for (int l = (warp - row0) & (kStemIssuers - 1); l < sw.len && ok; l += kStemIssuers, ++nt) {
+                const int b = p.acc_per == 2 ? warp * 2 + (nt & 1) : warp, aph = p.acc_per == 2 ? (nt >> 1) & 1 : nt & 1;
+                ok = mbar_wait(smem_u32(&ctl->acc_empty[b]), aph ^ 1, abort_flag, p.status, 60);
+                // (either team of converting warps fills its ring rows in order: behind the last two all are there)
+                for (int q = sw.q0 + l + p.U - 2; q < sw.q0 + l + p.U && ok; ++q)
+                    ok = mbar_wait(smem_u32(&ctl->full[q & (kStemRing - 1)]), (q / kStemRing) & 1, abort_flag, p.status, 61);
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t d_tmem = tmem_base + (uint32_t)(b * p.BN);
+                uint64_t bd = desc0 | desc_addr(w_base);
+                const uint64_t b_step = w_tile >> 4;
+                for (int u = 0; u < p.U; ++u) {
+                    const uint64_t ad = desc0 | desc_addr(ring_base + (uint32_t)((sw.q0 + l + u) & (kStemRing - 1)) * kStemSlot);
+#pragma unroll
+                    for (int v = 0; v < 4; ++v)
+                        if (v < p.V) umma_bf16_lead(d_tmem, ad + 2ull * v, bd + b_step * v, idesc, v == 0 ? (u ? 1u : 0u) : 1u, leader);
+                    bd += b_step * p.V;
+                }
+                umma_commit_lead(smem_u32(&ctl->acc_full[b]), leader);
+                // ring rows that this issuer needs no more: up to its next output row's first one, behind its last one all (those that
+                // it never reads once they are there: an arrival belongs to the row's own turn in the ring)
+                const int upto = l + kStemIssuers < sw.len ? sw.q0 + l + kStemIssuers : end;
+                for (; rel < upto && ok; ++rel) {
+                    const uint32_t bar = smem_u32(&ctl->empty[rel & (kStemRing - 1)]);
+                    if (rel < sw.q0 + l + p.U) umma_commit_lead(bar, leader);
+                    else {
+                        ok = mbar_wait(smem_u32(&ctl->full[rel & (kStemRing - 1)]), (rel / kStemRing) & 1, abort_flag, p.status, 62);
+                        if (ok && lane == 0) mbar_arrive(bar);
+                    }
+                }
+            }
+            for (; rel < end && ok; ++rel) {                          // (a segment without a row of this issuer)
+                ok = mbar_wait(smem_u32(&ctl->full[rel & (kStemRing - 1)]), (rel / kStemRing) & 1, abort_flag, p.status, 63);
+                if (ok && lane == 0) mbar_arrive(smem_u32(&ctl->empty[rel & (kStemRing - 1)]));
+            }
+        }
+    } else if (warp < kStemIssuers + 8) {
+        // ---------------- epilogue: group g (four warps) has every other output row
+        const int ew = warp - kStemIssuers, quarter = warp & 3, group = ew >> 2;
+        const uint32_t slab0 = staging_base + (uint32_t)ew * (kSlabs * 4096u);
+        const uint32_t st_acc = smem_base + (uint32_t)p.stats_off + (uint32_t)ew * (uint32_t)p.stats_warp;
+        const int n_chunks = (p.BN + 63) / 64;
+        if (STATS) {
+            stats_clear(st_acc, lane, n_chunks);
+            __syncwarp();
+        }
+        const int valid = p.Q - quarter * 32;                         // pixels of this warp's 32 that exist
+        const uint32_t rows = valid >= 32 ? 0xffffffffu : valid > 0 ? (1u << valid) - 1u : 0u;
+        bool ok = true;
+        int row0 = 0, sl = 0;
+        for (; sw.left > 0 && ok; row0 += sw.len, sw.next(p))
+            for (int l = (group - row0) & 1; l < sw.len; l += 2) {
+                // the nt-th row of issuer `iss`
+                const int iss = (row0 + l) & (kStemIssuers - 1), nt = (row0 + l) / kStemIssuers;
+                const int b = p.acc_per == 2 ? iss * 2 + (nt & 1) : iss, aph = p.acc_per == 2 ? (nt >> 1) & 1 : nt & 1;
+                ok = mbar_wait(smem_u32(&ctl->acc_full[b]), aph, abort_flag, p.status, 64);
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t lane_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * p.BN);
+                for (int ch = 0; ch < n_chunks; ++ch, sl ^= 1) {
+                    const uint32_t slab = slab0 + (uint32_t)sl * 4096u;
+                    if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");   // the slab's previous store has read it
+                    __syncwarp();
+                    const int groups = min(4, (p.BN - ch * 64) / 16);
+                    uint32_t v[4][16];
+#pragma unroll
+                    for (int g = 0; g < 4; ++g)
+                        if (g < groups) tmem_ld16(lane_addr + (uint32_t)(ch * 64 + g * 16), v[g]);
+                    tmem_ld_wait();
+                    if (ch + 1 >= n_chunks) {
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(smem_u32(&ctl->acc_empty[b]));
+                    }
+#pragma unroll
+                    for (int g = 0; g < 4; ++g) {
+                        if (g >= groups) break;
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            __nv_bfloat162 e[4];
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) e[k] = __floats2bfloat162_rn(__uint_as_float(v[g][8 * h + 2 * k]), __uint_as_float(v[g][8 * h + 2 * k + 1]));
+                            const uint32_t j = (uint32_t)(g * 2 + h);
+                            st_shared_v4(slab + (uint32_t)lane * 128u + ((j ^ ((uint32_t)lane & 7u)) << 4), *reinterpret_cast<uint4 *>(e));
+                        }
+                    }
+                    fence_proxy_async();
+                    __syncwarp();
+                    if (lane == 0) {
+                        if (valid > 0) tma_store_4d(&tmC, slab, ch * 64, quarter * 32, sw.p0 + l, sw.n);
+                        tma_store_commit();
+                    }
+                    if (STATS) chunk_stats(slab, 0, rows, lane, st_acc + (uint32_t)ch * 512u);
+                }
+            }
+        if (STATS) {
+            named_barrier(1, 256);
+            stats_store_cta(smem_base + (uint32_t)p.stats_off, (uint32_t)p.stats_warp, 8, (int)threadIdx.x - kStemIssuers * 32, 256,
+                            p.stats + (size_t)blockIdx.x * (1 + p.stats_lo) * 2 * p.ld_out, p.ld_out, p.stats_lo, p.K, 0, p.ld_out);
+        }
+        if (lane == 0) tma_store_wait_read();                          // the staging slabs must outlive the stores' reads
+        tc_fence_before();
+    } else {
+        // ---------------- converting warps: a team has every other ring row, a thread a position of it; the pixels of the team's next
+        // kStemAhead rows are on their way meanwhile
+        const int team = (warp - kStemIssuers - 8) >> 2, jp = (int)threadIdx.x - (kStemIssuers + 8 + team * 4) * 32;
+        const bool on = jp < p.Wp;
+        const uint32_t at = ring_base + (uint32_t)jp * 32u;
+        uint2 px[kStemAhead][4];
+        int total = 0;
+        StemWalk lw = sw;                                              // where the next load is: row li of image lw.n, lrest more of the segment
+        int li = lw.p0 - p.pl, lrest = lw.len + p.U - 1;
+        for (; sw.left > 0; sw.next(p)) total += sw.len + p.U - 1;
+        const auto skip = [&]() {
+            ++li;
+            if (--lrest == 0) { lw.next(p); li = lw.p0 - p.pl; lrest = lw.len + p.U - 1; }
+        };
+        const auto load = [&](uint2 (&d)[4]) {
+            if (lw.left <= 0) return;
+            if (on) stem_load(p, lw.n, li, jp, d);
+            skip();
+            if (lw.left > 0) skip();
+        };
+        grid_dependency_wait();
+        if (team == 1) skip();
+#pragma unroll
+        for (int k = 0; k < kStemAhead; ++k) load(px[k]);
+        bool ok = true;
+        for (int q0 = team; q0 < total && ok; q0 += 2 * kStemAhead) {
+#pragma unroll
+            for (int k = 0; k < kStemAhead; ++k) {
+                const int q = q0 + 2 * k, s = q & (kStemRing - 1);
+                if (q >= total || !ok) break;
+                ok = mbar_wait(smem_u32(&ctl->empty[s]), ((q / kStemRing) & 1) ^ 1, abort_flag, p.status, 65);
+                if (!ok) break;
+                if (on) {
+                    uint4 lo, hi;
+                    stem_pack(p.C, px[k], lo, hi);
+                    const uint32_t a = at + (uint32_t)s * kStemSlot, x = (a >> 3) & 16u;
+                    st_shared_v4(a + x, lo);
+                    st_shared_v4(a + (16u ^ x), hi);
+                }
+                fence_proxy_async();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&ctl->full[s]));
+                load(px[k]);
+            }
+        }
+    }
+    __syncthreads();
+    if (warp == 0) {
+        tc_fence_after();
+        tmem_dealloc(tmem_base, (uint32_t)p.tmem_cols);
+    }
+}
+
 // CT = channel count as a compile-time constant (1..4): the 16 output lanes are then plain registers
 template <int CT>
 __global__ void __launch_bounds__(256) stem_s2d_x_kernel_t(const __nv_bfloat16 *__restrict__ x, __nv_bfloat16 *__restrict__ xs, int N, int H,
@@ -2530,6 +2830,53 @@ void halo_spec_stride1(const pt_conv_desc *d, HaloSpec *h, const void *src, int 
 // frees only after a CTA that cannot start has arrived), so a split launch asks for more than half of an SM's shared
 // memory: at most one of them per SM, whatever else runs beside it (kernels that wait for nobody always finish).
 constexpr size_t kSplitSmemFloor = 116 * 1024;
+
+// Launches the stem's forward kernel; PT_ERR_UNSUPPORTED where the space-to-depth copy serves the layer.
+pt_status run_stem(pt_ctx *c, const pt_conv_desc *d, const StemPlan &sp, const void *x, const void *w, void *y, cudaStream_t st)
+{
+    // (narrower images would leave most of a row's 128 matrix rows empty; more channels do not fit beside two accumulators an issuer)
+    if (d->out_f32 || sp.U < 2 || sp.Q < 64 || sp.Q > 128 || sp.Wp > 128 || sp.Q + sp.V - 1 > 128 + 3 || d->K > 128 || !c->encode_tiled) return PT_ERR_UNSUPPORTED;
+    StemP p;
+    memset(&p, 0, sizeof(p));
+    p.N = d->N; p.H = d->H; p.W = d->W; p.C = d->C; p.K = d->K; p.R = d->R; p.S = d->S; p.ldw = d->ldw;
+    p.P = sp.P; p.Q = sp.Q; p.Hs = sp.Hs; p.Ws = sp.Ws; p.Wp = sp.Wp; p.pl = sp.pl; p.off = sp.off; p.U = sp.U; p.V = sp.V;
+    p.BN = pt_ceil_div(d->K, 16) * 16;
+    p.rows = d->N * sp.P;
+    p.rows_per_cta = pt_ceil_div(p.rows, c->sm_count);
+    p.acc_per = 2 * kStemIssuers * p.BN <= 512 ? 2 : 1;
+    p.tmem_cols = pow2_cols(kStemIssuers * p.acc_per * p.BN);
+    p.x = (const __nv_bfloat16 *)x; p.w = (const __nv_bfloat16 *)w;
+    p.status = c->d_status;
+    p.ld_out = d->ldy;
+    const int grid = pt_ceil_div(p.rows, p.rows_per_cta);
+    p.stats_warp = pt_ceil_div(p.BN, 64) * (int)kStatsChunkBytes;
+    const size_t st_smem = c->stats_mode ? (size_t)8 * p.stats_warp : 0;
+    const size_t smem = 2048 + 8 * kSlabs * 4096 + (size_t)kStemRing * kStemSlot + (size_t)sp.U * sp.V * p.BN * 32 + st_smem;
+    p.stats_off = (int)(smem - st_smem);
+    CUtensorMap tmC;
+    cuuint64_t dims[4] = {(cuuint64_t)store_cols(d->K, d->ldy), (cuuint64_t)sp.Q, (cuuint64_t)sp.P, (cuuint64_t)d->N};
+    cuuint64_t strides[3] = {(cuuint64_t)d->ldy * 2, (cuuint64_t)sp.Q * d->ldy * 2, (cuuint64_t)sp.P * sp.Q * d->ldy * 2};
+    cuuint32_t box[4] = {64, 32, 1, 1}, estr[4] = {1, 1, 1, 1};
+    CUresult r = ((EncodeTiledFn)c->encode_tiled)(&tmC, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, y, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                                                  CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (!map_ok(r, __LINE__)) return PT_ERR_CUDA;
+    void (*kernel)(CUtensorMap, StemP) = c->stats_mode ? conv_stem_kernel<true> : conv_stem_kernel<false>;
+    if (!(c->attr_done & kAttrStem)) {
+        PT_CUDA_OK(cudaFuncSetAttribute(conv_stem_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+        PT_CUDA_OK(cudaFuncSetAttribute(conv_stem_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+        c->attr_done |= kAttrStem;
+    }
+    if (c->stats_mode) {
+        p.stats_lo = grid < kStatsFewRows ? 1 : 0;
+        c->stats_parts = grid * (1 + p.stats_lo);
+        if ((size_t)c->stats_parts * 2 * p.ld_out * sizeof(float) > c->stats_cap) return PT_ERR_WORKSPACE;
+        p.stats = c->stats_out;
+    }
+    PT_CUDA_OK(pt_launch_pdl(kernel, dim3((unsigned)grid), dim3(kStemThreads), smem, st, tmC, p));
+    c->launches += 1;
+    PT_CUDA_OK(cudaGetLastError());
+    return PT_OK;
+}
 
 // ---- launch shape of a weight gradient
 // The kernels cut the work three ways: tiles of dw (channels), groups of taps, and the pixels of the reduction over `splits` CTAs
@@ -3264,6 +3611,8 @@ pt_status pt_sm100_conv(pt_ctx *c, const pt_conv_desc *d, int which, const void 
     p.out = out;
     p.out_f32 = d->out_f32;
     if (which == PT_CONV_FWD && sp.ok) {
+        const pt_status direct = run_stem(c, d, sp, a, b, out, st);
+        if (direct != PT_ERR_UNSUPPORTED) return direct;
         char *wsb = (char *)ws;
         __nv_bfloat16 *xs = (__nv_bfloat16 *)wsb, *w2 = (__nv_bfloat16 *)(wsb + sp.xs_bytes);
         const size_t tot = (size_t)d->N * sp.Hs * sp.Wp;

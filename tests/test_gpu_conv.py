@@ -86,6 +86,35 @@ def test_config3_pruned_bottleneck(algo):
         Hh.check_conv(dw, l.C, oracle.conv_wgrad(x.numpy(), dy.numpy(), l.R, l.R, l.stride, pad), what=l.name + " wgrad")
 
 
+# (N, H, W, C, K, R, extra pitch of y) of the stem's kernel that reads the image itself: the narrowest and widest rows, every channel count, 3x3
+# to 7x7 filters, one and two 64-channel chunks, one and two accumulators an issuer, CTAs of one and several output rows, of several images
+@pytest.mark.parametrize("shape", [(2, 6, 128, 3, 16, 7, 0), (1, 2, 250, 1, 9, 3, 8), (3, 10, 200, 4, 65, 5, 0), (30, 42, 130, 2, 128, 3, 0), (31, 22, 160, 3, 55, 7, 8),
+                                   (200, 2, 224, 3, 20, 7, 0), (2, 224, 224, 3, 70, 7, 0)])
+def test_stem_straight_from_the_image(shape):
+    N, H, Wd, C, K, R, ey = shape
+    x, w, _, pad = _case(N, H, Wd, C, K, R, 2, seed=W.BASE_SEED + 47)
+    d = B.make_conv_desc(N, H, Wd, C, K, R, R, 2, pad, 8, W.pad8(K) + ey, W.pad8(C), 0, 2)
+    P, Q = (H + 2 * pad - R) // 2 + 1, (Wd + 2 * pad - R) // 2 + 1
+    xd, wd = Hh.to_dev_padded(x, 8), Hh.to_dev_padded(w, d.ldw)
+    y, y2 = Hh.out_buffer((N, P, Q), K, d.ldy, 0), Hh.out_buffer((N, P, Q), K, d.ldy, 0)
+    c = B.Context(0)
+    before = c.launch_count()
+    B.pt_conv_fwd(c, d, xd, wd, y, Hh.conv_ws(d, B.PT_CONV_FWD))
+    assert c.launch_count() == before + 1                        # (the space-to-depth copy would be two launches more)
+    stats = torch.full((B.pt_conv_fwd_stats_bytes(c, d) // 4,), float("nan"), device="cuda")
+    parts = B.pt_conv_fwd_stats(c, d, xd, wd, y2, stats, Hh.conv_ws(d, B.PT_CONV_FWD))
+    torch.cuda.synchronize()
+    c.poll()
+    Hh.check_conv(y, K, oracle.conv_fwd(x.numpy(), w.numpy(), 2, pad), what="stem")
+    assert torch.equal(y, y2)
+    sums = stats[:parts * 2 * d.ldy].view(parts, 2, d.ldy).double().sum(0)
+    v = y[..., :K].double()
+    # fp32 chains of a few hundred values, combined in fp64
+    assert torch.all((sums[0, :K] - v.sum((0, 1, 2))).abs() <= 1e-5 * v.abs().sum((0, 1, 2)))
+    assert torch.all((sums[1, :K] - (v * v).sum((0, 1, 2))).abs() <= 1e-5 * (v * v).sum((0, 1, 2)))
+    c.close()
+
+
 # (N, H, W, C, K, R, stride): stride-2 weight gradients with few input channels (the generic kernel and the stem path):
 # odd and even tap groups, K above and below 64, 5x5 and 7x7 stems
 STRIDED_SMALL_C = [
