@@ -8,9 +8,12 @@
 //                      position, 32-byte swizzle, one MMA per tap) runs the space-to-depth stem.
 //   conv_wgrad_kernel  weight gradient: both operands MN-major, reduction over pixels split across CTAs, partial tiles
 //                      summed in-kernel in a fixed order.
+//   conv_wgrad_taps_kernel  weight gradient by filter rows: the staged pixels of one serve all of its taps (stride 1 or 2, up to 170 channels).
+//   conv_wgrad_packed_kernel  weight gradient of narrow stride-1 layers: several pixels to a staged row.
 //   conv_wgrad_rows_kernel  weight gradient of stride-1 layers with at most 64 input channels: row blocks of x staged
 //                      once, taps as row-shifted descriptors, two or four taps per MMA on the M side; same finish phase.
-//   stem_* kernels     space-to-depth layout kernels of the few-channel stride-2 stem.
+//   conv_stem_kernel   forward pass of the few-channel stride-2 stem straight from the image.
+//   stem_* kernels     space-to-depth layout kernels of its weight gradient (and of forward passes that conv_stem_kernel does not take).
 // Ragged channel counts are handled by the TMA unit (true extents in the tensor maps: zero-fill on load, clipping on
 // store) and by skipping the 16-wide k-steps past the last valid channel.
 // Issue is spread over warps in all three kernels: one thread spends ~200 cycles per TMA instruction and 50-100 per
@@ -1153,9 +1156,11 @@ struct WgradP {
                             // channels; accumulator lanes = (tap, c), columns = k
     int lanes, dy_lanes;    // row-block form: channel lanes per staged pixel of x and of dy (rows of 128 or 64 bytes)
     int lane_shift;         // log2 of `lanes`
+    int row_lanes;          // packed form: channel lanes from one pixel of dy to the next (16 or 32)
     int acc_row;            // 32 lanes: accumulators per filter row, ceil(S / 4): each holds four neighbouring taps
     // filter-row form: the taps of one filter row share a unit; a tap is plane tap_plane[s] of the unit's x rows (stride 2: the columns of
     // either parity are a plane each), tap_shift[s] pixels on
+    int G;                  // packed form: pixels side by side in a staged row of x (64 / lanes)
     int planes;
     int plane_lo[2];                                    // first column of a unit's rows in either plane
     unsigned char tap_plane[kMaxRow], tap_shift[kMaxRow];
@@ -1315,6 +1320,84 @@ struct WgradShare {
     }
 };
 
+// One thread, behind a barrier of the threads that stored this split's partial sums: announces them, waits (bounded) for the tile's other
+// splits, and the last CTA to see that all have arrived clears the counters (nobody looks at them again). Every split CTA of a tile is
+// resident (the grid is at most one CTA per SM).
+__device__ __forceinline__ void wgrad_arrive(const WgradP &p, int split, volatile int *abort_flag)
+{
+    unsigned int *arrived = p.sync + 2 * blockIdx.x;
+    __threadfence();                                             // the CTA's stores (ordered before this by the barrier), then its arrival
+    // (test hook: split 0 stays silent, so that every split of the tile runs into the bounded wait below)
+    if (!(p.test_skip && split == 0)) atomicAdd(arrived, 1u);
+    const uint64_t t0 = globaltimer_ns();
+    unsigned int seen, polls = 0;
+    for (;;) {
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(arrived) : "memory");
+        if (seen >= (unsigned)p.splits || *abort_flag) break;
+        if ((++polls & 63u) == 0u && globaltimer_ns() - t0 > *(volatile unsigned long long *)&g_wait_limit_ns) {
+            record_timeout(p.status, 8);
+            *abort_flag = 1;
+            break;
+        }
+    }
+    if (seen >= (unsigned)p.splits && atomicAdd(arrived + 1, 1u) == (unsigned)p.splits - 1u) {
+        arrived[0] = 0u;
+        arrived[1] = 0u;
+    }
+}
+
+// Pieces of a chunk that `bytes` of shared memory hold from each of Z sources: an odd number (see wgrad_bring), at least one.
+__device__ __forceinline__ int wgrad_chunk(uint32_t bytes, int Z)
+{
+    const int cap = (int)(bytes / ((uint32_t)Z * 16u));
+    return cap - 1 + (cap & 1);
+}
+// All threads: the run of `n` 16-byte pieces at `src` of each of Z sources, `stride` pieces apart, into shared memory: piece i of source z
+// at z * (n | 1) + i (an odd pitch: lanes on neighbouring sources do not share a bank; with a source's pieces apart instead, the copies'
+// writes do: 418 -> 111 1x1 at 28x28, batch 64 20.4 -> 22.9 us).
+__device__ __forceinline__ void wgrad_bring(uint32_t dst, const float4 *src, size_t stride, int Z, int n)
+{
+    // copies are dealt out evenly, i fastest
+    const int pitch = n | 1;
+    int z = threadIdx.x / n, i = threadIdx.x - z * n;
+    const int dz = kThreads / n, di = kThreads - dz * n;
+    while (z < Z) {
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + (uint32_t)(z * pitch + i) * 16u), "l"(src + (size_t)z * stride + i) : "memory");
+        z += dz; i += di;
+        if (i >= n) { i -= n; ++z; }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+}
+
+// log2 of the lanes that share the sum of a piece: a share of few pieces of many sources is one thread's long chain of adds otherwise
+// (8 -> 8 3x3 at 32x32, batch 128 in the packed form: two pieces of 512 sources, 14.9 us against 10.7).
+__device__ __forceinline__ int wgrad_sum_lanes(int n, int Z)
+{
+    int ls = 0;
+    while (ls < 5 && (n << (ls + 1)) <= kThreads && (Z >> (ls + 1)) >= 4) ++ls;
+    return ls;
+}
+// Piece k of what wgrad_bring brought (k >= n: none), summed over the sources: each of L = 2^ls neighbouring lanes every L-th of them in
+// ascending order, then the lanes' sums pairwise: always the same way. Whole warps; the sum is in the first of the lanes.
+__device__ __forceinline__ float4 wgrad_sum(uint32_t base, int k, int n, int Z, int ls)
+{
+    float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int step = 1 << ls, z0 = (int)(threadIdx.x & (unsigned)(step - 1)), z1 = k < n ? Z : 0;
+    uint32_t a = base + (uint32_t)(z0 * (n | 1) + k) * 16u;
+#pragma unroll 4
+    for (int y = z0; y < z1; y += step, a += (uint32_t)(step * (n | 1)) * 16u) {
+        float4 t;
+        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(t.x), "=f"(t.y), "=f"(t.z), "=f"(t.w) : "r"(a) : "memory");
+        sum.x += t.x; sum.y += t.y; sum.z += t.z; sum.w += t.w;
+    }
+    for (int o = 1; o < step; o <<= 1) {
+        sum.x += __shfl_down_sync(0xffffffffu, sum.x, o); sum.y += __shfl_down_sync(0xffffffffu, sum.y, o);
+        sum.z += __shfl_down_sync(0xffffffffu, sum.z, o); sum.w += __shfl_down_sync(0xffffffffu, sum.w, o);
+    }
+    return sum;
+}
+
 // Everything after the main loop of a weight-gradient kernel: the accumulators leave TMEM (directly to dw, or as this
 // split's partial tile), the splits of a tile meet, and every CTA sums its share of the tile over the splits.
 // `ring_bytes` of shared memory at `data_base` are free by then and serve as staging. `tap0` is the CTA's first tap (generic form) or
@@ -1359,28 +1442,7 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, Ctl *ctl, uint32_t
                 if (warp == 2) WTRACE(4);
                 named_barrier(1, 256);
                 // ---- (2) every split CTA of this tile is resident (the grid is at most one CTA per SM): wait for all of them
-                unsigned int *arrived = p.sync + 2 * blockIdx.x;
-                if (gtid == 0) {
-                    __threadfence();                             // the CTA's stores (ordered before this by the barrier), then its arrival
-                    // (test hook: split 0 stays silent, so that every split of the tile runs into the bounded wait below)
-                    if (!(p.test_skip && split == 0)) atomicAdd(arrived, 1u);
-                    const uint64_t t0 = globaltimer_ns();
-                    unsigned int seen, polls = 0;
-                    for (;;) {
-                        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(arrived) : "memory");
-                        if (seen >= (unsigned)p.splits || *abort_flag) break;
-                        if ((++polls & 63u) == 0u && globaltimer_ns() - t0 > *(volatile unsigned long long *)&g_wait_limit_ns) {
-                            record_timeout(p.status, 8);
-                            *abort_flag = 1;
-                            break;
-                        }
-                    }
-                    // the last CTA to see that all have arrived clears the counters (nobody looks at them again)
-                    if (seen >= (unsigned)p.splits && atomicAdd(arrived + 1, 1u) == (unsigned)p.splits - 1u) {
-                        arrived[0] = 0u;
-                        arrived[1] = 0u;
-                    }
-                }
+                if (gtid == 0) wgrad_arrive(p, split, abort_flag);
                 named_barrier(1, 256);
                 if (warp == 2) WTRACE(5);
             } else if (p.pair) {
@@ -1460,30 +1522,16 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, Ctl *ctl, uint32_t
         const int it_beg = split * per_cta, it_end = min(total, it_beg + per_cta);
         const float4 *const pbase = reinterpret_cast<const float4 *>(p.partial + sh.split_off(p, 0, acc_cols));
         const size_t zstride = (size_t)p.apc * acc_cols * 32;                    // in pieces
-        const int cap = (int)(ring_bytes / ((uint32_t)p.splits * 16u));         // pieces the stage memory holds
+        const int cap = wgrad_chunk(ring_bytes, p.splits);         // pieces the stage memory holds
         const float inv_rows = 1.0f / (float)sh.rows, inv_quads = 1.0f / (float)sh.quads;
         for (int c_beg = it_beg; c_beg < it_end; c_beg += cap) {
             const int n_chunk = min(cap, it_end - c_beg);
-            // copies are dealt out evenly: piece i of split z, i fastest
-            int z = threadIdx.x / n_chunk, i = threadIdx.x - z * n_chunk;
-            const int dz = kThreads / n_chunk, di = kThreads - dz * n_chunk;
-            while (z < p.splits) {
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
-                             ::"r"(data_base + (uint32_t)(z * n_chunk + i) * 16u), "l"(pbase + (size_t)z * zstride + c_beg + i) : "memory");
-                z += dz; i += di;
-                if (i >= n_chunk) { i -= n_chunk; ++z; }
-            }
-            asm volatile("cp.async.wait_all;" ::: "memory");
-            __syncthreads();
-            for (int k = threadIdx.x; k < n_chunk; k += kThreads) {
-                float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
-                uint32_t a = data_base + (uint32_t)k * 16u;
-#pragma unroll 4
-                for (int y = 0; y < p.splits; ++y, a += (uint32_t)n_chunk * 16u) {
-                    float4 t;
-                    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(t.x), "=f"(t.y), "=f"(t.z), "=f"(t.w) : "r"(a) : "memory");
-                    sum.x += t.x; sum.y += t.y; sum.z += t.z; sum.w += t.w;
-                }
+            wgrad_bring(data_base, pbase + c_beg, zstride, p.splits, n_chunk);
+            const int ls = wgrad_sum_lanes(n_chunk, p.splits);
+            for (int i = threadIdx.x; i < (((n_chunk << ls) + 31) & ~31); i += kThreads) {
+                const int k = i >> ls;
+                const float4 sum = wgrad_sum(data_base, k, n_chunk, p.splits, ls);
+                if (k >= n_chunk || (i & ((1 << ls) - 1))) continue;
                 const int piece = c_beg + k, tq = fast_div(piece, sh.rows, inv_rows), row = piece - tq * sh.rows;
                 const int tt = fast_div(tq, sh.quads, inv_quads), col = (tq - tt * sh.quads) * 4;
                 if (p.pair) {
@@ -1951,6 +1999,208 @@ __global__ void __launch_bounds__(kThreads, 1) conv_wgrad_taps_kernel(const __gr
         if (warp == 1) WTRACE(2);
     }
     wgrad_finish(p, ctl, data_base, tmem_base, r * p.S, k0, c0, split, iters, p.data_bytes, p.S, p.BN);
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem_base, (uint32_t)p.tmem_cols);
+    }
+}
+
+// Packed form of the weight gradient: stride-1 filters of several columns whose pixels are 16 or 32 channels apart on both sides. G = 4 (or
+// 2) neighbouring pixels make one 128-byte row, pad lanes and all (they only reach sums that are not stored), so that the reduction runs
+// over rows of G pixels and a matrix instruction does 16 G pixels: with x rows of pixels G j .. and the row of the next G pixels on its M
+// side (2 G x 64 / G lanes) and G pixels of dy on its N side, the sums of the tap s are the blocks (pixel a + s of x, pixel a of dy),
+// a = 0 .. G - 1; the other blocks are dropped and these added when the splits are. A unit is `nr` such columns of an image, each a box of
+// 64 elements x all rows of the image (and the R - 1 that the filter reaches over, zeros on the dy side), column behind column, so that the
+// filter rows are row shifts with an accumulator each and the next G pixels are one column (`Wp` rows) on. Against the row-block form at
+// 32x32, 8 -> 14 channels: 17 x 3 instructions per image instead of 68 x 3, and half as many
+// staged rows: with 48 CTAs 22.3 -> 13.2 us at batch 128, alone 16.6 -> 11.3; 19 -> 19 at 56x56, batch 256 80.8 -> 53.1 and 37.2 -> 29.9. What is
+// left there is the exchange (the dropped blocks are not stored, but the G pixels are G sources each) and a box per column, 0.2 us a thread.
+__global__ void __launch_bounds__(kThreads, 1) conv_wgrad_packed_kernel(const __grid_constant__ CUtensorMap tmDy,
+                                                                     const __grid_constant__ CUtensorMap tmX, const WgradP p)
+{
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    Ctl *ctl = reinterpret_cast<Ctl *>(smem_raw);
+    const uint32_t smem_base = smem_u32(smem_raw);
+    const uint32_t data_base = (smem_base + (uint32_t)sizeof(Ctl) + 1023u) & ~1023u;
+    const uint32_t a_bytes = (uint32_t)p.nb_a * p.a_box, stage_bytes = a_bytes + p.b_box;
+    volatile int *abort_flag = &ctl->abort_flag;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int split = blockIdx.y, G = p.G, R = p.taps / p.S;
+    const int u_beg = split * p.units_per_split, u_end = min(p.units, u_beg + p.units_per_split);
+    const int iters = u_end > u_beg ? u_end - u_beg : 0;
+    const uint32_t dy_row = (uint32_t)p.dy_lanes * 2u;                // bytes of a staged row of dy: 128, or 64 (two pixels of 16 channels)
+    const uint32_t x_col = (uint32_t)p.Wp * 128u, dy_col = (uint32_t)p.Wp * dy_row;
+    const int boxes = p.nr + 1 + p.nr * p.nb_a, NP = boxes < 5 ? boxes : 5;          // of a unit; producer warps 0, 2, 3, 4, 5
+    const int NI = R < 4 ? R : 4;                                     // MMA issuer warps in use: filter rows i, i + NI, ...
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < p.stages; ++s) {
+            mbar_init(smem_u32(&ctl->full[s]), (uint32_t)NP);
+            mbar_init(smem_u32(&ctl->empty[s]), (uint32_t)NI);
+        }
+        mbar_init(smem_u32(&ctl->accum), (uint32_t)NI);
+        ctl->abort_flag = 0;
+        fence_mbar_init();
+        prefetch_tmap(&tmDy);
+        prefetch_tmap(&tmX);
+    }
+    // rows past the last column, up to the last 16-row step and the largest shift: dy zeros, x times zero and must be finite
+    {
+        const uint32_t a_used = (uint32_t)p.nr * dy_col, b_used = (uint32_t)(p.nr + 1) * x_col;
+        const uint32_t a_rest = (p.a_box - a_used) / 16u, b_rest = (p.b_box - b_used) / 16u, a_all = (uint32_t)p.nb_a * a_rest, per_stage = a_all + b_rest;
+        for (uint32_t i = threadIdx.x; i < (uint32_t)p.stages * per_stage; i += kThreads) {
+            const uint32_t st = i / per_stage, o = i - st * per_stage;
+            const uint32_t at = o < a_all ? o / a_rest * p.a_box + a_used + o % a_rest * 16u : a_bytes + b_used + (o - a_all) * 16u;
+            asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(data_base + st * stage_bytes + at), "r"(0u) : "memory");
+        }
+    }
+    fence_proxy_async();
+    if (warp == 1) {
+        tmem_alloc(smem_u32(&ctl->tmem_base), (uint32_t)p.tmem_cols);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = ctl->tmem_base;
+    const int issuer = warp == 1 ? 0 : warp - 5;                      // warps 6, 7, 8 -> issuers 1, 2, 3
+    const int pid = warp == 0 ? 0 : warp >= 2 && warp <= 5 ? warp - 1 : 5;
+    // nothing above touches global memory; the producer threads wait after their set-up
+    if (!(pid < NP && lane == 0)) grid_dependency_wait();
+    grid_launch_dependents();
+    if (threadIdx.x == 0) WTRACE(0);
+
+    if (pid < NP) {
+        if (lane == 0) {
+            // ---------------- producers: the boxes pid, pid + NP, ... of every unit: nr + 1 columns of x, then nr of each dy block
+            uint32_t my_bytes = 0;
+            for (int b = pid; b < boxes; b += NP) my_bytes += b <= p.nr ? x_col : dy_col;
+            const int x_step = G * p.lanes, dy_px = G * p.row_lanes;       // elements from one column to the next
+            int n = u_beg / p.RB, rb = u_beg - n * p.RB;
+            int s = 0, ph = 0, issued = 0;
+            grid_dependency_wait();
+            for (int it = 0; it < iters; ++it) {
+                if (!mbar_wait(smem_u32(&ctl->empty[s]), ph ^ 1, abort_flag, p.status, 4)) break;
+                const uint32_t bar = smem_u32(&ctl->full[s]);
+                const uint32_t a_dst = data_base + (uint32_t)s * stage_bytes, b_dst = a_dst + a_bytes;
+                mbar_arrive_expect_tx(bar, my_bytes);
+                const int j0 = rb * p.nr;
+                for (int b = pid; b < boxes; b += NP) {
+                    if (b <= p.nr) {
+                        tma_load_3d(b_dst + (uint32_t)b * x_col, &tmX, bar, (j0 + b) * x_step + p.lo_w * p.lanes, p.lo_h, n);
+                    } else {
+                        int j = b - p.nr - 1, blk = 0;
+                        if (j >= p.nr) { j -= p.nr; blk = 1; }
+                        tma_load_3d(a_dst + (uint32_t)blk * p.a_box + (uint32_t)j * dy_col, &tmDy, bar, (j0 + j) * dy_px + blk * 64, 0, n);
+                    }
+                }
+                if (++rb == p.RB) { rb = 0; ++n; }
+                issued = it + 1;
+                if (++s == p.stages) { s = 0; ph ^= 1; }
+            }
+            if (*abort_flag) drain_ring(smem_u32(&ctl->full[0]), p.stages, issued);
+        }
+        __syncwarp();
+    }
+    if (warp == 1 || (warp >= 6 && issuer < NI)) {
+        // ---------------- MMA issuer `issuer`: the warp walks the loop in lockstep, lane 0 issues
+        const uint32_t leader = lane == 0 ? 1u : 0u;
+        const uint32_t idesc = make_idesc_bf16(128, p.acc_cols, 1, 1);
+        const uint64_t dy_step = dy_row;                              // 16 rows further on, in units of 16 bytes
+        bool ok = true;
+        int s = 0, ph = 0;
+        for (int it = 0; it < iters && ok; ++it) {
+            ok = mbar_wait(smem_u32(&ctl->full[s]), ph, abort_flag, p.status, 5);
+            if (!ok) break;
+            if (it == 0 && warp == 1) WTRACE(1);
+            tc_fence_after();
+            const uint32_t a_src = data_base + (uint32_t)s * stage_bytes, b_src = a_src + a_bytes;
+            const uint64_t dyd = make_desc_mn(a_src, p.a_box, dy_row);
+            const uint32_t acc = it != 0 ? 1u : 0u;
+            for (int r = issuer; r < R; r += NI) {
+                const uint64_t xd = make_desc_mn(b_src + (uint32_t)r * 128u, x_col, 128u);
+                const uint32_t d_tmem = tmem_base + (uint32_t)(r * p.acc_cols);
+                umma_bf16_lead(d_tmem, xd, dyd, idesc, acc, leader);
+                for (int k = 1; k < p.ksteps; ++k) umma_bf16_lead(d_tmem, xd + 128ull * k, dyd + dy_step * k, idesc, 1u, leader);
+            }
+            umma_commit_lead(smem_u32(&ctl->empty[s]), leader);
+            if (++s == p.stages) { s = 0; ph ^= 1; }
+        }
+        if (ok) umma_commit_lead(smem_u32(&ctl->accum), leader);
+        if (warp == 1) WTRACE(2);
+    }
+
+    // ---------------- the sums: every split leaves G sources, one per pixel of dy in a row, of 16-byte pieces [filter row][four output
+    // channels][tap column, input channel]; then each sums its share over the sources of all splits (as wgrad_finish does)
+    const int KQ = pt_ceil_div_dev(p.K, 4), SC = p.S * p.C, total = R * KQ * SC;
+    float4 *const part = reinterpret_cast<float4 *>(p.partial);
+    if (warp >= 1) {
+        const int quarter = warp & 3, wset = (warp >= 2 && warp < 6) ? 0 : 1;
+        bool ok = true;
+        if (iters > 0) ok = mbar_wait(smem_u32(&ctl->accum), 0, abort_flag, p.status, 6);
+        if (warp == 2) WTRACE(3);
+        tc_fence_after();
+        if (ok) {
+            const uint32_t lane_addr = tmem_base + ((uint32_t)(quarter * 32) << 16);
+            const int l = quarter * 32 + lane, px = l >> p.lane_shift, c = l & (p.lanes - 1);
+            // (all of a row's loads before the one wait: a load and its wait take 0.2 us, and there are up to 24)
+            const bool here = c < p.C;
+            int ci = 0;
+            for (int r = 0; r < R; ++r)
+                for (int h = 0; h < p.K; h += 16, ++ci) {
+                    if ((ci & 1) != wset) continue;
+                    uint32_t v[4][16];
+#pragma unroll
+                    for (int a = 0; a < 4; ++a)
+                        if (a < G && iters > 0) tmem_ld16(lane_addr + (uint32_t)(r * p.acc_cols + a * p.row_lanes + h), v[a]);
+                    tmem_ld_wait();
+                    float4 *const d4 = part + (size_t)(split * G) * total + (size_t)(r * KQ + (h >> 2)) * SC + c;
+#pragma unroll
+                    for (int a = 0; a < 4; ++a) {
+                        const int t = px - a;
+                        if (a >= G || t < 0 || t >= p.S || !here) continue;
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            if ((h >> 2) + j < KQ)
+                                __stcg(d4 + (size_t)a * total + (size_t)j * SC + t * p.C,
+                                       iters > 0 ? make_float4(__uint_as_float(v[a][4 * j]), __uint_as_float(v[a][4 * j + 1]), __uint_as_float(v[a][4 * j + 2]),
+                                                               __uint_as_float(v[a][4 * j + 3]))
+                                                 : make_float4(0.f, 0.f, 0.f, 0.f));
+                    }
+                }
+        }
+        if (warp == 2) WTRACE(4);
+        named_barrier(1, 256);
+        if (warp == 1 && lane == 0) wgrad_arrive(p, split, abort_flag);
+        named_barrier(1, 256);
+        if (warp == 2) WTRACE(5);
+        tc_fence_before();
+    }
+    __syncthreads();
+    if (!*abort_flag) {
+        const int Z = p.splits * G, per_cta = (total + p.splits - 1) / p.splits;
+        const int it_beg = split * per_cta, it_end = min(total, it_beg + per_cta);
+        const int cap = wgrad_chunk(p.data_bytes, Z);
+        const float inv_sc = 1.0f / (float)SC, inv_kq = 1.0f / (float)KQ;
+        for (int c_beg = it_beg; c_beg < it_end; c_beg += cap) {
+            const int n_chunk = min(cap, it_end - c_beg);
+            wgrad_bring(data_base, part + c_beg, (size_t)total, Z, n_chunk);
+            const int ls = wgrad_sum_lanes(n_chunk, Z);
+            for (int i = threadIdx.x; i < (((n_chunk << ls) + 31) & ~31); i += kThreads) {
+                const int k = i >> ls;
+                const float4 sum = wgrad_sum(data_base, k, n_chunk, Z, ls);
+                if (k >= n_chunk || (i & ((1 << ls) - 1))) continue;
+                const int piece = c_beg + k, rq = fast_div(piece, SC, inv_sc), sc = piece - rq * SC, r = fast_div(rq, KQ, inv_kq), kk = (rq - r * KQ) * 4;
+                const float v4[4] = {sum.x, sum.y, sum.z, sum.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (kk + e < p.K) p.out[((size_t)(kk + e) * p.taps + r * p.S) * p.C + sc] = v4[e];      // (taps of a row side by side)
+            }
+            __syncthreads();
+        }
+        if (threadIdx.x == 0) WTRACE(6);
+    }
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem_base, (uint32_t)p.tmem_cols);
@@ -2992,21 +3242,21 @@ double wgrad_gen_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, pt_w
     return best;
 }
 
-// The row-block kernel (stride-1 filters with at most 64 input channels); false where the generic kernel is used.
-bool wgrad_rows_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, pt_wgrad_plan *w)
+// The row-block kernel (stride-1 filters with at most 64 input channels): the estimated time, 1e30 where it does not apply.
+double wgrad_rows_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, pt_wgrad_plan *w)
 {
     memset(w, 0, sizeof(*w));
     const int taps = d->R * d->S;
-    if (d->stride != 1 || taps > kMaxTaps) return false;
+    if (d->stride != 1 || taps > kMaxTaps) return 1e30;
     // a 1x1 filter has no halo to save, but the orientation (x on the M side, all of dy's channels on the N side: one tile
     // where the generic kernel needs two for K > 128) and the plain tiled loads (no im2col boxes on 96-byte pixel pitches)
     // still pay on large maps (56x56, 59 -> 143: 53 -> 31 us at 49 CTAs); small maps have too few units to split
-    if (taps < 2 && P * Q < 784) return false;
+    if (taps < 2 && P * Q < 784) return 1e30;
     w->Wp = Q + d->S - 1;
-    if (w->Wp > 256 || P < 1 || Q < 1) return false;
+    if (w->Wp > 256 || P < 1 || Q < 1) return 1e30;
     // paired form only: the x tile is the M side (two taps x 64 channel lanes), dy's output channels the N side
     w->acc_cols = pt_ceil_div(d->K, 16) * 16;
-    if (d->C > 64 || w->acc_cols > 256) return false;
+    if (d->C > 64 || w->acc_cols > 256) return 1e30;
     w->bn = tile_n(d->C, &w->n_tiles);
     w->m_tiles = 1;
     w->lanes = d->C <= 32 ? 32 : 64;
@@ -3051,7 +3301,7 @@ bool wgrad_rows_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, pt_wg
             w->splits = s; w->cluster = cl;
         }
     }
-    if (w->nr == 0) return false;
+    if (w->nr == 0) return 1e30;
     w->units_per_split = pt_ceil_div(w->units, w->splits);
     w->splits = pt_ceil_div(w->units, w->units_per_split);
     if (w->splits < 2) w->cluster = 0;
@@ -3059,7 +3309,7 @@ bool wgrad_rows_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, pt_wg
     w->smem = 2048 + (size_t)w->stages * w->stage_bytes;
     if (w->smem < 2048 + 8 * 2 * 4096) w->smem = 2048 + 8 * 2 * 4096;    // the epilogue's staging slabs reuse the ring
     w->rows = 1;
-    return true;
+    return best_us;
 }
 
 // Columns of an accumulator, and tiles of them, of the filter-row form: S accumulators fit the tensor memory.
@@ -3126,6 +3376,64 @@ double wgrad_taps_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, pt_
     return best;
 }
 
+// The packed kernel: pixels of x 16 or 32 channels apart, of dy too; a staged row of x (64 / ldx pixels, G) and the next one hold what the
+// S taps of G pixels read.
+bool wgrad_packed_ok(const pt_conv_desc *d, int P)
+{
+    if (d->stride != 1 || (d->ldx != 16 && d->ldx != 32) || (d->ldy != 16 && d->ldy != 32) || d->S < 2) return false;
+    const int G = 64 / d->ldx, N = G * d->ldy;
+    return d->S - 1 <= G && d->R * N <= 512 && P >= 1 && P + d->R <= 256;
+}
+// 16-byte pieces that a split leaves (one source per pixel of dy in a row).
+long long wgrad_packed_pieces(const pt_conv_desc *d) { return (long long)(64 / d->ldx) * d->R * pt_ceil_div(d->K, 4) * d->S * d->C; }
+
+double wgrad_packed_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, pt_wgrad_plan *w)
+{
+    memset(w, 0, sizeof(*w));
+    if (!wgrad_packed_ok(d, P) || Q < 1) return 1e30;
+    const int G = 64 / d->ldx, cols = pt_ceil_div(Q, G), shift = d->R - 1;
+    w->acc_cols = w->bn = G * d->ldy;
+    w->n_tiles = w->m_tiles = w->tap_groups = 1;
+    w->apc = w->tpc = d->R;
+    w->lanes = d->ldx;
+    w->dy_lanes = w->acc_cols < 64 ? 32 : 64;
+    w->nb_a = w->acc_cols / w->dy_lanes;
+    w->Wp = P + shift;
+    if (w->dy_lanes == 32) w->Wp += w->Wp & 1;             // (a column of 64-byte rows starts on 128 bytes)
+    const double bytes = (double)wgrad_packed_pieces(d) * 16.0;
+    double best = 1e30;
+    for (int nc = 1; nc <= cols; ++nc) {
+        const int ks = pt_ceil_div(nc * w->Wp, 16);
+        const size_t a_box = pt_align_up((size_t)ks * 16 * w->dy_lanes * 2, 1024), b_box = pt_align_up(((size_t)w->Wp + shift + (size_t)ks * 16) * 128, 1024);
+        const size_t stage = w->nb_a * a_box + b_box;
+        int st = (int)((220 * 1024 - 2048) / stage);
+        if (st < 2) break;
+        if (st > kMaxStages) st = kMaxStages;
+        const int rb = pt_ceil_div(cols, nc), units = d->N * rb, boxes = nc + 1 + nc * w->nb_a;
+        const double mma = ks * d->R * wg_mma_us(w->acc_cols, d->R > 1), issue = pt_ceil_div(boxes, 5) * 0.2;
+        const double load = w->Wp * ((nc + 1) * 0.95e-3 + nc * w->nb_a * (w->dy_lanes == 64 ? 0.95e-3 : 0.55e-3)), lat = 1.4 / (st - 1);
+        double unit = mma > load ? mma : load;
+        if (unit < issue) unit = issue;
+        unit = (unit > lat ? unit : lat) + 0.1;
+        // splits: as few as share the units in the same number of turns
+        const int most = wgrad_budget(c) < units ? wgrad_budget(c) : units, turns = pt_ceil_div(units, most), s = pt_ceil_div(units, turns);
+        const double us = 1.4 + turns * unit + (s > 1 ? wg_exchange_us(1, s, false, bytes) : 3.0 + bytes / 33e3);
+        if (us >= best) continue;
+        best = us;
+        w->nr = nc; w->ksteps = ks; w->a_box = (unsigned)a_box; w->b_box = (unsigned)b_box;
+        w->stages = st; w->stage_bytes = stage; w->RB = rb; w->units = units; w->units_per_split = turns;
+        w->splits = s;
+    }
+    if (w->nr == 0) return 1e30;
+    if (w->stages > w->units_per_split && w->units_per_split >= 2) w->stages = w->units_per_split;
+    w->smem = 2048 + (size_t)w->stages * w->stage_bytes;
+    if (w->smem < 2048 + 8 * 2 * 4096) w->smem = 2048 + 8 * 2 * 4096;
+    w->packed = 1;
+    return best;
+}
+
+size_t wgrad_workspace_bound(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, const pt_wgrad_plan &w);
+
 // The plan of a descriptor at the context's CTA limit. rows_only: only a row-block plan is asked for (its `rows` is 0 if there is none).
 pt_wgrad_plan wgrad_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, bool rows_only = false)
 {
@@ -3136,8 +3444,12 @@ pt_wgrad_plan wgrad_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, b
     const auto known = c->wgrad_plans.find(key);
     if (known != c->wgrad_plans.end()) return known->second;
     pt_wgrad_plan w;
-    if (!wgrad_rows_plan(c, d, P, Q, &w)) {
-        w.rows = 0;
+    const double rows_us = wgrad_rows_plan(c, d, P, Q, &w);
+    if (!rows_only && wgrad_packed_ok(d, P)) {
+        pt_wgrad_plan k;
+        if (wgrad_packed_plan(c, d, P, Q, &k) < (w.rows ? rows_us : 1e29)) w = k;
+    }
+    if (!w.rows && !w.packed) {
         if (!rows_only) {
             pt_wgrad_plan g;
             // (measured against estimated times at all SMs and at 49: within 10 % of each other, so that near a tie either may be the faster;
@@ -3146,6 +3458,7 @@ pt_wgrad_plan wgrad_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, b
             if (0.98 * wgrad_gen_plan(c, d, P, Q, &g) <= wgrad_taps_plan(c, d, P, Q, &w)) w = g;
         }
     }
+    w.ws_bytes = wgrad_workspace_bound(c, d, P, Q, w);
     if (c->wgrad_plans.size() >= pt_ctx::kWgradPlans) c->wgrad_plans.clear();
     c->wgrad_plans.emplace(key, w);
     return w;
@@ -3153,8 +3466,9 @@ pt_wgrad_plan wgrad_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, b
 
 // Workspace of the split weight gradient: one padded 128 x columns fp32 tile per (tile, split). (A cluster needs none, but the test
 // hook of the arrival wait turns one into an exchange through the workspace.)
-size_t wgrad_partial_bytes(const pt_wgrad_plan &w)
+size_t wgrad_partial_bytes(const pt_wgrad_plan &w, const pt_conv_desc *d)
 {
+    if (w.packed) return (size_t)wgrad_packed_pieces(d) * 16 * (size_t)w.splits;
     if (w.splits <= 1) return 0;
     return (size_t)w.n_tiles * w.m_tiles * w.tap_groups * w.apc * w.splits * 128 * w.acc_cols * sizeof(float);
 }
@@ -3178,9 +3492,14 @@ size_t wgrad_workspace_bound(const pt_ctx *c, const pt_conv_desc *d, int P, int 
         return tiles128 * 128 * cols;
     };
     const long long units = (long long)d->N * P, unit_s = units > 3 ? units / 2 : 1;
-    if (w.rows)
-        return (size_t)floats(w.lanes == 64 ? pt_ceil_div(taps, 2) : d->R * pt_ceil_div(d->S, 4), 512 / w.acc_cols < 16 ? 512 / w.acc_cols : 16, 1,
-                              w.n_tiles * w.m_tiles, w.acc_cols, unit_s) * sizeof(float);
+    const size_t packed = wgrad_packed_ok(d, P) ? (size_t)wgrad_packed_pieces(d) * 16 * (size_t)budget : 0;
+    if (w.rows || w.packed) {
+        pt_wgrad_plan r = w;                               // (either may be the choice of a smaller limit)
+        if (w.packed && wgrad_rows_plan(c, d, P, Q, &r) > 1e29) return packed;
+        const size_t rows = (size_t)floats(r.lanes == 64 ? pt_ceil_div(taps, 2) : d->R * pt_ceil_div(d->S, 4), 512 / r.acc_cols < 16 ? 512 / r.acc_cols : 16, 1,
+                              r.n_tiles * r.m_tiles, r.acc_cols, unit_s) * sizeof(float);
+        return rows > packed ? rows : packed;
+    }
     int bn, n_tiles;
     const int m_tiles = pt_ceil_div(d->K, 128);
     long long most = 0;
@@ -3193,7 +3512,8 @@ size_t wgrad_workspace_bound(const pt_ctx *c, const pt_conv_desc *d, int P, int 
         const long long t = floats(taps, d->S, taps, n_tiles * m_tiles, bt, unit_s);
         if (t > most) most = t;
     }
-    return (size_t)most * sizeof(float);
+    const size_t bytes = (size_t)most * sizeof(float);
+    return bytes > packed ? bytes : packed;
 }
 
 // Launch of a weight-gradient kernel: with programmatic stream serialization and, where the splits of a tile meet in shared memory,
@@ -3219,6 +3539,7 @@ pt_status wgrad_attr(const pt_ctx *c)
     if (!(c->attr_done & kAttrWgrad)) {
         PT_CUDA_OK(cudaFuncSetAttribute(conv_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
         PT_CUDA_OK(cudaFuncSetAttribute(conv_wgrad_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
+        PT_CUDA_OK(cudaFuncSetAttribute(conv_wgrad_packed_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
         PT_CUDA_OK(cudaFuncSetAttribute(conv_wgrad_taps_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024));
         c->attr_done |= kAttrWgrad;
     }
@@ -3265,9 +3586,9 @@ pt_status wgrad_common(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const pt_
     p->status = c->d_status;
     p->out = out;
     if (c->test_skip == 1 && p->splits > 1) { p->test_skip = 1; p->cluster = 0; c->test_skip = 0; }
-    if (p->splits > 1 && !p->cluster) {
+    if ((p->splits > 1 && !p->cluster) || w.packed) {
         const int gx = p->n_tiles * p->m_tiles * p->tap_groups;
-        if (!ws || ws_bytes < wgrad_partial_bytes(w)) return PT_ERR_WORKSPACE;
+        if (!ws || ws_bytes < wgrad_partial_bytes(w, d)) return PT_ERR_WORKSPACE;
         p->partial = (float *)ws;
         // two self-resetting counters per tile from the context's ring (kernels of one stream run in order, and the ring
         // is far larger than the tiles of the few launches that can be in flight)
@@ -3342,6 +3663,36 @@ pt_status run_wgrad_rows(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const p
     const size_t smem = (p.splits > 1 && wr.smem < kSplitSmemFloor) ? kSplitSmemFloor : wr.smem;
     p.data_bytes = (unsigned)(smem - 2048);
     PT_CUDA_OK(launch_wgrad(conv_wgrad_rows_kernel, grid, p.cluster ? p.splits : 1, smem, st, tmA, tmX, p));
+    c->launches += 1;
+    PT_CUDA_OK(cudaGetLastError());
+    return PT_OK;
+}
+
+// Launches the packed weight-gradient kernel.
+pt_status run_wgrad_packed(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const pt_wgrad_plan &wk, const void *x, const void *dy, float *out, void *ws,
+                           size_t ws_bytes, cudaStream_t st)
+{
+    WgradP p;
+    CUtensorMap tmA, tmX;
+    const pt_status r0 = wgrad_common(c, d, P, Q, wk, out, ws, ws_bytes, &p);
+    if (r0 != PT_OK) return r0;
+    p.G = 64 / d->ldx; p.lanes = d->ldx; p.lane_shift = d->ldx == 32 ? 5 : 4; p.dy_lanes = wk.dy_lanes; p.row_lanes = d->ldy;
+    p.lo_h = p.lo_w = -d->pad;
+    p.nr = wk.nr; p.Wp = wk.Wp; p.RB = wk.RB; p.units = wk.units; p.units_per_split = wk.units_per_split;
+    p.ksteps = wk.ksteps; p.nb_a = wk.nb_a; p.a_box = wk.a_box; p.b_box = wk.b_box; p.stages = wk.stages;
+    // image rows as rows of W x ld elements: a box of 64 (32) of them is the next pixels side by side, zeros past either end of the row
+    const auto map = [&](CUtensorMap *tm, const void *base, int W, int H, int ld, int lanes) {
+        cuuint64_t dims[3] = {(cuuint64_t)W * ld, (cuuint64_t)H, (cuuint64_t)d->N};
+        cuuint64_t strides[2] = {(cuuint64_t)W * ld * 2, (cuuint64_t)H * W * ld * 2};
+        cuuint32_t box[3] = {(cuuint32_t)lanes, (cuuint32_t)wk.Wp, 1}, estr[3] = {1, 1, 1};
+        return map_ok(((EncodeTiledFn)c->encode_tiled)(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), dims, strides, box, estr,
+                                                       CU_TENSOR_MAP_INTERLEAVE_NONE, lanes_swizzle(lanes), CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                                                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE), __LINE__);
+    };
+    if (!c->encode_tiled || !map(&tmA, dy, Q, P, d->ldy, wk.dy_lanes) || !map(&tmX, x, d->W, d->H, d->ldx, 64)) return PT_ERR_CUDA;
+    const size_t smem = (p.splits > 1 && wk.smem < kSplitSmemFloor) ? kSplitSmemFloor : wk.smem;
+    p.data_bytes = (unsigned)(smem - 2048);
+    PT_CUDA_OK(launch_wgrad(conv_wgrad_packed_kernel, dim3(1u, (unsigned)p.splits), 1, smem, st, tmA, tmX, p));
     c->launches += 1;
     PT_CUDA_OK(cudaGetLastError());
     return PT_OK;
@@ -3540,12 +3891,12 @@ size_t pt_sm100_conv_workspace(const pt_ctx *c, const pt_conv_desc *d, int which
     if (sp.ok && which == PT_CONV_WGRAD) {
         const pt_conv_desc v = stem_virtual_desc(d, sp), vr = stem_rows_desc(d, sp);
         const pt_wgrad_plan wa = wgrad_plan(c, &v, sp.P, sp.Q), wb = wgrad_plan(c, &vr, sp.P, sp.Q, true);
-        const size_t pa = wgrad_workspace_bound(c, &v, sp.P, sp.Q, wa), pb = wb.rows ? wgrad_workspace_bound(c, &vr, sp.P, sp.Q, wb) : 0;
+        const size_t pa = wa.ws_bytes, pb = wb.rows ? wb.ws_bytes : 0;
         return sp.xs_bytes + pt_align_up(sp.w2_elems * 4, 1024) + (pa > pb ? pa : pb);
     }
     if (which != PT_CONV_WGRAD) return 0;
     const int P = pt_out_dim(d->H, d->R, d->stride, d->pad), Q = pt_out_dim(d->W, d->S, d->stride, d->pad);
-    return wgrad_workspace_bound(c, d, P, Q, wgrad_plan(c, d, P, Q));
+    return wgrad_plan(c, d, P, Q).ws_bytes;
 }
 
 pt_status pt_sm100_conv(pt_ctx *c, const pt_conv_desc *d, int which, const void *a, const void *b, void *out, void *ws,
@@ -3586,6 +3937,7 @@ pt_status pt_sm100_conv(pt_ctx *c, const pt_conv_desc *d, int which, const void 
             return PT_OK;
         }
         pt_wgrad_plan w = wgrad_plan(c, d, P, Q);
+        if (w.packed) return run_wgrad_packed(c, d, P, Q, w, a, b, (float *)out, ws, ws_bytes, st);
         if (w.rows) {
             const pt_status r = run_wgrad_rows(c, d, P, Q, w, a, b, (float *)out, ws, ws_bytes, st);
             if (r != PT_ERR_UNSUPPORTED) return r;

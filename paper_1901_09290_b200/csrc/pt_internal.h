@@ -62,6 +62,8 @@ struct pt_wgrad_plan {
     int lanes, dy_lanes;            // channel lanes per staged pixel of x (64: two taps per accumulator, 32: four) and of dy
     unsigned a_box, b_box;
     size_t stage_bytes, smem;
+    size_t ws_bytes;                // workspace that a caller is asked for
+    int packed;                     // packed form (nr: columns per unit; Wp: rows of a column; RB, units, ... as above)
     int filter_row, planes;         // filter-row form (nr, Wp, RB, units, ksteps, nb_a, stages, boxes as above); x boxes per unit and block
 };
 

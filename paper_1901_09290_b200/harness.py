@@ -183,9 +183,9 @@ class TrainStep:
         self.h_reg = torch.zeros(1, dtype=torch.float64).pin_memory()
 
     def _wgrad_work(self, li: int) -> float:
-        """Rough device time (us on one SM) of a layer's weight gradient: the largest of its MMA count at 55+ cycles each,
-        its tensor bytes at the ~35 GB/s one SM pulls and, for the row-block kernel, its staged pixel rows at 2.4 ns each; only
-        ratios between layers are used."""
+        """Rough device time (us on one SM) of a layer's weight gradient: the largest of its MMA count at 48+ cycles each,
+        its tensor bytes at the ~35 GB/s one SM pulls and, for the row-block and packed kernels, its staged rows; only ratios between
+        layers are used."""
         l = self.net.layers[li]
         px = self.N * l.P * l.P
         taps = l.R * l.R
@@ -193,6 +193,11 @@ class TrainStep:
         if l.stride == 2 and l.C <= 4:                       # space-to-depth stem: (R+1)/2 vertical taps of 64 lanes, two per MMA
             mmas = px / 16 * (((l.R + 1) // 2 + 1) // 2)
             cyc = 55
+        elif l.stride == 1 and 2 <= l.R <= 3 and l.C > 4 and max(l.C, l.K) <= 32:    # packed kernel: G pixels of x in a row of 64 lanes
+            g = 64 // W.pad16(l.C)
+            mmas = px / (16 * g) * l.R * (l.P + l.R - 1) / l.P
+            t_rows = px / g * (1.2 + -(-g * W.pad16(l.K) // 64)) * 0.95e-3
+            cyc = 48 if g * W.pad16(l.K) <= 64 else 64
         elif l.stride == 1 and l.C <= 64:                    # row-block kernel: two taps per MMA (four of a row), N = K
             mmas = px / 16 * (l.R * -(-l.R // 4) if l.C <= 32 else (taps + 1) // 2)
             t_rows = px * (1 + -(-W.pad16(l.K) // 64) + (l.R - 1) / 3) * 2.4e-3

@@ -225,6 +225,34 @@ def test_filter_row_weight_gradient(shape):
     c.close()
 
 
+# (N, H, W, C, K, R, S, pad, ldx, ldy) of the packed form: either pitch on either side, one and two blocks of dy, rows that do not divide into
+# groups of four or two pixels, all padding and none, one to five filter rows and columns, an image of one column group, many images
+@pytest.mark.parametrize("shape", [(5, 12, 12, 11, 13, 3, 3, 1, 16, 16), (40, 32, 32, 16, 16, 3, 3, 1, 16, 16), (3, 9, 13, 8, 20, 3, 3, 1, 16, 32), (4, 14, 15, 27, 9, 3, 3, 1, 32, 16),
+                                   (20, 16, 16, 32, 32, 3, 3, 1, 32, 32), (3, 10, 11, 17, 31, 3, 3, 2, 32, 32), (3, 11, 10, 16, 7, 3, 3, 0, 16, 16), (2, 8, 9, 13, 12, 4, 5, 2, 16, 32),
+                                   (2, 7, 21, 30, 30, 1, 2, 0, 32, 32), (3, 2, 3, 5, 6, 3, 3, 1, 16, 16), (2, 56, 56, 19, 19, 3, 3, 1, 32, 32), (2, 200, 6, 9, 9, 5, 3, 2, 16, 16)])
+def test_packed_weight_gradient(shape):
+    N, H, Wd, C, K, R, S, pad, ldx, ldy = shape
+    x = W.gen_act(N, H, Wd, C, W.BASE_SEED + 45)
+    P, Q = H + 2 * pad - R + 1, Wd + 2 * pad - S + 1
+    dy = W.gen_dy(N, P, Q, K, W.BASE_SEED + 46)
+    ref = oracle.conv_wgrad(x.numpy(), dy.numpy(), R, S, 1, pad)
+    c = B.Context(0)
+    d = B.make_conv_desc(N, H, Wd, C, K, R, S, 1, pad, ldx, ldy, W.pad8(C), 0, 2)
+    xd, dyd = Hh.to_dev_padded(x, ldx), Hh.to_dev_padded(dy, ldy)
+    for limit in (0, 49, 5, 1):
+        B.pt_set_wgrad_cta_limit(c, limit)
+        ws = torch.empty(max(16, B.pt_conv_workspace_bytes(c, d, B.PT_CONV_WGRAD)), dtype=torch.uint8, device="cuda")
+        dw = torch.full((K, R, S, C), 7680.0, device="cuda")
+        B.pt_conv_wgrad(c, d, xd, dyd, dw, ws)
+        again = torch.full_like(dw, 7680.0)
+        B.pt_conv_wgrad(c, d, xd, dyd, again, ws)
+        torch.cuda.synchronize()
+        c.poll()
+        Hh.check_conv(dw, C, ref, what=f"wgrad at limit {limit}")
+        assert torch.equal(dw, again)
+    c.close()
+
+
 def test_wgrad_is_run_to_run_identical():
     N, H, C, K, R = 4, 14, 27, 19, 3
     x, w, dy, pad = _case(N, H, H, C, K, R, 1, W.BASE_SEED + 5)
