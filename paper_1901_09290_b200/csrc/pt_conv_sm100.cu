@@ -1160,6 +1160,7 @@ struct WgradP {
     int acc_row;            // 32 lanes: accumulators per filter row, ceil(S / 4): each holds four neighbouring taps
     // filter-row form: the taps of one filter row share a unit; a tap is plane tap_plane[s] of the unit's x rows (stride 2: the columns of
     // either parity are a plane each), tap_shift[s] pixels on
+    struct { int C, R, S, off; } stem;      // the space-to-depth stem: channels of the image (0: not the stem) and the real filter, for dw
     int G;                  // packed form: pixels side by side in a staged row of x (64 / lanes)
     int planes;
     int plane_lo[2];                                    // first column of a unit's rows in either plane
@@ -1192,6 +1193,21 @@ __device__ __forceinline__ int wgrad_tap(const WgradP &p, int acc, int g)
     if (p.lanes == 64) return min(2 * acc + g, p.taps);
     const int r = p.acc_row == 1 ? acc : acc / p.acc_row, s = (acc - r * p.acc_row) * 4 + g;
     return s < p.S ? r * p.S + s : p.taps;
+}
+
+// Row-block form: the sum of (output channel k, tap, lane c) goes to dw. In the stem a tap is a pair of filter rows and a lane one of four
+// neighbouring positions' (a, b, channel): filter row 2 tap + a - off, column 2 (c / 16) + b - off, where the filter has them. (A launch of
+// its own for this took 2 us and its start.)
+__device__ __forceinline__ void wgrad_pair_store(const WgradP &p, int k, int tap, int c, float v)
+{
+    if (k >= p.K) return;
+    if (p.stem.C) {
+        const int e = c & 15, ab = (e >= p.stem.C ? 1 : 0) + (e >= 2 * p.stem.C ? 1 : 0) + (e >= 3 * p.stem.C ? 1 : 0);
+        const int r = 2 * tap + (ab >> 1) - p.stem.off, s = 2 * (c >> 4) + (ab & 1) - p.stem.off, ch = e - ab * p.stem.C;
+        if (ch < p.stem.C && r >= 0 && r < p.stem.R && s >= 0 && s < p.stem.S) p.out[((size_t)(k * p.stem.R + r) * p.stem.S + s) * p.stem.C + ch] = v;
+        return;
+    }
+    p.out[((size_t)k * p.taps + tap) * p.C + c] = v;
 }
 
 // 32 columns (16 where the accumulator ends) of a warp's 32 TMEM lanes; zeros for a CTA that had no work.
@@ -1282,7 +1298,7 @@ __device__ __forceinline__ void wgrad_cluster_sum(const WgradP &p, Ctl *ctl, uin
                     const float v4[4] = {sum.x, sum.y, sum.z, sum.w};
 #pragma unroll
                     for (int e = 0; e < 4; ++e)
-                        if (col + e < p.K) p.out[((size_t)(col + e) * p.taps + tap) * p.C + c] = v4[e];
+                        wgrad_pair_store(p, col + e, tap, c, v4[e]);
                 }
             } else if (k0 + row < p.K && col < acc_cols && c0 + col < p.C) {
                 wgrad_store4(p.out + ((size_t)(k0 + row) * p.taps + tap0 + tt) * p.C + c0 + col, sum, min(4, p.C - (c0 + col)));
@@ -1465,7 +1481,7 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, Ctl *ctl, uint32_t
                     if (c >= p.C || tap >= p.taps) continue;
 #pragma unroll
                     for (int e = 0; e < 16; ++e)
-                        if (cc + e < p.K) p.out[((size_t)(cc + e) * p.taps + tap) * p.C + c] = __uint_as_float(v[e]);
+                        wgrad_pair_store(p, cc + e, tap, c, __uint_as_float(v[e]));
                 }
             } else {
             float *obase = p.out;
@@ -1542,7 +1558,7 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, Ctl *ctl, uint32_t
                         const float v4[4] = {sum.x, sum.y, sum.z, sum.w};
 #pragma unroll
                         for (int e = 0; e < 4; ++e)
-                            if (col + e < p.K) p.out[((size_t)(col + e) * p.taps + tap) * p.C + c] = v4[e];
+                            wgrad_pair_store(p, col + e, tap, c, v4[e]);
                     }
                     continue;
                 }
@@ -2574,6 +2590,8 @@ __global__ void __launch_bounds__(256) stem_s2d_x_kernel_t(const __nv_bfloat16 *
     dst[1] = *reinterpret_cast<uint4 *>(&o[8]);
 }
 
+// (Launched plainly: a dependency wait in each of the thousands of blocks costs more than an earlier start saves, 142 -> 159 us for the
+// weight gradient of 3 -> 19 at batch 256.)
 void stem_s2d_x_kernel_launch(unsigned blocks, cudaStream_t st, const __nv_bfloat16 *x, __nv_bfloat16 *xs, int N, int H, int W, int C,
                               int Hs, int Ws, int Wp, int pl)
 {
@@ -3638,9 +3656,10 @@ pt_status run_wgrad(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const pt_wgr
 
 // Launches the row-block weight-gradient kernel.
 // `x_row_pixels` > 0 and (lo_h, lo_w): x is a view whose rows are x_row_pixels apart and whose raster origin for tap (0, 0)
-// is at (lo_h, lo_w) instead of (-pad, -pad) -- the space-to-depth stem, whose "pixels" are overlapping 4-pixel windows.
+// is at (lo_h, lo_w) instead of (-pad, -pad) -- the space-to-depth stem, whose "pixels" are overlapping 4-pixel windows; `stem` is that
+// layer and out its dw.
 pt_status run_wgrad_rows(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const pt_wgrad_plan &wr, const void *x, const void *dy, float *out, void *ws,
-                         size_t ws_bytes, cudaStream_t st, int x_row_pixels = 0, int lo_h = 0, int lo_w = 0)
+                         size_t ws_bytes, cudaStream_t st, int x_row_pixels = 0, int lo_h = 0, int lo_w = 0, const pt_conv_desc *stem = nullptr, int off = 0)
 {
     if (!c->encode_tiled) return PT_ERR_CUDA;
     WgradP p;
@@ -3650,6 +3669,7 @@ pt_status run_wgrad_rows(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const p
     p.pair = 1;
     p.stride = 1; p.lo_h = -d->pad; p.lo_w = -d->pad;
     if (x_row_pixels > 0) { p.lo_h = lo_h; p.lo_w = lo_w; }
+    if (stem) { p.stem.C = stem->C; p.stem.R = stem->R; p.stem.S = stem->S; p.stem.off = off; }
     p.nr = wr.nr; p.Wp = wr.Wp; p.RB = wr.RB; p.units = wr.units; p.units_per_split = wr.units_per_split;
     p.ksteps = wr.ksteps; p.nb_a = wr.nb_a; p.lo_span = d->R - 1; p.a_box = wr.a_box; p.b_box = wr.b_box;
     p.stages = wr.stages;
@@ -3914,15 +3934,17 @@ pt_status pt_sm100_conv(pt_ctx *c, const pt_conv_desc *d, int which, const void 
             char *part = wsb + sp.xs_bytes + pt_align_up(sp.w2_elems * 4, 1024);
             const pt_conv_desc v = stem_virtual_desc(d, sp);
             const size_t tot = (size_t)d->N * sp.Hs * sp.Wp;
-            stem_s2d_x_kernel_launch((unsigned)((tot + 255) / 256), st, (const __nv_bfloat16 *)a, xs, d->N, d->H, d->W, d->C, sp.Hs, sp.Ws,
-                                     sp.Wp, sp.pl);
+            stem_s2d_x_kernel_launch((unsigned)((tot + 255) / 256), st, (const __nv_bfloat16 *)a, xs, d->N, d->H, d->W, d->C, sp.Hs, sp.Ws, sp.Wp, sp.pl);
             c->launches += 1;
             // the row-block kernel first: the windows of a unit of rows are staged once for all U vertical taps and two taps share
             // an MMA (M = 128 lanes where the generic kernel has 55 output channels on its M side)
             const pt_conv_desc vr = stem_rows_desc(d, sp);
             const pt_wgrad_plan wr = wgrad_plan(c, &vr, sp.P, sp.Q, true);
             pt_status r = PT_ERR_UNSUPPORTED;
-            if (wr.rows) r = run_wgrad_rows(c, &vr, sp.P, sp.Q, wr, xs, b, dw2, part, ws_bytes - (size_t)(part - wsb), st, sp.Wp, -sp.pl, 0);
+            if (wr.rows) {
+                r = run_wgrad_rows(c, &vr, sp.P, sp.Q, wr, xs, b, (float *)out, part, ws_bytes - (size_t)(part - wsb), st, sp.Wp, -sp.pl, 0, d, sp.off);
+                if (r != PT_ERR_UNSUPPORTED) return r;
+            }
             if (r == PT_ERR_UNSUPPORTED) {
                 CUtensorMap tmX;
                 const int up_h = (sp.P - 1) - sp.pl - (sp.Hs - 1);
@@ -3968,8 +3990,7 @@ pt_status pt_sm100_conv(pt_ctx *c, const pt_conv_desc *d, int which, const void 
         char *wsb = (char *)ws;
         __nv_bfloat16 *xs = (__nv_bfloat16 *)wsb, *w2 = (__nv_bfloat16 *)(wsb + sp.xs_bytes);
         const size_t tot = (size_t)d->N * sp.Hs * sp.Wp;
-        stem_s2d_x_kernel_launch((unsigned)((tot + 255) / 256), st, (const __nv_bfloat16 *)a, xs, d->N, d->H, d->W, d->C, sp.Hs, sp.Ws, sp.Wp,
-                                 sp.pl);
+        stem_s2d_x_kernel_launch((unsigned)((tot + 255) / 256), st, (const __nv_bfloat16 *)a, xs, d->N, d->H, d->W, d->C, sp.Hs, sp.Ws, sp.Wp, sp.pl);
         stem_s2d_w_kernel<<<(unsigned)((sp.w2_elems + 255) / 256), 256, 0, st>>>((const __nv_bfloat16 *)b, w2, d->K, d->R, d->S, d->C, d->ldw,
                                                                               sp.U, sp.V, sp.off);
         c->launches += 2;
