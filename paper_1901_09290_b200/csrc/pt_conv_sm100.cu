@@ -747,8 +747,20 @@ constexpr int kHaloThreads = 512;
 // kernel therefore runs up to four issuer warps, each on its own scheduler: issuer i owns accumulator buffer i and
 // an A ring of its own (a waiter may lag an mbarrier by at most one phase, so issuers cannot share a ring), and takes
 // the tiles i, i + I, i + 2I, ... of the CTA. Weights that stream through a ring keep a single issuer.
-template <bool B_MN, bool STATS>
-__global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid_constant__ CUtensorMap tmA,
+//   PL = 4: the forward pass at stride 2. The source pixels of either row and column parity are a plane (every other pixel: a tensor map of its
+// own) in which the taps that read it are shifts of one pixel as at stride 1, so that every chunk of 64 channels is four boxes, each with its
+// own taps, all into one accumulator. The im2col form loads a tile's 128 pixels once per tap (2304 rows a tile of 106 channels and nine taps
+// against 1160). At PL = 1 the loops' bounds are read from the parameters as they stand: held in variables they cost the streamed layers 1 %
+// (28x28, 106 -> 103, batch 64 19.1 and 19.35 us).
+template <int PL> struct HaloMaps {
+    CUtensorMap m[PL];
+    int tap[PL + 1];           // the taps of plane i are tap[i] .. tap[i + 1] - 1
+    int lo_h[PL], lo_w[PL];    // source coordinate of raster position (0, 0) in it
+};
+template <> struct HaloMaps<1> { CUtensorMap m[1]; };
+
+template <bool B_MN, bool STATS, int PL>
+__global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid_constant__ HaloMaps<PL> tmA,
                                                                      const __grid_constant__ CUtensorMap tmB,
                                                                      const __grid_constant__ CUtensorMap tmC, const HaloP p)
 {
@@ -769,6 +781,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
     const int m_tiles = p.N * p.row_tiles;
     const int total_tiles = m_tiles * p.n_tiles;
     const int NI = p.n_issuers, SR = p.stages_a / NI;        // issuers, A stages per issuer ring
+    const int boxes = p.k_chunks * PL;                       // activation boxes of a tile: chunk by chunk, every plane of it
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < p.stages_a; ++s) { mbar_init(smem_u32(&ctl->full_a[s]), 1); mbar_init(smem_u32(&ctl->empty_a[s]), 1); }
@@ -777,7 +790,8 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
         for (int b = 0; b < 2 * kHaloMaxIssuers; ++b) { mbar_init(smem_u32(&ctl->acc_full[b]), 1); mbar_init(smem_u32(&ctl->acc_empty[b]), 4); }
         ctl->abort_flag = 0;
         fence_mbar_init();
-        prefetch_tmap(&tmA);
+#pragma unroll
+        for (int i = 0; i < PL; ++i) prefetch_tmap(&tmA.m[i]);
         prefetch_tmap(&tmB);
         if (p.tma_store) prefetch_tmap(&tmC);
     }
@@ -829,10 +843,10 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
             int tc = pid;
             TileWalk tw;
             tw.init((int)blockIdx.x + pid * (int)gridDim.x, n_prod * (int)gridDim.x, p.n_tiles, p.row_tiles);
-            // ring = tc % NI; every ring has carried (tc / NI) * k_chunks chunks before its tile of this round: position and
+            // ring = tc % NI; every ring has carried (tc / NI) * boxes boxes before its tile of this round: position and
             // phase of that count in a ring of SR stages, advanced per round
             int ring = pid % NI, base_pos = 0, base_ph = 0;
-            const int kdiv = p.k_chunks / SR, kmod = p.k_chunks - kdiv * SR;
+            const int kdiv = boxes / SR, kmod = boxes - kdiv * SR;
             int sb_pos = 0, sb_ph = 0;                         // position in this pipeline's weight ring
             const int skip_a = p.test_skip;
             int issued_a = 0, issued_b = 0;                    // stages filled (a producer of activations feeds one ring)
@@ -841,7 +855,10 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
                 const int n0 = tw.n_tile * p.BN;
                 bool ok = true;
                 int pos = base_pos, pha = base_ph;
-                for (int kc = 0; kc < p.k_chunks && ok; ++kc) {
+                for (int bx = 0; bx < p.k_chunks * PL && ok; ++bx) {
+                    const int kc = bx / PL, pl = bx % PL;
+                    [[maybe_unused]] int tap0 = 0, tap1 = 0, lo_h = p.lo_h, lo_w = p.lo_w;
+                    if constexpr (PL > 1) { tap0 = tmA.tap[pl]; tap1 = tmA.tap[pl + 1]; lo_h = tmA.lo_h[pl]; lo_w = tmA.lo_w[pl]; }
                     const int sa = ring * SR + pos, ph_use = pha;
                     if (++pos == SR) { pos = 0; pha ^= 1; }
                     if (a_role) {
@@ -852,11 +869,11 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
                         mbar_arrive_expect_tx(bar, (uint32_t)p.a_box_bytes);
                         if (!dep_waited) { grid_dependency_wait(); dep_waited = true; }
                         if (issued_a >= skip_a)                // (test hook: the first stage never becomes full)
-                            tma_load_4d(a_base + (uint32_t)sa * (uint32_t)p.a_alloc, &tmA, bar, kc * kKC, p.lo_w, p0 + p.lo_h, img);
+                            tma_load_4d(a_base + (uint32_t)sa * (uint32_t)p.a_alloc, &tmA.m[pl], bar, kc * kKC, lo_w, p0 + lo_h, img);
                         ++issued_a;
                     }
                     if (!b_role) continue;
-                    for (int tap = 0; tap < p.taps; ++tap) {
+                    for (int tap = PL > 1 ? tap0 : 0; tap < (PL > 1 ? tap1 : p.taps); ++tap) {
                         const int sb = (p.shared_b ? 0 : pid * SB) + sb_pos, phb = sb_ph;
                         if (++sb_pos == SB) { sb_pos = 0; sb_ph ^= 1; }
                         ok = mbar_wait(smem_u32(&ctl->empty_b[sb]), phb ^ 1, abort_flag, p.status, 12);
@@ -873,7 +890,7 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
                 if (!ok) break;
                 tw.next();
                 ring += n_prod;
-                while (ring >= NI) {                           // next round: every ring has carried k_chunks more
+                while (ring >= NI) {                           // next round: every ring has carried `boxes` more
                     ring -= NI;
                     base_pos += kmod;
                     int wraps = kdiv;
@@ -921,7 +938,10 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
             tc_fence_after();
             const uint32_t d_tmem = tmem_base + (uint32_t)(b * p.BN);
             uint32_t accumulate = 0u;
-            for (int kc = 0; kc < p.k_chunks && ok; ++kc) {
+            for (int bx = 0; bx < p.k_chunks * PL && ok; ++bx) {
+                const int kc = bx / PL;
+                [[maybe_unused]] int t0 = 0, t1 = 0;
+                if constexpr (PL > 1) { t0 = tmA.tap[bx % PL]; t1 = tmA.tap[bx % PL + 1]; }
                 const int sa = issuer * SR + s_loc;
                 ok = mbar_wait(smem_u32(&ctl->full_a[sa]), pha, abort_flag, p.status, 15);
                 if (!ok) break;
@@ -932,27 +952,27 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
                 const uint64_t abase = a_desc0 | desc_addr(a_base + (uint32_t)sa * (uint32_t)p.a_alloc);
                 if (p.resident) {
                     // every tap is the same A tile read through a descriptor that starts (r*Wp + s) rows further on
-                    uint64_t bd0 = b_desc0 | desc_addr(b_base + (uint32_t)kc * b_slot);
+                    uint64_t bd0 = b_desc0 | desc_addr(b_base + (uint32_t)(t0 * p.k_chunks + kc) * b_slot);
                     const uint64_t b_tap_step = (uint64_t)(((uint32_t)p.k_chunks * b_slot) >> 4);
                     if (ksteps == 1) {
-                        for (int tap = 0; tap < p.taps; ++tap, bd0 += b_tap_step) {
+                        for (int tap = PL > 1 ? t0 : 0; tap < (PL > 1 ? t1 : p.taps); ++tap, bd0 += b_tap_step) {
                             umma_bf16_lead(d_tmem, abase + ctl->tap_aoff[tap], bd0, idesc, accumulate, leader);
                             accumulate = 1u;
                         }
                     } else if (ksteps == 4) {
-                        for (int tap = 0; tap < p.taps; ++tap, bd0 += b_tap_step) {
+                        for (int tap = PL > 1 ? t0 : 0; tap < (PL > 1 ? t1 : p.taps); ++tap, bd0 += b_tap_step) {
                             const uint64_t ad0 = abase + ctl->tap_aoff[tap];
 #pragma unroll
                             for (int k = 0; k < 4; ++k) { umma_bf16_lead(d_tmem, ad0 + 2ull * k, bd0 + bstep * k, idesc, accumulate, leader); accumulate = 1u; }
                         }
                     } else {
-                        for (int tap = 0; tap < p.taps; ++tap, bd0 += b_tap_step) {
+                        for (int tap = PL > 1 ? t0 : 0; tap < (PL > 1 ? t1 : p.taps); ++tap, bd0 += b_tap_step) {
                             const uint64_t ad0 = abase + ctl->tap_aoff[tap];
                             for (int k = 0; k < ksteps; ++k) { umma_bf16_lead(d_tmem, ad0 + 2ull * k, bd0 + bstep * k, idesc, accumulate, leader); accumulate = 1u; }
                         }
                     }
                 } else {
-                    for (int tap = 0; tap < p.taps; ++tap) {
+                    for (int tap = PL > 1 ? t0 : 0; tap < (PL > 1 ? t1 : p.taps); ++tap) {
                         const int sb = (p.shared_b ? 0 : issuer * SB) + sb_pos, phb = sb_ph;
                         if (++sb_pos == SB) { sb_pos = 0; sb_ph ^= 1; }
                         ok = mbar_wait(smem_u32(&ctl->full_b[sb]), phb, abort_flag, p.status, 16);
@@ -2881,15 +2901,16 @@ bool make_halo_in_map(const pt_ctx *c, CUtensorMap *tm, const void *base, int C,
 
 // The pixels (a + i * stride, b + j * stride) of bf16 activations as a tiled 4-D tensor (C, columns j, rows i, N): box 64 channels x box_w x
 // box_h x 1.
-bool make_plane_map(const pt_ctx *c, CUtensorMap *tm, const void *base, int C, int W, int H, int N, int ld, int stride, int a, int b, int box_w, int box_h)
+bool make_plane_map(const pt_ctx *c, CUtensorMap *tm, const void *base, int C, int W, int H, int N, int ld, int stride, int a, int b, int box_w, int box_h,
+                    int lanes = kKC)
 {
     if (!c->encode_tiled || box_w > 256 || box_h > 256 || a >= H || b >= W) return false;
     const char *first = (const char *)base + ((size_t)a * W + b) * ld * 2;
     cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)pt_ceil_div(W - b, stride), (cuuint64_t)pt_ceil_div(H - a, stride), (cuuint64_t)N};
     cuuint64_t strides[3] = {(cuuint64_t)stride * ld * 2, (cuuint64_t)stride * W * ld * 2, (cuuint64_t)H * W * ld * 2};
-    cuuint32_t box[4] = {(cuuint32_t)kKC, (cuuint32_t)box_w, (cuuint32_t)box_h, 1}, estr[4] = {1, 1, 1, 1};
+    cuuint32_t box[4] = {(cuuint32_t)lanes, (cuuint32_t)box_w, (cuuint32_t)box_h, 1}, estr[4] = {1, 1, 1, 1};
     CUresult r = ((EncodeTiledFn)c->encode_tiled)(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<char *>(first), dims, strides, box, estr,
-                                                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                                                  CU_TENSOR_MAP_INTERLEAVE_NONE, lanes_swizzle(lanes), CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                                                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return map_ok(r, __LINE__);
 }
@@ -2905,14 +2926,15 @@ struct HaloSpec {
     int n_cols, ld_out;                              // output channels and pitch
     int oH, oW, o_step, o_h0, o_w0;                  // output view: raster (i, j) -> pixel (i*o_step + o_h0, j*o_step + o_w0) of oH x oW
     int row32, w_taps;                               // 16-lane pixels (32-byte rows); taps per output channel in the weight tensor
+    int plane_tap[5], plane_lo_h[4], plane_lo_w[4];  // stride-2 forward: the taps in the order of their parity planes, and where those start
     int max_ctas;                                    // > 0: grid limit (launches meant to run side by side share the SMs)
 };
 
-template <bool B_MN>
+template <bool B_MN, int PL = 1>
 pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const void *w, void *out, cudaStream_t st)
 {
     const int Wp = h.Q + h.span_w - 1;
-    if (h.n_taps < 1 || h.n_taps > kMaxTaps || Wp > 128 || h.Ws > 250) return PT_ERR_UNSUPPORTED;
+    if (h.n_taps < 1 || h.n_taps > kMaxTaps || Wp > 128 || (PL == 1 && h.Ws > 250)) return PT_ERR_UNSUPPORTED;
     HaloP p;
     memset(&p, 0, sizeof(p));
     p.N = d->N; p.P = h.P; p.Q = h.Q; p.Wp = Wp;
@@ -2920,6 +2942,11 @@ pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const
     p.row_tiles = pt_ceil_div(h.P, p.nr);
     p.n_cols = h.n_cols;
     p.BN = tile_n(h.n_cols, &p.n_tiles);
+    // The planes pay where a CTA has several tiles, so that the boxes of one are on their way while another's are multiplied; with one or two
+    // the im2col form's many small loads are sooner there (3x3/2, planes against im2col: 106 -> 103 at 56x56, batch 64, 448 tiles 23.6 and 25.7 us,
+    // 38 -> 38 at 56x56, batch 256 33.7 and 48.5, 8 -> 17 at 32x32, batch 128, 384 tiles 6.4 and 10.6; 64 -> 128 at 32x32, batch 64, 192
+    // tiles 11.1 and 7.9; 200 -> 200 at 28x28, batch 64, 128 tiles 23.4 and 19.6).
+    if (PL > 1 && (long long)p.N * p.row_tiles * p.n_tiles <= 2 * c->sm_count) return PT_ERR_UNSUPPORTED;
     p.c_red = h.Cs; p.k_chunks = pt_ceil_div(h.Cs, kKC); p.taps = h.n_taps;
     // Channel lanes per staged pixel: narrow layers take rows of 64 or 32 bytes. The TMA unit's time is per row, and a row whose tensor
     // ends in the middle of a sector costs it twice as much in a 128-byte box (4.5 ns for 19 channels) as a whole one (2.3 ns); in a
@@ -2977,7 +3004,7 @@ pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const
         // of its own -- a chunk that waits for the previous chunk's MMAs to free its stage exposes a DRAM round trip per tile
         // (28x28, 69 -> 93 channels, MN-major weights: two stages against four, 30 -> 22 us) -- as long as four weight stages
         // remain for the shared stream.
-        const int want_a = 2 * p.k_chunks > 4 ? 4 : 2 * p.k_chunks;
+        const int want_a = 2 * p.k_chunks * PL > 4 ? 4 : 2 * p.k_chunks * PL;
         if (two_pipes && p.n_tiles == 1 && left >= (size_t)want_a * p.a_alloc + 4 * b_bytes) {
             const size_t sb2 = (left - (size_t)want_a * p.a_alloc) / b_bytes;
             if ((size_t)p.stages_b > sb2) p.stages_b = (int)sb2;
@@ -3009,11 +3036,17 @@ pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const
     p.out = out; p.ld_out = h.ld_out; p.out_f32 = d->out_f32;
     p.oH = h.oH; p.oW = h.oW; p.o_step = h.o_step; p.o_h0 = h.o_h0; p.o_w0 = h.o_w0;
     p.status = c->d_status;
-    CUtensorMap tmA, tmB, tmC;
+    HaloMaps<PL> tmA;
+    if constexpr (PL > 1) {
+        memcpy(tmA.tap, h.plane_tap, sizeof(tmA.tap));
+        memcpy(tmA.lo_h, h.plane_lo_h, sizeof(tmA.lo_h));
+        memcpy(tmA.lo_w, h.plane_lo_w, sizeof(tmA.lo_w));
+    }
+    CUtensorMap tmB, tmC;
     memset(&tmC, 0, sizeof(tmC));
     if (h.row32) {
         if (!p.resident) return PT_ERR_UNSUPPORTED;
-        if (!make_halo_in_map(c, &tmA, h.src, h.Cs, h.Ws, h.Hs, d->N, h.lds, Wp, box_h, 16)) return PT_ERR_CUDA;
+        if (!make_halo_in_map(c, &tmA.m[0], h.src, h.Cs, h.Ws, h.Hs, d->N, h.lds, Wp, box_h, 16)) return PT_ERR_CUDA;
         // weights [K][w_taps][16]: one 32-byte row per output channel and tap
         cuuint64_t dims[3] = {16, (cuuint64_t)h.w_taps, (cuuint64_t)h.n_cols};
         cuuint64_t strides[2] = {32, (cuuint64_t)h.w_taps * 32};
@@ -3023,7 +3056,9 @@ pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const
                                                       CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (!map_ok(r, __LINE__)) return PT_ERR_CUDA;
     } else {
-        if (!make_halo_in_map(c, &tmA, h.src, h.Cs, h.Ws, h.Hs, d->N, h.lds, Wp, box_h, p.lanes)) return PT_ERR_CUDA;
+        for (int i = 0; i < PL; ++i)
+            if (PL == 1 ? !make_halo_in_map(c, &tmA.m[0], h.src, h.Cs, h.Ws, h.Hs, d->N, h.lds, Wp, box_h, p.lanes)
+                        : !make_plane_map(c, &tmA.m[i], h.src, h.Cs, h.Ws, h.Hs, d->N, h.lds, 2, i >> 1, i & 1, Wp, box_h, p.lanes)) return PT_ERR_CUDA;
         if (!make_weight_map(c, &tmB, w, d->C, d->R * d->S, d->K, d->ldw, B_MN ? p.lanes : p.b_rows, B_MN ? kKC : p.lanes)) return PT_ERR_CUDA;
     }
     if (p.tma_store) {
@@ -3042,9 +3077,9 @@ pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const
     const size_t smem = 2048 + 2 * (size_t)p.slabs * p.staging + (p.resident ? w_all : (size_t)p.stages_b * b_bytes) + (size_t)p.stages_a * p.a_alloc + a_tail +
                         st_smem;
     p.stats_off = (int)(smem - st_smem);
-    void (*kernel)(CUtensorMap, CUtensorMap, CUtensorMap, HaloP) =
-        (!B_MN && c->stats_mode) ? conv_halo_kernel<false, true> : conv_halo_kernel<B_MN, false>;
-    const int kid = (!B_MN && c->stats_mode) ? 2 : (B_MN ? 1 : 0);
+    void (*kernel)(HaloMaps<PL>, CUtensorMap, CUtensorMap, HaloP) =
+        (!B_MN && c->stats_mode) ? conv_halo_kernel<false, true, PL> : conv_halo_kernel<B_MN, false, PL>;
+    const int kid = PL > 1 ? (c->stats_mode ? 13 : 12) : (!B_MN && c->stats_mode) ? 2 : (B_MN ? 1 : 0);
     if (!(c->attr_done & (kAttrHalo << kid))) {
         PT_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
         c->attr_done |= kAttrHalo << kid;
@@ -3144,6 +3179,38 @@ pt_status run_stem(pt_ctx *c, const pt_conv_desc *d, const StemPlan &sp, const v
     c->launches += 1;
     PT_CUDA_OK(cudaGetLastError());
     return PT_OK;
+}
+
+// Stride-2 forward by parity planes; false where some plane has no tap or the image not both parities.
+bool halo_spec_stride2(const pt_conv_desc *d, HaloSpec *h, const void *src, int P, int Q)
+{
+    memset(h, 0, sizeof(*h));
+    if (d->stride != 2 || d->H < 2 || d->W < 2 || d->R * d->S > kMaxTaps) return false;
+    h->src = src; h->Cs = d->C; h->Ws = d->W; h->Hs = d->H; h->lds = d->ldx;
+    h->P = P; h->Q = Q; h->span_h = h->span_w = 1;
+    // filter row r reads image row 2 i + r - pad of output row i: row i + floor((r - pad) / 2) of the plane of its parity
+    for (int pl = 0; pl < 4; ++pl) {
+        h->plane_tap[pl] = h->n_taps;
+        h->plane_lo_h[pl] = h->plane_lo_w[pl] = 1 << 20;
+        for (int r = 0; r < d->R; ++r)
+            for (int s = 0; s < d->S; ++s) {
+                if (((r - d->pad) & 1) != pl >> 1 || ((s - d->pad) & 1) != (pl & 1)) continue;
+                const int oh = (r - d->pad) >> 1, ow = (s - d->pad) >> 1, t = h->n_taps++;
+                h->tap_oh[t] = oh; h->tap_ow[t] = ow; h->tap_wt[t] = r * d->S + s;
+                if (oh < h->plane_lo_h[pl]) h->plane_lo_h[pl] = oh;
+                if (ow < h->plane_lo_w[pl]) h->plane_lo_w[pl] = ow;
+            }
+        if (h->n_taps == h->plane_tap[pl]) return false;
+        for (int t = h->plane_tap[pl]; t < h->n_taps; ++t) {
+            h->tap_oh[t] -= h->plane_lo_h[pl]; h->tap_ow[t] -= h->plane_lo_w[pl];
+            if (h->tap_oh[t] + 1 > h->span_h) h->span_h = h->tap_oh[t] + 1;
+            if (h->tap_ow[t] + 1 > h->span_w) h->span_w = h->tap_ow[t] + 1;
+        }
+    }
+    h->plane_tap[4] = h->n_taps;
+    h->n_cols = d->K; h->ld_out = d->ldy;
+    h->oH = P; h->oW = Q; h->o_step = 1;
+    return true;
 }
 
 // ---- launch shape of a weight gradient
@@ -4038,6 +4105,13 @@ pt_status pt_sm100_conv(pt_ctx *c, const pt_conv_desc *d, int which, const void 
         halo_spec_stride1(d, &h, a, d->C, d->W, d->H, d->ldx, d->K, P, Q, d->ldy, d->pad, d->pad, false);
         pt_status r = launch_halo<false>(c, d, h, b, out, st);
         if (r != PT_ERR_UNSUPPORTED) return r;
+    }
+    if (!sparse_tiles && which == PT_CONV_FWD && d->stride == 2 && d->R * d->S > 1) {
+        HaloSpec h;
+        if (halo_spec_stride2(d, &h, a, P, Q)) {
+            const pt_status r = launch_halo<false, 4>(c, d, h, b, out, st);
+            if (r != PT_ERR_UNSUPPORTED) return r;
+        }
     }
     if (!sparse_tiles && which == PT_CONV_DGRAD && d->stride == 1 && d->R * d->S > 1 && d->R * d->S <= kMaxTaps && d->pad <= d->R - 1 &&
         d->pad <= d->S - 1) {

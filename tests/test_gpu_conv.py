@@ -115,6 +115,28 @@ def test_stem_straight_from_the_image(shape):
     c.close()
 
 
+# (N, H, W, C, K, R, pad) of the stride-2 forward by parity planes (more than two tiles a CTA): rows of 16, 32 and 64 lanes, one and several
+# chunks, resident and streamed weights, several channel tiles, odd sizes, no padding, an even filter
+@pytest.mark.parametrize("shape", [(150, 32, 32, 9, 17, 3, 1), (110, 33, 31, 32, 20, 3, 1), (80, 30, 60, 40, 33, 3, 0), (50, 56, 56, 70, 100, 3, 1), (100, 16, 130, 130, 24, 3, 1),
+                                   (60, 40, 42, 17, 300, 3, 1), (130, 24, 40, 20, 12, 2, 0), (100, 26, 34, 24, 40, 5, 2)])
+def test_stride_2_forward_by_planes(shape):
+    N, H, Wd, C, K, R, pad = shape
+    x = W.gen_act(N, H, Wd, C, W.BASE_SEED + 48)
+    w = W.bf16_round(W.gen_weight(K, R, R, C, W.BASE_SEED + 49))
+    P, Q = (H + 2 * pad - R) // 2 + 1, (Wd + 2 * pad - R) // 2 + 1
+    d = B.make_conv_desc(N, H, Wd, C, K, R, R, 2, pad, algo=2)
+    c = Hh.ctx()
+    y = Hh.out_buffer((N, P, Q), K, d.ldy, 0)
+    B.pt_conv_fwd(c, d, Hh.to_dev_padded(x, d.ldx), Hh.to_dev_padded(w, d.ldw), y, Hh.conv_ws(d, B.PT_CONV_FWD))
+    torch.cuda.synchronize()
+    c.poll()
+    # (the oracle for images of either end and the middle; fp64 torch for all)
+    ref = torch.nn.functional.conv2d(x.double().permute(0, 3, 1, 2), w.double().permute(0, 3, 1, 2), stride=2, padding=pad).permute(0, 2, 3, 1).numpy()
+    Hh.check_conv(y, K, ref, what="fwd")
+    for n in (0, N // 2, N - 1):
+        np.testing.assert_allclose(ref[n:n + 1], oracle.conv_fwd(x[n:n + 1].numpy(), w.numpy(), 2, pad), rtol=1e-9, atol=1e-9)
+
+
 # (N, H, W, C, K, R, stride): stride-2 weight gradients with few input channels (the generic kernel and the stem path):
 # odd and even tap groups, K above and below 64, 5x5 and 7x7 stems
 STRIDED_SMALL_C = [
