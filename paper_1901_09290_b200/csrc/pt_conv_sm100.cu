@@ -3,9 +3,9 @@
 //   conv_gemm_kernel   fwd and dgrad of 1x1 / strided layers: persistent CTAs, im2col-mode (or plain 2-D) TMA loads of
 //                      128 pixels x 64 channels, K-major (fwd) or MN-major (dgrad) weight tiles from the same bf16 shadow,
 //                      double/triple-buffered fp32 accumulators in TMEM, TMA-store epilogue.
-//   conv_halo_kernel   stride-1 RxS fwd/dgrad and the parities of a stride-2 dgrad: one halo tile per 64-channel chunk,
+//   conv_halo_kernel   stride-1 RxS fwd/dgrad, the parities of a stride-2 dgrad, stride-2 fwd by parity planes: one halo tile per 64-channel chunk,
 //                      filter taps as row-shifted UMMA descriptors of that tile; a 32-byte-pixel mode (16 lanes per
-//                      position, 32-byte swizzle, one MMA per tap) runs the space-to-depth stem.
+//                      position, 32-byte swizzle, one MMA per tap) runs the space-to-depth stem where conv_stem_kernel does not.
 //   conv_wgrad_kernel  weight gradient: both operands MN-major, reduction over pixels split across CTAs, partial tiles
 //                      summed in-kernel in a fixed order.
 //   conv_wgrad_taps_kernel  weight gradient by filter rows: the staged pixels of one serve all of its taps (stride 1 or 2, up to 170 channels).

@@ -133,6 +133,18 @@ def test_stride_2_forward_by_planes(shape):
     # (the oracle for images of either end and the middle; fp64 torch for all)
     ref = torch.nn.functional.conv2d(x.double().permute(0, 3, 1, 2), w.double().permute(0, 3, 1, 2), stride=2, padding=pad).permute(0, 2, 3, 1).numpy()
     Hh.check_conv(y, K, ref, what="fwd")
+    # bf16 is the rounding of the fp32 output, and the statistics are those of the stored values
+    xd, wd, d32 = Hh.to_dev_padded(x, d.ldx), Hh.to_dev_padded(w, d.ldw), B.make_conv_desc(N, H, Wd, C, K, R, R, 2, pad, out_f32=1, algo=2)
+    y32, ys = Hh.out_buffer((N, P, Q), K, d.ldy, True), Hh.out_buffer((N, P, Q), K, d.ldy, False)
+    B.pt_conv_fwd(c, d32, xd, wd, y32, Hh.conv_ws(d32, B.PT_CONV_FWD))
+    stats = torch.full((B.pt_conv_fwd_stats_bytes(c, d) // 4,), float("nan"), device="cuda")
+    parts = B.pt_conv_fwd_stats(c, d, xd, wd, ys, stats, Hh.conv_ws(d, B.PT_CONV_FWD))
+    torch.cuda.synchronize()
+    c.poll()
+    assert torch.equal(y32[..., :K].to(torch.bfloat16), y[..., :K]) and torch.equal(ys[..., :K], y[..., :K])
+    st, v = stats[: parts * 2 * d.ldy].view(parts, 2, d.ldy).double().sum(0), y[..., :K].double().reshape(-1, K)
+    # (fp32 sums of at most P Q N values each: the bounds of the statistics' own test)
+    assert torch.allclose(st[0, :K], v.sum(0), rtol=1e-5, atol=1e-5 * v.abs().sum(0).max().item()) and torch.allclose(st[1, :K], (v * v).sum(0), rtol=1e-5)
     for n in (0, N // 2, N - 1):
         np.testing.assert_allclose(ref[n:n + 1], oracle.conv_fwd(x[n:n + 1].numpy(), w.numpy(), 2, pad), rtol=1e-9, atol=1e-9)
 
