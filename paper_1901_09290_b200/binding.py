@@ -17,6 +17,8 @@ LIB_PATH = os.path.join(_HERE, "libpt_b200.so")
 
 PT_OK = 0
 PT_CONV_FWD, PT_CONV_DGRAD, PT_CONV_WGRAD = 0, 1, 2
+PT_FORM_ANY, PT_FORM_WGRAD_PIXELS, PT_FORM_WGRAD_ROWS, PT_FORM_WGRAD_TAPS, PT_FORM_WGRAD_PACKED = 0, 1, 2, 3, 4
+PT_FORM_GEMM, PT_FORM_HALO, PT_FORM_PLANES, PT_FORM_STEM = 5, 6, 7, 8
 STATUS_NAMES = ["PT_OK", "PT_ERR_INVALID_ARG", "PT_ERR_UNSUPPORTED", "PT_ERR_WORKSPACE", "PT_ERR_CUDA",
                 "PT_ERR_TIMEOUT", "PT_ERR_ARCH"]
 
@@ -82,6 +84,8 @@ EXPORTS = {
     "pt_launch_count": (c_uint64, [c_void_p]),
     "pt_test_set_wait_limit": (c_int32, [c_void_p, ctypes.c_uint32]),
     "pt_test_skip_next_arrive": (c_int32, [c_void_p, c_int32]),
+    "pt_test_wgrad_form": (c_int32, [c_void_p, c_int32]),
+    "pt_test_last_form": (c_int32, [c_void_p]),
     "pt_set_wgrad_cta_limit": (c_int32, [c_void_p, c_int32]),
     "pt_set_dgrad_cta_limit": (c_int32, [c_void_p, c_int32]),
     "pt_conv_wgrad_ctas": (c_int32, [c_void_p, POINTER(pt_conv_desc), POINTER(c_int32)]),
@@ -216,6 +220,14 @@ def pt_test_set_wait_limit(ctx: Context, milliseconds: int):
 
 def pt_test_skip_next_arrive(ctx: Context, which: int):
     _check(lib().pt_test_skip_next_arrive(ctx.handle, which), "pt_test_skip_next_arrive")
+
+
+def pt_test_wgrad_form(ctx: Context, form: int):
+    _check(lib().pt_test_wgrad_form(ctx.handle, form), "pt_test_wgrad_form")
+
+
+def pt_test_last_form(ctx: Context) -> int:
+    return int(lib().pt_test_last_form(ctx.handle))
 
 
 def pt_set_wgrad_cta_limit(ctx: Context, max_ctas: int):

@@ -147,6 +147,15 @@ extern "C" pt_status pt_test_skip_next_arrive(pt_ctx *c, int32_t which)
     return PT_OK;
 }
 
+extern "C" pt_status pt_test_wgrad_form(pt_ctx *c, int32_t form)
+{
+    if (!c || form < PT_FORM_ANY || form > PT_FORM_WGRAD_PACKED) return PT_ERR_INVALID_ARG;
+    c->test_form = form;
+    return PT_OK;
+}
+
+extern "C" int32_t pt_test_last_form(const pt_ctx *c) { return c ? c->last_form : PT_FORM_ANY; }
+
 extern "C" pt_status pt_poll_device_status(pt_ctx *c, void *stream)
 {
     if (!c) return PT_ERR_INVALID_ARG;

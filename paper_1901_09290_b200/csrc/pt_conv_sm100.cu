@@ -2878,6 +2878,7 @@ pt_status launch_gemm(pt_ctx *c, const GemmMaps &tm, GemmP &p, cudaStream_t st)
     if (c->test_skip == 2) { p.test_skip = 1; c->test_skip = 0; }
     PT_CUDA_OK(pt_launch_pdl(kernel, dim3((unsigned)grid), dim3(kGemmThreads), smem, st, tm.a, tm.tail, tm.b, tmC, p));
     c->launches += 1;
+    c->last_form = PT_FORM_GEMM;
     PT_CUDA_OK(cudaGetLastError());
     return PT_OK;
 }
@@ -3108,6 +3109,7 @@ pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const
     if (c->test_skip == 5) { p.test_skip = 1; c->test_skip = 0; }
     PT_CUDA_OK(pt_launch_pdl(kernel, dim3((unsigned)grid), dim3(kHaloThreads), smem, st, tmA, tmB, tmC, p));
     c->launches += 1;
+    c->last_form = PL > 1 ? PT_FORM_PLANES : PT_FORM_HALO;
     PT_CUDA_OK(cudaGetLastError());
     return PT_OK;
 }
@@ -3177,6 +3179,7 @@ pt_status run_stem(pt_ctx *c, const pt_conv_desc *d, const StemPlan &sp, const v
     }
     PT_CUDA_OK(pt_launch_pdl(kernel, dim3((unsigned)grid), dim3(kStemThreads), smem, st, tmC, p));
     c->launches += 1;
+    c->last_form = PT_FORM_STEM;
     PT_CUDA_OK(cudaGetLastError());
     return PT_OK;
 }
@@ -3519,23 +3522,30 @@ double wgrad_packed_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, p
 
 size_t wgrad_workspace_bound(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, const pt_wgrad_plan &w);
 
+double wgrad_form_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, int form, pt_wgrad_plan *w)
+{
+    return form == PT_FORM_WGRAD_ROWS ? wgrad_rows_plan(c, d, P, Q, w) : form == PT_FORM_WGRAD_TAPS ? wgrad_taps_plan(c, d, P, Q, w)
+         : form == PT_FORM_WGRAD_PACKED ? wgrad_packed_plan(c, d, P, Q, w) : wgrad_gen_plan(c, d, P, Q, w);
+}
+
 // The plan of a descriptor at the context's CTA limit. rows_only: only a row-block plan is asked for (its `rows` is 0 if there is none).
 pt_wgrad_plan wgrad_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, bool rows_only = false)
 {
     pt_ctx::WgradKey key{*d, wgrad_budget(c), P, Q};
     static_assert(sizeof(key) == sizeof(pt_conv_desc) + 12, "the key is compared and hashed as words");
-    key.d.ldw = key.d.out_f32 = 0; key.d.algo = rows_only ? 1 : 0;
+    const int form = rows_only ? PT_FORM_ANY : c->test_form;
+    key.d.ldw = key.d.out_f32 = 0; key.d.algo = rows_only ? 1 : 2 * form;
     std::lock_guard<std::mutex> lock(c->wgrad_mutex);
     const auto known = c->wgrad_plans.find(key);
     if (known != c->wgrad_plans.end()) return known->second;
     pt_wgrad_plan w;
-    const double rows_us = wgrad_rows_plan(c, d, P, Q, &w);
-    if (!rows_only && wgrad_packed_ok(d, P)) {
-        pt_wgrad_plan k;
-        if (wgrad_packed_plan(c, d, P, Q, &k) < (w.rows ? rows_us : 1e29)) w = k;
-    }
-    if (!w.rows && !w.packed) {
-        if (!rows_only) {
+    if (!form || wgrad_form_plan(c, d, P, Q, form, &w) > 1e29) {
+        const double rows_us = wgrad_rows_plan(c, d, P, Q, &w);
+        if (!rows_only && wgrad_packed_ok(d, P)) {
+            pt_wgrad_plan k;
+            if (wgrad_packed_plan(c, d, P, Q, &k) < (w.rows ? rows_us : 1e29)) w = k;
+        }
+        if (!w.rows && !w.packed && !rows_only) {
             pt_wgrad_plan g;
             // (measured against estimated times at all SMs and at 49: within 10 % of each other, so that near a tie either may be the faster;
             // 106 -> 103 3x3 at 28x28, batch 64 22.9 us generic, 21.8 by filter rows, 49.5 and 34.6 at 49; 128 -> 128 at 32x32 25.7 and 28.2,
@@ -3717,6 +3727,7 @@ pt_status run_wgrad(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const pt_wgr
     p.data_bytes = (unsigned)(smem - 2048);
     PT_CUDA_OK(launch_wgrad(conv_wgrad_kernel, grid, p.cluster ? p.splits : 1, smem, st, tmA, tmX, p));
     c->launches += 1;
+    c->last_form = PT_FORM_WGRAD_PIXELS;
     PT_CUDA_OK(cudaGetLastError());
     return PT_OK;
 }
@@ -3751,6 +3762,7 @@ pt_status run_wgrad_rows(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const p
     p.data_bytes = (unsigned)(smem - 2048);
     PT_CUDA_OK(launch_wgrad(conv_wgrad_rows_kernel, grid, p.cluster ? p.splits : 1, smem, st, tmA, tmX, p));
     c->launches += 1;
+    c->last_form = PT_FORM_WGRAD_ROWS;
     PT_CUDA_OK(cudaGetLastError());
     return PT_OK;
 }
@@ -3781,6 +3793,7 @@ pt_status run_wgrad_packed(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const
     p.data_bytes = (unsigned)(smem - 2048);
     PT_CUDA_OK(launch_wgrad(conv_wgrad_packed_kernel, dim3(1u, (unsigned)p.splits), 1, smem, st, tmA, tmX, p));
     c->launches += 1;
+    c->last_form = PT_FORM_WGRAD_PACKED;
     PT_CUDA_OK(cudaGetLastError());
     return PT_OK;
 }
@@ -3820,6 +3833,7 @@ pt_status run_wgrad_taps(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const p
     p.data_bytes = (unsigned)(smem - 2048);
     PT_CUDA_OK(launch_wgrad(conv_wgrad_taps_kernel, grid, p.cluster ? p.splits : 1, smem, st, tmA, tmX, p));
     c->launches += 1;
+    c->last_form = PT_FORM_WGRAD_TAPS;
     PT_CUDA_OK(cudaGetLastError());
     return PT_OK;
 }

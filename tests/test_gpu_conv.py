@@ -118,7 +118,7 @@ def test_stem_straight_from_the_image(shape):
 # (N, H, W, C, K, R, pad) of the stride-2 forward by parity planes (more than two tiles a CTA): rows of 16, 32 and 64 lanes, one and several
 # chunks, resident and streamed weights, several channel tiles, odd sizes, no padding, an even filter
 @pytest.mark.parametrize("shape", [(150, 32, 32, 9, 17, 3, 1), (110, 33, 31, 32, 20, 3, 1), (80, 30, 60, 40, 33, 3, 0), (50, 56, 56, 70, 100, 3, 1), (100, 16, 130, 130, 24, 3, 1),
-                                   (60, 40, 42, 17, 300, 3, 1), (130, 24, 40, 20, 12, 2, 0), (100, 26, 34, 24, 40, 5, 2)])
+                                   (60, 40, 42, 17, 300, 3, 1), (170, 24, 40, 20, 12, 2, 0), (120, 26, 34, 24, 40, 5, 2)])
 def test_stride_2_forward_by_planes(shape):
     N, H, Wd, C, K, R, pad = shape
     x = W.gen_act(N, H, Wd, C, W.BASE_SEED + 48)
@@ -128,6 +128,7 @@ def test_stride_2_forward_by_planes(shape):
     c = Hh.ctx()
     y = Hh.out_buffer((N, P, Q), K, d.ldy, 0)
     B.pt_conv_fwd(c, d, Hh.to_dev_padded(x, d.ldx), Hh.to_dev_padded(w, d.ldw), y, Hh.conv_ws(d, B.PT_CONV_FWD))
+    assert B.pt_test_last_form(c) == B.PT_FORM_PLANES
     torch.cuda.synchronize()
     c.poll()
     # (the oracle for images of either end and the middle; fp64 torch for all)
@@ -193,6 +194,10 @@ def test_row_block_weight_gradient(shape):
     Hh.check_conv(dx, C, oracle.conv_dgrad(dy.numpy(), w.numpy(), H, Wd, 1, pad), what="dgrad")
     again = Hh.run_conv_all(N, H, Wd, C, K, R, 1, pad, x, w, dy, algo=2)[2]
     assert torch.equal(dw, again)
+    d = B.make_conv_desc(N, H, Wd, C, K, R, R, 1, pad, algo=2)
+    rows, took = _wgrad_of_form(Hh.ctx(), d, Hh.to_dev_padded(x, d.ldx), Hh.to_dev_padded(dy, d.ldy), B.PT_FORM_WGRAD_ROWS, 0)
+    assert (took == B.PT_FORM_WGRAD_ROWS) == (C <= 64)
+    Hh.check_conv(rows, C, oracle.conv_wgrad(x.numpy(), dy.numpy(), R, R, 1, pad), what="wgrad, row blocks")
 
 
 @pytest.mark.parametrize("shape", [(2, 16, 16, 20, 36, 3, 1), (2, 14, 14, 37, 70, 3, 1), (2, 8, 8, 7, 33, 1, 1), (2, 16, 16, 41, 20, 3, 2)])
@@ -232,12 +237,31 @@ def test_weight_gradient_of_nan_pad_lanes(shape):
     Hh.check_conv(dw, C, oracle.conv_wgrad(x.numpy(), dy.numpy(), R, R, stride, pad), what="wgrad")
 
 
+def _wgrad_of_form(c, d, xd, dyd, form, limit):
+    """The weight gradient in the given form (PT_FORM_ANY: the library's choice) at a CTA limit, computed twice, and the form that it took."""
+    B.pt_test_wgrad_form(c, form)
+    B.pt_set_wgrad_cta_limit(c, limit)
+    try:
+        ws = torch.empty(max(16, B.pt_conv_workspace_bytes(c, d, B.PT_CONV_WGRAD)), dtype=torch.uint8, device="cuda")
+        dw = torch.full((d.K, d.R, d.S, d.C), 7680.0, device="cuda")
+        again = torch.full_like(dw, 7680.0)
+        B.pt_conv_wgrad(c, d, xd, dyd, dw, ws)
+        B.pt_conv_wgrad(c, d, xd, dyd, again, ws)
+        torch.cuda.synchronize()
+        c.poll()
+    finally:
+        B.pt_test_wgrad_form(c, B.PT_FORM_ANY)
+        B.pt_set_wgrad_cta_limit(c, 0)
+    assert torch.equal(dw, again)
+    return dw, B.pt_test_last_form(c)
+
+
 # (N, H, W, C, K, R, S, stride, pad) of the filter-row form of the weight gradient: one and two blocks of channels on either side and just
 # past them, units that leave rows over, both parities (odd and even sizes, no padding, more padding than the filter), filters of 2, 4, 5 and
 # 8 columns, other than square, a wide image, a single output row
 @pytest.mark.parametrize("shape", [(5, 14, 14, 65, 64, 3, 3, 1, 1), (4, 28, 28, 106, 129, 3, 3, 1, 1), (3, 13, 9, 160, 40, 3, 3, 1, 0), (2, 6, 100, 70, 20, 3, 3, 1, 1),
                                    (4, 28, 28, 106, 103, 3, 3, 2, 1), (3, 15, 17, 20, 70, 3, 3, 2, 1), (3, 15, 16, 33, 65, 3, 3, 2, 0), (2, 17, 12, 90, 30, 5, 5, 2, 2),
-                                   (3, 12, 12, 66, 50, 2, 2, 2, 0), (3, 16, 16, 60, 130, 4, 4, 2, 3), (2, 24, 24, 64, 40, 8, 8, 2, 3), (2, 9, 20, 100, 24, 1, 5, 1, 2),
+                                   (3, 12, 12, 66, 50, 2, 2, 2, 0), (3, 16, 16, 60, 130, 4, 4, 2, 3), (2, 24, 24, 64, 40, 8, 8, 2, 3), (2, 9, 20, 90, 24, 1, 5, 1, 2),
                                    (2, 3, 30, 80, 64, 3, 3, 1, 0), (64, 14, 14, 77, 77, 3, 3, 1, 1), (64, 28, 28, 38, 38, 3, 3, 2, 1)])
 def test_filter_row_weight_gradient(shape):
     N, H, Wd, C, K, R, S, stride, pad = shape
@@ -249,13 +273,10 @@ def test_filter_row_weight_gradient(shape):
     d = B.make_conv_desc(N, H, Wd, C, K, R, S, stride, pad, W.pad8(C), W.pad16(K), W.pad8(C), 0, 2)
     xd, dyd = Hh.to_dev_padded(x, d.ldx), Hh.to_dev_padded(dy, d.ldy)
     for limit in (0, 49, 3):                                    # (all SMs, a share of them, one CTA per filter row)
-        B.pt_set_wgrad_cta_limit(c, limit)
-        ws = torch.empty(max(16, B.pt_conv_workspace_bytes(c, d, B.PT_CONV_WGRAD)), dtype=torch.uint8, device="cuda")
-        dw = torch.full((K, R, S, C), 7680.0, device="cuda")
-        B.pt_conv_wgrad(c, d, xd, dyd, dw, ws)
-        torch.cuda.synchronize()
-        c.poll()
-        Hh.check_conv(dw, C, ref, what=f"wgrad at limit {limit}")
+        for form in (B.PT_FORM_WGRAD_TAPS, B.PT_FORM_WGRAD_PIXELS, B.PT_FORM_ANY):
+            dw, took = _wgrad_of_form(c, d, xd, dyd, form, limit)
+            assert took == form or form == B.PT_FORM_ANY
+            Hh.check_conv(dw, C, ref, what=f"wgrad at limit {limit}, form {took}")
     c.close()
 
 
@@ -274,16 +295,10 @@ def test_packed_weight_gradient(shape):
     d = B.make_conv_desc(N, H, Wd, C, K, R, S, 1, pad, ldx, ldy, W.pad8(C), 0, 2)
     xd, dyd = Hh.to_dev_padded(x, ldx), Hh.to_dev_padded(dy, ldy)
     for limit in (0, 49, 5, 1):
-        B.pt_set_wgrad_cta_limit(c, limit)
-        ws = torch.empty(max(16, B.pt_conv_workspace_bytes(c, d, B.PT_CONV_WGRAD)), dtype=torch.uint8, device="cuda")
-        dw = torch.full((K, R, S, C), 7680.0, device="cuda")
-        B.pt_conv_wgrad(c, d, xd, dyd, dw, ws)
-        again = torch.full_like(dw, 7680.0)
-        B.pt_conv_wgrad(c, d, xd, dyd, again, ws)
-        torch.cuda.synchronize()
-        c.poll()
-        Hh.check_conv(dw, C, ref, what=f"wgrad at limit {limit}")
-        assert torch.equal(dw, again)
+        for form in (B.PT_FORM_WGRAD_PACKED, B.PT_FORM_ANY):
+            dw, took = _wgrad_of_form(c, d, xd, dyd, form, limit)
+            assert took == form or form == B.PT_FORM_ANY
+            Hh.check_conv(dw, C, ref, what=f"wgrad at limit {limit}, form {took}")
     c.close()
 
 
