@@ -166,7 +166,9 @@ pt_status pt_conv_dgrad(pt_ctx *ctx, const pt_conv_desc *d, const void *dy, cons
                         void *ws, size_t ws_bytes, void *stream);
 
 /* dw[k,r,s,c] = sum_{n,p,q} dy[n,p,q,k] * x[n, p*stride-pad+r, q*stride-pad+s, c]   (Eq. 4).
- * dw: fp32 [K][R][S][C] dense. Deterministic: partial sums are combined in a fixed order. */
+ * dw: fp32 [K][R][S][C] dense. Deterministic: partial sums are combined in a fixed order.
+ * Infinities and NaN in x or dy reach the sums that they are part of and no other, the zeros outside the image counting as factors
+ * (0 x Inf = NaN); sums that are NaN may take the call longer (milliseconds in a large layer). */
 pt_status pt_conv_wgrad(pt_ctx *ctx, const pt_conv_desc *d, const void *x, const void *dy, float *dw,
                         void *ws, size_t ws_bytes, void *stream);
 

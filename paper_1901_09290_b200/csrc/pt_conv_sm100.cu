@@ -1154,6 +1154,11 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
 //   waits (bounded) until all splits of its tile have arrived, and then sums its share of the tile's rows over the
 //   splits in ascending order: deterministic, and no second kernel.
 constexpr int kMaxRow = 8;  // filter rows and columns of the filter-row form
+// The layer itself, for the sums that the raster forms cannot take from their accumulators (wgrad_pure).
+struct WgradRaw {
+    const __nv_bfloat16 *x, *dy;
+    int N, H, W, C, K, P, Q, R, S, stride, pad, ldx, ldy;
+};
 struct WgradP {
     int K, C, taps;         // true channel counts, number of taps (R*S)
     int BN, n_tiles;        // input-channel tile
@@ -1194,6 +1199,7 @@ struct WgradP {
     unsigned data_bytes;    // shared memory behind the control block: the stages, and what the exchange of the splits may use
     float *out;             // dw
     int test_skip;          // test hook (pt_test_skip_next_arrive): split 0 does not announce its partial tile
+    WgradRaw raw;           // raster forms (row-block, filter-row, packed)
     float *partial;         // splits > 1: workspace [blockIdx.x][split], room for the accumulators of 128 x acc_cols floats (WgradShare)
     unsigned int *sync;     // splits > 1: two zeroed counters per blockIdx.x (arrived, seen by); left zero again at exit
     unsigned int *status;
@@ -1215,19 +1221,83 @@ __device__ __forceinline__ int wgrad_tap(const WgradP &p, int acc, int g)
     return s < p.S ? r * p.S + s : p.taps;
 }
 
-// Row-block form: the sum of (output channel k, tap, lane c) goes to dw. In the stem a tap is a pair of filter rows and a lane one of four
+// The raster forms stage whole rows of pixels. Where a row of dy ends (or its last unit, or a column group) its staged zeros meet pixels of x
+// that no tap pairs them with: 0 x Inf, a NaN in a sum that the pixel is no part of. A NaN among the sums that a thread has stored, the four at
+// (k + e dk, tap, c + e dc), is therefore taken again from the layer itself: one product per output pixel, with zeros outside the image, as
+// the pixel form multiplies. Whole warps: eight `bad` lanes or more take their own sums, fewer are done one after the other by the warp, a lane
+// to an output row (a NaN in the last image, each lane its own sums or rows dealt out: 106 -> 103 3x3 at 28x28, batch 64, all lanes bad 6 and
+// 36 ms; 19 -> 19 at 56x56, batch 256, packed, a lane or two of a warp 106 and 20). A sum that is a NaN in its own right takes the rows up to
+// the first that makes it one (all of x NaN: 0.06 and 0.09 ms, against 0.035 and 0.04 of finite x). (Inline, and behind the store: a call costs the kernels hundreds of bytes of spilled registers.)
+__device__ __forceinline__ bool wgrad_nan(const float4 &v, int nv)
+{
+    return v.x != v.x || (nv > 1 && v.y != v.y) || (nv > 2 && v.z != v.z) || (nv > 3 && v.w != v.w);
+}
+__device__ __forceinline__ void wgrad_pure(const WgradRaw &q, float *out, bool bad, int k_, int dk, int tap_, int c_, int dc)
+{
+    unsigned left = __ballot_sync(0xffffffffu, bad);
+    const int lane = threadIdx.x & 31, rows = q.N * q.P;
+    const bool own = __popc(left) >= 8;
+    while (left) {
+        const int src = own ? lane : __ffs((int)left) - 1;
+        const int k = __shfl_sync(0xffffffffu, k_, src), tap = __shfl_sync(0xffffffffu, tap_, src), c = __shfl_sync(0xffffffffu, c_, src);
+        const int r = tap / q.S, s = tap - r * q.S;
+        float sum[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
+        for (int row0 = 0; row0 < rows; row0 += own ? 1 : 32) {
+            const int row = row0 + (own ? 0 : lane), n = row / q.P, h = (row - n * q.P) * q.stride - q.pad + r;
+            const bool in_h = h >= 0 && h < q.H;
+            const __nv_bfloat16 *const xr = q.x + ((size_t)n * q.H + (in_h ? h : 0)) * q.W * q.ldx, *const yr = q.dy + (size_t)row * q.Q * q.ldy;
+            float part[4] = {0.f, 0.f, 0.f, 0.f};          // (a row's sum by itself: shorter chains)
+            if (own ? bad : row < rows) {
+#pragma unroll 4
+                for (int j = 0; j < q.Q; ++j) {
+                    const int w = j * q.stride - q.pad + s;
+                    const bool in = in_h && w >= 0 && w < q.W;
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        part[e] = fmaf(__bfloat162float(yr[(size_t)j * q.ldy + min(k + e * dk, q.K - 1)]),
+                                       in ? __bfloat162float(xr[(size_t)w * q.ldx + min(c + e * dc, q.C - 1)]) : 0.f, part[e]);
+                }
+            }
+            bool numbers = false;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) { sum[e] += part[e]; numbers |= sum[e] == sum[e]; }
+            if (own ? __all_sync(0xffffffffu, !bad || !numbers) : __any_sync(0xffffffffu, !numbers)) break;
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            if (!own)
+#pragma unroll
+                for (int o = 16; o; o >>= 1) sum[e] += __shfl_xor_sync(0xffffffffu, sum[e], o);
+            if (!bad || lane != src || k + e * dk >= q.K || c + e * dc >= q.C) continue;
+            float *const at = out + ((size_t)(k + e * dk) * q.R * q.S + tap) * q.C + c + e * dc;
+            if (*at != *at) *at = sum[e];
+        }
+        left = own ? 0u : left & (left - 1u);
+    }
+}
+
+// Row-block form: where the sums of (tap, lane c) are in dw; false: nowhere. In the stem a tap is a pair of filter rows and a lane one of four
 // neighbouring positions' (a, b, channel): filter row 2 tap + a - off, column 2 (c / 16) + b - off, where the filter has them. (A launch of
 // its own for this took 2 us and its start.)
-__device__ __forceinline__ void wgrad_pair_store(const WgradP &p, int k, int tap, int c, float v)
+__device__ __forceinline__ bool wgrad_pair_place(const WgradP &p, int &tap, int &c)
 {
-    if (k >= p.K) return;
-    if (p.stem.C) {
-        const int e = c & 15, ab = (e >= p.stem.C ? 1 : 0) + (e >= 2 * p.stem.C ? 1 : 0) + (e >= 3 * p.stem.C ? 1 : 0);
-        const int r = 2 * tap + (ab >> 1) - p.stem.off, s = 2 * (c >> 4) + (ab & 1) - p.stem.off, ch = e - ab * p.stem.C;
-        if (ch < p.stem.C && r >= 0 && r < p.stem.R && s >= 0 && s < p.stem.S) p.out[((size_t)(k * p.stem.R + r) * p.stem.S + s) * p.stem.C + ch] = v;
-        return;
-    }
-    p.out[((size_t)k * p.taps + tap) * p.C + c] = v;
+    if (!p.stem.C) return tap < p.taps && c < p.C;
+    const int e = c & 15, ab = (e >= p.stem.C ? 1 : 0) + (e >= 2 * p.stem.C ? 1 : 0) + (e >= 3 * p.stem.C ? 1 : 0);
+    const int r = 2 * tap + (ab >> 1) - p.stem.off, s = 2 * (c >> 4) + (ab & 1) - p.stem.off;
+    c = e - ab * p.stem.C;
+    tap = r * p.stem.S + s;
+    return c < p.stem.C && r >= 0 && r < p.stem.R && s >= 0 && s < p.stem.S;
+}
+// The sums of the output channels k .. k + 3 at (tap, c) of dw (wgrad_pair_place).
+__device__ __forceinline__ void wgrad_pair_store(const WgradP &p, int k, int tap, int c, const float4 &v)
+{
+    const int C = p.raw.C, pitch = p.raw.R * p.raw.S * C;
+    float *const dst = p.out + (size_t)k * pitch + (size_t)tap * C + c;
+    const float v4[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+        if (k + e < p.K) dst[(size_t)e * pitch] = v4[e];
 }
 
 // 32 columns (16 where the accumulator ends) of a warp's 32 TMEM lanes; zeros for a CTA that had no work.
@@ -1265,6 +1335,7 @@ __device__ __forceinline__ void wgrad_store4(float *dst, const float4 &v, int nv
 // here it is two cluster barriers and the bytes (about 2.5 us). At most eight splits: what a portable cluster can be.
 // Every thread of every CTA of the cluster calls this, with the same trip counts, and aborting CTAs too (they hand on zeros; dw is
 // then undefined and the time-out already recorded): the barriers always complete.
+template <bool RASTER, bool PAIR>
 __device__ __forceinline__ void wgrad_cluster_sum(const WgradP &p, Ctl *ctl, uint32_t data_base, uint32_t tmem_base, int tap0, int k0, int c0,
                                                   int split, int iters, uint32_t ring_bytes, int n_acc, int acc_cols)
 {
@@ -1312,16 +1383,15 @@ __device__ __forceinline__ void wgrad_cluster_sum(const WgradP &p, Ctl *ctl, uin
                 asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(t.x), "=f"(t.y), "=f"(t.z), "=f"(t.w) : "r"(a + (uint32_t)z * 4096u) : "memory");
                 sum.x += t.x; sum.y += t.y; sum.z += t.z; sum.w += t.w;
             }
-            if (p.pair) {
-                const int tap = wgrad_tap(p, tap0 + tt, row >> p.lane_shift), c = row & (p.lanes - 1);
-                if (c < p.C && tap < p.taps) {
-                    const float v4[4] = {sum.x, sum.y, sum.z, sum.w};
-#pragma unroll
-                    for (int e = 0; e < 4; ++e)
-                        wgrad_pair_store(p, col + e, tap, c, v4[e]);
-                }
-            } else if (k0 + row < p.K && col < acc_cols && c0 + col < p.C) {
-                wgrad_store4(p.out + ((size_t)(k0 + row) * p.taps + tap0 + tt) * p.C + c0 + col, sum, min(4, p.C - (c0 + col)));
+            if (PAIR) {
+                int tap = wgrad_tap(p, tap0 + tt, row >> p.lane_shift), c = row & (p.lanes - 1);
+                const bool here = wgrad_pair_place(p, tap, c) && col < p.K;
+                if (here) wgrad_pair_store(p, col, tap, c, sum);
+                wgrad_pure(p.raw, p.out, here && wgrad_nan(sum, p.K - col), col, 1, tap, c, 0);
+            } else {
+                const int nv = k0 + row < p.K && col < acc_cols ? min(4, p.C - (c0 + col)) : 0;
+                if (nv > 0) wgrad_store4(p.out + ((size_t)(k0 + row) * p.taps + tap0 + tt) * p.C + c0 + col, sum, nv);
+                if (RASTER) wgrad_pure(p.raw, p.out, nv > 0 && wgrad_nan(sum, nv), k0 + row, 0, tap0 + tt, c0 + col, 1);
             }
         }
     }
@@ -1437,7 +1507,8 @@ __device__ __forceinline__ float4 wgrad_sum(uint32_t base, int k, int n, int Z, 
 // Everything after the main loop of a weight-gradient kernel: the accumulators leave TMEM (directly to dw, or as this
 // split's partial tile), the splits of a tile meet, and every CTA sums its share of the tile over the splits.
 // `ring_bytes` of shared memory at `data_base` are free by then and serve as staging. `tap0` is the CTA's first tap (generic form) or
-// accumulator (row-block form).
+// accumulator (row-block form). RASTER: a form that pairs staged zeros of dy with pixels of x (wgrad_pure); PAIR: the row-block form.
+template <bool RASTER, bool PAIR>
 __device__ __forceinline__ void wgrad_finish(const WgradP &p, Ctl *ctl, uint32_t data_base, uint32_t tmem_base,
                                              int tap0, int k0, int c0, int split, int iters, uint32_t ring_bytes, int n_acc, int acc_cols)
 {
@@ -1449,6 +1520,7 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, Ctl *ctl, uint32_t
         const int quarter = warp & 3, wset = (warp >= 2 && warp < 6) ? 0 : 1;
         bool ok = true;
         if (iters > 0) ok = mbar_wait(smem_u32(&ctl->accum), 0, abort_flag, p.status, 6);
+        ok = __all_sync(0xffffffffu, ok);                    // (the warp stays together below)
         if (warp == 2) WTRACE(3);
         tc_fence_after();
         if (ok) {
@@ -1481,15 +1553,15 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, Ctl *ctl, uint32_t
                 if (gtid == 0) wgrad_arrive(p, split, abort_flag);
                 named_barrier(1, 256);
                 if (warp == 2) WTRACE(5);
-            } else if (p.pair) {
+            } else if (PAIR) {
                 // lanes are (tap of the accumulator, input channel), columns are output channels: for one column a warp's lanes
                 // write consecutive floats of dw
-                const int l = quarter * 32 + lane, c = l & (p.lanes - 1);
+                const int l = quarter * 32 + lane;
                 int ci = 0;
                 for (int tt = 0; tt < n_acc; ++tt)
                 for (int cc = 0; cc < acc_cols; cc += 16, ++ci) {
                     if ((ci & 1) != wset) continue;
-                    const int tap = wgrad_tap(p, tap0 + tt, l >> p.lane_shift);
+                    int tap = wgrad_tap(p, tap0 + tt, l >> p.lane_shift), c = l & (p.lanes - 1);
                     uint32_t v[16];
                     if (iters > 0) {
                         tmem_ld16(lane_addr + (uint32_t)(tt * acc_cols + cc), v);
@@ -1498,10 +1570,18 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, Ctl *ctl, uint32_t
 #pragma unroll
                         for (int e = 0; e < 16; ++e) v[e] = 0u;
                     }
-                    if (c >= p.C || tap >= p.taps) continue;
+                    const bool here = wgrad_pair_place(p, tap, c);
+                    unsigned bad = 0u;                       // a bit per four sums
 #pragma unroll
-                    for (int e = 0; e < 16; ++e)
-                        wgrad_pair_store(p, cc + e, tap, c, __uint_as_float(v[e]));
+                    for (int e = 0; e < 4; ++e) {
+                        const float4 t = make_float4(__uint_as_float(v[4 * e]), __uint_as_float(v[4 * e + 1]), __uint_as_float(v[4 * e + 2]), __uint_as_float(v[4 * e + 3]));
+                        if (!here || cc + 4 * e >= p.K) break;
+                        wgrad_pair_store(p, cc + 4 * e, tap, c, t);
+                        if (wgrad_nan(t, p.K - cc - 4 * e)) bad |= 1u << e;
+                    }
+                    if (__any_sync(0xffffffffu, bad != 0u))
+#pragma unroll 1
+                        for (int e = 0; e < 4; ++e) wgrad_pure(p.raw, p.out, (bad >> e) & 1u, cc + 4 * e, 1, tap, c, 0);
                 }
             } else {
             float *obase = p.out;
@@ -1531,20 +1611,28 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, Ctl *ctl, uint32_t
                     asm volatile("st.shared.b32 [%0], %1;" ::"r"(sq + (uint32_t)(lane * 33 + e) * 4u), "r"(v[e]) : "memory");
                 __syncwarp();
                 const int col = c0 + cc + lane;
+                [[maybe_unused]] unsigned bad = 0u;          // a bit per row
                 for (int rr = 0; rr < 32; ++rr) {
                     const int kk = k0 + quarter * 32 + rr;
                     if (kk >= p.K) break;
                     uint32_t t;
                     asm volatile("ld.shared.b32 %0, [%1];" : "=r"(t) : "r"(sq + (uint32_t)(rr * 33 + lane) * 4u) : "memory");
-                    if (col < p.C && cc + lane < p.BN) obase[((size_t)kk * p.taps + tap) * p.C + col] = __uint_as_float(t);
+                    if (col < p.C && cc + lane < p.BN) {
+                        const float f = __uint_as_float(t);
+                        obase[((size_t)kk * p.taps + tap) * p.C + col] = f;
+                        if (RASTER && f != f) bad |= 1u << rr;
+                    }
                 }
+                if (RASTER && __any_sync(0xffffffffu, bad != 0u))
+#pragma unroll 1
+                    for (int rr = 0; rr < 32; ++rr) wgrad_pure(p.raw, p.out, (bad >> rr) & 1u, k0 + quarter * 32 + rr, 0, tap, col, 0);
             }
             }
         }
         tc_fence_before();
     }
     if (p.cluster) {
-        wgrad_cluster_sum(p, ctl, data_base, tmem_base, tap0, k0, c0, split, iters, ring_bytes, n_acc, acc_cols);
+        wgrad_cluster_sum<RASTER, PAIR>(p, ctl, data_base, tmem_base, tap0, k0, c0, split, iters, ring_bytes, n_acc, acc_cols);
         return;
     }
     __syncthreads();
@@ -1567,22 +1655,21 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, Ctl *ctl, uint32_t
             for (int i = threadIdx.x; i < (((n_chunk << ls) + 31) & ~31); i += kThreads) {
                 const int k = i >> ls;
                 const float4 sum = wgrad_sum(data_base, k, n_chunk, p.splits, ls);
-                if (k >= n_chunk || (i & ((1 << ls) - 1))) continue;
+                const bool mine = k < n_chunk && !(i & ((1 << ls) - 1));
                 const int piece = c_beg + k, tq = fast_div(piece, sh.rows, inv_rows), row = piece - tq * sh.rows;
                 const int tt = fast_div(tq, sh.quads, inv_quads), col = (tq - tt * sh.quads) * 4;
-                if (p.pair) {
+                if (PAIR) {
                     // row = (tap of the accumulator, input channel), columns = output channels: consecutive threads, consecutive floats
                     const int g = (row >= p.C ? 1 : 0) + (row >= 2 * p.C ? 1 : 0) + (row >= 3 * p.C ? 1 : 0);
-                    const int tap = wgrad_tap(p, tap0 + tt, g), c = row - g * p.C;
-                    if (tap < p.taps) {
-                        const float v4[4] = {sum.x, sum.y, sum.z, sum.w};
-#pragma unroll
-                        for (int e = 0; e < 4; ++e)
-                            wgrad_pair_store(p, col + e, tap, c, v4[e]);
-                    }
-                    continue;
+                    int tap = wgrad_tap(p, tap0 + tt, g), c = row - g * p.C;
+                    const bool here = wgrad_pair_place(p, tap, c) && mine;
+                    if (here) wgrad_pair_store(p, col, tap, c, sum);
+                    wgrad_pure(p.raw, p.out, here && wgrad_nan(sum, p.K - col), col, 1, tap, c, 0);
+                } else {
+                    const int nv = min(4, p.C - (c0 + col));
+                    if (mine) wgrad_store4(p.out + ((size_t)(k0 + row) * p.taps + tap0 + tt) * p.C + c0 + col, sum, nv);
+                    if (RASTER) wgrad_pure(p.raw, p.out, mine && wgrad_nan(sum, nv), k0 + row, 0, tap0 + tt, c0 + col, 1);
                 }
-                wgrad_store4(p.out + ((size_t)(k0 + row) * p.taps + tap0 + tt) * p.C + c0 + col, sum, min(4, p.C - (c0 + col)));
             }
             __syncthreads();
         }
@@ -1591,7 +1678,7 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, Ctl *ctl, uint32_t
 }
 
 __global__ void __launch_bounds__(kThreads, 1) conv_wgrad_kernel(const __grid_constant__ CUtensorMap tmDy,
-                                                              const __grid_constant__ CUtensorMap tmX, const WgradP p)
+                                                              const __grid_constant__ CUtensorMap tmX, const __grid_constant__ WgradP p)
 {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     Ctl *ctl = reinterpret_cast<Ctl *>(smem_raw);
@@ -1737,7 +1824,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_wgrad_kernel(const __grid_co
         if (ok) umma_commit_lead(smem_u32(&ctl->accum), leader);
         if (warp == 1) WTRACE(2);
     }
-    wgrad_finish(p, ctl, data_base, tmem_base, tap0, k0, c0, split, iters, p.data_bytes, ntap, p.BN);
+    wgrad_finish<false, false>(p, ctl, data_base, tmem_base, tap0, k0, c0, split, iters, p.data_bytes, ntap, p.BN);
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem_base, (uint32_t)p.tmem_cols);
@@ -1760,7 +1847,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_wgrad_kernel(const __grid_co
 // for a 3x3 filter. The MMAs (29 ns each however narrow) and the TMA unit's time per row bound the narrow layers, and a 64-byte
 // row that ends inside a sector takes it 3.1 ns instead of 4.5.
 __global__ void __launch_bounds__(kThreads, 1) conv_wgrad_rows_kernel(const __grid_constant__ CUtensorMap tmDy,
-                                                                   const __grid_constant__ CUtensorMap tmX, const WgradP p)
+                                                                   const __grid_constant__ CUtensorMap tmX, const __grid_constant__ WgradP p)
 {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     Ctl *ctl = reinterpret_cast<Ctl *>(smem_raw);
@@ -1895,7 +1982,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_wgrad_rows_kernel(const __gr
         if (ok) umma_commit_lead(smem_u32(&ctl->accum), leader);
         if (warp == 1) WTRACE(2);
     }
-    wgrad_finish(p, ctl, data_base, tmem_base, acc0, k0, c0, split, iters, p.data_bytes, n_acc, p.acc_cols);
+    wgrad_finish<true, true>(p, ctl, data_base, tmem_base, acc0, k0, c0, split, iters, p.data_bytes, n_acc, p.acc_cols);
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem_base, (uint32_t)p.tmem_cols);
@@ -1912,7 +1999,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_wgrad_rows_kernel(const __gr
 // instructions (N = 112: 60 cycles) take as long as its loads.
 struct TapMaps { CUtensorMap m[4]; };        // x: [row parity * 2 + column parity]; at stride 1 the first only
 
-__global__ void __launch_bounds__(kThreads, 1) conv_wgrad_taps_kernel(const __grid_constant__ CUtensorMap tmDy, const __grid_constant__ TapMaps tmX, const WgradP p)
+__global__ void __launch_bounds__(kThreads, 1) conv_wgrad_taps_kernel(const __grid_constant__ CUtensorMap tmDy, const __grid_constant__ TapMaps tmX, const __grid_constant__ WgradP p)
 {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     Ctl *ctl = reinterpret_cast<Ctl *>(smem_raw);
@@ -2034,7 +2121,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_wgrad_taps_kernel(const __gr
         if (ok) umma_commit_lead(smem_u32(&ctl->accum), leader);
         if (warp == 1) WTRACE(2);
     }
-    wgrad_finish(p, ctl, data_base, tmem_base, r * p.S, k0, c0, split, iters, p.data_bytes, p.S, p.BN);
+    wgrad_finish<true, false>(p, ctl, data_base, tmem_base, r * p.S, k0, c0, split, iters, p.data_bytes, p.S, p.BN);
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem_base, (uint32_t)p.tmem_cols);
@@ -2052,7 +2139,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_wgrad_taps_kernel(const __gr
 // staged rows: with 48 CTAs 22.3 -> 13.2 us at batch 128, alone 16.6 -> 11.3; 19 -> 19 at 56x56, batch 256 80.8 -> 53.1 and 37.2 -> 29.9. What is
 // left there is the exchange (the dropped blocks are not stored, but the G pixels are G sources each) and a box per column, 0.2 us a thread.
 __global__ void __launch_bounds__(kThreads, 1) conv_wgrad_packed_kernel(const __grid_constant__ CUtensorMap tmDy,
-                                                                     const __grid_constant__ CUtensorMap tmX, const WgradP p)
+                                                                     const __grid_constant__ CUtensorMap tmX, const __grid_constant__ WgradP p)
 {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     Ctl *ctl = reinterpret_cast<Ctl *>(smem_raw);
@@ -2226,12 +2313,14 @@ __global__ void __launch_bounds__(kThreads, 1) conv_wgrad_packed_kernel(const __
             for (int i = threadIdx.x; i < (((n_chunk << ls) + 31) & ~31); i += kThreads) {
                 const int k = i >> ls;
                 const float4 sum = wgrad_sum(data_base, k, n_chunk, Z, ls);
-                if (k >= n_chunk || (i & ((1 << ls) - 1))) continue;
+                const bool mine = k < n_chunk && !(i & ((1 << ls) - 1));
                 const int piece = c_beg + k, rq = fast_div(piece, SC, inv_sc), sc = piece - rq * SC, r = fast_div(rq, KQ, inv_kq), kk = (rq - r * KQ) * 4;
                 const float v4[4] = {sum.x, sum.y, sum.z, sum.w};
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
-                    if (kk + e < p.K) p.out[((size_t)(kk + e) * p.taps + r * p.S) * p.C + sc] = v4[e];      // (taps of a row side by side)
+                    if (mine && kk + e < p.K) p.out[((size_t)(kk + e) * p.taps + r * p.S) * p.C + sc] = v4[e];      // (taps of a row side by side)
+                if (__any_sync(0xffffffffu, mine && wgrad_nan(sum, p.K - kk)))
+                    wgrad_pure(p.raw, p.out, mine && wgrad_nan(sum, p.K - kk), kk, 1, r * p.S + sc / p.C, sc % p.C, 0);
             }
             __syncthreads();
         }
@@ -3667,7 +3756,12 @@ int wg_max_clusters(const pt_ctx *c, int size)
     return c->max_clusters[size] < 0 ? 0 : c->max_clusters[size];
 }
 
-// What both forms have in common: tiles, splits and where the partial tiles go.
+WgradRaw wgrad_raw(const pt_conv_desc *d, int P, int Q, const void *x, const void *dy)
+{
+    return WgradRaw{(const __nv_bfloat16 *)x, (const __nv_bfloat16 *)dy, d->N, d->H, d->W, d->C, d->K, P, Q, d->R, d->S, d->stride, d->pad, d->ldx, d->ldy};
+}
+
+// What all forms have in common: tiles, splits and where the partial tiles go.
 pt_status wgrad_common(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const pt_wgrad_plan &w, float *out, void *ws, size_t ws_bytes, WgradP *p)
 {
     memset(p, 0, sizeof(*p));
@@ -3735,9 +3829,9 @@ pt_status run_wgrad(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const pt_wgr
 // Launches the row-block weight-gradient kernel.
 // `x_row_pixels` > 0 and (lo_h, lo_w): x is a view whose rows are x_row_pixels apart and whose raster origin for tap (0, 0)
 // is at (lo_h, lo_w) instead of (-pad, -pad) -- the space-to-depth stem, whose "pixels" are overlapping 4-pixel windows; `stem` is that
-// layer and out its dw.
+// layer, `image` its input and out its dw.
 pt_status run_wgrad_rows(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const pt_wgrad_plan &wr, const void *x, const void *dy, float *out, void *ws,
-                         size_t ws_bytes, cudaStream_t st, int x_row_pixels = 0, int lo_h = 0, int lo_w = 0, const pt_conv_desc *stem = nullptr, int off = 0)
+                         size_t ws_bytes, cudaStream_t st, int x_row_pixels = 0, int lo_h = 0, int lo_w = 0, const pt_conv_desc *stem = nullptr, const void *image = nullptr, int off = 0)
 {
     if (!c->encode_tiled) return PT_ERR_CUDA;
     WgradP p;
@@ -3745,6 +3839,7 @@ pt_status run_wgrad_rows(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const p
     const pt_status r0 = wgrad_common(c, d, P, Q, wr, out, ws, ws_bytes, &p);
     if (r0 != PT_OK) return r0;
     p.pair = 1;
+    p.raw = wgrad_raw(stem ? stem : d, P, Q, stem ? image : x, dy);
     p.stride = 1; p.lo_h = -d->pad; p.lo_w = -d->pad;
     if (x_row_pixels > 0) { p.lo_h = lo_h; p.lo_w = lo_w; }
     if (stem) { p.stem.C = stem->C; p.stem.R = stem->R; p.stem.S = stem->S; p.stem.off = off; }
@@ -3777,6 +3872,7 @@ pt_status run_wgrad_packed(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const
     if (r0 != PT_OK) return r0;
     p.G = 64 / d->ldx; p.lanes = d->ldx; p.lane_shift = d->ldx == 32 ? 5 : 4; p.dy_lanes = wk.dy_lanes; p.row_lanes = d->ldy;
     p.lo_h = p.lo_w = -d->pad;
+    p.raw = wgrad_raw(d, P, Q, x, dy);
     p.nr = wk.nr; p.Wp = wk.Wp; p.RB = wk.RB; p.units = wk.units; p.units_per_split = wk.units_per_split;
     p.ksteps = wk.ksteps; p.nb_a = wk.nb_a; p.a_box = wk.a_box; p.b_box = wk.b_box; p.stages = wk.stages;
     // image rows as rows of W x ld elements: a box of 64 (32) of them is the next pixels side by side, zeros past either end of the row
@@ -3809,6 +3905,7 @@ pt_status run_wgrad_taps(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const p
     memset(&tmX, 0, sizeof(tmX));
     const pt_status r0 = wgrad_common(c, d, P, Q, wt, out, ws, ws_bytes, &p);
     if (r0 != PT_OK) return r0;
+    p.raw = wgrad_raw(d, P, Q, x, dy);
     p.nr = wt.nr; p.Wp = wt.Wp; p.RB = wt.RB; p.units = wt.units; p.units_per_split = wt.units_per_split;
     p.ksteps = wt.ksteps; p.nb_a = wt.nb_a; p.a_box = wt.a_box; p.b_box = wt.b_box; p.stages = wt.stages; p.planes = wt.planes;
     // tap column s reads pixel stride * j + s - pad of output column j: plane (s - pad) mod stride, column j + floor((s - pad) / stride) of it
@@ -4023,7 +4120,7 @@ pt_status pt_sm100_conv(pt_ctx *c, const pt_conv_desc *d, int which, const void 
             const pt_wgrad_plan wr = wgrad_plan(c, &vr, sp.P, sp.Q, true);
             pt_status r = PT_ERR_UNSUPPORTED;
             if (wr.rows) {
-                r = run_wgrad_rows(c, &vr, sp.P, sp.Q, wr, xs, b, (float *)out, part, ws_bytes - (size_t)(part - wsb), st, sp.Wp, -sp.pl, 0, d, sp.off);
+                r = run_wgrad_rows(c, &vr, sp.P, sp.Q, wr, xs, b, (float *)out, part, ws_bytes - (size_t)(part - wsb), st, sp.Wp, -sp.pl, 0, d, a, sp.off);
                 if (r != PT_ERR_UNSUPPORTED) return r;
             }
             if (r == PT_ERR_UNSUPPORTED) {

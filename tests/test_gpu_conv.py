@@ -302,6 +302,64 @@ def test_packed_weight_gradient(shape):
     c.close()
 
 
+def _dw_of_products(x, dy, R, S, stride, pad):
+    """dw from every product of an output pixel's dy with the pixel of x that a tap has there, zeros outside the image among them (0 x Inf is a
+    NaN), in fp64."""
+    N, P, Q, K = dy.shape
+    xp = torch.nn.functional.pad(x.double(), (0, 0, pad, pad + stride, pad, pad + stride))
+    dw = torch.empty((K, R, S, x.shape[3]), dtype=torch.float64)
+    for r in range(R):
+        for s in range(S):
+            v = xp[:, r:r + stride * (P - 1) + 1:stride, s:s + stride * (Q - 1) + 1:stride]
+            dw[:, r, s] = (dy.double()[..., :, None] * v[..., None, :]).sum((0, 1, 2))
+    return dw
+
+
+# Infinities and NaN at the edges of the images, where a row of pixels meets the next one, a unit's last row the rows behind it or a column
+# group the next: they reach the sums that they are part of and no other, in every form, however the splits exchange their sums
+# (N, H, W, C, K, R, S, stride, pad, ldx, ldy, form)
+@pytest.mark.parametrize("shape", [(3, 10, 9, 70, 40, 3, 3, 1, 1, 72, 40, "TAPS"), (2, 9, 12, 66, 130, 3, 3, 1, 0, 80, 136, "TAPS"), (3, 11, 14, 20, 70, 3, 3, 2, 1, 24, 72, "TAPS"),
+                                   (40, 7, 8, 68, 24, 3, 3, 2, 1, 72, 24, "TAPS"), (3, 10, 9, 70, 40, 3, 3, 1, 1, 72, 40, "PIXELS"), (3, 11, 14, 20, 70, 3, 3, 2, 1, 24, 72, "PIXELS"),
+                                   (3, 9, 13, 8, 20, 3, 3, 1, 1, 16, 32, "PACKED"), (40, 10, 11, 30, 9, 3, 3, 1, 1, 32, 16, "PACKED"), (2, 8, 9, 13, 12, 4, 5, 1, 2, 16, 32, "PACKED"),
+                                   (3, 10, 13, 20, 33, 3, 3, 1, 1, 24, 40, "ROWS"), (3, 9, 9, 41, 30, 3, 3, 1, 1, 48, 32, "ROWS"), (40, 7, 9, 12, 21, 5, 5, 1, 2, 16, 24, "ROWS"),
+                                   (2, 30, 30, 9, 12, 1, 1, 1, 0, 16, 16, "ROWS"), (2, 38, 32, 3, 16, 7, 7, 2, 3, 8, 16, "ANY"), (3, 12, 12, 4, 9, 3, 3, 2, 1, 8, 16, "ANY")])
+def test_infinities_and_nan_reach_their_own_weight_gradients_only(shape):
+    N, H, Wd, C, K, R, S, stride, pad, ldx, ldy, form = shape
+    P, Q = (H + 2 * pad - R) // stride + 1, (Wd + 2 * pad - S) // stride + 1
+    x, dy = W.gen_act(N, H, Wd, C, W.BASE_SEED + 91), W.gen_dy(N, P, Q, K, W.BASE_SEED + 92)
+    inf, nan = float("inf"), float("nan")
+    # one pixel in a channel of its own each: the corners of the first and the last image, the middles of the edges, an inner one
+    spots = [(0, 0, 0, inf), (N - 1, H - 1, Wd - 1, inf), (0, H - 1, 0, -inf), (0, 0, Wd - 1, nan), (0, H // 2, 0, inf), (N - 1, H // 2, Wd - 1, -inf), (0, 0, Wd // 2, nan), (0, H - 1, Wd // 2, inf),
+             (N // 2, H // 2, Wd // 2, nan)]
+    for c, (n, h, w_, v) in zip(range(C - 1, 0, -1), spots):      # (channel 0 stays finite)
+        x[n, h, w_, c] = v
+    for k, (n, p, q, v) in zip(range(K - 1, 1, -1), [(0, 0, 0, inf), (N - 1, P - 1, Q - 1, nan), (N // 2, P // 2, Q // 2, -inf)]):
+        dy[n, p, q, k] = v
+    ref = _dw_of_products(x, dy, R, S, stride, pad)
+    c = B.Context(0)
+    d = B.make_conv_desc(N, H, Wd, C, K, R, S, stride, pad, ldx, ldy, W.pad8(C), 0, 2)
+    xd, dyd = Hh.to_dev_padded(x, ldx), Hh.to_dev_padded(dy, ldy)
+    want = B.PT_FORM_ANY if form == "ANY" else getattr(B, "PT_FORM_WGRAD_" + form)
+    for limit in (0, 40, 1):
+        B.pt_test_wgrad_form(c, want)
+        B.pt_set_wgrad_cta_limit(c, limit)
+        ws = torch.empty(max(16, B.pt_conv_workspace_bytes(c, d, B.PT_CONV_WGRAD)), dtype=torch.uint8, device="cuda")
+        dw = torch.full((K, R, S, C), 7680.0, device="cuda")
+        B.pt_conv_wgrad(c, d, xd, dyd, dw, ws)
+        torch.cuda.synchronize()
+        c.poll()
+        assert want == B.PT_FORM_ANY or B.pt_test_last_form(c) == want
+        got = dw.cpu().double()
+        for what in (torch.isnan, torch.isposinf, torch.isneginf):
+            assert torch.equal(what(got), what(ref)), (limit, what.__name__, int((what(got) & ~what(ref)).sum()), int((what(ref) & ~what(got)).sum()))
+        fin = torch.isfinite(ref)
+        assert fin.any() and (~fin).any()
+        err = (got - ref)[fin]
+        # (fp32 sums of products of bf16 values: the bound of the other tests, of the finite part)
+        assert err.norm() <= 5e-3 * ref[fin].norm()
+    c.close()
+
+
 def test_wgrad_is_run_to_run_identical():
     N, H, C, K, R = 4, 14, 27, 19, 3
     x, w, dy, pad = _case(N, H, H, C, K, R, 1, W.BASE_SEED + 5)
