@@ -2416,14 +2416,15 @@ struct StemWalk {
 };
 
 // One position of a space-to-depth row: the four channels of four pixels of the image, zeros outside (i: the row, jp: the position), and
-// the 16 lanes they make, pixel by pixel.
+// the 16 lanes they make, pixel by pixel. (Plain loads: the kernel is on the SM before its predecessor, which may be writing the image, has
+// ended; the read-only path is for what nothing writes while the kernel runs.)
 __device__ __forceinline__ void stem_load(const StemP &p, int n, int i, int jp, uint2 (&px)[4])
 {
     const int j = jp - p.pl;
     const bool in = i >= 0 && i < p.Hs && j >= 0 && j < p.Ws;
 #pragma unroll
     for (int ab = 0; ab < 4; ++ab)
-        px[ab] = in ? __ldg(reinterpret_cast<const uint2 *>(p.x + ((size_t)(n * p.H + 2 * i + (ab >> 1)) * p.W + 2 * j + (ab & 1)) * 8)) : make_uint2(0, 0);
+        px[ab] = in ? *reinterpret_cast<const uint2 *>(p.x + ((size_t)(n * p.H + 2 * i + (ab >> 1)) * p.W + 2 * j + (ab & 1)) * 8) : make_uint2(0, 0);
 }
 __device__ __forceinline__ void stem_pack(int C, const uint2 (&px)[4], uint4 &lo, uint4 &hi)
 {

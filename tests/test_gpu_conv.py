@@ -115,6 +115,38 @@ def test_stem_straight_from_the_image(shape):
     c.close()
 
 
+def test_stem_behind_the_kernel_that_writes_its_image():
+    """The stem's kernel starts before its predecessor has ended (a batch norm, which releases its dependents early): every pass sees the image of
+    its own predecessor, whatever the same addresses held the pass before."""
+    N, H, C, K, R = 16, 128, 3, 40, 7
+    c = B.Context(0)
+    gen = torch.Generator(device="cuda").manual_seed(W.BASE_SEED + 50)
+    src = [torch.randn((N, H, H, 8), generator=gen, device="cuda").to(torch.bfloat16) for _ in range(2)]
+    w = Hh.to_dev_padded(W.bf16_round(W.gen_weight(K, R, R, C, W.BASE_SEED + 51)), 8)
+    d = B.make_conv_desc(N, H, H, C, K, R, R, 2, 3, 8, W.pad8(K), 8, 0, 2)
+    bn = B.make_bn_desc(N, H, H, C, 8)
+    g, b, sm, si = torch.ones(C, device="cuda"), torch.zeros(C, device="cuda"), torch.empty(C, device="cuda"), torch.empty(C, device="cuda")
+    wsb = torch.empty(B.pt_bn_workspace_bytes(c, bn), dtype=torch.uint8, device="cuda")
+    ws = torch.empty(B.pt_conv_workspace_bytes(c, d, B.PT_CONV_FWD), dtype=torch.uint8, device="cuda")
+    image = torch.empty_like(src[0])
+    ys = [torch.zeros((N, H // 2, H // 2, d.ldy), dtype=torch.bfloat16, device="cuda") for _ in range(40)]
+    for i, y in enumerate(ys):
+        B.pt_bn_relu_fwd(c, bn, src[i & 1], None, g, b, None, None, sm, si, image, wsb)
+        B.pt_conv_fwd(c, d, image, w, y, ws)
+    torch.cuda.synchronize()
+    c.poll()
+    assert B.pt_test_last_form(c) == B.PT_FORM_STEM
+    for i in range(2):
+        B.pt_bn_relu_fwd(c, bn, src[i], None, g, b, None, None, sm, si, image, wsb)
+        torch.cuda.synchronize()
+        alone = torch.zeros_like(ys[0])
+        B.pt_conv_fwd(c, d, image, w, alone, ws)
+        torch.cuda.synchronize()
+        assert all(torch.equal(y, alone) for y in ys[i::2])
+    assert not torch.equal(ys[0], ys[1])
+    c.close()
+
+
 # (N, H, W, C, K, R, pad) of the stride-2 forward by parity planes (more than two tiles a CTA): rows of 16, 32 and 64 lanes, one and several
 # chunks, resident and streamed weights, several channel tiles, odd sizes, no padding, an even filter
 @pytest.mark.parametrize("shape", [(150, 32, 32, 9, 17, 3, 1), (110, 33, 31, 32, 20, 3, 1), (80, 30, 60, 40, 33, 3, 0), (50, 56, 56, 70, 100, 3, 1), (100, 16, 130, 130, 24, 3, 1),
