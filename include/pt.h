@@ -76,7 +76,8 @@ pt_status pt_poll_device_status(pt_ctx *ctx, void *stream);
  *   which = 2: the next forward / data-gradient launch of the pixel-linear (GEMM-form) kernel -- the activation producer of
  *              every CTA leaves out the first pipeline stage;
  *   which = 3, 4, 5: the same for the next pass of a batch normalisation, the next channel gate that stages its rows in shared
- *              memory, the next convolution launch of the halo kernel;   which = 0 disarms.
+ *              memory, the next convolution launch of the halo kernel;
+ *   which = 6: the next forward pass of a stem straight from the image -- a row of its ring never becomes full;   which = 0 disarms.
  * The outputs of that launch are undefined. Not for production use. */
 pt_status pt_test_set_wait_limit(pt_ctx *ctx, uint32_t milliseconds);
 pt_status pt_test_skip_next_arrive(pt_ctx *ctx, int32_t which);

@@ -142,7 +142,7 @@ extern "C" pt_status pt_test_set_wait_limit(pt_ctx *c, uint32_t milliseconds)
 
 extern "C" pt_status pt_test_skip_next_arrive(pt_ctx *c, int32_t which)
 {
-    if (!c || which < 0 || which > 5) return PT_ERR_INVALID_ARG;
+    if (!c || which < 0 || which > 6) return PT_ERR_INVALID_ARG;
     c->test_skip = which;
     return PT_OK;
 }

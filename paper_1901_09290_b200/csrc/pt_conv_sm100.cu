@@ -2389,6 +2389,7 @@ struct StemP {
     float *stats;
     const __nv_bfloat16 *x, *w;
     unsigned int *status;
+    int test_skip;                      // test hook (pt_test_skip_next_arrive)
 };
 
 struct __align__(8) StemCtl {
@@ -2656,7 +2657,8 @@ __global__ void __launch_bounds__(kStemThreads, 1) conv_stem_kernel(const __grid
                 }
                 fence_proxy_async();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&ctl->full[s]));
+                // (test hook: the last ring row of the CTA's first output row never becomes full)
+                if (lane == 0 && !(p.test_skip && q == p.U - 1)) mbar_arrive(smem_u32(&ctl->full[s]));
                 load(px[k]);
             }
         }
@@ -3267,6 +3269,7 @@ pt_status run_stem(pt_ctx *c, const pt_conv_desc *d, const StemPlan &sp, const v
         if ((size_t)c->stats_parts * 2 * p.ld_out * sizeof(float) > c->stats_cap) return PT_ERR_WORKSPACE;
         p.stats = c->stats_out;
     }
+    if (c->test_skip == 6) { p.test_skip = 1; c->test_skip = 0; }
     PT_CUDA_OK(pt_launch_pdl(kernel, dim3((unsigned)grid), dim3(kStemThreads), smem, st, tmC, p));
     c->launches += 1;
     c->last_form = PT_FORM_STEM;

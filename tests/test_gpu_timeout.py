@@ -77,6 +77,72 @@ def test_split_weight_gradient_wait_runs_out_and_the_context_recovers():
     Hh.check_conv(dwb, 256, oracle.conv_wgrad(xb.numpy(), dyb.numpy(), 1, 1, 1, 0), what="wide wgrad after a time-out")
 
 
+# the forms that other layers choose: filter rows at both strides, packed rows, rows of blocks
+@pytest.mark.parametrize("form,N,H,C,K,stride,ld", [("TAPS", 6, 14, 70, 40, 1, 8), ("TAPS", 6, 15, 20, 130, 2, 8), ("PACKED", 8, 16, 13, 27, 1, 16), ("ROWS", 8, 16, 40, 27, 1, 8),
+                                                    ("PIXELS", 8, 16, 40, 27, 1, 8)])
+def test_every_form_of_the_weight_gradient_gives_up_and_recovers(form, N, H, C, K, stride, ld):
+    ctx = Hh.ctx()
+    P = (H + 2 - 3) // stride + 1
+    x, dy = W.gen_act(N, H, H, C, W.BASE_SEED + 69), W.gen_dy(N, P, P, K, W.BASE_SEED + 70)
+    up = lambda n: -(-n // ld) * ld
+    d = B.make_conv_desc(N, H, H, C, K, 3, 3, stride, 1, up(C), up(K), algo=2)
+    xd, dyd = Hh.to_dev_padded(x, d.ldx), Hh.to_dev_padded(dy, d.ldy)
+    want = getattr(B, "PT_FORM_WGRAD_" + form)
+    B.pt_test_wgrad_form(ctx, want)
+    try:
+        ctas, waits = B.pt_conv_wgrad_ctas(ctx, d)
+        assert waits and ctas > 1
+        dw = torch.zeros((K, 3, 3, C), dtype=torch.float32, device="cuda")
+        ws = Hh.conv_ws(d, B.PT_CONV_WGRAD)
+
+        def launch():
+            B.pt_test_skip_next_arrive(ctx, 1)
+            B.pt_conv_wgrad(ctx, d, xd, dyd, dw, ws)
+
+        _expect_timeout(ctx, launch)
+        ref = oracle.conv_wgrad(x.numpy(), dy.numpy(), 3, 3, stride, 1)
+        for _ in range(3):
+            dw.fill_(7680.0)
+            B.pt_conv_wgrad(ctx, d, xd, dyd, dw, ws)
+            torch.cuda.synchronize()
+            ctx.poll()
+            assert B.pt_test_last_form(ctx) == want
+            Hh.check_conv(dw, C, ref, what="wgrad after a time-out")
+    finally:
+        B.pt_test_wgrad_form(ctx, B.PT_FORM_ANY)
+
+
+# one and two accumulators an issuer, with and without statistics; a CTA of one output row and of several
+@pytest.mark.parametrize("N,H,K,stats", [(2, 128, 20, False), (12, 128, 90, True)])
+def test_stem_wait_runs_out_and_the_context_recovers(N, H, K, stats):
+    ctx = Hh.ctx()
+    x, w = W.gen_act(N, H, H, 3, W.BASE_SEED + 71), W.bf16_round(W.gen_weight(K, 7, 7, 3, W.BASE_SEED + 72))
+    d = B.make_conv_desc(N, H, H, 3, K, 7, 7, 2, 3, algo=2)
+    xd, wd = Hh.to_dev_padded(x, d.ldx), Hh.to_dev_padded(w, d.ldw)
+    y = torch.zeros((N, H // 2, H // 2, d.ldy), dtype=torch.bfloat16, device="cuda")
+    ws = Hh.conv_ws(d, B.PT_CONV_FWD)
+    st = torch.empty(B.pt_conv_fwd_stats_bytes(ctx, d) // 4, device="cuda")
+    run = lambda out: B.pt_conv_fwd_stats(ctx, d, xd, wd, out, st, ws) if stats else B.pt_conv_fwd(ctx, d, xd, wd, out, ws)
+
+    def launch():
+        B.pt_test_skip_next_arrive(ctx, 6)
+        run(y)
+
+    _expect_timeout(ctx, launch)
+    ref = oracle.conv_fwd(x.numpy(), w.numpy(), 2, 3)
+    for _ in range(3):
+        yo = Hh.out_buffer((N, H // 2, H // 2), K, d.ldy, False)
+        run(yo)
+        torch.cuda.synchronize()
+        ctx.poll()
+        assert B.pt_test_last_form(ctx) == B.PT_FORM_STEM
+        Hh.check_conv(yo, K, ref, what="stem after a time-out")
+    # a launch that takes all 512 columns of every SM's tensor memory
+    xb, wb, dyb = _inputs(4, 28, 256, 256, 1, W.BASE_SEED + 73)
+    dwb = Hh.run_conv_all(4, 28, 28, 256, 256, 1, 1, 0, xb, wb, dyb, algo=2)[2]
+    Hh.check_conv(dwb, 256, oracle.conv_wgrad(xb.numpy(), dyb.numpy(), 1, 1, 1, 0), what="wide wgrad after a time-out")
+
+
 def test_pipeline_barrier_wait_runs_out_and_the_context_recovers():
     ctx = Hh.ctx()
     N, H, C, K, R = 8, 16, 16, 32, 1                            # a 1x1 layer: the pixel-linear kernel
