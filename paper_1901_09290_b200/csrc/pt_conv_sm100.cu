@@ -2577,26 +2577,32 @@ __global__ void __launch_bounds__(kStemThreads, 1) conv_stem_kernel(const __grid
                     if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");   // the slab's previous store has read it
                     __syncwarp();
                     const int groups = min(4, (p.BN - ch * 64) / 16);
-                    uint32_t v[4][16];
+                    // (with statistics two groups of 16 columns at a time: four of them do not fit the registers of 640 threads beside the sums)
+                    constexpr int G = STATS ? 2 : 4;
 #pragma unroll
-                    for (int g = 0; g < 4; ++g)
-                        if (g < groups) tmem_ld16(lane_addr + (uint32_t)(ch * 64 + g * 16), v[g]);
-                    tmem_ld_wait();
-                    if (ch + 1 >= n_chunks) {
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(smem_u32(&ctl->acc_empty[b]));
-                    }
+                    for (int g0 = 0; g0 < 4; g0 += G) {
+                        if (g0 >= groups) break;
+                        uint32_t v[G][16];
 #pragma unroll
-                    for (int g = 0; g < 4; ++g) {
-                        if (g >= groups) break;
+                        for (int g = 0; g < G; ++g)
+                            if (g0 + g < groups) tmem_ld16(lane_addr + (uint32_t)(ch * 64 + (g0 + g) * 16), v[g]);
+                        tmem_ld_wait();
+                        if (ch + 1 >= n_chunks && g0 + G >= groups) {
+                            tc_fence_before();
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(smem_u32(&ctl->acc_empty[b]));
+                        }
 #pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            __nv_bfloat162 e[4];
+                        for (int g = 0; g < G; ++g) {
+                            if (g0 + g >= groups) break;
 #pragma unroll
-                            for (int k = 0; k < 4; ++k) e[k] = __floats2bfloat162_rn(__uint_as_float(v[g][8 * h + 2 * k]), __uint_as_float(v[g][8 * h + 2 * k + 1]));
-                            const uint32_t j = (uint32_t)(g * 2 + h);
-                            st_shared_v4(slab + (uint32_t)lane * 128u + ((j ^ ((uint32_t)lane & 7u)) << 4), *reinterpret_cast<uint4 *>(e));
+                            for (int h = 0; h < 2; ++h) {
+                                __nv_bfloat162 e[4];
+#pragma unroll
+                                for (int k = 0; k < 4; ++k) e[k] = __floats2bfloat162_rn(__uint_as_float(v[g][8 * h + 2 * k]), __uint_as_float(v[g][8 * h + 2 * k + 1]));
+                                const uint32_t j = (uint32_t)((g0 + g) * 2 + h);
+                                st_shared_v4(slab + (uint32_t)lane * 128u + ((j ^ ((uint32_t)lane & 7u)) << 4), *reinterpret_cast<uint4 *>(e));
+                            }
                         }
                     }
                     fence_proxy_async();
