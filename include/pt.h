@@ -81,16 +81,17 @@ pt_status pt_poll_device_status(pt_ctx *ctx, void *stream);
  * The outputs of that launch are undefined. Not for production use. */
 pt_status pt_test_set_wait_limit(pt_ctx *ctx, uint32_t milliseconds);
 pt_status pt_test_skip_next_arrive(pt_ctx *ctx, int32_t which);
-/* Testing hooks for the choice of a convolution kernel. pt_test_wgrad_form: from now on the context's weight gradients (and what
- * pt_conv_workspace_bytes and pt_conv_wgrad_ctas say of them) take the given form wherever it can serve the descriptor, whatever its estimated time;
- * PT_FORM_ANY (the default) chooses by time. PT_ERR_INVALID_ARG for a form that is not one of a weight gradient. pt_test_last_form: the form
- * of the last convolution that the tcgen05 kernels ran for this context, PT_FORM_ANY before the first. Not for production use. */
+/* Testing hooks for the choice of a convolution kernel. pt_test_form: from now on the context's calls take the given form wherever it can serve
+ * the descriptor, whether or not it pays: one of the four of a weight gradient (pt_conv_workspace_bytes and pt_conv_wgrad_ctas follow), or
+ * the parity planes of a stride-2 forward pass; PT_FORM_ANY (the default) leaves the choice to the library, PT_ERR_INVALID_ARG for any other.
+ * pt_test_last_form: the form of the last convolution that the tcgen05 kernels ran for this context, PT_FORM_ANY before the first.
+ * Not for production use. */
 enum {
     PT_FORM_ANY = 0,
     PT_FORM_WGRAD_PIXELS = 1, PT_FORM_WGRAD_ROWS = 2, PT_FORM_WGRAD_TAPS = 3, PT_FORM_WGRAD_PACKED = 4,
     PT_FORM_GEMM = 5, PT_FORM_HALO = 6, PT_FORM_PLANES = 7, PT_FORM_STEM = 8
 };
-pt_status pt_test_wgrad_form(pt_ctx *ctx, int32_t form);
+pt_status pt_test_form(pt_ctx *ctx, int32_t form);
 int32_t pt_test_last_form(const pt_ctx *ctx);
 /* Number of kernels this context has launched since creation (for launch accounting). */
 uint64_t pt_launch_count(const pt_ctx *ctx);

@@ -84,7 +84,7 @@ EXPORTS = {
     "pt_launch_count": (c_uint64, [c_void_p]),
     "pt_test_set_wait_limit": (c_int32, [c_void_p, ctypes.c_uint32]),
     "pt_test_skip_next_arrive": (c_int32, [c_void_p, c_int32]),
-    "pt_test_wgrad_form": (c_int32, [c_void_p, c_int32]),
+    "pt_test_form": (c_int32, [c_void_p, c_int32]),
     "pt_test_last_form": (c_int32, [c_void_p]),
     "pt_set_wgrad_cta_limit": (c_int32, [c_void_p, c_int32]),
     "pt_set_dgrad_cta_limit": (c_int32, [c_void_p, c_int32]),
@@ -222,8 +222,8 @@ def pt_test_skip_next_arrive(ctx: Context, which: int):
     _check(lib().pt_test_skip_next_arrive(ctx.handle, which), "pt_test_skip_next_arrive")
 
 
-def pt_test_wgrad_form(ctx: Context, form: int):
-    _check(lib().pt_test_wgrad_form(ctx.handle, form), "pt_test_wgrad_form")
+def pt_test_form(ctx: Context, form: int):
+    _check(lib().pt_test_form(ctx.handle, form), "pt_test_form")
 
 
 def pt_test_last_form(ctx: Context) -> int:

@@ -147,9 +147,9 @@ extern "C" pt_status pt_test_skip_next_arrive(pt_ctx *c, int32_t which)
     return PT_OK;
 }
 
-extern "C" pt_status pt_test_wgrad_form(pt_ctx *c, int32_t form)
+extern "C" pt_status pt_test_form(pt_ctx *c, int32_t form)
 {
-    if (!c || form < PT_FORM_ANY || form > PT_FORM_WGRAD_PACKED) return PT_ERR_INVALID_ARG;
+    if (!c || form < PT_FORM_ANY || (form > PT_FORM_WGRAD_PACKED && form != PT_FORM_PLANES)) return PT_ERR_INVALID_ARG;
     c->test_form = form;
     return PT_OK;
 }

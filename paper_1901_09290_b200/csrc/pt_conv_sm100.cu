@@ -3029,6 +3029,33 @@ struct HaloSpec {
     int max_ctas;                                    // > 0: grid limit (launches meant to run side by side share the SMs)
 };
 
+// Whether the parity planes pay, given a launch's rings: against the im2col form they have four boxes a chunk to wait for, whole raster rows in
+// tiles of 128, and weights that stream once per round of tiles where they are not resident. By the times of 480 random stride-2 layers (5 to
+// 400 channels, 2x2 to 5x5 filters, forward alone and with statistics; planes and im2col):
+//   a tap to a plane (2x2): rows of at most 32 lanes (17 -> 149 at 14x14, batch 478 16 and 25 us; 151 -> 94 at 17x17, batch 117 25 and 13);
+//   resident weights: always, but not with single stages for two issuers and more than two chunks (315 -> 32 at 27x27, batch 102 96 and 65) or, two
+//     chunks or more a stage, in tiles that hold few output pixels (170 -> 7 at 13x13, batch 445 45 and 31; 159 -> 19 at 27x27 22 and 30);
+//   streamed weights: rounds of tiles of which 55 % is work (354 -> 51 at 28x28, batch 12 58 and 41; 365 -> 190 at 28x28, batch 65 73 and 86), fewer
+//     with up to two chunks (94 -> 82 at 8x8 19 and 16; 52 -> 177 at 28x22 17 and 21); one issuer with many taps only (64 -> 209 at 27x27,
+//     batch 64 22 and 17; 41 -> 192 5x5 123 and 155); several channel tiles with narrow rows of one chunk only (83 -> 305 at 16x16 84 and 62; 17 ->
+//     352 at 28x16 21 and 28).
+// The layers take 0.71 of the im2col form's time by this rule, 0.74 without it and 0.71 by the faster of the two each.
+bool planes_pay(const pt_ctx *c, const HaloP &p, int taps)
+{
+    const double useful = (double)p.P * p.Q / (p.row_tiles * 128.0), slot = (double)p.N * p.row_tiles * p.n_tiles / c->sm_count / p.n_issuers;
+    const bool busy = useful * slot >= 0.55 * ceil(slot);
+    const int per = p.stages_a / p.n_issuers;
+    if (taps <= 4) return p.lanes < 64 && p.resident && (p.n_issuers == 4 || busy);
+    if (p.resident) {
+        if (taps >= 16 || per >= 2) return true;
+        if (p.n_issuers == 2 && p.k_chunks > 2) return false;
+        return useful >= 0.72 || p.k_chunks * (p.n_issuers == 2 ? 2 : 1) <= 2;
+    }
+    if (p.n_tiles > 1) return p.k_chunks == 1 && p.lanes < 64 && busy;
+    if (p.n_issuers == 1) return taps >= 16 && busy;
+    return busy || (p.k_chunks <= 2 && (taps >= 16 || useful >= 0.6));
+}
+
 template <bool B_MN, int PL = 1>
 pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const void *w, void *out, cudaStream_t st)
 {
@@ -3045,7 +3072,7 @@ pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const
     // the im2col form's many small loads are sooner there (3x3/2, planes against im2col: 106 -> 103 at 56x56, batch 64, 448 tiles 23.6 and 25.7 us,
     // 38 -> 38 at 56x56, batch 256 33.7 and 48.5, 8 -> 17 at 32x32, batch 128, 384 tiles 6.4 and 10.6; 64 -> 128 at 32x32, batch 64, 192
     // tiles 11.1 and 7.9; 200 -> 200 at 28x28, batch 64, 128 tiles 23.4 and 19.6).
-    if (PL > 1 && (long long)p.N * p.row_tiles * p.n_tiles <= 2 * c->sm_count) return PT_ERR_UNSUPPORTED;
+    if (PL > 1 && c->test_form != PT_FORM_PLANES && (long long)p.N * p.row_tiles * p.n_tiles <= 2 * c->sm_count) return PT_ERR_UNSUPPORTED;
     p.c_red = h.Cs; p.k_chunks = pt_ceil_div(h.Cs, kKC); p.taps = h.n_taps;
     // Channel lanes per staged pixel: narrow layers take rows of 64 or 32 bytes. The TMA unit's time is per row, and a row whose tensor
     // ends in the middle of a sector costs it twice as much in a 128-byte box (4.5 ns for 19 channels) as a whole one (2.3 ns); in a
@@ -3075,62 +3102,72 @@ pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const
     p.b_slot = (int)b_bytes;
     // narrow outputs are stored from registers (the 16-byte vectors of a pixel must be whole: room in the pitch)
     p.direct_cols = pt_ceil_div(h.n_cols, 16) * 16 <= h.ld_out ? pt_ceil_div(h.n_cols, 16) * 16 : pt_ceil_div(h.n_cols, 8) * 8;
-    p.direct = (!d->out_f32 && !c->stats_mode && p.n_tiles == 1 && p.BN <= 32) ? 1 : 0;
-    // epilogue staging: a slab of the tile's raster rows x 128 bytes per group, two where the launch's other needs leave room (direct-store
-    // launches use none)
-    p.tma_store = (d->out_f32 || p.direct) ? 0 : 1;
-    p.staging = !p.tma_store ? 0 : (int)pt_align_up((size_t)(p.nr * Wp < 128 ? p.nr * Wp : 128) * 128, 1024);
-    p.slabs = 1;
-    p.stats_warp = pt_ceil_div(p.BN, 64) * (int)kStatsChunkBytes;
-    const size_t st_smem = c->stats_mode ? (size_t)8 * p.stats_warp : 0;        // statistics accumulators of the eight epilogue warps
-    const size_t budget = 227 * 1024 - 2048 - 2 * (size_t)p.staging - a_tail - st_smem;
     const size_t w_all = (size_t)h.n_taps * p.k_chunks * b_bytes;
-    p.resident = (p.n_tiles == 1 && w_all + 2 * (size_t)p.a_alloc <= budget) ? 1 : 0;
-    size_t left = budget - (p.resident ? w_all : 0);
-    bool two_pipes = false;
-    if (!p.resident) {
-        // ring: at least two A stages, the rest for weight stages (at least 3)
-        p.stages_a = 2;
-        if (left < 2 * (size_t)p.a_alloc + 3 * b_bytes) return PT_ERR_UNSUPPORTED;
-        size_t sb = (left - 2 * (size_t)p.a_alloc) / b_bytes;
-        p.stages_b = sb > kMaxStages ? kMaxStages : (int)sb;
-        // two pipelines (one per tile parity) when each can have three weight stages and the CTAs get several tiles
-        // (a launch that shares the SMs with others has fewer CTAs, each with more tiles)
-        const int ctas_avail = (h.max_ctas > 0 && h.max_ctas < c->sm_count) ? h.max_ctas : c->sm_count;
-        two_pipes = p.stages_b >= 6 && pt_ceil_div(p.N * p.row_tiles * p.n_tiles, ctas_avail) >= 2;
-        if (two_pipes) p.stages_b = p.stages_b / 2 * 2;
-        // Two pipelines on one weight stream (a single channel tile): every chunk of both tiles should have an activation stage
-        // of its own -- a chunk that waits for the previous chunk's MMAs to free its stage exposes a DRAM round trip per tile
-        // (28x28, 69 -> 93 channels, MN-major weights: two stages against four, 30 -> 22 us) -- as long as four weight stages
-        // remain for the shared stream.
-        const int want_a = 2 * p.k_chunks * PL > 4 ? 4 : 2 * p.k_chunks * PL;
-        if (two_pipes && p.n_tiles == 1 && left >= (size_t)want_a * p.a_alloc + 4 * b_bytes) {
-            const size_t sb2 = (left - (size_t)want_a * p.a_alloc) / b_bytes;
-            if ((size_t)p.stages_b > sb2) p.stages_b = (int)sb2;
+    // The rings of a launch, for outputs in fp32 or bf16, with statistics or without; false where they do not fit.
+    const auto rings = [&](HaloP &p, bool f32, bool stats) {
+        p.direct = (!f32 && !stats && p.n_tiles == 1 && p.BN <= 32) ? 1 : 0;
+        // epilogue staging: a slab of the tile's raster rows x 128 bytes per group, two where the launch's other needs leave room (direct-store
+        // launches use none)
+        p.tma_store = (f32 || p.direct) ? 0 : 1;
+        p.staging = !p.tma_store ? 0 : (int)pt_align_up((size_t)(p.nr * Wp < 128 ? p.nr * Wp : 128) * 128, 1024);
+        p.slabs = 1;
+        p.stats_warp = pt_ceil_div(p.BN, 64) * (int)kStatsChunkBytes;
+        const size_t st_smem = stats ? (size_t)8 * p.stats_warp : 0;             // statistics accumulators of the eight epilogue warps
+        const size_t budget = 227 * 1024 - 2048 - 2 * (size_t)p.staging - a_tail - st_smem;
+        p.resident = (p.n_tiles == 1 && w_all + 2 * (size_t)p.a_alloc <= budget) ? 1 : 0;
+        size_t left = budget - (p.resident ? w_all : 0);
+        bool two_pipes = false;
+        if (!p.resident) {
+            // ring: at least two A stages, the rest for weight stages (at least 3)
+            p.stages_a = 2;
+            if (left < 2 * (size_t)p.a_alloc + 3 * b_bytes) return false;
+            size_t sb = (left - 2 * (size_t)p.a_alloc) / b_bytes;
+            p.stages_b = sb > kMaxStages ? kMaxStages : (int)sb;
+            // two pipelines (one per tile parity) when each can have three weight stages and the CTAs get several tiles
+            // (a launch that shares the SMs with others has fewer CTAs, each with more tiles)
+            const int ctas_avail = (h.max_ctas > 0 && h.max_ctas < c->sm_count) ? h.max_ctas : c->sm_count;
+            two_pipes = p.stages_b >= 6 && pt_ceil_div(p.N * p.row_tiles * p.n_tiles, ctas_avail) >= 2;
+            if (two_pipes) p.stages_b = p.stages_b / 2 * 2;
+            // Two pipelines on one weight stream (a single channel tile): every chunk of both tiles should have an activation stage
+            // of its own -- a chunk that waits for the previous chunk's MMAs to free its stage exposes a DRAM round trip per tile
+            // (28x28, 69 -> 93 channels, MN-major weights: two stages against four, 30 -> 22 us) -- as long as four weight stages
+            // remain for the shared stream.
+            const int want_a = 2 * p.k_chunks * PL > 4 ? 4 : 2 * p.k_chunks * PL;
+            if (two_pipes && p.n_tiles == 1 && left >= (size_t)want_a * p.a_alloc + 4 * b_bytes) {
+                const size_t sb2 = (left - (size_t)want_a * p.a_alloc) / b_bytes;
+                if ((size_t)p.stages_b > sb2) p.stages_b = (int)sb2;
+            }
+            left -= (size_t)p.stages_b * b_bytes;
+            int sa = (int)(left / p.a_alloc);
+            p.stages_a = sa > 4 ? 4 : sa;
+        } else {
+            // (one stage per issuer leaves its load latency exposed on every tile: 19 -> 19 at 56x56, batch 256, 46 us with 4 stages, 36 with 8)
+            int sa = (int)(left / p.a_alloc);
+            p.stages_a = sa > kHaloMaxA ? kHaloMaxA : sa;
+            p.stages_b = 1;
         }
-        left -= (size_t)p.stages_b * b_bytes;
-        int sa = (int)(left / p.a_alloc);
-        p.stages_a = sa > 4 ? 4 : sa;
-    } else {
-        // (one stage per issuer leaves its load latency exposed on every tile: 19 -> 19 at 56x56, batch 256, 46 us with 4 stages, 36 with 8)
-        int sa = (int)(left / p.a_alloc);
-        p.stages_a = sa > kHaloMaxA ? kHaloMaxA : sa;
-        p.stages_b = 1;
+        if (p.stages_a < 2) return false;
+        if (p.tma_store && p.resident && left >= kHaloMaxA * (size_t)p.a_alloc + 2 * (size_t)p.staging) p.slabs = 2;
+        // issuer warps: several only with resident weights; each needs an A stage of its own and an accumulator buffer
+        p.n_issuers = 1;
+        p.acc_per = 2;
+        if (p.resident) {
+            p.n_issuers = (p.stages_a >= 4 && 4 * p.BN <= 512) ? 4 : 2;
+            p.acc_per = p.n_issuers * 2 * p.BN <= 512 ? 2 : 1;
+        } else if (two_pipes) {
+            p.n_issuers = 2;
+            p.acc_per = 4 * p.BN <= 512 ? 2 : 1;
+            p.shared_b = p.n_tiles == 1 ? 1 : 0;          // the tiles of a round then use the same weight columns
+        }
+        p.stages_a = p.stages_a / p.n_issuers * p.n_issuers;
+        return true;
+    };
+    // (planes or not by the rings of the plain bf16 output, so that the same sums leave in every form: with statistics, in fp32)
+    if (PL > 1 && c->test_form != PT_FORM_PLANES) {
+        HaloP q = p;
+        if (!rings(q, false, false) || !planes_pay(c, q, h.n_taps)) return PT_ERR_UNSUPPORTED;
     }
-    if (p.stages_a < 2) return PT_ERR_UNSUPPORTED;
-    if (p.tma_store && p.resident && left >= kHaloMaxA * (size_t)p.a_alloc + 2 * (size_t)p.staging) p.slabs = 2;
-    // issuer warps: several only with resident weights; each needs an A stage of its own and an accumulator buffer
-    p.n_issuers = 1;
-    p.acc_per = 2;
-    if (p.resident) {
-        p.n_issuers = (p.stages_a >= 4 && 4 * p.BN <= 512) ? 4 : 2;
-        p.acc_per = p.n_issuers * 2 * p.BN <= 512 ? 2 : 1;
-    } else if (two_pipes) {
-        p.n_issuers = 2;
-        p.acc_per = 4 * p.BN <= 512 ? 2 : 1;
-        p.shared_b = p.n_tiles == 1 ? 1 : 0;          // the tiles of a round then use the same weight columns
-    }
-    p.stages_a = p.stages_a / p.n_issuers * p.n_issuers;
+    if (!rings(p, d->out_f32 != 0, c->stats_mode != 0)) return PT_ERR_UNSUPPORTED;
     p.tmem_cols = pow2_cols(p.n_issuers * p.acc_per * p.BN);
     p.out = out; p.ld_out = h.ld_out; p.out_f32 = d->out_f32;
     p.oH = h.oH; p.oW = h.oW; p.o_step = h.o_step; p.o_h0 = h.o_h0; p.o_w0 = h.o_w0;
@@ -3173,6 +3210,7 @@ pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const
                                                       CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (!map_ok(r, __LINE__)) return PT_ERR_CUDA;
     }
+    const size_t st_smem = c->stats_mode ? (size_t)8 * p.stats_warp : 0;
     const size_t smem = 2048 + 2 * (size_t)p.slabs * p.staging + (p.resident ? w_all : (size_t)p.stages_b * b_bytes) + (size_t)p.stages_a * p.a_alloc + a_tail +
                         st_smem;
     p.stats_off = (int)(smem - st_smem);
@@ -3632,7 +3670,7 @@ pt_wgrad_plan wgrad_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, b
 {
     pt_ctx::WgradKey key{*d, wgrad_budget(c), P, Q};
     static_assert(sizeof(key) == sizeof(pt_conv_desc) + 12, "the key is compared and hashed as words");
-    const int form = rows_only ? PT_FORM_ANY : c->test_form;
+    const int form = rows_only || c->test_form > PT_FORM_WGRAD_PACKED ? (int)PT_FORM_ANY : c->test_form;
     key.d.ldw = key.d.out_f32 = 0; key.d.algo = rows_only ? 1 : 2 * form;
     std::lock_guard<std::mutex> lock(c->wgrad_mutex);
     const auto known = c->wgrad_plans.find(key);
@@ -4227,7 +4265,7 @@ pt_status pt_sm100_conv(pt_ctx *c, const pt_conv_desc *d, int which, const void 
         pt_status r = launch_halo<false>(c, d, h, b, out, st);
         if (r != PT_ERR_UNSUPPORTED) return r;
     }
-    if (!sparse_tiles && which == PT_CONV_FWD && d->stride == 2 && d->R * d->S > 1) {
+    if ((!sparse_tiles || c->test_form == PT_FORM_PLANES) && which == PT_CONV_FWD && d->stride == 2 && d->R * d->S > 1) {
         HaloSpec h;
         if (halo_spec_stride2(d, &h, a, P, Q)) {
             const pt_status r = launch_halo<false, 4>(c, d, h, b, out, st);

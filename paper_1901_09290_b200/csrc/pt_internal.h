@@ -111,7 +111,7 @@ struct pt_ctx {
     size_t stats_cap = 0;
     int test_skip = 0;                  // pt_test_skip_next_arrive: 1 = next split weight gradient, 2 = next fwd/dgrad GEMM-form launch,
                                         // 3 = next batch-norm pass, 4 = next staged gate, 5 = next halo-form launch, 6 = next direct stem
-    int test_form = 0, last_form = 0;   // pt_test_wgrad_form, pt_test_last_form
+    int test_form = 0, last_form = 0;   // pt_test_form, pt_test_last_form
     int dgrad_ctas = 0;                 // pt_set_dgrad_cta_limit (0: none)
     // Plans of the weight-gradient descriptors met so far: choosing one walks a few hundred candidates (about 10 us), a call must not.
     // A network has about fifty, each at a few CTA limits; past kWgradPlans the table starts again.

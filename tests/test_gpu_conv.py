@@ -147,11 +147,25 @@ def test_stem_behind_the_kernel_that_writes_its_image():
     c.close()
 
 
-# (N, H, W, C, K, R, pad) of the stride-2 forward by parity planes (more than two tiles a CTA): rows of 16, 32 and 64 lanes, one and several
+# (N, H, W, C, K, R, pad) of the stride-2 forward by parity planes, taken whether they pay or not, and in the form of the library's choice: rows of 16, 32 and 64 lanes, one and several
 # chunks, resident and streamed weights, several channel tiles, odd sizes, no padding, an even filter
 @pytest.mark.parametrize("shape", [(150, 32, 32, 9, 17, 3, 1), (110, 33, 31, 32, 20, 3, 1), (80, 30, 60, 40, 33, 3, 0), (50, 56, 56, 70, 100, 3, 1), (100, 16, 130, 130, 24, 3, 1),
-                                   (60, 40, 42, 17, 300, 3, 1), (170, 24, 40, 20, 12, 2, 0), (120, 26, 34, 24, 40, 5, 2)])
+                                   (60, 40, 42, 17, 300, 3, 1), (170, 24, 40, 20, 12, 2, 0), (120, 26, 34, 24, 40, 5, 2),
+                                   (2, 15, 14, 70, 300, 3, 1), (1, 7, 9, 8, 8, 4, 1), (3, 9, 70, 200, 40, 3, 0), (2, 56, 56, 260, 210, 3, 1)])
 def test_stride_2_forward_by_planes(shape):
+    c = Hh.ctx()
+    B.pt_test_form(c, B.PT_FORM_PLANES)
+    try:
+        _stride_2_forward(shape)
+        assert B.pt_test_last_form(c) == B.PT_FORM_PLANES
+    finally:
+        B.pt_test_form(c, B.PT_FORM_ANY)
+    _stride_2_forward(shape)
+    with pytest.raises(B.PtError):
+        B.pt_test_form(c, B.PT_FORM_STEM)
+
+
+def _stride_2_forward(shape):
     N, H, Wd, C, K, R, pad = shape
     x = W.gen_act(N, H, Wd, C, W.BASE_SEED + 48)
     w = W.bf16_round(W.gen_weight(K, R, R, C, W.BASE_SEED + 49))
@@ -160,7 +174,6 @@ def test_stride_2_forward_by_planes(shape):
     c = Hh.ctx()
     y = Hh.out_buffer((N, P, Q), K, d.ldy, 0)
     B.pt_conv_fwd(c, d, Hh.to_dev_padded(x, d.ldx), Hh.to_dev_padded(w, d.ldw), y, Hh.conv_ws(d, B.PT_CONV_FWD))
-    assert B.pt_test_last_form(c) == B.PT_FORM_PLANES
     torch.cuda.synchronize()
     c.poll()
     # (the oracle for images of either end and the middle; fp64 torch for all)
@@ -271,7 +284,7 @@ def test_weight_gradient_of_nan_pad_lanes(shape):
 
 def _wgrad_of_form(c, d, xd, dyd, form, limit):
     """The weight gradient in the given form (PT_FORM_ANY: the library's choice) at a CTA limit, computed twice, and the form that it took."""
-    B.pt_test_wgrad_form(c, form)
+    B.pt_test_form(c, form)
     B.pt_set_wgrad_cta_limit(c, limit)
     try:
         ws = torch.empty(max(16, B.pt_conv_workspace_bytes(c, d, B.PT_CONV_WGRAD)), dtype=torch.uint8, device="cuda")
@@ -282,7 +295,7 @@ def _wgrad_of_form(c, d, xd, dyd, form, limit):
         torch.cuda.synchronize()
         c.poll()
     finally:
-        B.pt_test_wgrad_form(c, B.PT_FORM_ANY)
+        B.pt_test_form(c, B.PT_FORM_ANY)
         B.pt_set_wgrad_cta_limit(c, 0)
     assert torch.equal(dw, again)
     return dw, B.pt_test_last_form(c)
@@ -373,7 +386,7 @@ def test_infinities_and_nan_reach_their_own_weight_gradients_only(shape):
     xd, dyd = Hh.to_dev_padded(x, ldx), Hh.to_dev_padded(dy, ldy)
     want = B.PT_FORM_ANY if form == "ANY" else getattr(B, "PT_FORM_WGRAD_" + form)
     for limit in (0, 40, 1):
-        B.pt_test_wgrad_form(c, want)
+        B.pt_test_form(c, want)
         B.pt_set_wgrad_cta_limit(c, limit)
         ws = torch.empty(max(16, B.pt_conv_workspace_bytes(c, d, B.PT_CONV_WGRAD)), dtype=torch.uint8, device="cuda")
         dw = torch.full((K, R, S, C), 7680.0, device="cuda")

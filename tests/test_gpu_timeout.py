@@ -88,7 +88,7 @@ def test_every_form_of_the_weight_gradient_gives_up_and_recovers(form, N, H, C, 
     d = B.make_conv_desc(N, H, H, C, K, 3, 3, stride, 1, up(C), up(K), algo=2)
     xd, dyd = Hh.to_dev_padded(x, d.ldx), Hh.to_dev_padded(dy, d.ldy)
     want = getattr(B, "PT_FORM_WGRAD_" + form)
-    B.pt_test_wgrad_form(ctx, want)
+    B.pt_test_form(ctx, want)
     try:
         ctas, waits = B.pt_conv_wgrad_ctas(ctx, d)
         assert waits and ctas > 1
@@ -109,7 +109,7 @@ def test_every_form_of_the_weight_gradient_gives_up_and_recovers(form, N, H, C, 
             assert B.pt_test_last_form(ctx) == want
             Hh.check_conv(dw, C, ref, what="wgrad after a time-out")
     finally:
-        B.pt_test_wgrad_form(ctx, B.PT_FORM_ANY)
+        B.pt_test_form(ctx, B.PT_FORM_ANY)
 
 
 # one and two accumulators an issuer, with and without statistics; a CTA of one output row and of several
