@@ -1556,32 +1556,38 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, Ctl *ctl, uint32_t
             } else if (PAIR) {
                 // lanes are (tap of the accumulator, input channel), columns are output channels: for one column a warp's lanes
                 // write consecutive floats of dw
-                const int l = quarter * 32 + lane;
+                // (addresses once per accumulator and a pitch per column: with the place in dw found anew for each float, two accumulators of 176
+                // columns took 11 us, 6 before that)
+                const int l = quarter * 32 + lane, C = p.raw.C;
+                const size_t pitch = (size_t)p.raw.R * p.raw.S * C;
                 int ci = 0;
-                for (int tt = 0; tt < n_acc; ++tt)
-                for (int cc = 0; cc < acc_cols; cc += 16, ++ci) {
-                    if ((ci & 1) != wset) continue;
+                for (int tt = 0; tt < n_acc; ++tt) {
                     int tap = wgrad_tap(p, tap0 + tt, l >> p.lane_shift), c = l & (p.lanes - 1);
-                    uint32_t v[16];
-                    if (iters > 0) {
-                        tmem_ld16(lane_addr + (uint32_t)(tt * acc_cols + cc), v);
-                        tmem_ld_wait();
-                    } else {
-#pragma unroll
-                        for (int e = 0; e < 16; ++e) v[e] = 0u;
-                    }
                     const bool here = wgrad_pair_place(p, tap, c);
-                    unsigned bad = 0u;                       // a bit per four sums
+                    float *const dst = p.out + (here ? (size_t)tap * C + c : 0);
+                    for (int cc = 0; cc < acc_cols; cc += 16, ++ci) {
+                        if ((ci & 1) != wset) continue;
+                        uint32_t v[16];
+                        if (iters > 0) {
+                            tmem_ld16(lane_addr + (uint32_t)(tt * acc_cols + cc), v);
+                            tmem_ld_wait();
+                        } else {
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const float4 t = make_float4(__uint_as_float(v[4 * e]), __uint_as_float(v[4 * e + 1]), __uint_as_float(v[4 * e + 2]), __uint_as_float(v[4 * e + 3]));
-                        if (!here || cc + 4 * e >= p.K) break;
-                        wgrad_pair_store(p, cc + 4 * e, tap, c, t);
-                        if (wgrad_nan(t, p.K - cc - 4 * e)) bad |= 1u << e;
-                    }
-                    if (__any_sync(0xffffffffu, bad != 0u))
+                            for (int e = 0; e < 16; ++e) v[e] = 0u;
+                        }
+                        const int n = here ? min(16, p.K - cc) : 0;
+                        float *d = dst + (size_t)cc * pitch;
+                        unsigned bad = 0u;                   // a bit per four sums
+#pragma unroll
+                        for (int e = 0; e < 16; ++e, d += pitch) {
+                            const float f = __uint_as_float(v[e]);
+                            if (e < n) *d = f;
+                            if (e < n && f != f) bad |= 1u << (e >> 2);
+                        }
+                        if (__any_sync(0xffffffffu, bad != 0u))
 #pragma unroll 1
-                        for (int e = 0; e < 4; ++e) wgrad_pure(p.raw, p.out, (bad >> e) & 1u, cc + 4 * e, 1, tap, c, 0);
+                            for (int e = 0; e < 4; ++e) wgrad_pure(p.raw, p.out, (bad >> e) & 1u, cc + 4 * e, 1, tap, c, 0);
+                    }
                 }
             } else {
             float *obase = p.out;
