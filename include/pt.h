@@ -21,9 +21,9 @@
  * Physical layouts
  *   activations x, y, dy, dx : [N][H][W][ld]   bf16 (or fp32 outputs when out_f32 = 1), channels
  *                              innermost, channel pitch ld >= channels, ld a multiple of 8 elements.
- *                              Pad lanes (channel index >= channels) never affect a result, whatever they hold
- *                              (the weight gradient may load those up to the next multiple of 16 channels, into sums
- *                              that it drops; nothing else reads them). bf16 outputs may get zeros
+ *                              Pad lanes (channel index >= channels) within the pitch may be loaded (the weight
+ *                              gradients take whole sectors or whole rows of them, a stem of few channels the first
+ *                              four lanes) and never affect a result, whatever they hold. bf16 outputs may get zeros
  *                              written into the pad lanes up to the next multiple of 16 channels where the pitch has
  *                              room for them (whole 32-byte sectors are stored: a half-written sector costs a
  *                              read-modify-write in the memory system), else up to the end of the last 16-byte

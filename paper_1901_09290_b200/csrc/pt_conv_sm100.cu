@@ -8,7 +8,8 @@
 //                      position, 32-byte swizzle, one MMA per tap) runs the space-to-depth stem where conv_stem_kernel does not.
 //   conv_wgrad_kernel  weight gradient: both operands MN-major, reduction over pixels split across CTAs, partial tiles
 //                      summed in-kernel in a fixed order.
-//   conv_wgrad_taps_kernel  weight gradient by filter rows: the staged pixels of one serve all of its taps (stride 1 or 2, up to 170 channels).
+//   conv_wgrad_taps_kernel  weight gradient by filter rows: the staged pixels of one serve all of its taps (stride 1 or 2, one tile of input channels: 160 for three
+//                      columns, 256 for two, 64 for eight).
 //   conv_wgrad_packed_kernel  weight gradient of narrow stride-1 layers: several pixels to a staged row.
 //   conv_wgrad_rows_kernel  weight gradient of stride-1 layers with at most 64 input channels: row blocks of x staged
 //                      once, taps as row-shifted descriptors, two or four taps per MMA on the M side; same finish phase.
@@ -1150,9 +1151,9 @@ __global__ void __launch_bounds__(kHaloThreads, 1) conv_halo_kernel(const __grid
 //   B operand: x through the im2col map (same pixel raster as the forward pass, tap offset added by the TMA unit),
 //              c contiguous -> MN-major tiles (one 64-channel box per 64 columns).
 //   The pixel range is split across CTAs (blockIdx.y), at most one CTA per SM in total so that all of them are resident.
-//   With more than one split every CTA TMA-stores its fp32 partial tile to the workspace, announces it on a counter,
-//   waits (bounded) until all splits of its tile have arrived, and then sums its share of the tile's rows over the
-//   splits in ascending order: deterministic, and no second kernel.
+//   With more than one split every CTA stores its fp32 partial sums to the workspace from its registers, announces them on a
+//   counter, waits (bounded) until all splits of its tile have arrived, and then sums its share of them over the splits in a
+//   fixed order (wgrad_sum): deterministic, and no second kernel. Up to eight splits can meet in shared memory instead (wgrad_cluster_sum).
 constexpr int kMaxRow = 8;  // filter rows and columns of the filter-row form
 // The layer itself, for the sums that the raster forms cannot take from their accumulators (wgrad_pure).
 struct WgradRaw {
@@ -1183,10 +1184,10 @@ struct WgradP {
     int lane_shift;         // log2 of `lanes`
     int row_lanes;          // packed form: channel lanes from one pixel of dy to the next (16 or 32)
     int acc_row;            // 32 lanes: accumulators per filter row, ceil(S / 4): each holds four neighbouring taps
-    // filter-row form: the taps of one filter row share a unit; a tap is plane tap_plane[s] of the unit's x rows (stride 2: the columns of
-    // either parity are a plane each), tap_shift[s] pixels on
     struct { int C, R, S, off; } stem;      // the space-to-depth stem: channels of the image (0: not the stem) and the real filter, for dw
     int G;                  // packed form: pixels side by side in a staged row of x (64 / lanes)
+    // filter-row form: the taps of one filter row share a unit; a tap is plane tap_plane[s] of the unit's x rows (stride 2: the columns of
+    // either parity are a plane each), tap_shift[s] pixels on
     int planes;
     int plane_lo[2];                                    // first column of a unit's rows in either plane
     unsigned char tap_plane[kMaxRow], tap_shift[kMaxRow];
@@ -1645,7 +1646,7 @@ __device__ __forceinline__ void wgrad_finish(const WgradP &p, Ctl *ctl, uint32_t
     if (p.splits > 1 && !*abort_flag) {
         // ---- (3) all threads: this CTA sums its share of the tile's 16-byte pieces over the splits. The partial sums sit in L2 and what costs
         // time is a chain of dependent loads, so the asynchronous copies of the whole share, a run of every split's pieces, go out first, into
-        // the (now idle) stage memory; the copies are then summed from there in ascending split order: deterministic, whichever CTA
+        // the (now idle) stage memory; the copies are then summed from there in a fixed order (wgrad_sum): deterministic, whichever CTA
         // does the work.
         const WgradShare sh(p, k0, c0, acc_cols);
         const int total = n_acc * sh.quads * sh.rows, per_cta = (total + p.splits - 1) / p.splits;
@@ -2373,7 +2374,7 @@ StemPlan stem_plan(const pt_conv_desc *d)
     return s;
 }
 
-// Forward pass of a few-channel stride-2 stem straight from the image (U >= 2; 64 to 128 output columns, at most 128 channels, bf16 out).
+// Forward pass of a few-channel stride-2 stem straight from the image (U >= 2; 64 to 125 output columns, at most 128 channels, bf16 out).
 // A CTA has a run of consecutive output rows. Two teams of four warps turn each pair of image rows into one space-to-depth row in shared
 // memory (every one of them once: the next output row needs one new one of its U), in a ring of rows of 32-byte positions with the
 // swizzle of that width; an output row is then U x V matrix instructions on those rows (tap (u, v) starts at row u, v positions on) with the
@@ -3222,10 +3223,10 @@ pt_status launch_halo(pt_ctx *c, const pt_conv_desc *d, const HaloSpec &h, const
     p.stats_off = (int)(smem - st_smem);
     void (*kernel)(HaloMaps<PL>, CUtensorMap, CUtensorMap, HaloP) =
         (!B_MN && c->stats_mode) ? conv_halo_kernel<false, true, PL> : conv_halo_kernel<B_MN, false, PL>;
-    const int kid = PL > 1 ? (c->stats_mode ? 13 : 12) : (!B_MN && c->stats_mode) ? 2 : (B_MN ? 1 : 0);
-    if (!(c->attr_done & (kAttrHalo << kid))) {
+    const unsigned attr = PL > 1 ? kAttrPlanes << (c->stats_mode ? 1 : 0) : kAttrHalo << ((!B_MN && c->stats_mode) ? 2 : (B_MN ? 1 : 0));
+    if (!(c->attr_done & attr)) {
         PT_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-        c->attr_done |= kAttrHalo << kid;
+        c->attr_done |= attr;
     }
     const int total_tiles = p.N * p.row_tiles * p.n_tiles;
     int grid = total_tiles < c->sm_count ? total_tiles : c->sm_count;
@@ -3277,6 +3278,9 @@ void halo_spec_stride1(const pt_conv_desc *d, HaloSpec *h, const void *src, int 
 // frees only after a CTA that cannot start has arrived), so a split launch asks for more than half of an SM's shared
 // memory: at most one of them per SM, whatever else runs beside it (kernels that wait for nobody always finish).
 constexpr size_t kSplitSmemFloor = 116 * 1024;
+// The least that a weight gradient has behind its control block: the squares that its epilogue transposes (34 KB) and the sums of the splits reuse
+// the stages.
+constexpr size_t kWgradSmemMin = 2048 + 8 * 2 * 4096;
 
 // Launches the stem's forward kernel; PT_ERR_UNSUPPORTED where the space-to-depth copy serves the layer.
 pt_status run_stem(pt_ctx *c, const pt_conv_desc *d, const StemPlan &sp, const void *x, const void *w, void *y, cudaStream_t st)
@@ -3538,7 +3542,7 @@ double wgrad_rows_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, pt_
     if (w->splits < 2) w->cluster = 0;
     if (w->stages > w->units_per_split && w->units_per_split >= 2) w->stages = w->units_per_split;
     w->smem = 2048 + (size_t)w->stages * w->stage_bytes;
-    if (w->smem < 2048 + 8 * 2 * 4096) w->smem = 2048 + 8 * 2 * 4096;    // the epilogue's staging slabs reuse the ring
+    if (w->smem < kWgradSmemMin) w->smem = kWgradSmemMin;
     w->rows = 1;
     return best_us;
 }
@@ -3557,7 +3561,7 @@ bool wgrad_taps_ok(const pt_conv_desc *d)
     return d->S >= 2 && d->S <= kMaxRow && d->R <= kMaxRow && (d->stride == 1 || d->stride == 2) && d->pad <= 64 && d->H >= d->stride && d->W >= d->stride;
 }
 
-// The filter-row kernel; false where it does not apply.
+// The filter-row kernel: the estimated time, 1e30 where it does not apply.
 double wgrad_taps_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, pt_wgrad_plan *w)
 {
     memset(w, 0, sizeof(*w));
@@ -3602,7 +3606,7 @@ double wgrad_taps_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, pt_
     if (w->splits < 2) w->cluster = 0;
     if (w->stages > w->units_per_split && w->units_per_split >= 2) w->stages = w->units_per_split;
     w->smem = 2048 + (size_t)w->stages * w->stage_bytes;
-    if (w->smem < 2048 + 8 * 2 * 4096) w->smem = 2048 + 8 * 2 * 4096;    // the epilogue's staging slabs reuse the ring
+    if (w->smem < kWgradSmemMin) w->smem = kWgradSmemMin;
     w->filter_row = 1;
     return best;
 }
@@ -3658,7 +3662,7 @@ double wgrad_packed_plan(const pt_ctx *c, const pt_conv_desc *d, int P, int Q, p
     if (w->nr == 0) return 1e30;
     if (w->stages > w->units_per_split && w->units_per_split >= 2) w->stages = w->units_per_split;
     w->smem = 2048 + (size_t)w->stages * w->stage_bytes;
-    if (w->smem < 2048 + 8 * 2 * 4096) w->smem = 2048 + 8 * 2 * 4096;
+    if (w->smem < kWgradSmemMin) w->smem = kWgradSmemMin;
     w->packed = 1;
     return best;
 }
@@ -3869,7 +3873,7 @@ pt_status run_wgrad(pt_ctx *c, const pt_conv_desc *d, int P, int Q, const pt_wgr
     size_t smem = 0;
     const size_t stage = 2 * 8192 + (size_t)p.tpc * pt_ceil_div(p.BN, 64) * 8192;
     p.stages = pick_stages(stage, pt_ceil_div(p.pix_per_split, 64), 0, &smem);
-    if (smem < 2048 + 8 * 2 * 4096) smem = 2048 + 8 * 2 * 4096;        // the epilogue's staging slabs reuse the stage memory
+    if (smem < kWgradSmemMin) smem = kWgradSmemMin;
     if (p.splits > 1 && smem < kSplitSmemFloor) smem = kSplitSmemFloor;
     dim3 grid((unsigned)gx, (unsigned)p.splits);
     p.data_bytes = (unsigned)(smem - 2048);

@@ -50,8 +50,7 @@ struct pt_group_slot {
 // Kernels whose opt-in to more than 48 KB of dynamic shared memory a context has set (pt_ctx::attr_done). The attribute belongs to a
 // device, so it is remembered per context and not per process; setting it twice does no harm.
 enum : unsigned { kAttrGemm = 1u << 0 /* four variants */, kAttrHalo = 1u << 4 /* three */, kAttrWgrad = 1u << 7, kAttrBn = 1u << 8 /* four */,
-                  kAttrGate = 1u << 12 /* three */, kAttrStem = 1u << 15,
-                  kAttrPlanes = kAttrHalo << 12 /* two */ };
+                  kAttrGate = 1u << 12 /* three */, kAttrStem = 1u << 15, kAttrPlanes = 1u << 16 /* two */ };
 
 // Launch shape of a weight gradient. rows = 1: the row-block kernel (stride-1 filters with at most 64 input channels).
 struct pt_wgrad_plan {

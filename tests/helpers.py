@@ -16,7 +16,8 @@ def ctx():
 
 
 def to_dev_padded(t: torch.Tensor, ld: int, dtype=torch.bfloat16, fill=float("nan")) -> torch.Tensor:
-    """[..., C] fp32 host tensor -> [..., ld] device tensor; pad lanes hold `fill` (they must never be read)."""
+    """[..., C] fp32 host tensor -> [..., ld] device tensor; pad lanes hold `fill` (they may be loaded and must not
+    affect a result)."""
     C = t.shape[-1]
     out = torch.full(tuple(t.shape[:-1]) + (ld,), fill, dtype=torch.float32)
     out[..., :C] = t
@@ -48,7 +49,7 @@ def check_conv(out_dev: torch.Tensor, C: int, ref: np.ndarray, canary=7680.0, wh
     got = out_dev.float().cpu().numpy().astype(np.float64)
     if got.shape[-1] > C:
         pad = got[..., C:]
-        # pad lanes are never read; the TMA-store epilogue may zero those sharing the last 16-byte granule
+        # the TMA-store epilogue may zero pad lanes: those of the last sector, or of the last 16-byte granule
         assert np.all((pad == canary) | (pad == 0)), what + ": pad lanes hold something other than the canary or zero"
     got = got[..., :C]
     assert got.shape == ref.shape, (got.shape, ref.shape)
